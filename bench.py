@@ -53,6 +53,7 @@ PROFILES = {
                                    "paper_2607_01735_gb300/csrc/fp64.cuh"]),
 }
 PERSIST_MIN_N, PERSIST_MAX_N = 416, 1 << 15
+FUSED_WAVE_MIN_N = 512
 # side files of a run (nvidia-smi clock samples, trained U-Net parameters)
 OUT_DIR = os.environ.get("RBGS_BENCH_OUT", os.path.join(ROOT, "bench_out"))
 
@@ -186,8 +187,14 @@ def resolved_kernel(n, refine, kernel, tblock_k):
     if tblock_k:
         return 1, 1
     if refine:
-        return (3, 4) if n > 2048 else (1, 1)
+        return (3, 4) if n > 1000 else (1, 1)
     return 1, 1
+
+
+def fused_wavefront(args, n):
+    """The fused sweeps run as register-wavefront passes of up to 3 sweeps (the library's rule:
+    AUTO, no launch-shape option, FUSED_WAVE_MIN_N <= n)."""
+    return args.kernel == 0 and args.tile_rows == 0 and args.values == 0 and n >= FUSED_WAVE_MIN_N
 
 
 def device_peaks(dev):
@@ -994,7 +1001,7 @@ def main():
 
         kernel, kdepth = resolved_kernel(n, refine, args.kernel, args.tblock_k)
         if fma:
-            kernel, kdepth = 1, 1
+            kernel, kdepth = (3, 3) if fused_wavefront(margs, n) else (1, 1)
         blocked = kernel in (2, 3)  # several sweeps per launch (TMA tiles or register wavefront)
         persistent = uses_persistent(margs, n, refine)
         # pack f, pack u, ||b|| (2), the sweeps, residual, unpack.  The residual after
@@ -1002,7 +1009,9 @@ def main():
         # zero), else both colours (3)
         resid = 2 if sweeps > 0 and not fma else 3
         if fma:  # + max |h2 f| at load; per block of <= 1024 sweeps: max |u|, h2 f onto the grid
-            launches_per_step = 4 + 1 + 2 * -(-sweeps // 1024) + 2 * sweeps + resid + 1
+            blocks = [1024] * (sweeps // 1024) + ([sweeps % 1024] if sweeps % 1024 else [])
+            passes = sum(-(-m // 3) if blocked and m >= 4 else 2 * m for m in blocks)
+            launches_per_step = 4 + 1 + 2 * len(blocks) + passes + resid + 1
         elif refine:
             inner = args.inner or 100
             outer = -(-sweeps // inner)
@@ -1061,21 +1070,24 @@ def main():
                         "note": "per launch equivalent (a half-sweep, or a blocked pass), including the "
                                 "FP64 defect/correction passes in the time"}
         elif fma:
-            # dominant kernel: the fused half-sweep (integer arithmetic only), bound by HBM: 24
-            # algorithmic bytes per update (h2 f on the fixed-point grid, the other colour, the
-            # own colour written).  Per launch: half the points; the time includes the
-            # rescaling passes of each block of sweeps (max |u|, h2 f onto the grid).
-            launches = 2 * sweeps
-            kname = "fused_half_sweep"
+            # dominant kernel: a wavefront pass of 3 sweeps (integer arithmetic only; 16 bytes
+            # per point: h2 f on the fixed-point grid, the black values in and out) or the fused
+            # half-sweep (24 bytes per update: h2 f, the other colour, the own colour written).
+            # The time includes the rescaling passes of each block of sweeps (max |u|, h2 f onto
+            # the grid).
+            launches = -(-sweeps // 3) if blocked else 2 * sweeps
+            kname = "wavefront_kernel<int64, 3>" if blocked else "fused_half_sweep"
             launch_s = sweep_s / (launches * args.steps)
-            alg_bytes = BYTES_PER_LUP * n * n / 2.0
+            alg_bytes = 16.0 * n * n if blocked else BYTES_PER_LUP * n * n / 2.0
             achieved = alg_bytes / launch_s / 1e9
             roofline = {"bound": "hbm", "achieved": achieved, "peak": peak_hbm, "unit": "GB/s",
                         "frac": achieved / peak_hbm, "traffic": profiled_traffic(kname, args.emulate),
                         "kernel": kname, "peak_source": hbm_src, "launch_ms": 1e3 * launch_s,
                         "algorithmic_bytes_per_launch": alg_bytes,
-                        "note": "per half-sweep; the sweeps' device time includes the per-block rescaling "
-                                "passes (max |u|, h2 f onto the fixed-point grid)"}
+                        "note": ("per pass of 3 sweeps, bound by the integer ALU pipe (72% busy under ncu), not "
+                                 "by HBM" if blocked else "per half-sweep") +
+                                "; the sweeps' device time includes the per-block rescaling passes (max |u|, "
+                                "h2 f onto the fixed-point grid)"}
         else:
             # dominant kernel: the FP64 half-sweep, bound by the FP64 pipe: 4 correctly rounded
             # adds per update (the x0.25 runs on the integer pipe).  Peak: 2 FP64 instructions

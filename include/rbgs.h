@@ -70,7 +70,7 @@ typedef enum {
 typedef enum {
     RBGS_KERNEL_AUTO = 0,     /* FP64 sweeps: PERSISTENT for 416 <= n <= 32768 with the default
                                  launch-shape options, else COLOUR.  FP32 inner sweeps of
-                                 RBGS_FP32_REFINE: WAVEFRONT (depth 4) when n > 2048 and
+                                 RBGS_FP32_REFINE: WAVEFRONT (depth 4) when n > 1000 and
                                  tblock_k = 0, else COLOUR                                   */
     RBGS_KERNEL_COLOUR = 1,   /* one launch per colour (half-sweep kernels)               */
     RBGS_KERNEL_TEMPORAL = 2, /* several sweeps per shared-memory tile, halo recompute      */
@@ -112,8 +112,10 @@ typedef struct {
                             Integer arithmetic only, so the update leaves the FP64 pipe.  Agrees
                             with the bit-exact iterate to <= 1e-13 relative max-norm after the same
                             sweeps (the tolerance set for this mode); a non-finite value in u or h2 f makes
-                            that block of sweeps run the bit-exact update.  One launch per colour
-                            (the kernel option does not apply)                                   */
+                            that block of sweeps run the bit-exact update.  With kernel AUTO and
+                            no launch-shape option, register-wavefront passes from 512^2 on (two
+                            more FP64 arrays of half the grid each; without room for them, and
+                            otherwise, one launch per colour).  The same bits either way          */
     int stall_checks;  /* rbgs_solve and rbgs_solve_batched stop a problem with RBGS_ENOTCONV when
                           its residual has not reached a new minimum for this many consecutive
                           checks (0: 64; -1: never), so a tolerance below the rounding floor

@@ -47,6 +47,12 @@ constexpr int kPersistMaxN = 1 << 15;
 // max |u| + (sweeps) max |h2 f| / 2 a priori, so shorter blocks keep it tighter; the
 // rescaling pass (max |u|, h2 f onto the grid: about one sweep's traffic) repeats per block.
 constexpr long kFusedChunk = 1024;
+// Fused sweeps as register-wavefront passes (wavefront.cu) from this size on.  Measured per
+// sweep against cached graphs of one launch per colour: 5.6 against 4.4 us at 255^2, 5.7 / 5.8
+// at 511^2, 7.2 / 13.1 at 1023^2, 9.9 / 16.2 at 1500^2, 31 / 96 at 4095^2, 382 / 1021 at
+// 16384^2.
+constexpr int kFusedWaveMinN = 512;
+constexpr int kWave32MinN = 1001;    // FP32 inner sweeps as wavefront passes from this size on
 // Residual checks without a new minimum of rho after which a solve stops (opts.stall_checks 0).
 constexpr int kDefaultStallChecks = 64;
 
@@ -89,6 +95,9 @@ rbgs_status enqueue_pack(rbgs_ctx *c, const double *f_view, const double *u_view
     rbgs_status st;
     if (f_view && (st = launch_pack_f(g, c->h2, f_view, c->f64.hf[0], c->f64.hf[1], c->stream)) != RBGS_OK) return st;
     if ((st = launch_pack_u(g, u_view, c->f64.u[0], c->f64.u[1], c->stream)) != RBGS_OK) return st;
+    if (c->kernel == RBGS_KERNEL_WAVEFRONT &&
+        (st = launch_ring_to_rhs(g, c->f64.u[0], c->f64.u[1], c->f64.hf[0], c->f64.hf[1], c->stream)) != RBGS_OK)
+        return st;
     if (f_view && c->fused && (st = launch_fused_rhs_max(c, c->stream)) != RBGS_OK) return st;
     // ||h^2 b||^2 depends on f and the ring
     return launch_rhs_norm(c, c->stream);
@@ -128,6 +137,8 @@ void free_ctx(rbgs_ctx *c) {
     cudaFree(c->hq[0]);
     cudaFree(c->hq[1]);
     cudaFree(c->fwords);
+    cudaFree(c->tq[0]);
+    cudaFree(c->tq[1]);
     for (int q = 0; q < 2; ++q) {
         cudaFree(c->sin_f[q]);
         cudaFree(c->sin_u[q]);
@@ -216,10 +227,8 @@ rbgs_status enqueue_sweeps(rbgs_ctx *c, long nsweeps, cudaStream_t s) {
     if (c->kernel == RBGS_KERNEL_TEMPORAL) return launch_temporal_sweeps(c, nsweeps, s);
     if (c->kernel == RBGS_KERNEL_WAVEFRONT) {
         const long passes = nsweeps / c->tblock_k;
-        for (long q = 0; q < passes; ++q) {
-            rbgs_status st = launch_wavefront_pass<double>(c->f64, c->tblock_k, s);
-            if (st != RBGS_OK) return st;
-        }
+        const rbgs_status st = launch_wavefront_passes<double>(c->f64, c->tblock_k, passes, s);
+        if (st != RBGS_OK) return st;
         nsweeps -= passes * c->tblock_k;
     }
     return launch_sweeps_f64(c, nsweeps, s);
@@ -262,6 +271,10 @@ rbgs_status sweeps_f64(rbgs_ctx *c, long nsweeps) {
             nsweeps -= m;
             rbgs_status st = launch_fused_prepare(c, m, c->stream);
             if (st != RBGS_OK) return st;
+            if (c->tq[0] && m >= kFusedWaveMin) {
+                if ((st = launch_fused_wave_sweeps(c, m, c->stream)) != RBGS_OK) return st;
+                continue;
+            }
             if (m >= kGraphSweeps) {
                 if ((st = ensure_graph(c)) != RBGS_OK) return st;
                 while (m >= c->graph_sweeps) {
@@ -335,11 +348,14 @@ rbgs_status inner_sweeps_f32(rbgs_ctx *c, long m) {
     if (c->kernel32 == RBGS_KERNEL_TEMPORAL || c->kernel32 == RBGS_KERNEL_WAVEFRONT) {
         const int k = c->tblock_k32;
         const long passes = m / k;
-        for (long q = 0; q < passes; ++q) {
-            rbgs_status st = c->kernel32 == RBGS_KERNEL_TEMPORAL
-                                 ? launch_temporal_pass<float>(c->f32, k, c->dstatus, c->stream)
-                                 : launch_wavefront_pass<float>(c->f32, k, c->stream);
+        if (c->kernel32 == RBGS_KERNEL_WAVEFRONT) {
+            const rbgs_status st = launch_wavefront_passes<float>(c->f32, k, passes, c->stream);
             if (st != RBGS_OK) return st;
+        } else {
+            for (long q = 0; q < passes; ++q) {
+                const rbgs_status st = launch_temporal_pass<float>(c->f32, k, c->dstatus, c->stream);
+                if (st != RBGS_OK) return st;
+            }
         }
         m -= passes * k;
     }
@@ -522,8 +538,9 @@ rbgs_status rbgs_create(int n, double h2, const double *f, const double *u_init,
     // 416^2 to 32768^2 with the default launch shape (1.15x at 511^2 to 1.53x at 2047^2 and
     // 1.10x at 16383^2 over one launch per colour), else one launch per colour with cached
     // graphs (the register wavefront reaches the same FP64-pipe limit, with overlap work on
-    // top); the FP32 inner sweeps of the refinement run the register wavefront above 2048^2
-    // (1.6x) and one launch per colour (with graphs) on smaller grids
+    // top); the FP32 inner sweeps of the refinement run the register wavefront above 1000^2
+    // (a sweep at depth 4 against one launch per colour: 4.1 / 3.5 us at 700^2, 4.2 / 5.0 at
+    // 1023^2, 6.2 / 10 at 2047^2) and one launch per colour (with graphs) on smaller grids
     const bool auto_k = o.kernel == RBGS_KERNEL_AUTO && o.tblock_k == 0;
     const bool default_shape = o.fp64_emulate == -1 && o.int_rows <= 0 && (o.sweep_values == 0 || o.sweep_values == 2) &&
                                (o.sweep_rows == 0 || o.sweep_rows == 1) && o.tile_rows == 0;
@@ -555,8 +572,8 @@ rbgs_status rbgs_create(int n, double h2, const double *f, const double *u_init,
     // FP64 sweeps: temporal depth (used when kernel == TEMPORAL)
     c->tblock_k = (o.precision == RBGS_FP64 && o.tblock_k) ? o.tblock_k : 2;
     // FP32 inner sweeps of the refinement (the TMA-tiled temporal kernel measured slower
-    // than one launch per colour on GB300; the register wavefront faster above 2048^2)
-    c->kernel32 = o.kernel == RBGS_KERNEL_AUTO ? ((auto_k && n > 2048) ? RBGS_KERNEL_WAVEFRONT
+    // than one launch per colour on GB300; the register wavefront faster on large grids)
+    c->kernel32 = o.kernel == RBGS_KERNEL_AUTO ? ((auto_k && n >= kWave32MinN) ? RBGS_KERNEL_WAVEFRONT
                                                                        : RBGS_KERNEL_COLOUR)
                   : o.kernel == RBGS_KERNEL_PERSISTENT ? RBGS_KERNEL_COLOUR
                                                         : o.kernel;
@@ -583,6 +600,16 @@ rbgs_status rbgs_create(int n, double h2, const double *f, const double *u_init,
     ok = ok && cudaMallocHost(&c->hstatus, sizeof(int)) == cudaSuccess;
     for (int q = 0; q < 2 && ok && c->fused; ++q) ok = cudaMalloc(&c->hq[q], c->g.colour_elems() * sizeof(int64_t)) == cudaSuccess;
     ok = ok && (!c->fused || cudaMalloc(&c->fwords, 3 * sizeof(unsigned long long)) == cudaSuccess);
+    // the wavefront's buffers; without room for them the half-sweeps run one launch per colour
+    if (ok && c->fused && o.kernel == RBGS_KERNEL_AUTO && o.tile_rows == 0 && o.sweep_values == 0 &&
+        n >= kFusedWaveMinN) {
+        const size_t qbytes = c->g.colour_elems() * sizeof(int64_t);
+        if (cudaMalloc(&c->tq[0], qbytes) != cudaSuccess || cudaMalloc(&c->tq[1], qbytes) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(c->tq[0]);
+            c->tq[0] = c->tq[1] = nullptr;
+        }
+    }
     ok = ok && cudaMemsetAsync(c->dstatus, 0, sizeof(int), c->stream) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();

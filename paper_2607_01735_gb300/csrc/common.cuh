@@ -111,6 +111,9 @@ struct rbgs_ctx {
     bool fused;
     int64_t *hq[2];
     unsigned long long *fwords;
+    // fused wavefront (wavefront.cu): the black values on the fixed-point grid between passes,
+    // two buffers; NULL when the half-sweeps run one launch per colour
+    int64_t *tq[2];
     // rbgs_run_stream: double-buffered natural-layout device staging of the inputs (f, u) and
     // of the solution, one copy stream per direction, their events, and per-problem sums
     double *sin_f[2], *sin_u[2], *sout[2];
@@ -129,6 +132,8 @@ rbgs_status launch_pack_f(const Geometry &g, double h2, const double *f_nat, dou
                           double *hf_black, cudaStream_t s);
 rbgs_status launch_unpack_u(const Geometry &g, const double *red, const double *black,
                             double *u_nat, cudaStream_t s);
+rbgs_status launch_ring_to_rhs(const Geometry &g, const double *red, const double *black, double *hf_red,
+                               double *hf_black, cudaStream_t s);
 rbgs_status launch_half_sweep(const rbgs_ctx *c, int colour, cudaStream_t s);
 rbgs_status launch_sweeps_f64(const rbgs_ctx *c, long nsweeps, cudaStream_t s);
 rbgs_status launch_residual_sum(const rbgs_ctx *c, cudaStream_t s);   // -> dsum[0]
@@ -137,9 +142,10 @@ rbgs_status launch_temporal_sweeps(rbgs_ctx *c, long nsweeps, cudaStream_t s);
 template <typename T>
 rbgs_status launch_temporal_pass(ColourField<T> &fld, int k, int *status, cudaStream_t s);
 rbgs_status launch_sweeps_f32(const ColourField<float> &fld, long nsweeps, cudaStream_t s);
-// one register-wavefront pass of k sweeps from fld.u into fld.alt, then swaps them (wavefront.cu)
+// register-wavefront passes of k sweeps each between fld.u and fld.alt, which are swapped so
+// that the result is in fld.u (wavefront.cu)
 template <typename T>
-rbgs_status launch_wavefront_pass(ColourField<T> &fld, int k, cudaStream_t s);
+rbgs_status launch_wavefront_passes(ColourField<T> &fld, int k, long passes, cudaStream_t s);
 // nsweeps FP64 sweeps of fld in cooperative launches with a bounded grid barrier between
 // the colours (persistent.cu); a barrier that gives up sets *status
 template <typename T>
@@ -157,5 +163,8 @@ rbgs_status launch_correct(const rbgs_ctx *c, double scale, cudaStream_t s);
 rbgs_status launch_fused_rhs_max(const rbgs_ctx *c, cudaStream_t s);
 rbgs_status launch_fused_prepare(const rbgs_ctx *c, long long nsweeps, cudaStream_t s);
 rbgs_status launch_fused_half_sweep(const rbgs_ctx *c, int colour, cudaStream_t s);
+// nsweeps (>= kFusedWaveMin) fused sweeps at that scale in register-wavefront passes (wavefront.cu)
+constexpr long kFusedWaveMin = 4;
+rbgs_status launch_fused_wave_sweeps(const rbgs_ctx *c, long nsweeps, cudaStream_t s);
 
 }  // namespace rbgs

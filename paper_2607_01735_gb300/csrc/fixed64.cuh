@@ -58,6 +58,33 @@ __host__ __device__ __forceinline__ double fixed_quarter_to_double(int64_t s, in
     return a ? bitsd(bits) : 0.0;
 }
 
+// to_fixed(fixed_quarter_to_double(s, e), e) without leaving the integers, for |s| < 2^61:
+// trunc(RN53(s) / 4), where RN53 rounds an integer to 53 significant bits, half to even.
+// The number q of bits below the 53 follows from the position of the first bit that differs
+// from the sign (RN53 leaves an exact power of two as it is, so counting a negative s by
+// ~s instead of -s changes nothing).  Half to even on two's complement is the usual
+// s + (2^(q-1) - 1) + (bit q of s), low q bits dropped.  The truncated division adds 3 to a
+// negative value before the shift; where q = 1 the dropped low bit leaves 2 of the 3, and
+// from q = 2 the value is a multiple of 4: the bias is 3 with the low q bits dropped.  All of
+// it is one 64-bit add of at most 2^8 and 12 further 32-bit operations, against about 60 for
+// the way through binary64.
+__host__ __device__ __forceinline__ int64_t fixed_quarter(int64_t s) {
+    const int hi = (int)(s >> 32);
+    const uint32_t lo = (uint32_t)s;
+#if defined(__CUDA_ARCH__)
+    int top;  // highest bit of hi that differs from its sign, -1 when none does
+    asm("bfind.s32 %0, %1;" : "=r"(top) : "r"(hi));
+#else
+    const uint32_t hx = (uint32_t)(hi ^ (hi >> 31));
+    const int top = hx ? 31 - __builtin_clz(hx) : -1;
+#endif
+    const int q = top > 20 ? top - 20 : 0;  // at most 8
+    const uint32_t m = (1u << q) - 1u;
+    const uint32_t c = (m >> 1) + ((lo >> q) & m & 1u) + (((uint32_t)hi >> 30) & ~m);
+    const uint64_t x = (uint64_t)s + c;
+    return (int64_t)((x & 0xFFFFFFFF00000000ull) | ((uint32_t)x & ~m)) >> 2;
+}
+
 // Scale of one block of nsweeps fused sweeps.  B = max |u| over the whole grid (ring
 // included) and Q = max |h2 f| when the block starts.  An update changes no value by more
 // than Q/4 beyond the largest neighbour, so after t sweeps every |u| <= B + t Q / 2 and

@@ -15,12 +15,14 @@
 //   2. prepare_kernel: e = scale_exponent(B, Q, sweeps of the block) into words[2] (or
 //      kNoScale); h2 f of both colours converted once to the fixed-point grid (hq, int64),
 //      so the sweeps read it as is;
-//   3. the block's sweeps: per colour one launch of fused_half_sweep.
+//   3. the block's sweeps: register-wavefront passes of 2 or 3 sweeps (wavefront.cu) from
+//      512^2 on, else, or with a launch-shape option, one launch of fused_half_sweep per
+//      colour.
 // A non-finite B or Q (a NaN or Inf in the iterate or in f) leaves no valid scale: the
 // block's half-sweeps then write NaN to every point they update, so the next residual
 // reports RBGS_ENONFINITE.
 //
-// Work decomposition of a half-sweep: that of the bit-exact strip kernel (sweep.cu).  A
+// Work decomposition of fused_half_sweep: that of the bit-exact strip kernel (sweep.cu).  A
 // thread owns PTS neighbouring values of its colour row and walks down a strip of rows
 // with the other colour's rows i-1, i, i+1 in registers, here already converted to the
 // fixed-point grid, so each value of the other colour is converted once per strip; the
@@ -75,18 +77,34 @@ absmax_kernel(const double *__restrict__ a0, const double *__restrict__ a1, size
     }
 }
 
-// h2 f of both colours on the block's fixed-point grid (nothing to do without a scale).
+// h2 f of both colours on the block's fixed-point grid (nothing to do without a scale).  The
+// ring places, where h2 f is zero and no update reads it, take the ring's values of u on the
+// grid: the wavefront passes (wavefront.cu) read them there.  Element k of colour c in row i is
+// column 2k + ((i + c) & 1).
 __global__ void __launch_bounds__(kMaxThreads)
-prepare_kernel(const double *__restrict__ hf0, const double *__restrict__ hf1, int64_t *__restrict__ hq0,
-               int64_t *__restrict__ hq1, size_t count, unsigned long long *__restrict__ words,
-               long long nsweeps) {
+prepare_kernel(const double *__restrict__ hf0, const double *__restrict__ hf1, const double *__restrict__ u0,
+               const double *__restrict__ u1, int64_t *__restrict__ hq0, int64_t *__restrict__ hq1, int n, int W,
+               unsigned long long *__restrict__ words, long long nsweeps) {
     int e = 0;
     const bool ok = scale_exponent(bitsd(words[0]), bitsd(words[1]), nsweeps, &e);
-    if (blockIdx.x == 0 && threadIdx.x == 0) words[2] = ok ? (unsigned long long)(long long)e : kNoScale;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+        words[2] = ok ? (unsigned long long)(long long)e : kNoScale;
     if (!ok) return;
-    for (size_t q = (size_t)blockIdx.x * kMaxThreads + threadIdx.x; q < count; q += (size_t)gridDim.x * kMaxThreads) {
-        hq0[q] = to_fixed(__ldg(hf0 + q), e);
-        hq1[q] = to_fixed(__ldg(hf1 + q), e);
+    const int k = 2 * (blockIdx.x * kMaxThreads + threadIdx.x);
+    if (k >= W) return;
+    for (int i = blockIdx.y; i < n + 2; i += gridDim.y) {
+        const size_t q = (size_t)i * W + k;
+        double2 a = ldg2(hf0 + q), b = ldg2(hf1 + q);
+        const int p0 = i & 1, p1 = p0 ^ 1;  // column offsets of red and black in this row
+        const bool row = i == 0 || i == n + 1;
+        if (row || k == 0 || 2 * k + 3 >= n + 1) {
+            if (row || 2 * k + p0 == 0 || 2 * k + p0 == n + 1) a.x = u0[q];
+            if (row || 2 * k + 2 + p0 == n + 1) a.y = u0[q + 1];
+            if (row || 2 * k + p1 == 0 || 2 * k + p1 == n + 1) b.x = u1[q];
+            if (row || 2 * k + 2 + p1 == n + 1) b.y = u1[q + 1];
+        }
+        *reinterpret_cast<longlong2 *>(hq0 + q) = make_longlong2(to_fixed(a.x, e), to_fixed(a.y, e));
+        *reinterpret_cast<longlong2 *>(hq1 + q) = make_longlong2(to_fixed(b.x, e), to_fixed(b.y, e));
     }
 }
 
@@ -218,8 +236,10 @@ rbgs_status launch_fused_prepare(const rbgs_ctx *c, long long nsweeps, cudaStrea
     const int grid = reduce_grid(count);
     absmax_kernel<<<grid, kMaxThreads, 0, s>>>(c->f64.u[0], c->f64.u[1], count, c->fwords);
     RBGS_LAUNCH_CHECK();
-    prepare_kernel<<<grid, kMaxThreads, 0, s>>>(c->f64.hf[0], c->f64.hf[1], c->hq[0], c->hq[1], count, c->fwords,
-                                                nsweeps);
+    const Geometry &g = c->g;
+    const dim3 pgrid((g.W / 2 + kMaxThreads - 1) / kMaxThreads, g.rows < 65535 ? g.rows : 65535);
+    prepare_kernel<<<pgrid, kMaxThreads, 0, s>>>(c->f64.hf[0], c->f64.hf[1], c->f64.u[0], c->f64.u[1], c->hq[0],
+                                                 c->hq[1], g.n, g.W, c->fwords, nsweeps);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }

@@ -61,6 +61,22 @@ __global__ void unpack_u_kernel(const double *__restrict__ red, const double *__
     }
 }
 
+// The ring's values of u into the ring places of the right-hand side (zero after packing; no
+// update or norm reads them there), where the wavefront passes take them (wavefront.cu).
+__global__ void ring_to_rhs_kernel(const double *__restrict__ red, const double *__restrict__ black,
+                                   double *__restrict__ hf_red, double *__restrict__ hf_black, int n, int W) {
+    const int q = blockIdx.x * kThreads + threadIdx.x;  // place along the four sides
+    const int side = blockIdx.y;
+    if (q > n + 1) return;
+    const int i = side == 0 ? 0 : side == 1 ? n + 1 : q;
+    const int j = side == 2 ? 0 : side == 3 ? n + 1 : q;
+    const size_t at = (size_t)i * W + (j >> 1);
+    if ((i + j) & 1)
+        hf_black[at] = black[at];
+    else
+        hf_red[at] = red[at];
+}
+
 dim3 layout_grid(const Geometry &g) {
     int gy = g.rows < 65535 ? g.rows : 65535;
     return dim3((g.W + kThreads - 1) / kThreads, gy);
@@ -78,6 +94,14 @@ rbgs_status launch_pack_u(const Geometry &g, const double *u_nat, double *red, d
 rbgs_status launch_pack_f(const Geometry &g, double h2, const double *f_nat, double *hf_red,
                           double *hf_black, cudaStream_t s) {
     pack_f_kernel<<<layout_grid(g), kThreads, 0, s>>>(f_nat, h2, hf_red, hf_black, g.n, g.W);
+    RBGS_LAUNCH_CHECK();
+    return RBGS_OK;
+}
+
+rbgs_status launch_ring_to_rhs(const Geometry &g, const double *red, const double *black, double *hf_red,
+                               double *hf_black, cudaStream_t s) {
+    ring_to_rhs_kernel<<<dim3((g.rows + kThreads - 1) / kThreads, 4), kThreads, 0, s>>>(red, black, hf_red, hf_black,
+                                                                                        g.n, g.W);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }

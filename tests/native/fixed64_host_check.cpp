@@ -15,6 +15,10 @@ void check_fixed_quarter(long n, const long long *s, const int *e, double *out) 
     for (long q = 0; q < n; ++q) out[q] = rbgs::fixed_quarter_to_double((int64_t)s[q], e[q]);
 }
 
+void check_fixed_quarter_int(long n, const long long *s, long long *out) {
+    for (long q = 0; q < n; ++q) out[q] = (long long)rbgs::fixed_quarter((int64_t)s[q]);
+}
+
 // e, or -100000 when scale_exponent reports a non-finite bound
 void check_scale_exponent(long n, const double *B, const double *Q, const long long *sweeps, int *out) {
     for (long q = 0; q < n; ++q) {

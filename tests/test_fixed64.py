@@ -42,6 +42,7 @@ def lib():
     vp = ctypes.c_void_p
     l.check_to_fixed.argtypes = [ctypes.c_long, vp, vp, vp]
     l.check_fixed_quarter.argtypes = [ctypes.c_long, vp, vp, vp]
+    l.check_fixed_quarter_int.argtypes = [ctypes.c_long, vp, vp]
     l.check_scale_exponent.argtypes = [ctypes.c_long, vp, vp, vp, vp]
     return l
 
@@ -114,6 +115,27 @@ def test_fixed_quarter_rounds_once_to_nearest_even():
     # zero is +0, and no nonzero result is subnormal for e <= 1020
     assert _quarter(lib_, np.array([0], np.int64), 7)[0].hex() == "0x0.0p+0"
     assert np.all((got == 0) | (np.abs(got) >= 2.2250738585072014e-308))
+
+
+def test_fixed_quarter_stays_on_the_grid():
+    """fixed_quarter(s) = to_fixed(fixed_quarter_to_double(s, e), e): random magnitudes below
+    2^61, ties and near-ties at every rounding position, powers of two and their neighbours."""
+    lib_ = pytest.lib_fixed
+    rng = np.random.default_rng(5)
+    mags = [rng.integers(0, 1 << 61, 200000, dtype=np.int64) >> rng.integers(0, 61, 200000)]
+    for L in range(54, 62):
+        keep = rng.integers(1 << 52, 1 << 53, 4000, dtype=np.int64) << (L - 53)
+        for low in (0, 1, (1 << (L - 54)) - 1, 1 << (L - 54), (1 << (L - 54)) + 1, (1 << (L - 53)) - 1):
+            mags.append(keep + low)
+    for b in range(61):
+        mags.append(np.arange(-600, 600, dtype=np.int64) + (1 << b))
+    a = np.concatenate(mags)
+    a = a[(a >= 0) & (a < 1 << 61)]
+    s = np.concatenate([a, -a])
+    got = np.empty_like(s)
+    lib_.check_fixed_quarter_int(s.size, s.ctypes.data, got.ctypes.data)
+    for e in (-40, 0, 59, 1020):
+        assert np.array_equal(got, _to_fixed(lib_, _quarter(lib_, s, e), e))
 
 
 def test_scale_exponent_bounds_every_sum_below_2_61():

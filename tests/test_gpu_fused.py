@@ -207,3 +207,39 @@ def test_fused_full_size_16384_sampled():
         oracle.sweeps(up, fw, h2, sweeps, parity)
         want = up[i - a + 1, j - c + 1]
         assert abs(got - want) <= TOL * float(np.max(np.abs(up))), (i, j, got, want)
+
+
+@pytest.mark.parametrize("sweeps", [4, 5, 6, 7, 8, 9, 11])
+@pytest.mark.parametrize("n", [512, 513, 557, 558, 669, 1021])
+def test_fused_wavefront_bit_exact(n, sweeps):
+    """The default fused sweeps (register-wavefront passes of 2 to 4 sweeps on the fixed-point
+    grid, from 512^2 on): every split of a sweep count into passes, at the smallest such grid and
+    at grids that end at and just past a whole number of strips (60 stored values at depth 2,
+    56 at depth 3)."""
+    f, u0 = _problem(n, 77 + n)
+    h2 = synth.h_squared(n)
+    got, _ = _run(n, h2, f, u0, [sweeps])
+    ref = u0.copy()
+    oracle.sweeps_fused(ref, f, h2, sweeps)
+    _assert_bits(got, ref)
+
+
+def test_fused_wavefront_equals_one_launch_per_colour_on_a_large_grid():
+    """Whole waves of strips and segments: the same bits as one launch per colour."""
+    n, sweeps = 2999, 31
+    f, u0 = _problem(n, 5)
+    h2 = synth.h_squared(n)
+    got, _ = _run(n, h2, f, u0, [sweeps])
+    ref, _ = _run(n, h2, f, u0, [sweeps], kernel=rb.RBGS_KERNEL_COLOUR)
+    _assert_bits(got, ref)
+
+
+def test_fused_wavefront_reports_non_finite_input():
+    n = 70
+    f, u0 = _problem(n, 6)
+    f[3, 4] = np.inf
+    with rb.Solver(n, synth.h_squared(n), torch.from_numpy(f).cuda(), torch.from_numpy(u0).cuda(), fma=1) as s:
+        s.sweep(9)
+        with pytest.raises(rb.RbgsError) as e:
+            s.residual()
+    assert e.value.status == rb.RBGS_ENONFINITE
