@@ -8,14 +8,16 @@
 // its k-neighbours sit in the other colour's row of the same line, at m-1/m or m/m+1.
 // W = ceil((N+2)/2) rounded up to 32 values (256-byte rows).
 //
-// Half-sweep: the colour's (line, pair of values) items are flattened over a grid-stride
-// loop; each item reads the other colour's rows of lines (i-1, j), (i+1, j), (i, j-1),
-// (i, j+1) and (i, j) and h2 f, and writes its own two values.  Neighbouring lines in j are
-// adjacent in the item order and lines i+-1 one plane apart, so the re-reads of the other
-// colour hit the caches (a plane of a 511^3 grid is 1.2 MB).  Arithmetic: six adds in the
-// order above, each one correctly rounded fused multiply-add by a run-time 1.0, and one
-// correctly rounded division by 6 (div6 in div6.cuh: three FP64 operations instead of the
-// division sequence): the same bits as the plain sequential loop.
+// Half-sweep: the pairs of values of a plane (line j, pair of elements) are flattened over the
+// threads, and a thread walks its place (j, m) down a chunk of planes i.  The other colour's
+// values at planes i-1, i, i+1 stay in registers, so each is loaded once per chunk; lines j-1
+// and j+1 of plane i are other threads' places and come through L1.  (One flattened loop over
+// all (i, j, m) with five line loads and two index divisions per pair, and a division by 6 of
+// three FP64 operations, ran at 31 GLUP/s at 511^3, 2.12 ms a half-sweep.)  Arithmetic: six
+// adds in the order above, each one correctly rounded fused multiply-add by a run-time 1.0, and
+// one correctly rounded division by 6 on the integer pipes (div6.cuh): the same bits as the
+// plain sequential loop.  The FP64 pipe bounds it, six instructions
+// per update, 83% busy (ncu): 85.9 GLUP/s at 511^3, 0.78 ms a half-sweep, 79 at 255^3 (27 before).
 #include <algorithm>
 #include <cmath>
 #include <new>
@@ -32,7 +34,7 @@ struct rbgs3d_ctx {
     cudaStream_t stream;
     double *u[2], *hf[2];
     double *staging;   // natural-layout (N+2)^3 buffer for host inputs and outputs
-    double *partials;  // [2 * kBlocks3]: per block sum rt^2, sum hb^2
+    double *partials;  // [2 * kBlocks3]: per block sums, both colours
     double *dsum;      // [2]
     double *hsum;      // pinned mirror of dsum
     double den2;
@@ -91,120 +93,173 @@ __global__ void unpack3_kernel(const double *__restrict__ u0, const double *__re
     }
 }
 
-// One half-sweep of colour C: items (interior line, pair of values) over the grid.
+// A thread's place in every plane: line j and the pair of elements m0, m0 + 1.
+struct Place3 {
+    int j, m0;
+    bool act;
+};
+
+// Pairs per line and the multiplier ceil(2^32 / npairs) of the division by it: item / npairs =
+// umulhi(item, mul) exactly, as item (mul npairs - 2^32) < 2^22 2^10 (n <= 2048).  An integer
+// division costs FP64-pipe instructions, which a short chunk would notice.
+struct Pairs3 {
+    int npairs;
+    unsigned mul;
+};
+
+__device__ __forceinline__ Place3 place3(int block, int n, const Pairs3 &d) {
+    const int item = block * kThreads3 + (int)threadIdx.x;
+    const int npairs = d.npairs;
+    const int line = npairs == 1 ? item : (int)__umulhi((unsigned)item, d.mul);
+    return Place3{1 + line, 2 * (item - line * npairs), line < n};
+}
+
+// One half-sweep of colour C over planes [i0, i0 + chunk) by block (x: places, y: chunk).
 template <int C>
 __global__ void __launch_bounds__(kThreads3)
 half_sweep3_kernel(double *__restrict__ self, const double *__restrict__ other, const double *__restrict__ hf,
-                   int n, int W, int kact, double one) {
-    const int L = n + 2;
-    const int npairs = kact / 2;
-    const size_t items = (size_t)n * n * npairs;
-    for (size_t q = (size_t)blockIdx.x * kThreads3 + threadIdx.x; q < items; q += (size_t)gridDim.x * kThreads3) {
-        const int pr = (int)(q % npairs);
-        const size_t ln = q / npairs;
-        const int i = 1 + (int)(ln / n), j = 1 + (int)(ln % n);
-        const int m0 = 2 * pr;
-        const int p = (i + j + C) & 1;  // k offset of this colour on line (i, j)
-        const size_t row = ((size_t)i * L + j) * W;
-        const size_t plane = (size_t)L * W;
-        const double2 vn = __ldg(reinterpret_cast<const double2 *>(other + row - plane + m0));
-        const double2 vs = __ldg(reinterpret_cast<const double2 *>(other + row + plane + m0));
-        const double2 vw = __ldg(reinterpret_cast<const double2 *>(other + row - W + m0));
-        const double2 ve = __ldg(reinterpret_cast<const double2 *>(other + row + W + m0));
-        const double2 vm = __ldg(reinterpret_cast<const double2 *>(other + row + m0));
-        const double2 f2 = __ldg(reinterpret_cast<const double2 *>(hf + row + m0));
-        double d0, u0, d1, u1;  // k-1 and k+1 neighbours of the two values
-        if (p == 0) {  // value v at k = 2(m0+v): k-1 at m0+v-1, k+1 at m0+v
-            d0 = m0 > 0 ? __ldg(other + row + m0 - 1) : 0.0;
-            u0 = vm.x;
-            d1 = vm.x;
-            u1 = vm.y;
-        } else {  // at 2(m0+v)+1: k-1 at m0+v, k+1 at m0+v+1
-            d0 = vm.x;
-            u0 = vm.y;
-            d1 = vm.y;
-            u1 = m0 + 2 < W ? __ldg(other + row + m0 + 2) : 0.0;
+                   int n, int W, Pairs3 npairs, int chunk, double one) {
+    constexpr int NV = 2;  // 4 and 8 values measured 1.5% and 10% slower
+    const Place3 pl = place3(blockIdx.x, n, npairs);
+    if (!pl.act) return;
+    const int m0 = pl.m0;
+    const int i0 = 1 + blockIdx.y * chunk, i1 = min(n, i0 + chunk - 1);
+    const size_t plane = (size_t)(n + 2) * W;
+    size_t at = ((size_t)i0 * (n + 2) + pl.j) * W + m0;
+    double vn[NV], vm[NV], vs[NV], vw[NV], ve[NV], f[NV];
+    load_row<NV>(vn, other + at - plane, true);
+    load_row<NV>(vm, other + at, true);
+    for (int i = i0; i <= i1; ++i, at += plane) {
+        load_row<NV>(vs, other + at + plane, true);
+        load_row<NV>(vw, other + at - W, true);
+        load_row<NV>(ve, other + at + W, true);
+        load_row<NV>(f, hf + at, true);
+        // value v at k = 2(m0+v) + p: k-1 and k+1 at elements m0+v-1+p and m0+v+p
+        const int p = (i + pl.j + C) & 1;
+        const bool in = p ? m0 + NV < W : m0 > 0;
+        const double x = in ? __ldg(other + at + (p ? NV : -1)) : 0.0;
+        double r[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            r[v] = add_fma(add_fma(add_fma(add_fma(f[v], vn[v], one), vs[v], one), vw[v], one), ve[v], one);
+            r[v] = add_fma(r[v], p ? vm[v] : (v ? vm[v ? v - 1 : 0] : x), one);
+            r[v] = add_fma(r[v], p ? (v + 1 < NV ? vm[v + 1 < NV ? v + 1 : 0] : x) : vm[v], one);
         }
-        double s0 = add_fma(f2.x, vn.x, one);
-        s0 = add_fma(s0, vs.x, one);
-        s0 = add_fma(s0, vw.x, one);
-        s0 = add_fma(s0, ve.x, one);
-        s0 = add_fma(s0, d0, one);
-        s0 = add_fma(s0, u0, one);
-        double s1 = add_fma(f2.y, vn.y, one);
-        s1 = add_fma(s1, vs.y, one);
-        s1 = add_fma(s1, vw.y, one);
-        s1 = add_fma(s1, ve.y, one);
-        s1 = add_fma(s1, d1, one);
-        s1 = add_fma(s1, u1, one);
-        const int k0 = 2 * m0 + p;  // natural k of value 0; value 1 at k0 + 2
-        if (k0 >= 1 && k0 <= n) self[row + m0] = div6(s0);
-        if (k0 + 2 <= n) self[row + m0 + 1] = div6(s1);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) r[v] = div6(r[v]);
+        const int k0 = 2 * m0 + p;  // natural k of value 0; value v at k0 + 2v
+        if (k0 >= 1 && k0 + 2 * (NV - 1) <= n) {
+            store_row<NV>(self + at, r);
+        } else {
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+                if (k0 + 2 * v >= 1 && k0 + 2 * v <= n) self[at + v] = r[v];
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) vn[v] = vm[v], vm[v] = vs[v];
     }
 }
 
-// Per-block sums of rt^2 and (h^2 b)^2 over every interior point (both colours).
+// Per-block sums of rt^2 over the interior points of colour C, the same walk as a half-sweep
+// (places and chunks of planes as a grid-stride loop over `tasks` = x_blocks * chunks).
+template <int C>
 __global__ void __launch_bounds__(kThreads3)
-residual3_kernel(const double *__restrict__ u0, const double *__restrict__ u1, const double *__restrict__ hf0,
-                 const double *__restrict__ hf1, int n, int W, double *__restrict__ partials) {
+residual3_kernel(const double *__restrict__ self, const double *__restrict__ other, const double *__restrict__ hf,
+                 int n, int W, Pairs3 npairs, int chunk, int x_blocks, int tasks, double one,
+                 double *__restrict__ partials) {
+    __shared__ double smem[kThreads3 / 32];
+    const size_t plane = (size_t)(n + 2) * W;
+    double acc = 0.0;
+    for (int task = blockIdx.x; task < tasks; task += gridDim.x) {
+        const Place3 pl = place3(task % x_blocks, n, npairs);
+        if (!pl.act) continue;
+        const int i0 = 1 + task / x_blocks * chunk, i1 = min(n, i0 + chunk - 1);
+        size_t at = ((size_t)i0 * (n + 2) + pl.j) * W + pl.m0;
+        double2 vn = ldg2(other + at - plane), vm = ldg2(other + at);
+        for (int i = i0; i <= i1; ++i, at += plane) {
+            const double2 vs = ldg2(other + at + plane);
+            const double2 vw = ldg2(other + at - W), ve = ldg2(other + at + W);
+            const double2 f2 = ldg2(hf + at), me = ldg2(self + at);
+            const int p = (i + pl.j + C) & 1;
+            const bool in = p ? pl.m0 + 2 < W : pl.m0 > 0;
+            const double x = in ? __ldg(other + at + (p ? 2 : -1)) : 0.0;
+            double s0 = add_fma(add_fma(add_fma(add_fma(f2.x, vn.x, one), vs.x, one), vw.x, one), ve.x, one);
+            double s1 = add_fma(add_fma(add_fma(add_fma(f2.y, vn.y, one), vs.y, one), vw.y, one), ve.y, one);
+            s0 = add_fma(add_fma(s0, p ? vm.x : x, one), p ? vm.y : vm.x, one);
+            s1 = add_fma(add_fma(s1, p ? vm.y : vm.x, one), p ? x : vm.y, one);
+            const double r0 = add_fma(s0, -__dmul_rn(6.0, me.x), one), r1 = add_fma(s1, -__dmul_rn(6.0, me.y), one);
+            const int k0 = 2 * pl.m0 + p;
+            if (k0 >= 1 && k0 <= n) acc = __fma_rn(r0, r0, acc);
+            if (k0 + 2 <= n) acc = __fma_rn(r1, r1, acc);
+            vn = vm;
+            vm = vs;
+        }
+    }
+    const double t = block_sum<kThreads3>(acc, smem);
+    if (threadIdx.x == 0) partials[blockIdx.x] = t;
+}
+
+// Per-block sums of (h^2 b)^2 over the interior points of colour C: h2 f plus, in N, S, W, E, D,
+// U order, the neighbours on the shell.  The same walk and the same order of additions as
+// residual3_kernel, so rho is exactly 1 for u = 0 inside and on the shell.  Only points next
+// to the shell read u; everywhere else b is h2 f and the walk streams it.
+template <int C>
+__global__ void __launch_bounds__(kThreads3)
+norm3_kernel(const double *__restrict__ other, const double *__restrict__ hf, int n, int W, Pairs3 npairs, int chunk,
+             int x_blocks, int tasks, double *__restrict__ partials) {
     __shared__ double smem[kThreads3 / 32];
     const int L = n + 2;
-    const size_t total = (size_t)n * n * n;
-    double r2 = 0.0, b2 = 0.0;
-    auto at = [&](int i, int j, int k) {
-        const bool even = ((i + j + k) & 1) == 0;
-        return (even ? u0 : u1)[((size_t)i * L + j) * W + (k >> 1)];
-    };
-    for (size_t q = (size_t)blockIdx.x * kThreads3 + threadIdx.x; q < total; q += (size_t)gridDim.x * kThreads3) {
-        const int k = 1 + (int)(q % n);
-        const size_t t = q / n;
-        const int j = 1 + (int)(t % n), i = 1 + (int)(t / n);
-        const bool even = ((i + j + k) & 1) == 0;
-        const double hf = (even ? hf0 : hf1)[((size_t)i * L + j) * W + (k >> 1)];
-        const double vn = at(i - 1, j, k), vs = at(i + 1, j, k), vw = at(i, j - 1, k), ve = at(i, j + 1, k);
-        const double vd = at(i, j, k - 1), vu = at(i, j, k + 1);
-        double s = __dadd_rn(hf, vn);
-        s = __dadd_rn(s, vs);
-        s = __dadd_rn(s, vw);
-        s = __dadd_rn(s, ve);
-        s = __dadd_rn(s, vd);
-        s = __dadd_rn(s, vu);
-        const double r = __dadd_rn(s, -__dmul_rn(6.0, at(i, j, k)));
-        r2 = __fma_rn(r, r, r2);
-        double b = hf;
-        if (i == 1) b = __dadd_rn(b, vn);
-        if (i == n) b = __dadd_rn(b, vs);
-        if (j == 1) b = __dadd_rn(b, vw);
-        if (j == n) b = __dadd_rn(b, ve);
-        if (k == 1) b = __dadd_rn(b, vd);
-        if (k == n) b = __dadd_rn(b, vu);
-        b2 = __fma_rn(b, b, b2);
+    const size_t plane = (size_t)L * W;
+    // a shell neighbour of a point of colour C has the other colour
+    auto shell = [&](int i, int j, int k) { return other[((size_t)i * L + j) * W + (k >> 1)]; };
+    double acc = 0.0;
+    for (int task = blockIdx.x; task < tasks; task += gridDim.x) {
+        const Place3 pl = place3(task % x_blocks, n, npairs);
+        if (!pl.act) continue;
+        const int j = pl.j, i0 = 1 + task / x_blocks * chunk, i1 = min(n, i0 + chunk - 1);
+        const double *row = hf + ((size_t)i0 * L + j) * W + pl.m0;
+        const bool inner = j > 1 && j < n && pl.m0 > 0 && 2 * pl.m0 + 3 < n;  // for either parity
+        int i = i0;
+        if (inner && i0 > 1) {  // four planes' loads in flight, no index work
+            const int last = min(i1, n - 1);
+            for (; i + 3 <= last; i += 4, row += 4 * plane) {
+                const double2 a = ldg2(row), b = ldg2(row + plane), c = ldg2(row + 2 * plane), d = ldg2(row + 3 * plane);
+                acc = __fma_rn(a.x, a.x, acc), acc = __fma_rn(a.y, a.y, acc);
+                acc = __fma_rn(b.x, b.x, acc), acc = __fma_rn(b.y, b.y, acc);
+                acc = __fma_rn(c.x, c.x, acc), acc = __fma_rn(c.y, c.y, acc);
+                acc = __fma_rn(d.x, d.x, acc), acc = __fma_rn(d.y, d.y, acc);
+            }
+        }
+        for (; i <= i1; ++i, row += plane) {
+            const double2 f2 = ldg2(row);
+            const int k0 = 2 * pl.m0 + ((i + j + C) & 1);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int k = k0 + 2 * q;
+                if (k < 1 || k > n) continue;
+                double b = q ? f2.y : f2.x;
+                if (i == 1) b = __dadd_rn(b, shell(0, j, k));
+                if (i == n) b = __dadd_rn(b, shell(n + 1, j, k));
+                if (j == 1) b = __dadd_rn(b, shell(i, 0, k));
+                if (j == n) b = __dadd_rn(b, shell(i, n + 1, k));
+                if (k == 1) b = __dadd_rn(b, shell(i, j, 0));
+                if (k == n) b = __dadd_rn(b, shell(i, j, n + 1));
+                acc = __fma_rn(b, b, acc);
+            }
+        }
     }
-    const double tr = block_sum<kThreads3>(r2, smem);
-    __syncthreads();
-    const double tb = block_sum<kThreads3>(b2, smem);
-    if (threadIdx.x == 0) {
-        partials[2 * blockIdx.x] = tr;
-        partials[2 * blockIdx.x + 1] = tb;
-    }
+    const double t = block_sum<kThreads3>(acc, smem);
+    if (threadIdx.x == 0) partials[blockIdx.x] = t;
 }
 
 // The blocks' partial sums added in a fixed order (one block).
 __global__ void __launch_bounds__(kThreads3)
-final3_kernel(const double *__restrict__ partials, int blocks, double *__restrict__ out) {
+final3_kernel(const double *__restrict__ partials, int count, double *__restrict__ out) {
     __shared__ double smem[kThreads3 / 32];
-    double r2 = 0.0, b2 = 0.0;
-    for (int q = threadIdx.x; q < blocks; q += kThreads3) {
-        r2 = __dadd_rn(r2, partials[2 * q]);
-        b2 = __dadd_rn(b2, partials[2 * q + 1]);
-    }
-    const double tr = block_sum<kThreads3>(r2, smem);
-    __syncthreads();
-    const double tb = block_sum<kThreads3>(b2, smem);
-    if (threadIdx.x == 0) {
-        out[0] = tr;
-        out[1] = tb;
-    }
+    double v = 0.0;
+    for (int q = threadIdx.x; q < count; q += kThreads3) v = __dadd_rn(v, partials[q]);
+    const double t = block_sum<kThreads3>(v, smem);
+    if (threadIdx.x == 0) *out = t;
 }
 
 int grid_for(size_t items) {
@@ -243,14 +298,53 @@ void free3(rbgs3d_ctx *c) {
     delete c;
 }
 
-// rho's two sums into dsum (stream-ordered)
+// Launch shape of a walk over an n^3 grid: blocks of places, and planes per chunk.  Chunks of 8
+// planes load the other colour's planes 1.25 times (from L2; 8 / 16 / 64 planes: 1553 / 1567 /
+// 1585 us a sweep at 511^3); smaller grids take shorter chunks, so that there are about four
+// blocks for each one that is resident.
+struct Walk3 {
+    Pairs3 npairs;
+    int x_blocks, chunk, chunks;
+};
+
+Walk3 walk3(int n) {
+    Walk3 w;
+    const int np = active_width(n) / 2;
+    w.npairs = Pairs3{np, (unsigned)(((1ull << 32) + np - 1) / np)};
+    w.x_blocks = (n * np + kThreads3 - 1) / kThreads3;
+    const long want = 4L * grid_for((size_t)1 << 40);  // 4 x 8 blocks for each SM
+    long chunk = (long)n * w.x_blocks / want;
+    w.chunk = (int)(chunk < 1 ? 1 : chunk > 8 ? 8 : chunk);
+    w.chunks = (n + w.chunk - 1) / w.chunk;
+    return w;
+}
+
+// sum rt^2 into dsum[0] (stream-ordered)
 rbgs_status enqueue_residual3(rbgs3d_ctx *c) {
-    const size_t total = (size_t)c->n * c->n * c->n;
-    const int blocks = std::min(grid_for(total), kBlocks3);
-    residual3_kernel<<<blocks, kThreads3, 0, c->stream>>>(c->u[0], c->u[1], c->hf[0], c->hf[1], c->n, c->W,
-                                                          c->partials);
+    const Walk3 w = walk3(c->n);
+    const int tasks = w.x_blocks * w.chunks, blocks = std::min(tasks, kBlocks3);
+    residual3_kernel<0><<<blocks, kThreads3, 0, c->stream>>>(c->u[0], c->u[1], c->hf[0], c->n, c->W, w.npairs, w.chunk,
+                                                             w.x_blocks, tasks, 1.0, c->partials);
     RBGS_LAUNCH_CHECK();
-    final3_kernel<<<1, kThreads3, 0, c->stream>>>(c->partials, blocks, c->dsum);
+    residual3_kernel<1><<<blocks, kThreads3, 0, c->stream>>>(c->u[1], c->u[0], c->hf[1], c->n, c->W, w.npairs, w.chunk,
+                                                             w.x_blocks, tasks, 1.0, c->partials + blocks);
+    RBGS_LAUNCH_CHECK();
+    final3_kernel<<<1, kThreads3, 0, c->stream>>>(c->partials, 2 * blocks, c->dsum);
+    RBGS_LAUNCH_CHECK();
+    return RBGS_OK;
+}
+
+// sum (h^2 b)^2 into dsum[1] (stream-ordered)
+rbgs_status enqueue_norm3(rbgs3d_ctx *c) {
+    const Walk3 w = walk3(c->n);
+    const int tasks = w.x_blocks * w.chunks, blocks = std::min(tasks, kBlocks3);
+    norm3_kernel<0><<<blocks, kThreads3, 0, c->stream>>>(c->u[1], c->hf[0], c->n, c->W, w.npairs, w.chunk, w.x_blocks,
+                                                         tasks, c->partials);
+    RBGS_LAUNCH_CHECK();
+    norm3_kernel<1><<<blocks, kThreads3, 0, c->stream>>>(c->u[0], c->hf[1], c->n, c->W, w.npairs, w.chunk, w.x_blocks,
+                                                         tasks, c->partials + blocks);
+    RBGS_LAUNCH_CHECK();
+    final3_kernel<<<1, kThreads3, 0, c->stream>>>(c->partials, 2 * blocks, c->dsum + 1);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
@@ -328,8 +422,8 @@ rbgs_status rbgs3d_create(int n, double h2, const double *f, const double *u_ini
     pack3_kernel<<<grid_for(L * L * c->W), kThreads3, 0, c->stream>>>(uv, fv, h2, c->u[0], c->u[1], c->hf[0],
                                                                       c->hf[1], n, c->W);
     rbgs_status st = cudaGetLastError() == cudaSuccess ? RBGS_OK : RBGS_ECUDA;
-    if (st == RBGS_OK) st = enqueue_residual3(c);
-    if (st == RBGS_OK && (cudaMemcpyAsync(c->hsum, c->dsum, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream) !=
+    if (st == RBGS_OK) st = enqueue_norm3(c);
+    if (st == RBGS_OK && (cudaMemcpyAsync(c->hsum + 1, c->dsum + 1, sizeof(double), cudaMemcpyDeviceToHost, c->stream) !=
                               cudaSuccess ||
                           cudaStreamSynchronize(c->stream) != cudaSuccess)) {
         cudaGetLastError();
@@ -350,13 +444,14 @@ rbgs_status rbgs3d_sweep(rbgs3d_t c, long nsweeps) {
     clear_error();
     if (!c) { set_error("ctx is NULL"); return RBGS_EINVAL; }
     if (nsweeps < 0) { set_error("nsweeps < 0"); return RBGS_EINVAL; }
-    const int kact = active_width(c->n);
-    const size_t items = (size_t)c->n * c->n * (kact / 2);
-    const int grid = grid_for(items);
+    const Walk3 w = walk3(c->n);
+    const dim3 grid(w.x_blocks, w.chunks);
     for (long it = 0; it < nsweeps; ++it) {
-        half_sweep3_kernel<0><<<grid, kThreads3, 0, c->stream>>>(c->u[0], c->u[1], c->hf[0], c->n, c->W, kact, 1.0);
+        half_sweep3_kernel<0><<<grid, kThreads3, 0, c->stream>>>(c->u[0], c->u[1], c->hf[0], c->n, c->W, w.npairs,
+                                                                      w.chunk, 1.0);
         RBGS_LAUNCH_CHECK();
-        half_sweep3_kernel<1><<<grid, kThreads3, 0, c->stream>>>(c->u[1], c->u[0], c->hf[1], c->n, c->W, kact, 1.0);
+        half_sweep3_kernel<1><<<grid, kThreads3, 0, c->stream>>>(c->u[1], c->u[0], c->hf[1], c->n, c->W, w.npairs,
+                                                                      w.chunk, 1.0);
         RBGS_LAUNCH_CHECK();
     }
     return RBGS_OK;
@@ -367,7 +462,7 @@ rbgs_status rbgs3d_residual(rbgs3d_t c, double *rel) {
     if (!c || !rel) { set_error("ctx and rel must not be NULL"); return RBGS_EINVAL; }
     rbgs_status st = enqueue_residual3(c);
     if (st != RBGS_OK) return st;
-    RBGS_CUDA(cudaMemcpyAsync(c->hsum, c->dsum, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    RBGS_CUDA(cudaMemcpyAsync(c->hsum, c->dsum, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     RBGS_CUDA(cudaStreamSynchronize(c->stream));
     const double r2 = c->hsum[0];
     *rel = c->den2 > 0.0 ? std::sqrt(r2) / std::sqrt(c->den2) : std::sqrt(r2);

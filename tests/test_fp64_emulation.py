@@ -179,3 +179,19 @@ def test_div6_is_the_correctly_rounded_quotient(lib):
     nan = np.array([np.nan])
     lib.check_div6(1, _p(nan), _p(out[:1]))
     assert np.isnan(out[0])
+
+
+def test_div6_next_to_the_subnormal_range(lib):
+    """div6 for biased exponents 0..8 (its integer path for results in or next to the subnormal
+    range, and the first exponents of the common path): random and extreme significands, exact
+    multiples and ties, both signs; infinities stay as they are."""
+    rng = np.random.default_rng(8)
+    parts = []
+    for e in range(9):
+        mant = np.concatenate([rng.integers(0, 2 ** 52, 20000, dtype=np.uint64), np.arange(0, 200, dtype=np.uint64),
+                               np.uint64(2 ** 52) - np.arange(1, 200, dtype=np.uint64)])
+        parts += [(np.uint64(s) << np.uint64(63)) | (np.uint64(e) << np.uint64(52)) | mant for s in (0, 1)]
+    a = np.concatenate([_bits_to_f(np.concatenate(parts)), [np.inf, -np.inf]])
+    out = np.empty_like(a)
+    lib.check_div6(a.size, _p(a), _p(out))
+    assert _same_bits(out, a / 6.0)
