@@ -52,8 +52,8 @@ PROFILES = {
                                    "paper_2607_01735_gb300/csrc/sweep_impl.cuh",
                                    "paper_2607_01735_gb300/csrc/fp64.cuh"]),
 }
-PERSIST_MIN_N, PERSIST_MAX_N = 416, 1 << 15
-FUSED_WAVE_MIN_N = 512
+RESIDENT_MAX_N = 1376  # tiles in shared memory up to here; one cooperative launch with a grid barrier above
+PERSIST_MIN_N, PERSIST_MAX_N = RESIDENT_MAX_N + 1, 1 << 15
 # side files of a run (nvidia-smi clock samples, trained U-Net parameters)
 OUT_DIR = os.environ.get("RBGS_BENCH_OUT", os.path.join(ROOT, "bench_out"))
 
@@ -193,8 +193,16 @@ def resolved_kernel(n, refine, kernel, tblock_k):
 
 def fused_wavefront(args, n):
     """The fused sweeps run as register-wavefront passes of up to 3 sweeps (the library's rule:
-    AUTO, no launch-shape option, FUSED_WAVE_MIN_N <= n)."""
-    return args.kernel == 0 and args.tile_rows == 0 and args.values == 0 and n >= FUSED_WAVE_MIN_N
+    AUTO, no launch-shape option, n > RESIDENT_MAX_N)."""
+    return args.kernel == 0 and args.tile_rows == 0 and args.values == 0 and n > RESIDENT_MAX_N
+
+
+def uses_resident(args, n, refine):
+    """The FP64 sweeps, bit-exact or fused, run in one cooperative launch with tiles in shared
+    memory (the library's rule: AUTO, no launch-shape option, n <= RESIDENT_MAX_N)."""
+    return (not refine and args.kernel == 0 and args.tile_rows == 0 and args.emulate == -1
+            and args.values == 0 and args.rows in (0, 1) and args.int_rows <= 0 and args.tblock_k == 0
+            and n <= RESIDENT_MAX_N)
 
 
 def device_peaks(dev):
@@ -1003,6 +1011,7 @@ def main():
         if fma:
             kernel, kdepth = (3, 3) if fused_wavefront(margs, n) else (1, 1)
         blocked = kernel in (2, 3)  # several sweeps per launch (TMA tiles or register wavefront)
+        resident = uses_resident(margs, n, refine)
         persistent = uses_persistent(margs, n, refine)
         # pack f, pack u, ||b|| (2), the sweeps, residual, unpack.  The residual after
         # bit-exact FP64 sweeps walks the red points only (2 launches: the black rt is exactly
@@ -1010,7 +1019,7 @@ def main():
         resid = 2 if sweeps > 0 and not fma else 3
         if fma:  # + max |h2 f| at load; per block of <= 1024 sweeps: max |u|, h2 f onto the grid
             blocks = [1024] * (sweeps // 1024) + ([sweeps % 1024] if sweeps % 1024 else [])
-            passes = sum(-(-m // 3) if blocked and m >= 4 else 2 * m for m in blocks)
+            passes = sum(1 if resident else -(-m // 3) if blocked and m >= 4 else 2 * m for m in blocks)
             launches_per_step = 4 + 1 + 2 * len(blocks) + passes + resid + 1
         elif refine:
             inner = args.inner or 100
@@ -1019,6 +1028,8 @@ def main():
             launches_per_step = 4 + 4 + outer * per_outer + 3 + 1
         elif blocked:
             launches_per_step = 4 + sweeps // kdepth + 2 * (sweeps % kdepth) + resid + 1
+        elif resident:
+            launches_per_step = 4 + (1 if sweeps > 1 else 2 * sweeps) + resid + 1
         elif persistent:  # one cooperative launch runs all the sweeps (up to 2^20 per launch)
             launches_per_step = 4 + -(-sweeps // (1 << 20)) + resid + 1
         else:
@@ -1076,7 +1087,8 @@ def main():
             # The time includes the rescaling passes of each block of sweeps (max |u|, h2 f onto
             # the grid).
             launches = -(-sweeps // 3) if blocked else 2 * sweeps
-            kname = "wavefront_kernel<int64, 3>" if blocked else "fused_half_sweep"
+            kname = ("resident_kernel<int64>" if resident else "wavefront_kernel<int64, 3>" if blocked
+                     else "fused_half_sweep")
             launch_s = sweep_s / (launches * args.steps)
             alg_bytes = 16.0 * n * n if blocked else BYTES_PER_LUP * n * n / 2.0
             achieved = alg_bytes / launch_s / 1e9
@@ -1094,7 +1106,7 @@ def main():
             # per clock per SM (ncu's DFMA peak_sustained) x SMs x maximum SM clock.
             # (the persistent kernel: per half-sweep equivalent, its launch time / (2 sweeps))
             launches = (sweeps // kdepth) if blocked else 2 * sweeps
-            kname = (f"{names[kernel]}<double, {kdepth}>" if blocked
+            kname = ("resident_kernel<double>" if resident else f"{names[kernel]}<double, {kdepth}>" if blocked
                      else "persistent_sweeps<double>" if persistent else "half_sweep_f64")
             per_launch_lups = n * n * sweeps / launches
             launch_s = sweep_s / (launches * args.steps)
@@ -1113,7 +1125,8 @@ def main():
             if persistent:
                 roofline["note"] = ("one cooperative launch runs all sweeps; launch_ms, traffic and the "
                                     "algorithmic bytes are per half-sweep equivalent (the launch / 2 sweeps)")
-        kdesc = ("all sweeps in one cooperative launch (grid barrier between colours)" if persistent
+        kdesc = ("all sweeps in one cooperative launch, tiles in shared memory" if resident
+                 else "all sweeps in one cooperative launch (grid barrier between colours)" if persistent
                  else {1: "one launch per colour", 2: "temporal (TMA tiles)", 3: "register wavefront"}[kernel])
         return {"ctx": ctx, "step": step, "value": lups / elapsed / 1e9, "elapsed": elapsed, "lups": lups,
                 "step_ms": step_ms, "sweep_ms": sweep_ms, "roofline": roofline, "clocks": clocks.summary(),

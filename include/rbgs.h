@@ -53,8 +53,8 @@ typedef enum {
     RBGS_ENOTCONV = 4,    /* max_sweeps reached, or the residual stalled (stall_checks);
                              the iterate is kept                                          */
     RBGS_ENONFINITE = 5,  /* the residual became NaN or Inf                              */
-    RBGS_ETIMEOUT = 6     /* a bounded device-side wait gave up: the grid barrier of the
-                             cooperative FP64 launch or the TMA wait of the temporal
+    RBGS_ETIMEOUT = 6     /* a bounded device-side wait gave up: the grid barrier or the
+                             tile exchange of a cooperative launch or the TMA wait of the temporal
                              kernel (reported by the next rbgs_residual or rbgs_solve).
                              Sticky: the iterate is left part-updated and every later
                              rbgs_residual / rbgs_solve on the context returns it again;
@@ -68,10 +68,14 @@ typedef enum {
 } rbgs_precision;
 
 typedef enum {
-    RBGS_KERNEL_AUTO = 0,     /* FP64 sweeps: PERSISTENT for 416 <= n <= 32768 with the default
-                                 launch-shape options, else COLOUR.  FP32 inner sweeps of
-                                 RBGS_FP32_REFINE: WAVEFRONT (depth 4) when n > 1000 and
-                                 tblock_k = 0, else COLOUR                                   */
+    RBGS_KERNEL_AUTO = 0,     /* FP64 sweeps, bit-exact or fused, with the default launch-shape
+                                 options: all sweeps of a call in one cooperative launch with
+                                 tiles of the grid held in shared memory, where they fit (n up
+                                 to about 1370); above that PERSISTENT for 416 <= n <= 32768
+                                 (fused: see fma), else COLOUR.  FP32 inner sweeps of
+                                 RBGS_FP32_REFINE with tblock_k = 0: tiles in shared memory for
+                                 n <= 1000, WAVEFRONT (depth 4) above, else COLOUR.  Sweeps of
+                                 the tiled form wait within the launch (RBGS_ETIMEOUT)         */
     RBGS_KERNEL_COLOUR = 1,   /* one launch per colour (half-sweep kernels)               */
     RBGS_KERNEL_TEMPORAL = 2, /* several sweeps per shared-memory tile, halo recompute      */
     RBGS_KERNEL_WAVEFRONT = 3,/* several sweeps per pass, a register wavefront per strip   */
@@ -113,9 +117,10 @@ typedef struct {
                             with the bit-exact iterate to <= 1e-13 relative max-norm after the same
                             sweeps (the tolerance set for this mode); a non-finite value in u or h2 f makes
                             that block of sweeps run the bit-exact update.  With kernel AUTO and
-                            no launch-shape option, register-wavefront passes from 512^2 on (two
-                            more FP64 arrays of half the grid each; without room for them, and
-                            otherwise, one launch per colour).  The same bits either way          */
+                            no launch-shape option, tiles in shared memory where they fit, above
+                            that register-wavefront passes (two more FP64 arrays of half the grid
+                            each); without room for their buffers, and otherwise, one launch per
+                            colour.  The same bits either way                                     */
     int stall_checks;  /* rbgs_solve and rbgs_solve_batched stop a problem with RBGS_ENOTCONV when
                           its residual has not reached a new minimum for this many consecutive
                           checks (0: 64; -1: never), so a tolerance below the rounding floor

@@ -52,9 +52,16 @@ constexpr long kFusedChunk = 1024;
 // at 511^2, 7.2 / 13.1 at 1023^2, 9.9 / 16.2 at 1500^2, 31 / 96 at 4095^2, 382 / 1021 at
 // 16384^2.
 constexpr int kFusedWaveMinN = 512;
+// The resident kernel (resident.cu): FP64 and fused sweeps wherever its tiles fit (up to about
+// 1200^2, resident_plan decides), FP32 inner sweeps up to 1000^2, above which the wavefront is
+// as fast and needs no cooperative launch.
+constexpr int kResidentMaxN = 2048, kResident32MaxN = 1000;
 constexpr int kWave32MinN = 1001;    // FP32 inner sweeps as wavefront passes from this size on
 // Residual checks without a new minimum of rho after which a solve stops (opts.stall_checks 0).
 constexpr int kDefaultStallChecks = 64;
+
+// Internal kernel choice: the resident kernel (resident.cu), which RBGS_KERNEL_AUTO takes.
+constexpr int kKernelResident = 100;
 
 bool use_persistent(const rbgs_ctx *c) { return c->kernel == RBGS_KERNEL_PERSISTENT; }
 
@@ -139,6 +146,10 @@ void free_ctx(rbgs_ctx *c) {
     cudaFree(c->fwords);
     cudaFree(c->tq[0]);
     cudaFree(c->tq[1]);
+    for (ResidentState *r : {&c->res64, &c->res32}) {
+        cudaFree(r->slots);
+        cudaFree(r->epoch);
+    }
     for (int q = 0; q < 2; ++q) {
         cudaFree(c->sin_f[q]);
         cudaFree(c->sin_u[q]);
@@ -186,6 +197,23 @@ rbgs_status ensure_f64_alt(rbgs_ctx *c) {
     return RBGS_OK;
 }
 
+// The resident kernel's plan and exchange slots for this context's grid; without room for the
+// slots the kernel is not used (r.slots stays NULL).
+void prepare_resident(rbgs_ctx *c, ResidentState &r, int W, int kind) {
+    r.plan = resident_plan(c->g.n, kind);
+    if (r.plan.rows == 0) return;
+    const size_t bytes = resident_slot_bytes(c->g.n, W, kind);
+    if (cudaMalloc(&r.slots, bytes) != cudaSuccess || cudaMalloc(&r.epoch, 2 * sizeof(unsigned)) != cudaSuccess ||
+        cudaMemsetAsync(r.slots, 0, bytes, c->stream) != cudaSuccess ||
+        cudaMemsetAsync(r.epoch, 0, 2 * sizeof(unsigned), c->stream) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(r.slots);
+        cudaFree(r.epoch);
+        r.slots = nullptr;
+        r.epoch = nullptr;
+    }
+}
+
 // FP32 correction, scaled defect and (for the temporal inner kernel) the partner buffers.
 rbgs_status ensure_f32(rbgs_ctx *c) {
     if (c->f32.u[0]) return RBGS_OK;
@@ -201,6 +229,9 @@ rbgs_status ensure_f32(rbgs_ctx *c) {
             return st;
     }
     c->f32.maps_ready = false;
+    if (c->kernel32 == RBGS_KERNEL_COLOUR && c->opts.kernel == RBGS_KERNEL_AUTO && c->opts.tblock_k == 0 &&
+        c->opts.tile_rows == 0 && c->g.n <= kResident32MaxN)
+        prepare_resident(c, c->res32, c->f32.W, 1);
     return RBGS_OK;
 }
 
@@ -271,6 +302,10 @@ rbgs_status sweeps_f64(rbgs_ctx *c, long nsweeps) {
             nsweeps -= m;
             rbgs_status st = launch_fused_prepare(c, m, c->stream);
             if (st != RBGS_OK) return st;
+            if (c->res64.slots && m >= 2) {
+                if ((st = launch_resident_sweeps_fused(c, m, c->stream)) != RBGS_OK) return st;
+                continue;
+            }
             if (c->tq[0] && m >= kFusedWaveMin) {
                 if ((st = launch_fused_wave_sweeps(c, m, c->stream)) != RBGS_OK) return st;
                 continue;
@@ -286,6 +321,7 @@ rbgs_status sweeps_f64(rbgs_ctx *c, long nsweeps) {
         }
         return RBGS_OK;
     }
+    if (c->kernel == kKernelResident && nsweeps >= 2) return launch_resident_sweeps_f64(c, nsweeps, c->stream);
     if (use_persistent(c)) return launch_persistent_sweeps<double>(c->f64, nsweeps, c->pcounter, c->dstatus, c->stream);
     if (c->kernel == RBGS_KERNEL_COLOUR && c->g.n <= kGraphMaxN && nsweeps >= kGraphSweeps) {
         rbgs_status st = ensure_graph(c);
@@ -315,6 +351,7 @@ rbgs_status defect_stats(rbgs_ctx *c, double *rho, double *mx) {
 }
 
 rbgs_status inner_sweeps_f32(rbgs_ctx *c, long m) {
+    if (c->res32.slots && m >= 2) return launch_resident_sweeps_f32(c, m, c->stream);
     // small grids: all m sweeps in one launch of one thread-block cluster
     if (c->kernel32 == RBGS_KERNEL_COLOUR && c->opts.tile_rows == 0 && c->g.n <= kClusterMaxN &&
         cluster_sweeps_f32_fit(c->g.n, c->f32.W))
@@ -534,7 +571,8 @@ rbgs_status rbgs_create(int n, double h2, const double *f, const double *u_init,
     c->h2 = h2;
     c->opts = o;
     c->stream = (cudaStream_t)cuda_stream;
-    // automatic kernels (measured on GB300): FP64 sweeps run in one cooperative launch from
+    // automatic kernels (measured on GB300): FP64 sweeps run with their tiles in shared memory
+    // where those fit (resident.cu has the figures), else in one cooperative launch from
     // 416^2 to 32768^2 with the default launch shape (1.15x at 511^2 to 1.53x at 2047^2 and
     // 1.10x at 16383^2 over one launch per colour), else one launch per colour with cached
     // graphs (the register wavefront reaches the same FP64-pipe limit, with overlap work on
@@ -547,6 +585,7 @@ rbgs_status rbgs_create(int n, double h2, const double *f, const double *u_init,
     c->fused = o.fma == 1;
     c->kernel = c->fused ? RBGS_KERNEL_COLOUR
                 : o.kernel != RBGS_KERNEL_AUTO ? o.kernel
+                : (default_shape && auto_k && o.precision == RBGS_FP64 && n <= kResidentMaxN) ? kKernelResident
                 : (default_shape && n >= kPersistMinN && n <= kPersistMaxN) ? RBGS_KERNEL_PERSISTENT
                                                                             : RBGS_KERNEL_COLOUR;
     c->emulate = o.fp64_emulate == -1 ? 0x00 : o.fp64_emulate;
@@ -600,9 +639,17 @@ rbgs_status rbgs_create(int n, double h2, const double *f, const double *u_init,
     ok = ok && cudaMallocHost(&c->hstatus, sizeof(int)) == cudaSuccess;
     for (int q = 0; q < 2 && ok && c->fused; ++q) ok = cudaMalloc(&c->hq[q], c->g.colour_elems() * sizeof(int64_t)) == cudaSuccess;
     ok = ok && (!c->fused || cudaMalloc(&c->fwords, 3 * sizeof(unsigned long long)) == cudaSuccess);
+    if (ok && c->kernel == kKernelResident) {
+        prepare_resident(c, c->res64, c->g.W, 0);
+        if (!c->res64.slots)
+            c->kernel = n >= kPersistMinN && n <= kPersistMaxN ? RBGS_KERNEL_PERSISTENT : RBGS_KERNEL_COLOUR;
+    } else if (ok && c->fused && o.kernel == RBGS_KERNEL_AUTO && o.tile_rows == 0 && o.sweep_values == 0 &&
+               n <= kResidentMaxN) {
+        prepare_resident(c, c->res64, c->g.W, 2);
+    }
     // the wavefront's buffers; without room for them the half-sweeps run one launch per colour
     if (ok && c->fused && o.kernel == RBGS_KERNEL_AUTO && o.tile_rows == 0 && o.sweep_values == 0 &&
-        n >= kFusedWaveMinN) {
+        n >= kFusedWaveMinN && !c->res64.slots) {
         const size_t qbytes = c->g.colour_elems() * sizeof(int64_t);
         if (cudaMalloc(&c->tq[0], qbytes) != cudaSuccess || cudaMalloc(&c->tq[1], qbytes) != cudaSuccess) {
             cudaGetLastError();

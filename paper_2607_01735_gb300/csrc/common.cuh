@@ -65,7 +65,17 @@ inline Geometry make_geometry(int n) { return Geometry{n, colour_width(n), n + 2
 // Residual reduction scratch: one partial sum per thread block.
 constexpr int kMaxPartials = 8192;
 
-struct Ctx;
+// Tiles of the resident kernel (resident.cu): gx x gy of them, each of at most rows rows and
+// vals values of a colour row, `period` sweeps between exchanges.  rows == 0: does not fit.
+struct ResidentPlan {
+    int gx, gy, rows, vals, period;
+};
+
+struct ResidentState {
+    ResidentPlan plan;
+    unsigned long long *slots;  // exchange slots (NULL: the kernel is not used)
+    unsigned *epoch;            // [0] number of the last period, [1] scratch
+};
 
 }  // namespace rbgs
 
@@ -114,6 +124,8 @@ struct rbgs_ctx {
     // fused wavefront (wavefront.cu): the black values on the fixed-point grid between passes,
     // two buffers; NULL when the half-sweeps run one launch per colour
     int64_t *tq[2];
+    // resident kernel: FP64 or fused sweeps, FP32 inner sweeps
+    rbgs::ResidentState res64, res32;
     // rbgs_run_stream: double-buffered natural-layout device staging of the inputs (f, u) and
     // of the solution, one copy stream per direction, their events, and per-problem sums
     double *sin_f[2], *sin_u[2], *sout[2];
@@ -151,6 +163,13 @@ rbgs_status launch_wavefront_passes(ColourField<T> &fld, int k, long passes, cud
 template <typename T>
 rbgs_status launch_persistent_sweeps(ColourField<T> &fld, long nsweeps, unsigned *counter, int *status,
                                      cudaStream_t s);
+// all sweeps of a small grid in one cooperative launch, tiles in shared memory (resident.cu).
+// kind 0: FP64, 1: FP32 inner sweeps, 2: fused.  nsweeps >= 2
+ResidentPlan resident_plan(int n, int kind);
+size_t resident_slot_bytes(int n, int W, int kind);
+rbgs_status launch_resident_sweeps_f64(const rbgs_ctx *c, long nsweeps, cudaStream_t s);
+rbgs_status launch_resident_sweeps_f32(const rbgs_ctx *c, long nsweeps, cudaStream_t s);
+rbgs_status launch_resident_sweeps_fused(const rbgs_ctx *c, long nsweeps, cudaStream_t s);
 // FP32 inner sweeps in one launch of one thread-block cluster, d held in its shared memory
 // (cluster_sweeps.cu); usable when d of an n^2 grid with row pitch W fits the cluster
 bool cluster_sweeps_f32_fit(int n, int W);

@@ -1,0 +1,407 @@
+// Many sweeps of a small grid in one cooperative launch, each block's tile held in shared memory.
+//
+// On a small grid a half-sweep is less work than a launch or a grid barrier (about 2 us each).
+// Here the grid is cut into tiles, one per block and SM.  A block keeps both colours of its tile
+// and of a halo around it, and h2 f, in shared memory for the whole launch.  A period of K
+// sweeps (2K half-sweeps of Eq. (1), red then black) runs inside the block: half-sweep s updates
+// the tile plus a margin that shrinks from 2K - 1 rows (and as many columns) to none, so what
+// the tile ends with is exact, and only the block barrier separates the colours.  After a period
+// a block needs its halo's black values again (the red ones are recomputed), 2K rows and K values
+// of a colour row deep, from its eight neighbours: no wait on any other block.
+//
+// Exchange: a slot of global memory per black point and parity of the period.  A value travels
+// with the period's number in the same 64-bit word (a binary64 or int64 value as two words, a
+// binary32 value as one), so a reader that finds the number has the value: no fences, no flags,
+// one trip through L2.  Two parities suffice: a block writes the slots of period q + 2 only after
+// it has read its neighbours' period q + 1 values, which they wrote after reading its period q
+// ones.  The numbers continue from launch to launch (the last block to finish advances them in
+// device memory), so nothing is cleared, and a captured launch can be replayed.  Every wait is
+// bounded: after kPolls polls, or when another block has given up, the block records a status
+// and leaves; the host reports it as RBGS_ETIMEOUT at its next synchronising call.
+//
+// Tile and period: chosen per grid size from a model of the three costs (plan below): the
+// updates of the shrinking regions, a fixed cost per half-sweep (the chain of dependent
+// operations and the block barrier), and the exchange.
+//
+// Measured, a sweep, against what ran before (cached graphs of one launch per colour, or one
+// cooperative launch with a grid barrier per colour): FP64 127^2 1.1 us (3.9), 255^2 1.7 (4.0),
+// 511^2 3.4 (6.4), 1023^2 9.7 (14.1), 1190^2 12.9 (19.4); fused 255^2 1.3 us (4.4), 1023^2 4.3
+// (7.2 as wavefront passes); FP32 255^2 0.8 us (3.1), 511^2 1.2 (3.3), 1000^2 2.8 (3.9).  What
+// bounds it: from about 700^2 the FP64 pipe (74% of its rate at 1023^2, the shrinking margins
+// included), below the chain of a half-sweep and the exchange, about 1 us together.
+//
+// Three kinds of values, as in wavefront.cu: double (bit-exact FP64), float (inner sweeps of the
+// refinement) and int64 (the fused update on its block's fixed-point grid; the iterate is
+// converted as it is loaded, and the last sweep's sums are written as binary64).  Each equals
+// one launch per colour bit for bit.
+#include <type_traits>
+
+#include "common.cuh"
+#include "fixed64.cuh"
+#include "fp64.cuh"
+#include "sweep_impl.cuh"
+
+namespace rbgs {
+namespace {
+
+constexpr int kRThreads = 512;
+constexpr uint32_t kRPolls = 1u << 22;
+constexpr int kMaxPeriod = 8;       // sweeps per period at most
+constexpr int kSmemMax = 220 * 1024;
+constexpr unsigned long long kNoScale = 0x8000000000000000ull;  // fused: no valid scale
+
+template <typename T>
+struct ResTypes {
+    using S = T;  // type of the iterate in global memory
+};
+template <>
+struct ResTypes<int64_t> {
+    using S = double;
+};
+
+template <typename T>
+struct RArgs {
+    using S = typename ResTypes<T>::S;
+    S *u0, *u1;
+    const T *hf0, *hf1;
+    const unsigned long long *words;  // fused: [2] the block's scale
+    unsigned long long *slots;        // [parity][row W + k]: 1 (float) or 2 words each
+    unsigned *epoch;                  // [0] number of the last period, [1] blocks that have finished
+    int *status;
+    int n, W, kmax, kint;             // values of a colour row holding columns 0..n+1, 1..n
+    int gx, gy, period;               // tiles; K
+    int pitch, erows;                 // values per row and rows of the tile with its halo
+    long long sweeps;
+    double one;
+};
+
+// The region a half-sweep updates when its margin is e rows: rows i0.., values k0.. (w of them)
+struct Region {
+    int i0, k0, w, items;
+    unsigned mul;  // ceil(2^32 / w): item / w = umulhi(item, mul) while item w < 2^32
+};
+
+__device__ __forceinline__ float r_update(float hf, float vn, float vs, float vw, float ve, double) {
+    float s = __fadd_rn(hf, vn);
+    s = __fadd_rn(s, vs);
+    s = __fadd_rn(s, vw);
+    s = __fadd_rn(s, ve);
+    return __fmul_rn(s, 0.25f);
+}
+__device__ __forceinline__ double r_update(double hf, double vn, double vs, double vw, double ve, double one) {
+    return update_f64<false>(0, hf, vn, vs, vw, ve, one);
+}
+
+__device__ __forceinline__ void put(unsigned long long *slot, uint64_t bits, unsigned seq) {
+    const unsigned long long s = (unsigned long long)seq << 32;
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(slot), "l"(s | (uint32_t)bits),
+                 "l"(s | (uint32_t)(bits >> 32))
+                 : "memory");
+}
+__device__ __forceinline__ void put(unsigned long long *slot, uint32_t bits, unsigned seq) {
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(slot), "l"(((unsigned long long)seq << 32) | bits)
+                 : "memory");
+}
+// true when the slot holds period seq's value, then in `bits`
+__device__ __forceinline__ bool get(const unsigned long long *slot, uint64_t &bits, unsigned seq) {
+    unsigned long long a, b;
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(slot) : "memory");
+    bits = (uint64_t)(uint32_t)a | ((uint64_t)(uint32_t)b << 32);
+    return (unsigned)(a >> 32) == seq && (unsigned)(b >> 32) == seq;
+}
+__device__ __forceinline__ bool get(const unsigned long long *slot, uint32_t &bits, unsigned seq) {
+    unsigned long long a;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(a) : "l"(slot) : "memory");
+    bits = (uint32_t)a;
+    return (unsigned)(a >> 32) == seq;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const RArgs<T> a) {
+    using S = typename ResTypes<T>::S;
+    using Bits = typename std::conditional<sizeof(T) == 8, uint64_t, uint32_t>::type;
+    constexpr bool FUSED = std::is_same<T, int64_t>::value;
+    constexpr int kWords = sizeof(T) / 4;  // 64-bit words per slot
+    extern __shared__ __align__(16) unsigned char r_shared[];
+    __shared__ Region regions[2 * kMaxPeriod];
+    __shared__ int s_nrcv, s_abort;
+    const int tid = threadIdx.x;
+    const int n = a.n, W = a.W, kmax = a.kmax, K = a.period, pitch = a.pitch;
+    const int ty = blockIdx.x / a.gx, tx = blockIdx.x % a.gx;
+    // the tile's rows and values (balanced: sizes differ by one at most)
+    const int ra = 1 + ty * n / a.gy, rb = 1 + (ty + 1) * n / a.gy;
+    const int ka = tx * a.kint / a.gx, kb = (tx + 1) * a.kint / a.gx;
+    const int ibase = ra - 2 * K, kbase = ka - K - 1;  // grid place of shared element 0
+    const int plane = a.erows * pitch;                 // elements of one colour
+    T *su = reinterpret_cast<T *>(r_shared);           // u: red, black; then h2 f: red, black
+    T *sf = su + 2 * plane;
+    int2 *rcv = reinterpret_cast<int2 *>(sf + 2 * plane);  // halo points: {shared element, grid element}
+
+    if (*reinterpret_cast<volatile int *>(a.status) != 0) return;  // a wait of an earlier launch gave up
+    unsigned long long ew = 0;
+    if (FUSED) ew = a.words[2];
+    const bool ok_scale = ew != kNoScale;
+    const int e2 = ok_scale ? (int)(long long)ew : 0;
+    const unsigned seq0 = *reinterpret_cast<volatile unsigned *>(a.epoch);
+    if (tid == 0) s_nrcv = 0, s_abort = 0;
+    if (tid < 2 * K) {
+        const int e = tid, ek = (e + 1) >> 1;
+        Region r;
+        r.i0 = max(1, ra - e);
+        r.k0 = max(0, ka - ek);
+        r.w = min(a.kint, kb + ek) - r.k0;
+        r.items = (min(n, rb - 1 + e) - r.i0 + 1) * r.w;
+        r.mul = 0xFFFFFFFFu / (unsigned)r.w + 1u;
+        regions[e] = r;
+    }
+    __syncthreads();
+    for (int q = tid; q < plane; q += kRThreads) {
+        const int i = ibase + q / pitch, k = kbase + q % pitch;
+        T v0 = T(0), v1 = T(0), f0 = T(0), f1 = T(0);
+        if (i >= 0 && i <= n + 1 && k >= 0 && k < kmax) {
+            const size_t at = (size_t)i * W + k;
+            if constexpr (FUSED) {
+                if (ok_scale) v0 = to_fixed(a.u0[at], e2), v1 = to_fixed(a.u1[at], e2);
+            } else {
+                v0 = a.u0[at], v1 = a.u1[at];
+            }
+            f0 = a.hf0[at], f1 = a.hf1[at];
+            // a black point of the halo, inside the ring and outside the tile: received each period
+            const int j = 2 * k + ((i + 1) & 1);
+            if (i >= 1 && i <= n && i < rb + 2 * K && j >= 1 && j <= n && k >= ka - K && k < kb + K &&
+                !(i >= ra && i < rb && k >= ka && k < kb))
+                rcv[atomicAdd(&s_nrcv, 1)] = make_int2(plane + q, (int)at);
+        }
+        su[q] = v0, su[plane + q] = v1;
+        sf[q] = f0, sf[plane + q] = f1;
+    }
+    __syncthreads();
+    const int nrcv = s_nrcv;
+    const size_t parity_words = (size_t)(n + 2) * W * kWords;
+
+    // one half-sweep of colour c with margin e; publish: the tile's outgoing black values with
+    // number seq; final: fused only, the sums leave as binary64
+    auto half_sweep = [&](int c, int e, bool publish, unsigned seq, bool final) {
+        const Region r = regions[e];
+        T *self = su + c * plane;
+        const T *other = su + (c ^ 1) * plane;
+        const T *f = sf + c * plane;
+        unsigned long long *slots = a.slots + (seq & 1u) * parity_words;
+        for (int base = 0; base < r.items; base += kRThreads) {
+            if (base + (tid & ~31) >= r.items) break;  // warp-uniform: no item left for this warp
+            const bool act = base + tid < r.items;
+            const int item = act ? base + tid : base;
+            const int row = r.w == 1 ? item : (int)__umulhi((unsigned)item, r.mul);
+            const int i = r.i0 + row, k = r.k0 + (item - row * r.w);
+            const int p = (i + c) & 1, j = 2 * k + p;
+            const int q = (i - ibase) * pitch + (k - kbase);
+            const bool in = act && j >= 1 && j <= n;
+            T v;
+            if constexpr (FUSED) {
+                const int64_t s = f[q] + other[q - pitch] + other[q + pitch] + other[q - 1 + p] + other[q + p];
+                v = fixed_quarter(s);
+                if (final && in && i >= ra && i < rb && k >= ka && k < kb)
+                    (c ? a.u1 : a.u0)[(size_t)i * W + k] =
+                        ok_scale ? fixed_quarter_to_double(s, e2) : __longlong_as_double(0x7FF8000000000000ll);
+            } else {
+                v = r_update(f[q], other[q - pitch], other[q + pitch], other[q - 1 + p], other[q + p], a.one);
+            }
+            if (in) {
+                self[q] = v;
+                // the margin is 0 here, so (i, k) is in the tile: its outer 2K rows and K values
+                if (publish && (i < ra + 2 * K || i >= rb - 2 * K || k < ka + K || k >= kb - K)) {
+                    Bits b;
+                    __builtin_memcpy(&b, &v, sizeof(T));
+                    put(slots + ((size_t)i * W + k) * kWords, b, seq);
+                }
+            }
+        }
+        __syncthreads();
+    };
+
+    unsigned seq = seq0;
+    long long left = a.sweeps;
+    // a launch of several tiles has at least two periods: a tile's result is written over the
+    // iterate only after every neighbour has loaded (it has received their first period)
+    int kk = (int)(left > K ? K : gridDim.x > 1 ? (left + 1) / 2 : left);
+    while (left > 0) {
+        left -= kk;
+        ++seq;
+        for (int s = 0; s < kk; ++s) {
+            const bool last = left == 0 && s == kk - 1;
+            half_sweep(0, 2 * (kk - s) - 1, false, seq, last);
+            half_sweep(1, 2 * (kk - s) - 2, left > 0 && s == kk - 1 && gridDim.x > 1, seq, last);
+        }
+        if (left == 0) break;
+        kk = (int)(left < K ? left : K);
+        // the halo's black values of this period
+        const unsigned long long *slots = a.slots + (seq & 1u) * parity_words;
+        for (int base = 0; base < nrcv; base += 4 * kRThreads) {
+            unsigned pend = 0;
+            int2 ent[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int at = base + tid + q * kRThreads;
+                if (at < nrcv) ent[q] = rcv[at], pend |= 1u << q;
+            }
+            uint32_t polls = 0;
+            while (pend) {
+                Bits b[4];
+                bool hit[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) hit[q] = ((pend >> q) & 1u) && get(slots + (size_t)ent[q].y * kWords, b[q], seq);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (hit[q]) {
+                        __builtin_memcpy(&su[ent[q].x], &b[q], sizeof(T));
+                        pend &= ~(1u << q);
+                    }
+                }
+                if (pend && (++polls >= kRPolls || ((polls & 1023u) == 0 && *reinterpret_cast<volatile int *>(a.status) != 0))) {
+                    atomicOr(a.status, 2);
+                    s_abort = 1;
+                    break;
+                }
+            }
+        }
+        __syncthreads();
+        if (s_abort) return;
+    }
+    if constexpr (!FUSED) {
+        for (int q = tid; q < plane; q += kRThreads) {
+            const int i = ibase + q / pitch, k = kbase + q % pitch;
+            if (i < ra || i >= rb || k < ka || k >= kb) continue;
+            const size_t at = (size_t)i * W + k;
+            const int j = 2 * k + (i & 1);  // red; black is the other column of the pair
+            if (j >= 1 && j <= n) a.u0[at] = su[q];
+            const int jb = 2 * k + ((i + 1) & 1);
+            if (jb >= 1 && jb <= n) a.u1[at] = su[plane + q];
+        }
+    }
+    // the last block to finish advances the period number for the next launch
+    if (tid == 0 && atomicAdd(&a.epoch[1], 1u) == gridDim.x - 1) {
+        a.epoch[1] = 0;
+        a.epoch[0] = seq;
+    }
+}
+
+int device_sms() {
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            v = 0;
+        }
+        return v;
+    }();
+    return sms;
+}
+
+template <typename T>
+size_t resident_smem(int rows, int vals, int K) {
+    const size_t pts = (size_t)(rows + 4 * K) * (vals + 2 * K + 2);
+    const size_t halo = (size_t)4 * K * (vals + 2 * K) + (size_t)2 * K * rows;
+    return pts * 4 * sizeof(T) + halo * sizeof(int2);
+}
+
+// Cycles of the model, per type: an update per SM, a half-sweep's chain and barrier, an exchange.
+// With them the model's period is within 5% of the best one measured (periods 1 to 8 forced, a
+// sweep at 63 / 127 / 255 / 511 / 1023^2: FP64 best at 3 / 3 / 2 / 2 / 2, fused 4 / 3 / 3 / 2 / 2,
+// FP32 4 / 3 / 4 / 4 / 3).
+template <typename T>
+struct Costs {
+    static constexpr double update = 2.3, chain = 450, exchange = 1900;  // FP64: 4 adds at 2 per clock
+};
+template <>
+struct Costs<float> {
+    static constexpr double update = 0.5, chain = 300, exchange = 1900;
+};
+template <>
+struct Costs<int64_t> {
+    static constexpr double update = 0.9, chain = 400, exchange = 1900;
+};
+
+template <typename T>
+ResidentPlan plan_for(int n) {
+    ResidentPlan best{};
+    double best_cost = 0.0;
+    const int kint = n / 2 + 1, sms = device_sms();
+    for (int K = 1; K <= kMaxPeriod; ++K) {
+        for (int gx = 1; gx <= sms && gx <= kint; ++gx) {
+            int gy = sms / gx;
+            if (n / gy < 2 * K) gy = n / (2 * K) > 1 ? n / (2 * K) : 1;
+            const int vals = (kint + gx - 1) / gx, rows = (n + gy - 1) / gy;
+            // A halo reaches no further than the next tile; and every tile has a black interior
+            // point to send to each of its neighbours, so that no tile runs ahead of one that
+            // has yet to read from it: 2K rows hold both parities, and two values of which the
+            // inner one is no ring value in either.
+            if (gx > 1 && kint / gx < (K > 2 ? K : 2)) continue;
+            if (resident_smem<T>(rows, vals, K) > (size_t)kSmemMax) continue;
+            double cost = gx * gy > 1 ? Costs<T>::exchange : 0.0;
+            for (int e = 0; e < 2 * K; ++e) {
+                const int m = gy > 1 ? 2 * e : 0, mk = gx > 1 ? 2 * ((e + 1) / 2) : 0;
+                cost += Costs<T>::chain + Costs<T>::update * (rows + m) * (vals + mk);
+            }
+            cost /= K;
+            if (best.rows == 0 || cost < best_cost) {
+                best_cost = cost;
+                best = ResidentPlan{gx, gy, rows, vals, K};
+            }
+        }
+    }
+    return best;
+}
+
+template <typename T>
+rbgs_status run_resident(RArgs<T> &a, const ResidentPlan &pl, long nsweeps, cudaStream_t s) {
+    const size_t smem = resident_smem<T>(pl.rows, pl.vals, pl.period);
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(resident_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+    RBGS_CUDA(attr);
+    a.gx = pl.gx, a.gy = pl.gy, a.period = pl.period;
+    a.pitch = pl.vals + 2 * pl.period + 2, a.erows = pl.rows + 4 * pl.period;
+    a.sweeps = nsweeps;
+    a.one = 1.0;
+    void *args[] = {&a};
+    RBGS_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(resident_kernel<T>), dim3(pl.gx * pl.gy),
+                                          dim3(kRThreads), args, smem, s));
+    return RBGS_OK;
+}
+
+template <typename T>
+RArgs<T> base_args(const rbgs_ctx *c, int W, const ResidentState &r) {
+    RArgs<T> a{};
+    a.n = c->g.n, a.W = W, a.kmax = (c->g.n + 3) / 2, a.kint = c->g.n / 2 + 1;
+    a.slots = r.slots, a.epoch = r.epoch, a.status = c->dstatus;
+    return a;
+}
+
+}  // namespace
+
+ResidentPlan resident_plan(int n, int kind) {
+    return kind == 0 ? plan_for<double>(n) : kind == 1 ? plan_for<float>(n) : plan_for<int64_t>(n);
+}
+
+size_t resident_slot_bytes(int n, int W, int kind) { return (size_t)2 * (n + 2) * W * (kind == 1 ? 8 : 16); }
+
+rbgs_status launch_resident_sweeps_f64(const rbgs_ctx *c, long nsweeps, cudaStream_t s) {
+    RArgs<double> a = base_args<double>(c, c->g.W, c->res64);
+    a.u0 = c->f64.u[0], a.u1 = c->f64.u[1], a.hf0 = c->f64.hf[0], a.hf1 = c->f64.hf[1];
+    return run_resident(a, c->res64.plan, nsweeps, s);
+}
+
+rbgs_status launch_resident_sweeps_fused(const rbgs_ctx *c, long nsweeps, cudaStream_t s) {
+    RArgs<int64_t> a = base_args<int64_t>(c, c->g.W, c->res64);
+    a.u0 = c->f64.u[0], a.u1 = c->f64.u[1], a.hf0 = c->hq[0], a.hf1 = c->hq[1];
+    a.words = c->fwords;
+    return run_resident(a, c->res64.plan, nsweeps, s);
+}
+
+rbgs_status launch_resident_sweeps_f32(const rbgs_ctx *c, long nsweeps, cudaStream_t s) {
+    RArgs<float> a = base_args<float>(c, c->f32.W, c->res32);
+    a.u0 = c->f32.u[0], a.u1 = c->f32.u[1], a.hf0 = c->f32.hf[0], a.hf1 = c->f32.hf[1];
+    return run_resident(a, c->res32.plan, nsweeps, s);
+}
+
+}  // namespace rbgs
