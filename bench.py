@@ -52,8 +52,8 @@ PROFILES = {
                                    "paper_2607_01735_gb300/csrc/sweep_impl.cuh",
                                    "paper_2607_01735_gb300/csrc/fp64.cuh"]),
 }
-RESIDENT_MAX_N = 1376  # tiles in shared memory up to here; one cooperative launch with a grid barrier above
-PERSIST_MIN_N, PERSIST_MAX_N = RESIDENT_MAX_N + 1, 1 << 15
+PERSIST_MIN_N, PERSIST_MAX_N = 416, 1 << 15
+RESIDENT_MAX_N = 1376  # tiles in shared memory up to here (GB300: 152 SMs)
 # side files of a run (nvidia-smi clock samples, trained U-Net parameters)
 OUT_DIR = os.environ.get("RBGS_BENCH_OUT", os.path.join(ROOT, "bench_out"))
 
@@ -1012,7 +1012,7 @@ def main():
             kernel, kdepth = (3, 3) if fused_wavefront(margs, n) else (1, 1)
         blocked = kernel in (2, 3)  # several sweeps per launch (TMA tiles or register wavefront)
         resident = uses_resident(margs, n, refine)
-        persistent = uses_persistent(margs, n, refine)
+        persistent = not resident and uses_persistent(margs, n, refine)
         # pack f, pack u, ||b|| (2), the sweeps, residual, unpack.  The residual after
         # bit-exact FP64 sweeps walks the red points only (2 launches: the black rt is exactly
         # zero), else both colours (3)
