@@ -123,8 +123,7 @@ rbgs_status load_problem(rbgs_ctx *c, const double *f, const double *u_init) {
     }
     if ((st = stage_in(c, u_init, (size_t)g.rows * g.rows, &uview)) != RBGS_OK) return st;
     if ((st = enqueue_pack(c, fview, uview)) != RBGS_OK) return st;
-    RBGS_CUDA(cudaMemcpyAsync(c->hsum + 1, c->dsum + 1, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    RBGS_CUDA(cudaStreamSynchronize(c->stream));
+    RBGS_CUDA(cudaStreamSynchronize(c->stream));  // the reduction wrote hsum[1]
     c->den2 = c->hsum[1];
     return RBGS_OK;
 }
@@ -235,15 +234,26 @@ rbgs_status ensure_f32(rbgs_ctx *c) {
     return RBGS_OK;
 }
 
+rbgs_status status_error(int status) {
+    if (status) {
+        set_error("a bounded device-side wait timed out (status %d)", status);
+        return RBGS_ETIMEOUT;
+    }
+    return RBGS_OK;
+}
+
 // A bounded device-side wait gave up in an earlier launch?  (Reads after a stream sync.)
 rbgs_status check_device_status(rbgs_ctx *c) {
     RBGS_CUDA(cudaMemcpyAsync(c->hstatus, c->dstatus, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     RBGS_CUDA(cudaStreamSynchronize(c->stream));
-    if (*c->hstatus) {
-        set_error("a bounded device-side wait timed out (status %d)", *c->hstatus);
-        return RBGS_ETIMEOUT;
-    }
-    return RBGS_OK;
+    return status_error(*c->hstatus);
+}
+
+// Waits for a residual reduction, whose last block has written its sums and the device status
+// into hsum (page-locked: no copies).
+rbgs_status finish_residual(rbgs_ctx *c) {
+    RBGS_CUDA(cudaStreamSynchronize(c->stream));
+    return status_error((int)c->hsum[3]);
 }
 
 rbgs_status enqueue_sweeps(rbgs_ctx *c, long nsweeps, cudaStream_t s) {
@@ -338,8 +348,7 @@ rbgs_status sweeps_f64(rbgs_ctx *c, long nsweeps) {
 rbgs_status defect_stats(rbgs_ctx *c, double *rho, double *mx) {
     rbgs_status st = launch_defect(c, false, 1.0, c->stream);
     if (st != RBGS_OK) return st;
-    RBGS_CUDA(cudaMemcpyAsync(c->hsum, c->dsum, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    if ((st = check_device_status(c)) != RBGS_OK) return st;
+    if ((st = finish_residual(c)) != RBGS_OK) return st;
     const double r2 = c->hsum[0];
     *mx = c->hsum[2];
     *rho = c->den2 > 0.0 ? std::sqrt(r2) / std::sqrt(c->den2) : std::sqrt(r2);
@@ -634,7 +643,7 @@ rbgs_status rbgs_create(int n, double h2, const double *f, const double *u_init,
     ok = ok && cudaMalloc(&c->partials, 2 * kMaxPartials * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->dsum, 4 * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->dstatus, sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->pcounter, sizeof(unsigned)) == cudaSuccess;
+    ok = ok && cudaMalloc(&c->pcounter, 3 * sizeof(unsigned)) == cudaSuccess;
     ok = ok && cudaMallocHost(&c->hsum, 4 * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMallocHost(&c->hstatus, sizeof(int)) == cudaSuccess;
     for (int q = 0; q < 2 && ok && c->fused; ++q) ok = cudaMalloc(&c->hq[q], c->g.colour_elems() * sizeof(int64_t)) == cudaSuccess;
@@ -657,7 +666,8 @@ rbgs_status rbgs_create(int n, double h2, const double *f, const double *u_init,
             c->tq[0] = c->tq[1] = nullptr;
         }
     }
-    ok = ok && cudaMemsetAsync(c->dstatus, 0, sizeof(int), c->stream) == cudaSuccess;
+    ok = ok && cudaMemsetAsync(c->dstatus, 0, sizeof(int), c->stream) == cudaSuccess &&
+         cudaMemsetAsync(c->pcounter, 0, 3 * sizeof(unsigned), c->stream) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         free_ctx(c);
@@ -698,8 +708,7 @@ rbgs_status rbgs_residual(rbgs_t c, double *rel) {
     if (!c || !rel) { set_error("ctx and rel must not be NULL"); return RBGS_EINVAL; }
     rbgs_status st = launch_residual_sum(c, c->stream);
     if (st != RBGS_OK) return st;
-    RBGS_CUDA(cudaMemcpyAsync(c->hsum, c->dsum, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    if ((st = check_device_status(c)) != RBGS_OK) return st;
+    if ((st = finish_residual(c)) != RBGS_OK) return st;
     const double r2 = c->hsum[0];
     *rel = c->den2 > 0.0 ? std::sqrt(r2) / std::sqrt(c->den2) : std::sqrt(r2);
     if (!std::isfinite(*rel)) {

@@ -114,7 +114,8 @@ struct rbgs_ctx {
     int inner_sweeps;           // resolved FP32 sweeps per correction
     int kernel32;               // resolved inner kernel for the FP32 sweeps
     int *hstatus;               // pinned host mirror of dstatus
-    unsigned *pcounter;         // device: grid-barrier counter of the cooperative sweep launch
+    unsigned *pcounter;         // device: [0] grid-barrier counter of the cooperative sweep launch,
+                                // [1], [2] tickets of the residual and right-hand-side reductions
     bool black_fresh;           // the FP64 iterate is the result of a full sweep (black rt == 0)
     // fused FP64 update (opts.fma = 1): h2 f on the fixed-point grid of the current block of
     // sweeps, per colour, and [0] max |u| bits, [1] max |h2 f| bits, [2] the block's scale e

@@ -14,22 +14,33 @@ namespace rbgs {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kRows = 4;  // rows per block
 
+// A thread takes the pair of elements k, k + 1 of both colour rows: 16-byte loads and stores of u
+// and 8-byte loads of d (element by element at the ring columns).
 __global__ void __launch_bounds__(kThreads)
 correct_kernel(double *__restrict__ red, double *__restrict__ black, const float *__restrict__ d_red,
                const float *__restrict__ d_black, int n, int W, int W32, double scale) {
-    const int k = blockIdx.x * kThreads + threadIdx.x;
+    const int k = 2 * (blockIdx.x * kThreads + threadIdx.x);
     if (k > (n + 1) / 2) return;
-    for (int i = 1 + blockIdx.y; i <= n; i += gridDim.y) {
-        // colour c of row i holds natural column j = 2k + ((i + c) & 1)
+    const bool inner = k > 0 && 2 * k + 3 <= n;  // columns 2k .. 2k + 3 are all interior
+    for (int g = blockIdx.y; g * kRows < n; g += gridDim.y) {
+        for (int i = 1 + g * kRows; i <= min(n, g * kRows + kRows); ++i) {
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int j = 2 * k + ((i + c) & 1);
-            if (j < 1 || j > n) continue;
-            double *u = c ? black : red;
-            const float *d = c ? d_black : d_red;
-            const size_t q = (size_t)i * W + k;
-            u[q] = __dadd_rn(u[q], __dmul_rn((double)d[(size_t)i * W32 + k], scale));
+            for (int c = 0; c < 2; ++c) {
+                double *u = (c ? black : red) + (size_t)i * W + k;
+                const float2 d = __ldg(reinterpret_cast<const float2 *>((c ? d_black : d_red) + (size_t)i * W32 + k));
+                double2 v = *reinterpret_cast<const double2 *>(u);
+                v.x = __dadd_rn(v.x, __dmul_rn((double)d.x, scale));
+                v.y = __dadd_rn(v.y, __dmul_rn((double)d.y, scale));
+                if (inner) {
+                    *reinterpret_cast<double2 *>(u) = v;
+                } else {
+                    const int j = 2 * k + ((i + c) & 1);  // natural column of element k
+                    if (j >= 1 && j <= n) u[0] = v.x;
+                    if (j + 2 <= n) u[1] = v.y;
+                }
+            }
         }
     }
 }
@@ -38,9 +49,9 @@ correct_kernel(double *__restrict__ red, double *__restrict__ black, const float
 
 rbgs_status launch_correct(const rbgs_ctx *c, double scale, cudaStream_t s) {
     const int n = c->g.n;
-    const int kmax = (n + 1) / 2 + 1;
-    int gy = n < 65535 ? n : 65535;
-    dim3 grid((kmax + kThreads - 1) / kThreads, gy);
+    const int pairs = (n + 1) / 4 + 1;  // pairs that hold an element up to (n + 1) / 2
+    const int gy = (n + kRows - 1) / kRows;
+    dim3 grid((pairs + kThreads - 1) / kThreads, gy < 65535 ? gy : 65535);
     correct_kernel<<<grid, kThreads, 0, s>>>(c->f64.u[0], c->f64.u[1], c->f32.u[0], c->f32.u[1], n, c->g.W,
                                              c->f32.W, scale);
     RBGS_LAUNCH_CHECK();

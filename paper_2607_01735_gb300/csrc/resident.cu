@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const RArgs<T> a
     __shared__ Region regions[2 * kMaxPeriod];
     __shared__ int s_nrcv, s_abort;
     const int tid = threadIdx.x;
+    const double one = a.one;
     const int n = a.n, W = a.W, kmax = a.kmax, K = a.period, pitch = a.pitch;
     const int ty = blockIdx.x / a.gx, tx = blockIdx.x % a.gx;
     // the tile's rows and values (balanced: sizes differ by one at most)
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const RArgs<T> a
                     (c ? a.u1 : a.u0)[(size_t)i * W + k] =
                         ok_scale ? fixed_quarter_to_double(s, e2) : __longlong_as_double(0x7FF8000000000000ll);
             } else {
-                v = r_update(f[q], other[q - pitch], other[q + pitch], other[q - 1 + p], other[q + p], a.one);
+                v = r_update(f[q], other[q - pitch], other[q + pitch], other[q - 1 + p], other[q + p], one);
             }
             if (in) {
                 self[q] = v;
@@ -305,21 +306,21 @@ size_t resident_smem(int rows, int vals, int K) {
     return pts * 4 * sizeof(T) + halo * sizeof(int2);
 }
 
-// Cycles of the model, per type: an update per SM, a half-sweep's chain and barrier, an exchange.
-// With them the model's period is within 5% of the best one measured (periods 1 to 8 forced, a
-// sweep at 63 / 127 / 255 / 511 / 1023^2: FP64 best at 3 / 3 / 2 / 2 / 2, fused 4 / 3 / 3 / 2 / 2,
-// FP32 4 / 3 / 4 / 4 / 3).
+// Cycles of the model, per type: a warp's update of 32 points on its quarter of an SM (FP64: four
+// adds at half a lane per clock), a half-sweep's chain and barrier, an exchange.  A region of
+// items takes as long as the quarter with the most warps, so a plan is better off just below a
+// multiple of 128 items.  Fitted to sweeps at 63^2 and 1023^2 with the period forced to 1 to 4.
 template <typename T>
 struct Costs {
-    static constexpr double update = 2.3, chain = 450, exchange = 1900;  // FP64: 4 adds at 2 per clock
+    static constexpr double warp = 300, chain = 500, exchange = 1600;
 };
 template <>
 struct Costs<float> {
-    static constexpr double update = 0.5, chain = 300, exchange = 1900;
+    static constexpr double warp = 76, chain = 250, exchange = 1900;
 };
 template <>
 struct Costs<int64_t> {
-    static constexpr double update = 0.9, chain = 400, exchange = 1900;
+    static constexpr double warp = 117, chain = 590, exchange = 1550;
 };
 
 template <typename T>
@@ -341,7 +342,8 @@ ResidentPlan plan_for(int n) {
             double cost = gx * gy > 1 ? Costs<T>::exchange : 0.0;
             for (int e = 0; e < 2 * K; ++e) {
                 const int m = gy > 1 ? 2 * e : 0, mk = gx > 1 ? 2 * ((e + 1) / 2) : 0;
-                cost += Costs<T>::chain + Costs<T>::update * (rows + m) * (vals + mk);
+                const int warps = ((rows + m) * (vals + mk) + 31) / 32;
+                cost += Costs<T>::chain + Costs<T>::warp * ((warps + 3) / 4);
             }
             cost /= K;
             if (best.rows == 0 || cost < best_cost) {

@@ -1,11 +1,15 @@
 // Residual-norm reduction (the convergence test of the solver).
 //
 // For every interior point, rt = ((((h2f + N) + S) + W) + E) - 4 u equals h^2 (b - A u)
-// for the linear system of Eq. (1) with the ring folded into b.  The kernels walk the
-// colour-split grid the same way the half-sweeps do (strip of rows per block, other
-// colour's rows i-1, i, i+1 in registers), square each rt and reduce: warp shuffle,
-// then the block, then one partial per block; a single-block kernel adds the partials
-// in a fixed order.  The result is the same on every run.
+// for the linear system of Eq. (1) with the ring folded into b.  One kernel walks strips of rows
+// of the colour-split grid as the half-sweeps do (the other colour's rows i-1, i, i+1 in
+// registers), squares each rt and reduces: warp shuffle, then the block; the last block to
+// finish adds the blocks' partials in a fixed order and writes the results to the device and to
+// page-locked host memory, so a residual is one launch and a wait.  The result is the same on
+// every run.  Measured with the wait: 127^2 16 us (one launch per colour, a final sum and two
+// copies: 32-44), 511^2 20-24 us (30-45), 16384^2 2.91 ms for both colours (3.00), the FP64
+// pipe 93% busy there.  One value's chain of dependent operations after the other, each behind
+// its own test: with the two values' chains interleaved the pipe was 84% busy.
 //
 // The adds run as fused multiply-adds by a run-time 1.0 (one rounding of the exact sum,
 // the same value as the add, on GB300's faster-issuing DFMA path), and rt as
@@ -32,91 +36,150 @@
 namespace rbgs {
 namespace {
 
-constexpr int kFinalThreads = 1024;
+constexpr int kAhead = 8;  // partials loaded at once by the finishing block
 
-// MAX: also reduce max |rt| (into partials[kMaxPartials + block]).  WRITE: also store
-// (float)(rt * scale) into the FP32 colour array r32 (pitch W32) at interior points: the
-// scaled defect that the mixed-precision refinement hands to its FP32 inner solver.
-template <int COLOUR, bool MAX, bool WRITE>
-__global__ void __launch_bounds__(kSweepThreads)
-residual_colour_kernel(const double *__restrict__ self, const double *__restrict__ other,
-                       const double *__restrict__ hf, int n, int W, int kact,
-                       int rows_per_block, double *__restrict__ partials, float *__restrict__ r32,
-                       int W32, double scale, double one) {
-    __shared__ double red_smem[kSweepThreads / 32];
-    const int lane = threadIdx.x & 31;
-    const int k0 = 2 * (blockIdx.x * kSweepThreads + threadIdx.x);
-    const bool act = k0 < kact;
-    const int i0 = 1 + blockIdx.y * rows_per_block;
-    const int i1 = min(n, i0 + rows_per_block - 1);
-    const double2 zero = make_double2(0.0, 0.0);
-    double acc = 0.0, mx = 0.0;
-    if (i0 <= n) {
-        double2 up = act ? ldg2(other + (size_t)(i0 - 1) * W + k0) : zero;
-        double2 mid = act ? ldg2(other + (size_t)i0 * W + k0) : zero;
-        for (int i = i0; i <= i1; ++i) {
-            const size_t row = (size_t)i * W;
-            const double2 dn = act ? ldg2(other + row + W + k0) : zero;
-            const double2 f2 = act ? ldg2(hf + row + k0) : zero;
-            const double2 me = act ? ldg2(self + row + k0) : zero;
-            const int p = (i + COLOUR) & 1;
-            double w0, e0, w1, e1;
-            if (p == 0) {
-                double prev = __shfl_up_sync(0xffffffffu, mid.y, 1);
-                if (lane == 0) prev = (act && k0 > 0) ? __ldg(other + row + k0 - 1) : 0.0;
-                w0 = prev; e0 = mid.x; w1 = mid.x; e1 = mid.y;
-            } else {
-                double next = __shfl_down_sync(0xffffffffu, mid.x, 1);
-                if (lane == 31) next = (k0 + 2 < kact) ? __ldg(other + row + k0 + 2) : 0.0;
-                w0 = mid.x; e0 = mid.y; w1 = mid.y; e1 = next;
-            }
-            const int j0 = 2 * k0 + p;
-            if (act && j0 >= 1 && j0 <= n) {
-                const double s = add_fma(add_fma(add_fma(add_fma(f2.x, up.x, one), dn.x, one), w0, one), e0, one);
-                const double r = __fma_rn(-4.0, me.x, s);
-                acc = __fma_rn(r, r, acc);
-                if (MAX) mx = fmax(mx, fabs(r));
-                if (WRITE) r32[(size_t)i * W32 + k0] = __double2float_rn(__dmul_rn(r, scale));
-            }
-            if (act && j0 + 2 <= n) {
-                const double s = add_fma(add_fma(add_fma(add_fma(f2.y, up.y, one), dn.y, one), w1, one), e1, one);
-                const double r = __fma_rn(-4.0, me.y, s);
-                acc = __fma_rn(r, r, acc);
-                if (MAX) mx = fmax(mx, fabs(r));
-                if (WRITE) r32[(size_t)i * W32 + k0 + 1] = __double2float_rn(__dmul_rn(r, scale));
-            }
-            up = mid;
-            mid = dn;
+// The last block of a launch adds all its partials in a fixed order (whichever block is last),
+// so a reduction is one launch.  ticket: zero before the launch, zero again after it.
+// Every block calls this with its own partials written (by thread 0).
+template <int THREADS>
+__device__ __forceinline__ bool last_block(unsigned *ticket, unsigned blocks) {
+    __shared__ bool s_last;
+    if (threadIdx.x == 0) {
+        __threadfence();  // this block's partials before its ticket
+        s_last = atomicAdd(ticket, 1u) == blocks - 1;
+        if (s_last) {
+            *ticket = 0;
+            __threadfence();  // every partial is visible from here on
         }
     }
-    const size_t slot = (size_t)COLOUR * gridDim.x * gridDim.y + (size_t)blockIdx.y * gridDim.x + blockIdx.x;
-    const double t = block_sum<kSweepThreads>(acc, red_smem);
-    if (threadIdx.x == 0) partials[slot] = t;
+    __syncthreads();
+    return s_last;
+}
+
+template <int THREADS>
+__device__ __forceinline__ double sum_partials(const double *partials, int count, double *smem) {
+    double v = 0.0;
+    for (int q = threadIdx.x; q < count; q += kAhead * THREADS) {
+        double t[kAhead];
+#pragma unroll
+        for (int r = 0; r < kAhead; ++r) t[r] = q + r * THREADS < count ? __ldcg(partials + q + r * THREADS) : 0.0;
+#pragma unroll
+        for (int r = 0; r < kAhead; ++r) v = __dadd_rn(v, t[r]);
+    }
+    __syncthreads();
+    return block_sum<THREADS>(v, smem);
+}
+
+template <int THREADS>
+__device__ __forceinline__ double max_partials(const double *partials, int count, double *smem) {
+    double v = 0.0;
+    for (int q = threadIdx.x; q < count; q += THREADS) v = fmax(v, __ldcg(partials + q));
+    __syncthreads();
+    return block_max<THREADS>(v, smem);
+}
+
+struct ResidualArgs {
+    const double *u[2], *hf[2];
+    int n, W, kact;
+    int rows, bx, items, colours;  // strips: rows each, bx of them across, `items` per colour
+    int lanes;                     // blocks that share a colour's strips
+    double *partials;       // sums, then (from kMaxPartials) maxima
+    double *out;            // [0] sum rt^2, [2] max |rt|
+    double *host;           // the same in page-locked host memory, and [3] the device status
+    const int *status;
+    unsigned *ticket;
+    float *r32[2];          // WRITE: FP32 colour arrays of pitch W32
+    int W32;
+    double scale, one;
+};
+
+// MAX: also reduce max |rt|.  WRITE: only store (float)(rt * scale) into the FP32 colour arrays at
+// interior points: the scaled defect that the refinement hands to its FP32 inner solver.
+// Values per thread: PTS neighbouring ones of a colour row.  The grid is one wave of resident
+// blocks, each walking every gridDim.x-th strip of the red and then of the black points (a grid
+// of strips ran 1.4 waves at 16384^2).  Small grids give the black points blocks of their own.
+// Either way the red points' sum does not depend on whether the black ones are walked: their
+// partials keep their places and the black ones come after them.
+template <bool MAX, bool WRITE, int PTS>
+__global__ void __launch_bounds__(kSweepThreads) residual_kernel(const ResidualArgs a) {
+    __shared__ double smem[kSweepThreads / 32];
+    const int n = a.n, W = a.W;
+    const double one = a.one;
+    const int lane = threadIdx.x & 31;
+    double acc = 0.0, mx = 0.0;
+    const int own = (int)blockIdx.x >= a.lanes ? 1 : 0;  // blocks past `lanes`: the black points alone
+    const int last_colour = (int)gridDim.x > a.lanes ? own : a.colours - 1;
+    for (int colour = own; colour <= last_colour; ++colour) {
+    const double *__restrict__ self = colour ? a.u[1] : a.u[0], *__restrict__ other = colour ? a.u[0] : a.u[1];
+    const double *__restrict__ hf = colour ? a.hf[1] : a.hf[0];
+    float *__restrict__ r32 = colour ? a.r32[1] : a.r32[0];
+        for (int item = blockIdx.x - own * a.lanes; item < a.items; item += a.lanes) {
+            const int strip = item / a.bx;
+            const int k0 = PTS * ((item - strip * a.bx) * kSweepThreads + threadIdx.x);
+            const bool act = k0 < a.kact;
+            const int i0 = 1 + strip * a.rows, i1 = min(n, i0 + a.rows - 1);
+            double up[PTS], mid[PTS], dn[PTS], f[PTS], me[PTS];
+            load_row<PTS>(up, other + (size_t)(i0 - 1) * W + k0, act);
+            load_row<PTS>(mid, other + (size_t)i0 * W + k0, act);
+            for (int i = i0; i <= i1; ++i) {
+                const size_t row = (size_t)i * W;
+                load_row<PTS>(dn, other + row + W + k0, act);
+                load_row<PTS>(f, hf + row + k0, act);
+                load_row<PTS>(me, self + row + k0, act);
+                const int p = (i + colour) & 1;
+                // value q: west/east at k0+q-1, k0+q (p = 0) or k0+q, k0+q+1 (p = 1)
+                double w[PTS], e[PTS];
+                if (p == 0) {
+                    double x = __shfl_up_sync(0xffffffffu, mid[PTS - 1], 1);
+                    if (lane == 0) x = (act && k0 > 0) ? __ldg(other + row + k0 - 1) : 0.0;
+#pragma unroll
+                    for (int q = 0; q < PTS; ++q) w[q] = q ? mid[q ? q - 1 : 0] : x, e[q] = mid[q];
+                } else {
+                    double x = __shfl_down_sync(0xffffffffu, mid[0], 1);
+                    if (lane == 31) x = (k0 + PTS < a.kact) ? __ldg(other + row + k0 + PTS) : 0.0;
+#pragma unroll
+                    for (int q = 0; q < PTS; ++q) w[q] = mid[q], e[q] = q + 1 < PTS ? mid[q + 1 < PTS ? q + 1 : 0] : x;
+                }
+                const int j0 = 2 * k0 + p;
+#pragma unroll
+                for (int q = 0; q < PTS; ++q) {
+                    if (!(act && j0 + 2 * q >= 1 && j0 + 2 * q <= n)) continue;
+                    const double s =
+                        add_fma(add_fma(add_fma(add_fma(f[q], up[q], one), dn[q], one), w[q], one), e[q], one);
+                    const double r = __fma_rn(-4.0, me[q], s);
+                    if (WRITE) {
+                        r32[(size_t)i * a.W32 + k0 + q] = __double2float_rn(__dmul_rn(r, a.scale));
+                    } else {
+                        acc = __fma_rn(r, r, acc);
+                        // |r| compares as its bits do; a NaN sorts above everything and the sum shows it
+                        if (MAX) {
+                            const double m = __longlong_as_double(__double_as_longlong(r) & 0x7FFFFFFFFFFFFFFFll);
+                            mx = __double_as_longlong(m) > __double_as_longlong(mx) ? m : mx;
+                        }
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < PTS; ++q) up[q] = mid[q], mid[q] = dn[q];
+            }
+        }
+    }
+    if (WRITE) return;
+    const int blocks = gridDim.x, slot = blockIdx.x;
+    const double t = block_sum<kSweepThreads>(acc, smem);
+    if (threadIdx.x == 0) a.partials[slot] = t;
     if (MAX) {
         __syncthreads();
-        const double m = block_max<kSweepThreads>(mx, red_smem);
-        if (threadIdx.x == 0) partials[kMaxPartials + slot] = m;
+        const double m = block_max<kSweepThreads>(mx, smem);
+        if (threadIdx.x == 0) a.partials[kMaxPartials + slot] = m;
     }
-}
-
-// Max of `count` partials -> *out (order-independent, exact).
-__global__ void __launch_bounds__(kFinalThreads)
-final_max_kernel(const double *__restrict__ partials, int count, double *__restrict__ out) {
-    __shared__ double smem[kFinalThreads / 32];
-    double v = 0.0;
-    for (int q = threadIdx.x; q < count; q += kFinalThreads) v = fmax(v, partials[q]);
-    const double t = block_max<kFinalThreads>(v, smem);
-    if (threadIdx.x == 0) *out = t;
-}
-
-// Sum of `count` partials in a fixed order -> *out.
-__global__ void __launch_bounds__(kFinalThreads)
-final_sum_kernel(const double *__restrict__ partials, int count, double *__restrict__ out) {
-    __shared__ double smem[kFinalThreads / 32];
-    double v = 0.0;
-    for (int q = threadIdx.x; q < count; q += kFinalThreads) v = __dadd_rn(v, partials[q]);
-    const double t = block_sum<kFinalThreads>(v, smem);
-    if (threadIdx.x == 0) *out = t;
+    if (!last_block<kSweepThreads>(a.ticket, blocks)) return;
+    const double sum = sum_partials<kSweepThreads>(a.partials, blocks, smem);
+    if (threadIdx.x == 0) a.out[0] = a.host[0] = sum, a.host[3] = (double)*a.status;
+    if (MAX) {
+        __syncthreads();
+        const double m = max_partials<kSweepThreads>(a.partials + kMaxPartials, blocks, smem);
+        if (threadIdx.x == 0) a.out[2] = a.host[2] = m;
+    }
 }
 
 __device__ __forceinline__ double at(const double *const *u, int W, int i, int j) {
@@ -136,7 +199,8 @@ constexpr int kNormRowsAhead = 4;
 
 __global__ void __launch_bounds__(kNormThreads)
 rhs_norm_kernel(ColourPtrs u, ColourPtrs hf, int n, int W, int kact, int rows_per_block,
-                double *__restrict__ partials) {
+                double *__restrict__ partials, double *__restrict__ out, double *__restrict__ host,
+                unsigned *ticket) {
     __shared__ double smem[kNormThreads / 32];
     const int k0 = 2 * (blockIdx.x * kNormThreads + threadIdx.x);
     const int i0 = 1 + blockIdx.y * rows_per_block, i1 = min(n, i0 + rows_per_block - 1);
@@ -180,57 +244,81 @@ rhs_norm_kernel(ColourPtrs u, ColourPtrs hf, int n, int W, int kact, int rows_pe
     }
     const double t = block_sum<kNormThreads>(acc, smem);
     if (threadIdx.x == 0) partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
+    if (!last_block<kNormThreads>(ticket, gridDim.x * gridDim.y)) return;
+    const double sum = sum_partials<kNormThreads>(partials, gridDim.x * gridDim.y, smem);
+    if (threadIdx.x == 0) *out = *host = sum;
 }
 
-int residual_rows(int n, int kact) {
-    // enough blocks to fill the GPU, at most kMaxPartials / 2 per colour
-    const int bx = (kact + 2 * kSweepThreads - 1) / (2 * kSweepThreads);
-    int rows = 16;
-    while ((size_t)bx * ((n + rows - 1) / rows) > (size_t)kMaxPartials / 2) rows *= 2;
+// Rows per block: up to `most`, fewer where that would leave the GPU with fewer than about four
+// blocks per SM (a thread walks its rows one after another: 16 rows of a 127^2 grid took 17 us,
+// one row takes 4), and at most `blocks` blocks in all (a power-of-two number of rows then).
+int block_rows(int n, int bx, int most, int blocks) {
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) {
+            cudaGetLastError();
+            v = 152;
+        }
+        return v;
+    }();
+    const long r = (long)n * bx / (4L * sms);
+    int rows = (int)(r < 1 ? 1 : r > most ? most : r);
+    while ((size_t)bx * ((n + rows - 1) / rows) > (size_t)blocks) rows *= 2;
     return rows;
 }
-
-}  // namespace
-
-namespace {
 
 // red_only: the black points' rt is known to be zero (the iterate is the result of a full
 // sweep); only the red partials are formed and summed.
 template <bool MAX, bool WRITE>
-rbgs_status residual_passes(const rbgs_ctx *c, double scale, cudaStream_t s, bool red_only) {
+rbgs_status residual_pass(const rbgs_ctx *c, double scale, cudaStream_t s, bool red_only) {
     const Geometry &g = c->g;
-    const int kact = active_width(g.n);
-    const int rows = residual_rows(g.n, kact);
-    dim3 grid((kact + 2 * kSweepThreads - 1) / (2 * kSweepThreads), (g.n + rows - 1) / rows);
-    float *r0 = WRITE ? c->f32.hf[0] : nullptr, *r1 = WRITE ? c->f32.hf[1] : nullptr;
-    residual_colour_kernel<0, MAX, WRITE><<<grid, kSweepThreads, 0, s>>>(
-        c->f64.u[0], c->f64.u[1], c->f64.hf[0], g.n, g.W, kact, rows, c->partials, r0, c->f32.W, scale, 1.0);
-    RBGS_LAUNCH_CHECK();
-    if (!red_only) {
-        residual_colour_kernel<1, MAX, WRITE><<<grid, kSweepThreads, 0, s>>>(
-            c->f64.u[1], c->f64.u[0], c->f64.hf[1], g.n, g.W, kact, rows, c->partials, r1, c->f32.W, scale, 1.0);
-        RBGS_LAUNCH_CHECK();
+    ResidualArgs a;
+    for (int q = 0; q < 2; ++q) {
+        a.u[q] = c->f64.u[q], a.hf[q] = c->f64.hf[q];
+        a.r32[q] = WRITE ? c->f32.hf[q] : nullptr;
     }
-    const int count = (red_only ? 1 : 2) * (int)(grid.x * grid.y);
-    final_sum_kernel<<<1, kFinalThreads, 0, s>>>(c->partials, count, c->dsum);
+    a.n = g.n, a.W = g.W, a.kact = active_width(g.n), a.W32 = c->f32.W;
+    a.colours = red_only ? 1 : 2;
+    a.partials = c->partials, a.out = c->dsum, a.host = c->hsum;
+    a.status = c->dstatus, a.ticket = c->pcounter + 1;
+    a.scale = scale, a.one = 1.0;
+    static const int wave = [] {  // resident blocks of the GPU, per template instance
+        int dev = 0, sms = 0, per_sm = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, residual_kernel<MAX, WRITE, 2>, kSweepThreads, 0) !=
+                cudaSuccess ||
+            sms < 1 || per_sm < 1) {
+            cudaGetLastError();
+            return 1024;
+        }
+        return sms * per_sm < kMaxPartials ? sms * per_sm : kMaxPartials;
+    }();
+    // strips of up to 16 rows, and on large grids the tallest ones that give each block four:
+    // short strips start over too often (84% of the FP64 pipe at 8192^2 with 16 rows, 92% so)
+    a.bx = (a.kact + 2 * kSweepThreads - 1) / (2 * kSweepThreads);
+    a.rows = block_rows(g.n, a.bx, 16, 1 << 30);
+    const int strips = 4 * wave / a.bx;
+    if (strips > 0 && (g.n + strips - 1) / strips > a.rows) a.rows = (g.n + strips - 1) / strips;
+    a.items = a.bx * ((g.n + a.rows - 1) / a.rows);
+    a.lanes = a.items < wave ? a.items : wave;
+    const int grid = !red_only && 2 * a.lanes <= wave ? 2 * a.lanes : a.lanes;
+    residual_kernel<MAX, WRITE, 2><<<grid, kSweepThreads, 0, s>>>(a);
     RBGS_LAUNCH_CHECK();
-    if (MAX) {
-        final_max_kernel<<<1, kFinalThreads, 0, s>>>(c->partials + kMaxPartials, count, c->dsum + 2);
-        RBGS_LAUNCH_CHECK();
-    }
     return RBGS_OK;
 }
 
 }  // namespace
 
 rbgs_status launch_residual_sum(const rbgs_ctx *c, cudaStream_t s) {
-    return residual_passes<false, false>(c, 1.0, s, c->black_fresh);
+    return residual_pass<false, false>(c, 1.0, s, c->black_fresh);
 }
 
 // write_r32 = false: sum rt^2 -> dsum[0], max |rt| -> dsum[2].
-// write_r32 = true:  r32 = (float)(rt * scale) at interior points (and the sum again).
+// write_r32 = true:  r32 = (float)(rt * scale) at interior points.
 rbgs_status launch_defect(const rbgs_ctx *c, bool write_r32, double scale, cudaStream_t s) {
-    return write_r32 ? residual_passes<false, true>(c, scale, s, false) : residual_passes<true, false>(c, scale, s, false);
+    return write_r32 ? residual_pass<false, true>(c, scale, s, false) : residual_pass<true, false>(c, scale, s, false);
 }
 
 rbgs_status launch_rhs_norm(const rbgs_ctx *c, cudaStream_t s) {
@@ -238,12 +326,10 @@ rbgs_status launch_rhs_norm(const rbgs_ctx *c, cudaStream_t s) {
     ColourPtrs u{{c->f64.u[0], c->f64.u[1]}}, hf{{c->f64.hf[0], c->f64.hf[1]}};
     const int kact = active_width(g.n);
     const int bx = (kact + 2 * kNormThreads - 1) / (2 * kNormThreads);
-    int rows = 16;
-    while ((size_t)bx * ((g.n + rows - 1) / rows) > (size_t)kMaxPartials) rows *= 2;
+    const int rows = block_rows(g.n, bx, 16, kMaxPartials);
     const dim3 grid(bx, (g.n + rows - 1) / rows);
-    rhs_norm_kernel<<<grid, kNormThreads, 0, s>>>(u, hf, g.n, g.W, kact, rows, c->partials);
-    RBGS_LAUNCH_CHECK();
-    final_sum_kernel<<<1, kFinalThreads, 0, s>>>(c->partials, (int)(grid.x * grid.y), c->dsum + 1);
+    rhs_norm_kernel<<<grid, kNormThreads, 0, s>>>(u, hf, g.n, g.W, kact, rows, c->partials, c->dsum + 1,
+                                                     c->hsum + 1, c->pcounter + 2);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
