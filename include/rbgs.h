@@ -254,8 +254,8 @@ rbgs_status rbgs_solve_batched(int nprob, const rbgs_problem *probs, double tol,
  * Not in the paper: library mechanics.
  * Launch shape of the last rbgs_solve_batched call on this thread (zeros before the first):
  * threads per block, blocks per SM, team size (1: one block per problem; 2 or 4: the phased
- * plan), and for the phased plan the number of largest problems solved one per block in its
- * first phase and the number solved by clusters in its second.  Any pointer may be NULL.
+ * plan), and for the phased plan the number of largest problems solved in its first phase (one
+ * per block, or one per cluster of 2) and the number solved by clusters in its second.  Any pointer may be NULL.
  */
 void rbgs_batched_last_shape(int *threads, int *blocks_per_sm, int *team, int *first, int *nteam);
 

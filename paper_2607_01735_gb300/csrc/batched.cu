@@ -267,7 +267,7 @@ __device__ void block_half_sweep_band(T *__restrict__ self, const T *other, cons
 // are ordinary (coherent) loads, through L2 for multi-block teams: the team wrote it one
 // half-sweep earlier.
 template <int C, int VT, int CS>
-__device__ void block_half_sweep_f64(const DevProblem &P, int vt) {
+__device__ void block_half_sweep_f64(const DevProblem &P, int vt, double one) {
     double *self = P.u[C];
     const double *other = P.u[C ^ 1];
     const double *hf = P.hf[C];
@@ -293,8 +293,8 @@ __device__ void block_half_sweep_f64(const DevProblem &P, int vt) {
             w0 = mid.x; e0 = mid.y; w1 = mid.y;
             e1 = (k0 + 2 < kact) ? ldt<CS>(other + row + k0 + 2) : 0.0;
         }
-        const double r0 = update_f64<false>(0, f2.x, up.x, dn.x, w0, e0, 1.0);
-        const double r1 = update_f64<false>(0, f2.y, up.y, dn.y, w1, e1, 1.0);
+        const double r0 = update_f64<false>(0, f2.x, up.x, dn.x, w0, e0, one);
+        const double r1 = update_f64<false>(0, f2.y, up.y, dn.y, w1, e1, one);
         const int j0 = 2 * k0 + p;
         if (act && j0 >= 1 && j0 <= n) self[row + k0] = r0;
         if (act && j0 + 2 <= n) self[row + k0 + 1] = r1;
@@ -312,7 +312,7 @@ __device__ void block_half_sweep_f32(const DevProblem &P, int vt) {
 // zero (their values are s * 0.25 of the very sums s formed here, and 4 (s * 0.25) = s), so
 // the red points alone give the same sum bit for bit: colours = 1 there.
 template <int VT, int CS, bool WRITE>
-__device__ void block_residual(const DevProblem &P, double scale, double &r2, double &mx, int vt,
+__device__ void block_residual(const DevProblem &P, double scale, double &r2, double &mx, int vt, double one,
                                int colours = 2) {
     const int n = P.n, W = P.W, kact = kact_of(n);
     r2 = 0.0;
@@ -326,11 +326,11 @@ __device__ void block_residual(const DevProblem &P, double scale, double &r2, do
             const int j = 2 * k + p;
             if (j < 1 || j > n) continue;
             const size_t row = (size_t)i * W;
-            double s = __dadd_rn(hf[row + k], ldt<CS>(other + row - W + k));
-            s = __dadd_rn(s, ldt<CS>(other + row + W + k));
-            s = __dadd_rn(s, ldt<CS>(other + row + k - 1 + p));
-            s = __dadd_rn(s, ldt<CS>(other + row + k + p));
-            const double r = __dadd_rn(s, -__dmul_rn(4.0, ldt<CS>(self + row + k)));
+            double s = add_fma(hf[row + k], ldt<CS>(other + row - W + k), one);
+            s = add_fma(s, ldt<CS>(other + row + W + k), one);
+            s = add_fma(s, ldt<CS>(other + row + k - 1 + p), one);
+            s = add_fma(s, ldt<CS>(other + row + k + p), one);
+            const double r = __fma_rn(-4.0, ldt<CS>(self + row + k), s);  // 4u is exact
             r2 = __fma_rn(r, r, r2);
             mx = fmax(mx, fabs(r));
             if (WRITE) P.r[c][(size_t)i * P.W32 + k] = __double2float_rn(__dmul_rn(r, scale));
@@ -382,7 +382,7 @@ __device__ __forceinline__ bool budget_spent(const BatchLimits &L, int rank, dou
 template <int THREADS, int CS>
 __device__ void solve_problem(const DevProblem &P, DevResult &R, double tol, int check_every,
                               long long max_sweeps, int inner, bool refine, int cap_n, const BatchLimits &L,
-                              int rank, double *smem, double *slot) {
+                              int rank, double one, double *smem, double *slot) {
     constexpr int VT = THREADS * CS;
     const int vt = rank * THREADS + (int)threadIdx.x;
     const unsigned long long t0 = globaltimer();
@@ -393,7 +393,7 @@ __device__ void solve_problem(const DevProblem &P, DevResult &R, double tol, int
     }
     const double den2 = team_sum<THREADS, CS>(rhs_norm2_partial<VT>(P, vt), smem, slot);
     double r2, mx;
-    block_residual<VT, CS, false>(P, 1.0, r2, mx, vt);
+    block_residual<VT, CS, false>(P, 1.0, r2, mx, vt, one);
     r2 = team_sum<THREADS, CS>(r2, smem, slot);
     mx = team_max<THREADS, CS>(mx, smem, slot);
     double rho = rho_of(r2, den2);
@@ -407,9 +407,9 @@ __device__ void solve_problem(const DevProblem &P, DevResult &R, double tol, int
             long long k = check_every;
             if (k > max_sweeps - done) k = max_sweeps - done;
             for (long long it = 0; it < k; ++it) {
-                block_half_sweep_f64<0, VT, CS>(P, vt);
+                block_half_sweep_f64<0, VT, CS>(P, vt, one);
                 team_sync<CS>();
-                block_half_sweep_f64<1, VT, CS>(P, vt);
+                block_half_sweep_f64<1, VT, CS>(P, vt, one);
                 team_sync<CS>();
             }
             done += k;
@@ -418,7 +418,7 @@ __device__ void solve_problem(const DevProblem &P, DevResult &R, double tol, int
             frexp(mx, &e);
             const double down = ldexp(1.0, -e), up = ldexp(1.0, e);
             double t2, tm;
-            block_residual<VT, CS, true>(P, down, t2, tm, vt);  // writes the scaled defect
+            block_residual<VT, CS, true>(P, down, t2, tm, vt, one);  // writes the scaled defect
             const size_t elems = (size_t)(P.n + 2) * P.W32;
             for (size_t q = vt; q < elems; q += VT) {
                 P.d[0][q] = 0.0f;
@@ -448,7 +448,7 @@ __device__ void solve_problem(const DevProblem &P, DevResult &R, double tol, int
             done += k;
         }
         // after FP64 sweeps the black rt is zero; the refinement's correction moves every point
-        block_residual<VT, CS, false>(P, 1.0, r2, mx, vt, refine ? 2 : 1);
+        block_residual<VT, CS, false>(P, 1.0, r2, mx, vt, one, refine ? 2 : 1);
         r2 = team_sum<THREADS, CS>(r2, smem, slot);
         mx = team_max<THREADS, CS>(mx, smem, slot);
         rho = rho_of(r2, den2);
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(THREADS)
 batched_persistent_kernel(const DevProblem *__restrict__ probs, DevResult *__restrict__ res,
                           const int *__restrict__ order, int nprob, int nteam, int *queues, double tol,
                           int check_every, long long max_sweeps, int inner, int refine, int cap_n,
-                          const BatchLimits L) {
+                          const BatchLimits L, double one) {
     __shared__ double smem[THREADS / 32 + 1];
     __shared__ double slot;
     __shared__ int s_q;
@@ -498,7 +498,7 @@ batched_persistent_kernel(const DevProblem *__restrict__ probs, DevResult *__res
             const int p = order[q];
             const DevProblem P = probs[p];
             solve_problem<THREADS, CS>(P, res[p], tol, check_every, max_sweeps, inner, refine != 0, cap_n, L,
-                                       rank, smem, &slot);
+                                       rank, one, smem, &slot);
         }
     }
     for (;;) {
@@ -510,7 +510,7 @@ batched_persistent_kernel(const DevProblem *__restrict__ probs, DevResult *__res
         const int p = order[q];
         const DevProblem P = probs[p];
         solve_problem<THREADS, 1>(P, res[p], tol, check_every, max_sweeps, inner, refine != 0, cap_n, L, 0,
-                                  smem, &slot);
+                                  one, smem, &slot);
         __syncthreads();
     }
 }
@@ -574,7 +574,8 @@ struct LaunchConfig {
     int threads;       // 256, 512 or 1024
     int blocks_per_sm;
     int team;          // 1: one phase, one block per problem
-    int first = 0;     // problems (largest first) solved one per block in the first phase
+    int team1 = 1;     // blocks per problem in the first phase (1, or a cluster of 2)
+    int first = 0;     // problems (largest first) solved in the first phase
     int nteam = 0;     // problems after those solved by teams in the second phase
     int grid1 = 0, grid2 = 0;
 };
@@ -597,7 +598,7 @@ rbgs_status launch_one(int grid, const DevProblem *d_probs, DevResult *d_res, co
     cfg.attrs = at;
     cfg.numAttrs = CS > 1 ? 1 : 0;
     RBGS_CUDA(cudaLaunchKernelEx(&cfg, batched_persistent_kernel<THREADS, CS>, d_probs, d_res, d_order, nprob, nteam,
-                                 d_queues, tol, check_every, max_sweeps, inner, refine, cap_n, L));
+                                 d_queues, tol, check_every, max_sweeps, inner, refine, cap_n, L, 1.0));
     return RBGS_OK;
 }
 
@@ -632,9 +633,10 @@ void plan_phases(LaunchConfig &lc, const std::vector<int> &sizes_desc, int sms) 
     const int nmax = sizes_desc.empty() ? 0 : sizes_desc[0];
     int m = 0;
     while (m < (int)sizes_desc.size() && sizes_desc[m] == nmax) ++m;
-    lc.first = (m / sms) * sms;
+    const int wave = lc.team1 > 1 ? std::max(1, max_clusters_of(lc.team1)) : sms;
+    lc.first = (m / wave) * wave;
     lc.nteam = m - lc.first;
-    lc.grid1 = sms;
+    lc.grid1 = lc.team1 * wave;
     const int nc = max_clusters_of(lc.team);
     lc.grid2 = lc.team * std::max(1, nc);
 }
@@ -645,7 +647,10 @@ rbgs_status launch_persistent(const LaunchConfig &lc, int sms, const DevProblem 
                               cudaStream_t s) {
     if (lc.team > 1) {
         rbgs_status st = RBGS_OK;
-        if (lc.first > 0)
+        if (lc.first > 0 && lc.team1 == 2)
+            st = launch_one<1024, 2>(lc.grid1, d_probs, d_res, d_order, lc.first, lc.first, d_queues, tol, check_every,
+                                     max_sweeps, inner, refine, cap_n, L, s);
+        else if (lc.first > 0)
             st = launch_one<1024, 1>(lc.grid1, d_probs, d_res, d_order, lc.first, 0, d_queues, tol, check_every,
                                      max_sweeps, inner, refine, cap_n, L, s);
         if (st != RBGS_OK || lc.first >= nprob) return st;
@@ -864,6 +869,11 @@ extern "C" rbgs_status rbgs_solve_batched(int nprob, const rbgs_problem *probs, 
                     LaunchConfig c{1024, 1, cs};
                     plan_phases(c, sizes_desc, sms);
                     cands.push_back(c);
+                    if (cs == 4 && c.first == 0) {  // clusters of 2 for a first wave, if they fill one
+                        c.team1 = 2;
+                        plan_phases(c, sizes_desc, sms);
+                        if (c.first > 0) cands.push_back(c);
+                    }
                 }
             }
             cudaEvent_t e0, e1;

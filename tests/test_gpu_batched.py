@@ -263,3 +263,15 @@ def test_batched_time_budget_ends_the_batch():
     for p in late:
         _assert_bits(outs[p], batch[p][3])
     assert max(r["latency_ms"] for r in res) < 2000.0
+
+
+def test_batched_first_wave_of_clusters_matches_oracle():
+    """80 problems at the largest size (a wave of 2-block clusters and a few left over, among
+    the plans that the autotuner tries) with smaller ones: every problem has the oracle's bits."""
+    batch = _batch([31] * 80 + [15, 7, 3, 15], 12)
+    res, outs = _run(batch, 0.0, check_every=20, max_sweeps=40)
+    for (n, h2, f, u0), r, got in zip(batch, res, outs):
+        ref = u0.copy()
+        oracle.sweeps(ref, f, h2, 40)
+        assert r["status"] == rb.RBGS_ENOTCONV and r["sweeps"] == 40
+        _assert_bits(got, ref)
