@@ -232,15 +232,15 @@ __global__ void __launch_bounds__(kBiasThreads) bias_grad_kernel(const uint16_t 
     const int g = threadIdx.x % groups, r = threadIdx.x / groups;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (r < lanes) {
-        // four pixels per step, their loads issued together
+        // eight pixels per step, their loads issued together
         const long stride = (long)gridDim.x * lanes;
-        for (long p = (long)blockIdx.x * lanes + r; p < P; p += 4 * stride) {
-            uint4 v[4];
+        for (long p = (long)blockIdx.x * lanes + r; p < P; p += 8 * stride) {
+            uint4 v[8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < 8; ++u)
                 v[u] = p + u * stride < P ? ld16(G + (p + u * stride) * Cout + g * 8) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < 8; ++u) {
                 const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -253,13 +253,12 @@ __global__ void __launch_bounds__(kBiasThreads) bias_grad_kernel(const uint16_t 
 #pragma unroll
     for (int e = 0; e < 8; ++e) part[threadIdx.x][e] = acc[e];
     __syncthreads();
-    if (r == 0) {
-        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int q = 0; q < lanes; ++q)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) s[e] += part[q * groups + g][e];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) atomicAdd(db + g * 8 + e, s[e]);
+    // one thread per channel adds the lanes in order (8 channels per thread, a few threads at work,
+    // cost more than the loads)
+    for (int ch = threadIdx.x; ch < Cout; ch += kBiasThreads) {
+        float t = 0.f;
+        for (int q = 0; q < lanes; ++q) t += part[q * groups + (ch >> 3)][ch & 7];
+        atomicAdd(db + ch, t);
     }
 }
 
@@ -272,8 +271,9 @@ int g_wgrad_kind = RBGS_WGRAD_AUTO;
 
 rbgs_status umma_conv_forward(const uint16_t *X, const uint16_t *Wt, const float *bias, void *Y, int B, int H,
                               int W, int Cin, int Cout, int ks, int relu, int y_fp32, cudaStream_t s);
-rbgs_status umma_conv_backward_data(const uint16_t *Wtt, const uint16_t *G, float *dX, int B, int H, int W,
-                                    int Cin, int Cout, int ks, int accumulate, bool tma, cudaStream_t s);
+rbgs_status umma_conv_backward_data(const uint16_t *Wtt, const uint16_t *G, float *dX, const uint16_t *Y,
+                                    uint16_t *Gin, int B, int H, int W, int Cin, int Cout, int ks, int accumulate,
+                                    bool tma, cudaStream_t s);
 rbgs_status umma_conv_backward_weight(const uint16_t *X, const uint16_t *G, float *dW, int B, int H, int W,
                                       int Cin, int Cout, int ks, int kind, cudaStream_t s);
 rbgs_status umma_conv_check(cudaStream_t s);
@@ -290,16 +290,33 @@ rbgs_status conv_forward(const uint16_t *X, const uint16_t *Wt, const float *bia
     return RBGS_OK;
 }
 
-rbgs_status conv_backward(const uint16_t *X, const uint16_t *Wt, const uint16_t *G, float *dX, float *dW,
-                          float *db, uint16_t *Wtt, int B, int H, int W, int Cin, int Cout, int ks,
-                          int accumulate, cudaStream_t s) {
+namespace {
+
+// Gin = bf16(dX) where the activation Y is positive, else 0; 4 values per thread (n: a multiple of 4)
+__global__ void relu_grad_kernel(const float4 *__restrict__ dX, const uint2 *__restrict__ Y, uint2 *__restrict__ Gin,
+                                 long n4) {
+    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += (long)gridDim.x * blockDim.x) {
+        const float4 v = dX[q];
+        const uint2 y = Y[q];
+        auto pos = [](uint32_t bits) { return __uint_as_float(bits) > 0.f; };
+        auto bf = [](float f) { return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(f)); };
+        const uint32_t a = bf(pos(y.x << 16) ? v.x : 0.f), b = bf(pos(y.x & 0xFFFF0000u) ? v.y : 0.f);
+        const uint32_t c = bf(pos(y.y << 16) ? v.z : 0.f), d = bf(pos(y.y & 0xFFFF0000u) ? v.w : 0.f);
+        Gin[q] = make_uint2(a | (b << 16), c | (d << 16));
+    }
+}
+
+// Backward of one layer with its weights already transposed (Wtt).  Gin != NULL: the data
+// gradient goes through the ReLU of the layer before (whose output is X) into Gin as bf16; dX is
+// then scratch, used by the mma.sync engine only.
+rbgs_status backward_products(const uint16_t *X, const uint16_t *Wt, const uint16_t *G, float *dX, uint16_t *Gin,
+                              float *dW, float *db, const uint16_t *Wtt, int B, int H, int W, int Cin, int Cout, int ks,
+                              int accumulate, cudaStream_t s) {
     const long P = (long)B * H * W;
     const int taps = ks * ks;
     if (dX) {
-        transpose_weights_kernel<<<256, 256, 0, s>>>(Wt, Wtt, Cout, taps, Cin);
-        RBGS_LAUNCH_CHECK();
         if (g_engine != RBGS_CONV_MMA_SYNC) {
-            const rbgs_status st = umma_conv_backward_data(Wtt, G, dX, B, H, W, Cin, Cout, ks, accumulate,
+            const rbgs_status st = umma_conv_backward_data(Wtt, G, dX, X, Gin, B, H, W, Cin, Cout, ks, accumulate,
                                                            g_engine == RBGS_CONV_TCGEN05, s);
             if (st != RBGS_OK) return st;
         } else {
@@ -307,6 +324,10 @@ rbgs_status conv_backward(const uint16_t *X, const uint16_t *Wt, const uint16_t 
             dim3 grid((unsigned)((P + BM - 1) / BM), (unsigned)((Cin + BN - 1) / BN), 1);
             conv_igemm_kernel<BWD_DATA><<<grid, THREADS, 0, s>>>(a);
             RBGS_LAUNCH_CHECK();
+            if (Gin) {
+                relu_grad_kernel<<<2048, 256, 0, s>>>((const float4 *)dX, (const uint2 *)X, (uint2 *)Gin, P * Cin / 4);
+                RBGS_LAUNCH_CHECK();
+            }
         }
     }
     if (dW && g_engine != RBGS_CONV_MMA_SYNC) {
@@ -322,10 +343,28 @@ rbgs_status conv_backward(const uint16_t *X, const uint16_t *Wt, const uint16_t 
         RBGS_LAUNCH_CHECK();
     }
     if (db) {
-        bias_grad_kernel<<<2 * 152, kBiasThreads, 0, s>>>(G, db, P, Cout);
+        bias_grad_kernel<<<4 * 152, kBiasThreads, 0, s>>>(G, db, P, Cout);
         RBGS_LAUNCH_CHECK();
     }
     return RBGS_OK;
+}
+
+}  // namespace
+
+static rbgs_status conv_backward(const uint16_t *X, const uint16_t *Wt, const uint16_t *G, float *dX, float *dW,
+                                 float *db, uint16_t *Wtt, int B, int H, int W, int Cin, int Cout, int ks,
+                          int accumulate, cudaStream_t s) {
+    if (dX) {
+        transpose_weights_kernel<<<256, 256, 0, s>>>(Wt, Wtt, Cout, ks * ks, Cin);
+        RBGS_LAUNCH_CHECK();
+    }
+    return backward_products(X, Wt, G, dX, nullptr, dW, db, Wtt, B, H, W, Cin, Cout, ks, accumulate, s);
+}
+
+// One layer of the network's backward pass (unet.cu): see backward_products.
+rbgs_status conv_backward_layer(const uint16_t *X, const uint16_t *G, float *dX, uint16_t *Gin, float *dW, float *db,
+                                const uint16_t *Wtt, int B, int H, int W, int Cin, int Cout, int ks, cudaStream_t s) {
+    return backward_products(X, nullptr, G, dX, Gin, dW, db, Wtt, B, H, W, Cin, Cout, ks, 0, s);
 }
 
 bool conv_shapes_ok(int B, int H, int W, int Cin, int Cout, int ks) {

@@ -33,6 +33,8 @@ struct TMaps {
 struct TArgs {
     const float *bias;
     void *out;
+    const uint16_t *Y;  // data gradient with gin: as in UArgs
+    uint16_t *gin;
     int H, W, B, ks, pad, taps;
     int relu, y_fp32, accumulate;
     int M, N;  // pixels, output channels of this product
@@ -242,6 +244,10 @@ __global__ void __launch_bounds__(kTmaThreads, 1) conv_tma_kernel(const __grid_c
                                 make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
                                            pack_bf16(v[6], v[7]));
                         }
+                    } else if (a.gin) {
+                        const long o = m * a.N + n;
+                        *reinterpret_cast<uint4 *>(a.gin + o) =
+                            masked_bf16(v, __ldg(reinterpret_cast<const uint4 *>(a.Y + o)));
                     } else {
                         float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + m * a.N + n);
                         float4 p0 = make_float4(v[0], v[1], v[2], v[3]), p1 = make_float4(v[4], v[5], v[6], v[7]);
@@ -314,14 +320,14 @@ bool tma_chunks(int CK, TArgs &a) {
 // wts: Wt [Cout][taps][Cin] (forward) or Wt_t [taps][Cin][Cout] (data gradient).
 // Returns false (nothing launched) when the shape is not one the TMA path takes.
 template <int MODE>
-bool tma_conv_launch(const uint16_t *src, const uint16_t *wts, const float *bias, void *out, int B, int H, int W,
-                     int Cin, int Cout, int ks, int relu, int y_fp32, int accumulate, cudaStream_t s,
+bool tma_conv_launch(const uint16_t *src, const uint16_t *wts, const float *bias, void *out, const uint16_t *Y,
+                     uint16_t *gin, int B, int H, int W, int Cin, int Cout, int ks, int relu, int y_fp32, int accumulate, cudaStream_t s,
                      rbgs_status *st) {
     TArgs a{};
     const int CK = MODE == U_FWD ? Cin : Cout;
     const int N = MODE == U_FWD ? Cout : Cin;
     if (!tma_chunks(CK, a)) return false;
-    a.bias = bias, a.out = out;
+    a.bias = bias, a.out = out, a.Y = Y, a.gin = gin;
     a.H = H, a.W = W, a.B = B, a.ks = ks, a.pad = ks / 2, a.taps = ks * ks;
     a.kstages = a.group > 1 ? (a.taps + a.group - 1) / a.group : a.taps * a.nchunks;
     a.relu = relu, a.y_fp32 = y_fp32, a.accumulate = accumulate;

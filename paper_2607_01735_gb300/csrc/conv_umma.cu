@@ -103,6 +103,8 @@ struct UArgs {
     const uint16_t *G;   // NHWC bf16 gradient of the pre-activation output
     const float *bias;
     void *out;
+    const uint16_t *Y;   // data grad with gin: the input activation, whose sign masks the result
+    uint16_t *gin;       // data grad: bf16 output through that mask (NULL: FP32 to out)
     int H, W, Cin, Cout, ks;
     int relu, y_fp32, accumulate;
     int M, N, K;         // GEMM sizes
@@ -190,6 +192,17 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, vo
 
 __device__ __forceinline__ bool wait_or_abort_spin(uint64_t *bar, uint32_t parity, volatile int *abort_flag) {
     return rbgs::wait_or_abort_spin(bar, parity, abort_flag, kSpinPolls, &g_conv_wait_failed);
+}
+
+// 8 data-gradient values through the ReLU of the layer before, as bf16 (y: its 8 outputs)
+__device__ __forceinline__ uint4 masked_bf16(const float *v, uint4 y) {
+    const uint32_t w[4] = {y.x, y.y, y.z, y.w};
+    uint32_t o[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        o[e] = pack_bf16(__uint_as_float(w[e] << 16) > 0.f ? v[2 * e] : 0.f,
+                         __uint_as_float(w[e] & 0xFFFF0000u) > 0.f ? v[2 * e + 1] : 0.f);
+    return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
 struct Tile {
@@ -470,6 +483,9 @@ __device__ void drain(const UArgs &a, uint32_t tmem, uint64_t *tfull_bar, uint64
                             make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
                                        pack_bf16(v[6], v[7]));
                     }
+                } else if (MODE == U_BWD_DATA && a.gin) {
+                    const long o = (long)m * a.N + n;
+                    *reinterpret_cast<uint4 *>(a.gin + o) = masked_bf16(v, __ldg(reinterpret_cast<const uint4 *>(a.Y + o)));
                 } else if (MODE == U_BWD_DATA) {
                     float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + (long)m * a.N + n);
                     float4 p0 = make_float4(v[0], v[1], v[2], v[3]), p1 = make_float4(v[4], v[5], v[6], v[7]);
@@ -624,17 +640,18 @@ rbgs_status umma_conv_forward(const uint16_t *X, const uint16_t *Wt, const float
     return launch<U_FWD>(a, s);
 }
 
-rbgs_status umma_conv_backward_data(const uint16_t *Wtt, const uint16_t *G, float *dX, int B, int H, int W,
-                                    int Cin, int Cout, int ks, int accumulate, bool tma, cudaStream_t s) {
+rbgs_status umma_conv_backward_data(const uint16_t *Wtt, const uint16_t *G, float *dX, const uint16_t *Y,
+                                    uint16_t *Gin, int B, int H, int W, int Cin, int Cout, int ks, int accumulate,
+                                    bool tma, cudaStream_t s) {
     if (!sizes_fit(B, H, W)) {
         set_error("tcgen05 convolution: at most 2^31 - 64 pixels");
         return RBGS_EINVAL;
     }
     rbgs_status st = RBGS_OK;
-    if (tma && tma_conv_launch<U_BWD_DATA>(G, Wtt, nullptr, dX, B, H, W, Cin, Cout, ks, 0, 0, accumulate, s, &st))
+    if (tma && tma_conv_launch<U_BWD_DATA>(G, Wtt, nullptr, dX, Y, Gin, B, H, W, Cin, Cout, ks, 0, 0, accumulate, s, &st))
         return st;
     UArgs a{};
-    a.Wt = Wtt, a.G = G, a.out = dX;
+    a.Wt = Wtt, a.G = G, a.out = dX, a.Y = Y, a.gin = Gin;
     a.H = H, a.W = W, a.Cin = Cin, a.Cout = Cout, a.ks = ks, a.accumulate = accumulate;
     a.M = B * H * W, a.N = Cin, a.K = ks * ks * Cout;
     a.bn = pick_bn(a.N);

@@ -27,9 +27,8 @@ namespace rbgs {
 rbgs_status conv_forward(const uint16_t *X, const uint16_t *Wt, const float *bias, void *Y, int B, int H,
                          int W, int Cin, int Cout, int ks, int relu, int y_fp32, cudaStream_t s);
 rbgs_status umma_conv_check(cudaStream_t s);
-rbgs_status conv_backward(const uint16_t *X, const uint16_t *Wt, const uint16_t *G, float *dX, float *dW,
-                          float *db, uint16_t *Wtt, int B, int H, int W, int Cin, int Cout, int ks,
-                          int accumulate, cudaStream_t s);
+rbgs_status conv_backward_layer(const uint16_t *X, const uint16_t *G, float *dX, uint16_t *Gin, float *dW, float *db,
+                                const uint16_t *Wtt, int B, int H, int W, int Cin, int Cout, int ks, cudaStream_t s);
 
 namespace {
 
@@ -48,92 +47,129 @@ const int kSpec[15][5] = {
     {96, 32, 3, 1, 0},   {32, 32, 3, 1, 0},   {32, 8, 1, 0, 0}};
 
 // ------------------------------------------------------------------ elementwise kernels
-__global__ void pack_input_kernel(const float *__restrict__ x, __nv_bfloat16 *__restrict__ out, long P) {
+// All of them move 16-byte vectors (8 bf16 or 4 FP32 channels), one image row per blockIdx.y
+// step, with the channel counts of the network as template parameters, so that a vector's place
+// costs one division by a constant.  HBM bounds them.  At 16 x 264^2, before (one channel per
+// thread, 64-bit divisions) and now: up_concat 900 -> 100 us over the three levels, avgpool 106 ->
+// 25, pack_input 100 -> 10.
+
+constexpr int kEw = 256;  // threads per block
+
+__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
+__device__ __forceinline__ uint32_t bf_pack(float lo, float hi) {
+    const __nv_bfloat16 a = __float2bfloat16_rn(lo), b = __float2bfloat16_rn(hi);
+    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+}
+// v where the activation y is positive, else 0 (a pair of channels; y as bf16 bits)
+__device__ __forceinline__ uint32_t relu_grad2(float lo, float hi, uint32_t y) {
+    return bf_pack(bf_lo(y) > 0.f ? lo : 0.f, bf_hi(y) > 0.f ? hi : 0.f);
+}
+
+// VEC: x is 16-byte aligned (the caller's pointer need not be)
+template <bool VEC>
+__global__ void pack_input_kernel(const float *__restrict__ x, uint4 *__restrict__ out, long P) {
+    static_assert(kInCh == 16 && kXCh == 4, "one 16-byte load, two 16-byte stores per pixel");
     for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (long)gridDim.x * blockDim.x) {
+        const float4 v = VEC ? *reinterpret_cast<const float4 *>(x + 4 * p)
+                             : make_float4(x[4 * p], x[4 * p + 1], x[4 * p + 2], x[4 * p + 3]);
+        out[2 * p] = make_uint4(bf_pack(v.x, v.y), bf_pack(v.z, v.w), 0u, 0u);
+        out[2 * p + 1] = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
+// 2x2 average pooling: in [rows][W][C] -> out [rows/2][W/2][C] (rows = B H, H even)
+template <int C>
+__global__ void __launch_bounds__(kEw) avgpool_kernel(const uint4 *__restrict__ in, uint4 *__restrict__ out,
+                                                      long orows, int W) {
+    constexpr int C8 = C / 8;
+    const int w = W / 2, q = blockIdx.x * kEw + threadIdx.x;
+    if (q >= w * C8) return;
+    const int x = q / C8, c = q - x * C8;
+    for (long r = blockIdx.y; r < orows; r += gridDim.y) {
+        const uint4 *p = in + ((2 * r) * W + 2 * x) * C8 + c;
+        const uint4 v[4] = {p[0], p[C8], p[(long)W * C8], p[(long)W * C8 + C8]};
+        uint32_t o[4];
 #pragma unroll
-        for (int c = 0; c < kInCh; ++c) out[p * kInCh + c] = __float2bfloat16_rn(c < kXCh ? x[p * kXCh + c] : 0.f);
+        for (int e = 0; e < 4; ++e) {
+            float lo = 0.f, hi = 0.f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t t = e == 0 ? v[k].x : e == 1 ? v[k].y : e == 2 ? v[k].z : v[k].w;
+                lo = k ? lo + bf_lo(t) : bf_lo(t);
+                hi = k ? hi + bf_hi(t) : bf_hi(t);
+            }
+            o[e] = bf_pack(0.25f * lo, 0.25f * hi);
+        }
+        out[(r * w + x) * C8 + c] = make_uint4(o[0], o[1], o[2], o[3]);
     }
 }
 
-// G = bf16(dY * (Y > 0)) (relu != 0) or bf16(dY)
-__global__ void act_grad_kernel(const float *__restrict__ dY, const __nv_bfloat16 *__restrict__ Y,
-                                __nv_bfloat16 *__restrict__ G, long n, int relu) {
-    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
-        float v = dY[q];
-        if (relu && !(__bfloat162float(Y[q]) > 0.f)) v = 0.f;
-        G[q] = __float2bfloat16_rn(v);
+// concat(up(lo), skip): out [rows][W][CLO + CS]
+template <int CLO, int CS>
+__global__ void __launch_bounds__(kEw) up_concat_kernel(const uint4 *__restrict__ lo, const uint4 *__restrict__ skip,
+                                                        uint4 *__restrict__ out, long rows, int W) {
+    constexpr int L8 = CLO / 8, S8 = CS / 8, T8 = L8 + S8;
+    const int q = blockIdx.x * kEw + threadIdx.x;
+    if (q >= W * T8) return;
+    const int x = q / T8, c = q - x * T8;
+    for (long r = blockIdx.y; r < rows; r += gridDim.y)  // H is even: row r / 2 of lo is the same image's
+        out[r * W * T8 + q] = c < L8 ? lo[((r >> 1) * (W / 2) + x / 2) * L8 + c] : skip[(r * W + x) * S8 + (c - L8)];
+}
+
+// Gradient of a decoder tensor that was upsampled into a concatenation, through its ReLU: the sum
+// of dCat[.., :CLO] over each 2x2 block, where y (the tensor itself) is positive, as bf16.
+template <int CLO, int CS>
+__global__ void __launch_bounds__(kEw) up_grad_kernel(const float4 *__restrict__ dCat, const uint2 *__restrict__ y,
+                                                      uint2 *__restrict__ G, long lrows, int W) {
+    constexpr int L4 = CLO / 4, T4 = (CLO + CS) / 4;
+    const int w = W / 2, q = blockIdx.x * kEw + threadIdx.x;
+    if (q >= w * L4) return;
+    const int x = q / L4, c = q - x * L4;
+    for (long r = blockIdx.y; r < lrows; r += gridDim.y) {
+        const float4 *p = dCat + ((2 * r) * W + 2 * x) * T4 + c;
+        const float4 a = p[0], b = p[T4], d = p[(long)W * T4], e = p[(long)W * T4 + T4];
+        const uint2 m = y[r * w * L4 + q];
+        G[r * w * L4 + q] = make_uint2(relu_grad2(a.x + b.x + d.x + e.x, a.y + b.y + d.y + e.y, m.x),
+                                       relu_grad2(a.z + b.z + d.z + e.z, a.w + b.w + d.w + e.w, m.y));
     }
 }
 
-// 2x2 average pooling: in [B][H][W][C] -> out [B][H/2][W/2][C]
-__global__ void avgpool_kernel(const __nv_bfloat16 *__restrict__ in, __nv_bfloat16 *__restrict__ out, int B,
-                               int H, int W, int C) {
-    const int h = H / 2, w = W / 2;
-    const long total = (long)B * h * w * C;
-    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (long)gridDim.x * blockDim.x) {
-        const int c = (int)(q % C);
-        const long pix = q / C;
-        const int x = (int)(pix % w), y = (int)((pix / w) % h);
-        const long b = pix / ((long)w * h);
-        const long base = ((b * H + 2 * y) * W + 2 * x) * C + c;
-        const float s = __bfloat162float(in[base]) + __bfloat162float(in[base + C]) +
-                        __bfloat162float(in[base + (long)W * C]) + __bfloat162float(in[base + (long)W * C + C]);
-        out[q] = __float2bfloat16_rn(0.25f * s);
+// Gradient of an encoder tensor that went into a concatenation and into a pooling, through its
+// ReLU: dCat[.., CLO:] + dPool / 4, where y (the tensor itself) is positive, as bf16.
+template <int CLO, int CS>
+__global__ void __launch_bounds__(kEw) skip_grad_kernel(const float4 *__restrict__ dCat,
+                                                        const float4 *__restrict__ dPool,
+                                                        const uint2 *__restrict__ y, uint2 *__restrict__ G, long rows,
+                                                        int W) {
+    constexpr int L4 = CLO / 4, S4 = CS / 4, T4 = L4 + S4;
+    const int q = blockIdx.x * kEw + threadIdx.x;
+    if (q >= W * S4) return;
+    const int x = q / S4, c = q - x * S4;
+    for (long r = blockIdx.y; r < rows; r += gridDim.y) {
+        const float4 a = dCat[(r * W + x) * T4 + L4 + c], d = dPool[((r >> 1) * (W / 2) + x / 2) * S4 + c];
+        const uint2 m = y[r * W * S4 + q];
+        G[r * W * S4 + q] =
+            make_uint2(relu_grad2(__fmaf_rn(0.25f, d.x, a.x), __fmaf_rn(0.25f, d.y, a.y), m.x),
+                       relu_grad2(__fmaf_rn(0.25f, d.z, a.z), __fmaf_rn(0.25f, d.w, a.w), m.y));
     }
 }
 
-// backward of avg pooling: dIn[.., 2y+a, 2x+b, c] += dOut[.., y, x, c] / 4
-__global__ void avgpool_bwd_kernel(const float *__restrict__ dOut, float *__restrict__ dIn, int B, int H, int W,
-                                   int C) {
-    const long total = (long)B * H * W * C;
-    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (long)gridDim.x * blockDim.x) {
-        const int c = (int)(q % C);
-        const long pix = q / C;
-        const int x = (int)(pix % W), y = (int)((pix / W) % H);
-        const long b = pix / ((long)W * H);
-        dIn[q] += 0.25f * dOut[((b * (H / 2) + y / 2) * (W / 2) + x / 2) * C + c];
-    }
-}
+// The transposed weights Wt_t[t][c][o] of every layer's Wt[o][t][c], in one launch (blockIdx.y:
+// the layer).
+struct TransposeTable {
+    long off[15];
+    int cin[15], cout[15], taps[15];
+};
 
-// concat(up(lo), skip): out [B][H][W][Clo + Cs]
-__global__ void up_concat_kernel(const __nv_bfloat16 *__restrict__ lo, const __nv_bfloat16 *__restrict__ skip,
-                                 __nv_bfloat16 *__restrict__ out, int B, int H, int W, int Clo, int Cs) {
-    const int Ct = Clo + Cs;
-    const long total = (long)B * H * W * Ct;
-    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (long)gridDim.x * blockDim.x) {
-        const int c = (int)(q % Ct);
-        const long pix = q / Ct;
-        const int x = (int)(pix % W), y = (int)((pix / W) % H);
-        const long b = pix / ((long)W * H);
-        out[q] = c < Clo ? lo[((b * (H / 2) + y / 2) * (W / 2) + x / 2) * Clo + c] : skip[pix * Cs + (c - Clo)];
-    }
-}
-
-// split the concat gradient: dLo = sum over each 2x2 block of dCat[.., :Clo] (assigned);
-// dSkip (+)= dCat[.., Clo:]
-__global__ void up_concat_bwd_lo_kernel(const float *__restrict__ dCat, float *__restrict__ dLo, int B, int H,
-                                        int W, int Clo, int Cs) {
-    const int Ct = Clo + Cs, h = H / 2, w = W / 2;
-    const long total = (long)B * h * w * Clo;
-    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (long)gridDim.x * blockDim.x) {
-        const int c = (int)(q % Clo);
-        const long pix = q / Clo;
-        const int x = (int)(pix % w), y = (int)((pix / w) % h);
-        const long b = pix / ((long)w * h);
-        const long base = ((b * H + 2 * y) * W + 2 * x) * Ct + c;
-        dLo[q] = dCat[base] + dCat[base + Ct] + dCat[base + (long)W * Ct] + dCat[base + (long)W * Ct + Ct];
-    }
-}
-
-__global__ void concat_bwd_skip_kernel(const float *__restrict__ dCat, float *__restrict__ dSkip, long P, int Clo,
-                                       int Cs, int accumulate) {
-    const int Ct = Clo + Cs;
-    const long total = P * Cs;
-    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (long)gridDim.x * blockDim.x) {
-        const long pix = q / Cs;
-        const int c = (int)(q % Cs);
-        const float v = dCat[pix * Ct + Clo + c];
-        dSkip[q] = accumulate ? dSkip[q] + v : v;
+__global__ void transpose_all_kernel(const uint16_t *__restrict__ wb, uint16_t *__restrict__ wtt,
+                                     const TransposeTable t) {
+    const int li = blockIdx.y, ci = t.cin[li], co = t.cout[li], taps = t.taps[li];
+    const uint16_t *src = wb + t.off[li];
+    uint16_t *dst = wtt + t.off[li];
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < ci * co * taps; q += gridDim.x * blockDim.x) {
+        const int o = q % co, r = q / co;  // r = tap * cin + c
+        dst[q] = src[(long)o * taps * ci + r];
     }
 }
 
@@ -152,10 +188,11 @@ __global__ void mask_sum_kernel(const float *__restrict__ mask, float *__restric
     }
 }
 
-// prediction (channel 0 of the 8-channel output) and masked MSE: loss partials, dOut
+// prediction (channel 0 of the 8-channel output) and masked MSE: loss partials, and the output
+// layer's gradient as bf16 (the other seven channels are zero)
 __global__ void loss_kernel(const float *__restrict__ out8, const float *__restrict__ target,
                             const float *__restrict__ mask, const float *__restrict__ count,
-                            float *__restrict__ dOut8, float *__restrict__ loss, long P) {
+                            uint4 *__restrict__ G8, float *__restrict__ loss, long P) {
     __shared__ float sm[32];
     const float inv_count = *count > 0.f ? 1.f / *count : 0.f;
     float acc = 0.f;
@@ -163,8 +200,7 @@ __global__ void loss_kernel(const float *__restrict__ out8, const float *__restr
         const float d = out8[p * 8] - target[p];
         const float m = mask[p];
         acc += m * d * d;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) dOut8[p * 8 + c] = c == 0 ? 2.f * m * d * inv_count : 0.f;
+        G8[p] = make_uint4(bf_pack(2.f * m * d * inv_count, 0.f), 0u, 0u, 0u);
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = acc;
@@ -224,15 +260,15 @@ struct rbgs_unet {
     long nparams;
     float *w, *grad, *m, *v;   // FP32 master weights, gradient, Adam moments
     uint16_t *wb;               // bf16 copy used by the forward and backward
-    uint16_t *wtt;              // transposed-weight scratch (largest layer)
+    uint16_t *wtt;              // transposed weights of every layer (at the weights' offsets)
     long step;
     // activation / gradient buffers for one (B, H, W)
     int B, H, W;
     std::vector<void *> bufs;
     uint16_t *act[22];          // bf16 activations (see forward for the order)
     float *gr[22];              // fp32 gradients of the same tensors
-    uint16_t *gbf;              // bf16 pre-activation gradient scratch
-    float *out8, *dout8, *dloss, *hloss;
+    uint16_t *gbf[2];           // bf16 pre-activation gradients: a layer's and the next one's
+    float *out8, *dloss, *hloss;
 };
 
 namespace {
@@ -270,8 +306,8 @@ rbgs_status ensure_buffers(rbgs_unet *net, int B, int H, int W) {
         gmax = n > gmax ? n : gmax;
     }
     const size_t P = (size_t)B * H * W;
-    if (!alloc(gmax * 2, (void **)&net->gbf) || !alloc(P * 8 * 4, (void **)&net->out8) ||
-        !alloc(P * 8 * 4, (void **)&net->dout8) || !alloc(8, (void **)&net->dloss)) {
+    if (!alloc(gmax * 2, (void **)&net->gbf[0]) || !alloc(gmax * 2, (void **)&net->gbf[1]) ||
+        !alloc(P * 8 * 4, (void **)&net->out8) || !alloc(8, (void **)&net->dloss)) {
         set_error("U-Net buffers: out of device memory");
         return RBGS_ENOMEM;
     }
@@ -287,11 +323,19 @@ rbgs_status ensure_buffers(rbgs_unet *net, int B, int H, int W) {
         if (st_ != RBGS_OK) return st_;          \
     } while (0)
 
+// grid of an elementwise kernel: `per_row` vectors per image row
+dim3 ew_grid(int per_row, long rows) {
+    return dim3((unsigned)((per_row + kEw - 1) / kEw), (unsigned)(rows < 32768 ? rows : 32768));
+}
+
 rbgs_status forward(rbgs_unet *net, const float *x) {
     const int B = net->B, H = net->H, W = net->W;
     cudaStream_t s = net->stream;
     const long P = (long)B * H * W;
-    pack_input_kernel<<<nblocks(P), 256, 0, s>>>(x, (__nv_bfloat16 *)net->act[A_IN], P);
+    if ((reinterpret_cast<uintptr_t>(x) & 15u) == 0)
+        pack_input_kernel<true><<<nblocks(P), 256, 0, s>>>(x, (uint4 *)net->act[A_IN], P);
+    else
+        pack_input_kernel<false><<<nblocks(P), 256, 0, s>>>(x, (uint4 *)net->act[A_IN], P);
     RBGS_LAUNCH_CHECK();
     auto conv = [&](int li, int in, int out) {
         const Layer &L = net->layers[li];
@@ -299,17 +343,26 @@ rbgs_status forward(rbgs_unet *net, const float *x) {
                             W >> L.level, L.cin, L.cout, L.ks, L.relu, 0, s);
     };
     auto pool = [&](int in, int out) {
-        const int lv = kActLv[in];
-        avgpool_kernel<<<nblocks((long)B * (H >> lv) * (W >> lv) * kActCh[in] / 4), 256, 0, s>>>(
-            (const __nv_bfloat16 *)net->act[in], (__nv_bfloat16 *)net->act[out], B, H >> lv, W >> lv, kActCh[in]);
-        return cudaGetLastError() == cudaSuccess ? RBGS_OK : RBGS_ECUDA;
+        const int lv = kActLv[in], h = H >> lv, w = W >> lv, C = kActCh[in];
+        const uint4 *i = (const uint4 *)net->act[in];
+        uint4 *o = (uint4 *)net->act[out];
+        const dim3 g = ew_grid((w / 2) * (C / 8), (long)B * h / 2);
+        if (C == 32) avgpool_kernel<32><<<g, kEw, 0, s>>>(i, o, (long)B * h / 2, w);
+        else if (C == 64) avgpool_kernel<64><<<g, kEw, 0, s>>>(i, o, (long)B * h / 2, w);
+        else avgpool_kernel<128><<<g, kEw, 0, s>>>(i, o, (long)B * h / 2, w);
+        RBGS_LAUNCH_CHECK();
+        return RBGS_OK;
     };
     auto upcat = [&](int lo, int skip, int out) {
-        const int lv = kActLv[out];
-        up_concat_kernel<<<nblocks((long)B * (H >> lv) * (W >> lv) * kActCh[out]), 256, 0, s>>>(
-            (const __nv_bfloat16 *)net->act[lo], (const __nv_bfloat16 *)net->act[skip], (__nv_bfloat16 *)net->act[out],
-            B, H >> lv, W >> lv, kActCh[lo], kActCh[skip]);
-        return cudaGetLastError() == cudaSuccess ? RBGS_OK : RBGS_ECUDA;
+        const int lv = kActLv[out], h = H >> lv, w = W >> lv;
+        const uint4 *l = (const uint4 *)net->act[lo], *k = (const uint4 *)net->act[skip];
+        uint4 *o = (uint4 *)net->act[out];
+        const dim3 g = ew_grid(w * (kActCh[out] / 8), (long)B * h);
+        if (lv == 0) up_concat_kernel<64, 32><<<g, kEw, 0, s>>>(l, k, o, (long)B * h, w);
+        else if (lv == 1) up_concat_kernel<128, 64><<<g, kEw, 0, s>>>(l, k, o, (long)B * h, w);
+        else up_concat_kernel<256, 128><<<g, kEw, 0, s>>>(l, k, o, (long)B * h, w);
+        RBGS_LAUNCH_CHECK();
+        return RBGS_OK;
     };
     UNET_TRY(conv(0, A_IN, A_E0A));
     UNET_TRY(conv(1, A_E0A, A_S0));
@@ -336,72 +389,81 @@ rbgs_status forward(rbgs_unet *net, const float *x) {
                         L.ks, 0, 1, s);
 }
 
-// Backward from dout8 (gradient of the 8-channel output); fills net->grad.
+// Backward from gbf[0], the bf16 gradient of the 8-channel output; fills net->grad.  Along a
+// chain of convolutions the data gradient leaves its kernel as the next layer's bf16
+// pre-activation gradient (the ReLU's mask from that layer's output); at the concatenations and
+// poolings it leaves as FP32 and one kernel forms the sum and the mask.
 rbgs_status backward(rbgs_unet *net) {
     const int B = net->B, H = net->H, W = net->W;
     cudaStream_t s = net->stream;
     RBGS_CUDA(cudaMemsetAsync(net->grad, 0, net->nparams * sizeof(float), s));
-    // layer li: input activation `in` (bf16), output activation `out` whose fp32 gradient
-    // gr[out] is complete; writes gr[in] (assigned, or accumulated when acc != 0)
-    auto conv_bwd = [&](int li, int in, const float *dOut, const uint16_t *Yout, int acc, bool need_dx) {
+    TransposeTable tt;
+    for (int li = 0; li < 15; ++li) {
         const Layer &L = net->layers[li];
-        const int h = H >> L.level, w = W >> L.level;
-        const long n = (long)B * h * w * L.cout;
-        act_grad_kernel<<<nblocks(n), 256, 0, s>>>(dOut, (const __nv_bfloat16 *)Yout, (__nv_bfloat16 *)net->gbf, n,
-                                                  L.relu);
-        if (cudaGetLastError() != cudaSuccess) {
-            set_error("act_grad launch failed");
-            return RBGS_ECUDA;
-        }
-        return conv_backward(net->act[in], net->wb + L.w_off, net->gbf, need_dx ? net->gr[in] : nullptr,
-                             net->grad + L.w_off, net->grad + L.b_off, net->wtt, B, h, w, L.cin, L.cout, L.ks, acc,
-                             s);
-    };
-    auto upcat_bwd = [&](int cat, int lo, int skip, int acc_skip) {
-        const int lv = kActLv[cat];
-        const int h = H >> lv, w = W >> lv;
-        up_concat_bwd_lo_kernel<<<nblocks((long)B * h * w * kActCh[lo] / 4), 256, 0, s>>>(
-            net->gr[cat], net->gr[lo], B, h, w, kActCh[lo], kActCh[skip]);
-        concat_bwd_skip_kernel<<<nblocks((long)B * h * w * kActCh[skip]), 256, 0, s>>>(
-            net->gr[cat], net->gr[skip], (long)B * h * w, kActCh[lo], kActCh[skip], acc_skip);
-        return cudaGetLastError() == cudaSuccess ? RBGS_OK : RBGS_ECUDA;
-    };
-    auto pool_bwd = [&](int pooled, int src) {
-        const int lv = kActLv[src];
-        avgpool_bwd_kernel<<<nblocks((long)B * (H >> lv) * (W >> lv) * kActCh[src]), 256, 0, s>>>(
-            net->gr[pooled], net->gr[src], B, H >> lv, W >> lv, kActCh[src]);
-        return cudaGetLastError() == cudaSuccess ? RBGS_OK : RBGS_ECUDA;
-    };
-    // output layer (1x1, linear): its "output activation" is the fp32 out8
-    {
-        const Layer &L = net->layers[14];
-        const long n = (long)B * H * W * 8;
-        act_grad_kernel<<<nblocks(n), 256, 0, s>>>(net->dout8, nullptr, (__nv_bfloat16 *)net->gbf, n, 0);
-        RBGS_LAUNCH_CHECK();
-        UNET_TRY(conv_backward(net->act[A_D0B], net->wb + L.w_off, net->gbf, net->gr[A_D0B], net->grad + L.w_off,
-                               net->grad + L.b_off, net->wtt, B, H, W, L.cin, L.cout, L.ks, 0, s));
+        tt.off[li] = L.w_off, tt.cin[li] = L.cin, tt.cout[li] = L.cout, tt.taps[li] = L.ks * L.ks;
     }
-    UNET_TRY(conv_bwd(13, A_D0A, net->gr[A_D0B], net->act[A_D0B], 0, true));
-    UNET_TRY(conv_bwd(12, A_C0, net->gr[A_D0A], net->act[A_D0A], 0, true));
-    UNET_TRY(upcat_bwd(A_C0, A_D1B, A_S0, 0));
-    UNET_TRY(conv_bwd(11, A_D1A, net->gr[A_D1B], net->act[A_D1B], 0, true));
-    UNET_TRY(conv_bwd(10, A_C1, net->gr[A_D1A], net->act[A_D1A], 0, true));
-    UNET_TRY(upcat_bwd(A_C1, A_D2B, A_S1, 0));
-    UNET_TRY(conv_bwd(9, A_D2A, net->gr[A_D2B], net->act[A_D2B], 0, true));
-    UNET_TRY(conv_bwd(8, A_C2, net->gr[A_D2A], net->act[A_D2A], 0, true));
-    UNET_TRY(upcat_bwd(A_C2, A_B3B, A_S2, 0));
-    UNET_TRY(conv_bwd(7, A_B3A, net->gr[A_B3B], net->act[A_B3B], 0, true));
-    UNET_TRY(conv_bwd(6, A_P2, net->gr[A_B3A], net->act[A_B3A], 0, true));
-    UNET_TRY(pool_bwd(A_P2, A_S2));
-    UNET_TRY(conv_bwd(5, A_E2A, net->gr[A_S2], net->act[A_S2], 0, true));
-    UNET_TRY(conv_bwd(4, A_P1, net->gr[A_E2A], net->act[A_E2A], 0, true));
-    UNET_TRY(pool_bwd(A_P1, A_S1));
-    UNET_TRY(conv_bwd(3, A_E1A, net->gr[A_S1], net->act[A_S1], 0, true));
-    UNET_TRY(conv_bwd(2, A_P0, net->gr[A_E1A], net->act[A_E1A], 0, true));
-    UNET_TRY(pool_bwd(A_P0, A_S0));
-    UNET_TRY(conv_bwd(1, A_E0A, net->gr[A_S0], net->act[A_S0], 0, true));
-    UNET_TRY(conv_bwd(0, A_IN, net->gr[A_E0A], net->act[A_E0A], 0, false));
-    return RBGS_OK;
+    transpose_all_kernel<<<dim3(64, 15), 256, 0, s>>>(net->wb, net->wtt, tt);
+    RBGS_LAUNCH_CHECK();
+    int g = 0;  // gbf[g]: the gradient of the layer at hand
+    // layer li with input activation `in`: to_g: its data gradient becomes gbf[g ^ 1] (and g
+    // moves there), else the FP32 gr[in]
+    enum { TO_G, TO_F32, NONE };
+    auto conv_bwd = [&](int li, int in, int to) {
+        const Layer &L = net->layers[li];
+        const rbgs_status st = conv_backward_layer(
+            net->act[in], net->gbf[g], to == NONE ? nullptr : net->gr[in], to == TO_G ? net->gbf[g ^ 1] : nullptr,
+            net->grad + L.w_off, net->grad + L.b_off, net->wtt + L.w_off, B, H >> L.level, W >> L.level, L.cin, L.cout,
+            L.ks, s);
+        if (to == TO_G) g ^= 1;
+        return st;
+    };
+    // gbf[g] = gradient of act[lo] (level lv + 1), upsampled into the concatenation cat (level lv)
+    auto up_bwd = [&](int cat, int lo) {
+        const int lv = kActLv[cat], h = H >> lv, w = W >> lv;
+        const float4 *d = (const float4 *)net->gr[cat];
+        const uint2 *y = (const uint2 *)net->act[lo];
+        uint2 *o = (uint2 *)net->gbf[g];
+        const dim3 gr = ew_grid((w / 2) * (kActCh[lo] / 4), (long)B * h / 2);
+        if (lv == 0) up_grad_kernel<64, 32><<<gr, kEw, 0, s>>>(d, y, o, (long)B * h / 2, w);
+        else if (lv == 1) up_grad_kernel<128, 64><<<gr, kEw, 0, s>>>(d, y, o, (long)B * h / 2, w);
+        else up_grad_kernel<256, 128><<<gr, kEw, 0, s>>>(d, y, o, (long)B * h / 2, w);
+        RBGS_LAUNCH_CHECK();
+        return RBGS_OK;
+    };
+    // gbf[g] = gradient of act[skip], in the concatenation cat and pooled into `pooled`
+    auto skip_bwd = [&](int cat, int pooled, int skip) {
+        const int lv = kActLv[skip], h = H >> lv, w = W >> lv;
+        const float4 *d = (const float4 *)net->gr[cat], *pd = (const float4 *)net->gr[pooled];
+        const uint2 *y = (const uint2 *)net->act[skip];
+        uint2 *o = (uint2 *)net->gbf[g];
+        const dim3 gr = ew_grid(w * (kActCh[skip] / 4), (long)B * h);
+        if (lv == 0) skip_grad_kernel<64, 32><<<gr, kEw, 0, s>>>(d, pd, y, o, (long)B * h, w);
+        else if (lv == 1) skip_grad_kernel<128, 64><<<gr, kEw, 0, s>>>(d, pd, y, o, (long)B * h, w);
+        else skip_grad_kernel<256, 128><<<gr, kEw, 0, s>>>(d, pd, y, o, (long)B * h, w);
+        RBGS_LAUNCH_CHECK();
+        return RBGS_OK;
+    };
+    UNET_TRY(conv_bwd(14, A_D0B, TO_G));
+    UNET_TRY(conv_bwd(13, A_D0A, TO_G));
+    UNET_TRY(conv_bwd(12, A_C0, TO_F32));
+    UNET_TRY(up_bwd(A_C0, A_D1B));
+    UNET_TRY(conv_bwd(11, A_D1A, TO_G));
+    UNET_TRY(conv_bwd(10, A_C1, TO_F32));
+    UNET_TRY(up_bwd(A_C1, A_D2B));
+    UNET_TRY(conv_bwd(9, A_D2A, TO_G));
+    UNET_TRY(conv_bwd(8, A_C2, TO_F32));
+    UNET_TRY(up_bwd(A_C2, A_B3B));
+    UNET_TRY(conv_bwd(7, A_B3A, TO_G));
+    UNET_TRY(conv_bwd(6, A_P2, TO_F32));
+    UNET_TRY(skip_bwd(A_C2, A_P2, A_S2));
+    UNET_TRY(conv_bwd(5, A_E2A, TO_G));
+    UNET_TRY(conv_bwd(4, A_P1, TO_F32));
+    UNET_TRY(skip_bwd(A_C1, A_P1, A_S1));
+    UNET_TRY(conv_bwd(3, A_E1A, TO_G));
+    UNET_TRY(conv_bwd(2, A_P0, TO_F32));
+    UNET_TRY(skip_bwd(A_C0, A_P0, A_S0));
+    UNET_TRY(conv_bwd(1, A_E0A, TO_G));
+    return conv_bwd(0, A_IN, NONE);
 }
 
 }  // namespace
@@ -415,7 +477,7 @@ rbgs_status rbgs_unet_create(uint64_t seed, void *cuda_stream, rbgs_unet_t *out)
     rbgs_unet *net = new (std::nothrow) rbgs_unet();
     if (!net) { set_error("out of host memory"); return RBGS_ENOMEM; }
     net->stream = (cudaStream_t)cuda_stream;
-    long off = 0, wmax = 0;
+    long off = 0;
     for (int li = 0; li < 15; ++li) {
         Layer L{kSpec[li][0], kSpec[li][1], kSpec[li][2], kSpec[li][3], kSpec[li][4], 0, 0};
         const long nw = (long)L.cout * L.ks * L.ks * L.cin;
@@ -423,7 +485,6 @@ rbgs_status rbgs_unet_create(uint64_t seed, void *cuda_stream, rbgs_unet_t *out)
         off += nw;
         L.b_off = off;
         off += L.cout;
-        wmax = nw > wmax ? nw : wmax;
         net->layers.push_back(L);
     }
     net->nparams = off;
@@ -441,7 +502,7 @@ rbgs_status rbgs_unet_create(uint64_t seed, void *cuda_stream, rbgs_unet_t *out)
     }
     bool ok = cudaMalloc(&net->w, off * 4) == cudaSuccess && cudaMalloc(&net->grad, off * 4) == cudaSuccess &&
               cudaMalloc(&net->m, off * 4) == cudaSuccess && cudaMalloc(&net->v, off * 4) == cudaSuccess &&
-              cudaMalloc(&net->wb, off * 2) == cudaSuccess && cudaMalloc(&net->wtt, wmax * 2) == cudaSuccess &&
+              cudaMalloc(&net->wb, off * 2) == cudaSuccess && cudaMalloc(&net->wtt, off * 2) == cudaSuccess &&
               cudaMallocHost(&net->hloss, 4) == cudaSuccess;
     if (ok) {
         ok = cudaMemcpyAsync(net->w, h.data(), off * 4, cudaMemcpyHostToDevice, net->stream) == cudaSuccess &&
@@ -510,8 +571,8 @@ rbgs_status rbgs_unet_train_step(rbgs_unet_t net, const float *x, const float *t
     RBGS_CUDA(cudaMemsetAsync(net->dloss, 0, 8, net->stream));  // [0] loss, [1] sum(mask)
     mask_sum_kernel<<<nblocks(P), 256, 0, net->stream>>>(mask_loss, net->dloss + 1, P);
     RBGS_LAUNCH_CHECK();
-    loss_kernel<<<nblocks(P), 256, 0, net->stream>>>(net->out8, target, mask_loss, net->dloss + 1, net->dout8,
-                                                    net->dloss, P);
+    loss_kernel<<<nblocks(P), 256, 0, net->stream>>>(net->out8, target, mask_loss, net->dloss + 1,
+                                                    (uint4 *)net->gbf[0], net->dloss, P);
     RBGS_LAUNCH_CHECK();
     UNET_TRY(backward(net));
     if (grads) {
