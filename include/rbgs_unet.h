@@ -64,9 +64,11 @@ rbgs_status rbgs_conv_backward(const uint16_t *X, const uint16_t *Wt, const uint
  * Engine of the convolution kernels (process-wide; applies to the network too):
  *   RBGS_CONV_TCGEN05        (default) 5th-generation tensor cores: tcgen05.mma from shared-
  *                            memory descriptors, FP32 accumulators in tensor memory, 128-row
- *                            tiles; operand tiles of the data-gradient product loaded by TMA
- *                            when the output channels split into chunks of 64, 32 and 16,
- *                            all other operand tiles gathered by cp.async;
+ *                            tiles; forward and data-gradient products of 3x3 layers whose
+ *                            weights fit in shared memory read each input pixel once per
+ *                            tile; operand tiles of the other data-gradient products loaded
+ *                            by TMA when the output channels split into chunks of 64, 32 and
+ *                            16, all other operand tiles gathered by cp.async;
  *   RBGS_CONV_MMA_SYNC       warp-level mma.sync tiles with register accumulators;
  *   RBGS_CONV_TCGEN05_GATHER tcgen05 with every operand tile gathered by cp.async.
  * All compute the same sums in FP32 (the order of accumulation differs).  Returns

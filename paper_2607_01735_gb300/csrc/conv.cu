@@ -270,7 +270,7 @@ int g_wgrad_kind = RBGS_WGRAD_AUTO;
 }  // namespace
 
 rbgs_status umma_conv_forward(const uint16_t *X, const uint16_t *Wt, const float *bias, void *Y, int B, int H,
-                              int W, int Cin, int Cout, int ks, int relu, int y_fp32, cudaStream_t s);
+                              int W, int Cin, int Cout, int ks, int relu, int y_fp32, bool slab, cudaStream_t s);
 rbgs_status umma_conv_backward_data(const uint16_t *Wtt, const uint16_t *G, float *dX, const uint16_t *Y,
                                     uint16_t *Gin, int B, int H, int W, int Cin, int Cout, int ks, int accumulate,
                                     bool tma, cudaStream_t s);
@@ -281,7 +281,7 @@ rbgs_status umma_conv_check(cudaStream_t s);
 rbgs_status conv_forward(const uint16_t *X, const uint16_t *Wt, const float *bias, void *Y, int B, int H,
                          int W, int Cin, int Cout, int ks, int relu, int y_fp32, cudaStream_t s) {
     if (g_engine != RBGS_CONV_MMA_SYNC)
-        return umma_conv_forward(X, Wt, bias, Y, B, H, W, Cin, Cout, ks, relu, y_fp32, s);
+        return umma_conv_forward(X, Wt, bias, Y, B, H, W, Cin, Cout, ks, relu, y_fp32, g_engine == RBGS_CONV_TCGEN05, s);
     ConvArgs a{X, Wt, nullptr, bias, Y, B, H, W, Cin, Cout, ks, relu, y_fp32, 0, 0};
     const long P = (long)B * H * W;
     dim3 grid((unsigned)((P + BM - 1) / BM), (unsigned)((Cout + BN - 1) / BN), 1);

@@ -1,8 +1,9 @@
 // Convolution kernels of the learned initial guess on the 5th-generation tensor cores:
 // implicit GEMM with tcgen05.mma, FP32 accumulators in tensor memory (TMEM).
 //
-// The three products of a convolution layer are the GEMMs listed in conv.cu, tiled here
-// as (M x N output tile, K in stages of 64 bf16):
+// 3x3 layers whose weights fit in shared memory take conv_slab.cuh for the forward and the data
+// gradient.  The rest: the three products of a convolution layer are the GEMMs listed in conv.cu,
+// tiled here as (M x N output tile, K in stages of 64 bf16):
 //   forward      M = pixels,     N = Cout, K = taps*Cin    A, B K-major
 //   data grad    M = pixels,     N = Cin,  K = taps*Cout   A, B K-major
 //   weight grad  M = taps*Cin,   N = Cout, K = pixels      A, B MN-major, K split in chunks
@@ -616,6 +617,7 @@ rbgs_status launch(const UArgs &a, cudaStream_t s) {
 
 bool sizes_fit(int B, int H, int W) { return (long)B * H * W < (1L << 31) - UK; }
 
+#include "conv_slab.cuh"
 #include "conv_tma.cuh"
 #include "conv_wgrad.cuh"
 #include "conv_wgrad_ring.cuh"
@@ -623,11 +625,14 @@ bool sizes_fit(int B, int H, int W) { return (long)B * H * W < (1L << 31) - UK; 
 }  // namespace
 
 rbgs_status umma_conv_forward(const uint16_t *X, const uint16_t *Wt, const float *bias, void *Y, int B, int H,
-                              int W, int Cin, int Cout, int ks, int relu, int y_fp32, cudaStream_t s) {
+                              int W, int Cin, int Cout, int ks, int relu, int y_fp32, bool slab, cudaStream_t s) {
     if (!sizes_fit(B, H, W)) {
         set_error("tcgen05 convolution: at most 2^31 - 64 pixels");
         return RBGS_EINVAL;
     }
+    rbgs_status st = RBGS_OK;
+    if (slab && slab_conv_launch<U_FWD>(X, Wt, bias, Y, nullptr, nullptr, B, H, W, Cin, Cout, ks, relu, y_fp32, 0, s, &st))
+        return st;
     // (the TMA-fed kernel also takes the forward product, but measured slower there than
     // the cp.async gathers: its weight box reads bn rows 9 Cin apart per tap)
     UArgs a{};
@@ -648,6 +653,8 @@ rbgs_status umma_conv_backward_data(const uint16_t *Wtt, const uint16_t *G, floa
         return RBGS_EINVAL;
     }
     rbgs_status st = RBGS_OK;
+    if (tma && slab_conv_launch<U_BWD_DATA>(G, Wtt, nullptr, dX, Y, Gin, B, H, W, Cout, Cin, ks, 0, 0, accumulate, s, &st))
+        return st;
     if (tma && tma_conv_launch<U_BWD_DATA>(G, Wtt, nullptr, dX, Y, Gin, B, H, W, Cin, Cout, ks, 0, 0, accumulate, s, &st))
         return st;
     UArgs a{};

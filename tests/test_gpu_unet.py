@@ -141,6 +141,35 @@ def test_conv_engines_agree(B, H, W, Cin, Cout, k):
             assert float((a - b).abs().max()) <= 1e-5 * scale + 1e-6
 
 
+@pytest.mark.parametrize("Cin,Cout", [(16, 16), (48, 32), (96, 32), (128, 16), (16, 128), (80, 48), (112, 112)])
+@pytest.mark.parametrize("B,H,W", [(1, 1, 1), (2, 15, 7), (1, 16, 8), (3, 17, 9), (2, 33, 90), (5, 100, 100)])
+def test_conv_with_resident_weights_at_tile_edges(B, H, W, Cin, Cout):
+    """3x3 layers whose weights stay in shared memory (patches of 8 x 16 pixels; 112 x 112
+    channels no longer fit): one pixel, edges of the patch, several patches per block, every
+    number of copies per thread.  The sums run in the gather kernel's order, so both agree to
+    FP32 rounding of the sums (2^-24 x 9 x 128 terms < 1e-4 of the scale; bf16 results one ulp)."""
+    from paper_2607_01735_gb300 import unet as un
+    rng = np.random.default_rng(7 * Cin + Cout + H)
+    x = _bf(rng.normal(size=(B, H, W, Cin))).cuda()
+    w = _bf(rng.normal(size=(Cout, 3, 3, Cin)) / np.sqrt(9 * Cin)).cuda()
+    g = _bf(rng.normal(size=(B, H, W, Cout))).cuda()
+    bias = torch.from_numpy(rng.normal(size=Cout).astype(np.float32)).cuda()
+    outs = {}
+    for name in ("tcgen05", "tcgen05_gather"):
+        un.rbgs_conv_set_engine(ENGINES[name])
+        y = torch.full((B, H, W, Cout), 7.0, dtype=torch.float32, device="cuda")
+        yb = torch.full((B, H, W, Cout), 7.0, dtype=torch.bfloat16, device="cuda")
+        un.rbgs_conv_forward(x, w, None, y, relu=False)
+        un.rbgs_conv_forward(x, w, bias, yb, relu=True)
+        dx = torch.full((B, H, W, Cin), 0.5, dtype=torch.float32, device="cuda")
+        un.rbgs_conv_backward(x, w, g, dx, None, None, accumulate=True)
+        un.rbgs_conv_check()
+        outs[name] = (y, yb.float(), dx)
+    un.rbgs_conv_set_engine(un.RBGS_CONV_TCGEN05)
+    for (a, b), tol in zip(zip(outs["tcgen05"], outs["tcgen05_gather"]), (1e-4, 2.0 ** -7, 1e-4)):
+        assert float((a - b).abs().max()) <= tol * float(b.abs().max()) + 1e-6
+
+
 # the 3x3 layer shapes of the network (Cin, Cout at their level's resolution), at batch 2
 # and a quarter of the training resolution
 UNET_3X3 = [(64, 16, 32), (64, 32, 32), (32, 32, 64), (32, 64, 64), (16, 64, 128), (16, 128, 128),
