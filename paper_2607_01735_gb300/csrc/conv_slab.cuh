@@ -22,13 +22,15 @@
 // accumulators, four warps each (on the narrowest layers one tile's drain takes longer than its
 // MMAs).  Every wait is bounded as in the other kernels.
 //
-// What bounds it: an MMA without swizzle took about 78 cycles whatever N (16 to 96) here, so the
-// tensor pipe is mostly idle, and each tile costs another 1 us of barrier and issue latency.
-// Measured on 16 images of 264 x 264 (us; before: gathers forward, TMA data gradient):
-//   forward 16->32 123, now 88; 32->32 168, now 115; 96->32 393, now 217
-//   at 132 x 132: 32->64 53, now 41; 64->64 81, now 54
-//   data gradient 32->32 254, now 117; 96->32 270, now 180; at 132 x 132: 64->64 158, now 58; 32->64 154, now 54
-// (against two commits per tile, two accumulators and eight epilogue warps: 10 to 20% slower.)
+// What bounds it: the MMAs.  One takes 40 to 60 cycles from these layouts without swizzle
+// (128 x 16 bf16 of A at about 70 bytes per clock) for 16 to 32 cycles of products, and its thread
+// waits about 500 cycles per tile at the hand-over; copies alone would take a third of the time.
+// Measured on 16 images of 264 x 264 (us; before: gathers forward, TMA data gradient; in
+// brackets: the issuing thread chosen by lane number, see elect_one):
+//   forward 16->32 123, now 56 [88]; 32->32 168, now 82 [115]; 96->32 393, now 154 [217]
+//   at 132 x 132: 32->64 53, now 31 [41]; 64->64 81, now 39 [54]
+//   data gradient 32->32 254, now 105 [117]; 96->32 270, now 187 [180]; at 132 x 132:
+//   64->64 158, now 51 [58]; 32->64 154, now 45 [54]
 
 constexpr int kSlabW = 10, kSlabH = 18;
 constexpr uint32_t kPlane = (kSlabW * kSlabH + 1) * 16;  // an odd number of 16-byte rows: 8 groups of a pixel hit 8 banks
@@ -69,16 +71,6 @@ struct SlabTile {
         b += db + cy;
     }
 };
-
-// tcgen05.mma issued by the lanes whose `leader` is nonzero (one of the warp)
-__device__ __forceinline__ void umma_bf16_if(uint32_t leader, uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                             uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-        "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate), "r"(leader)
-        : "memory");
-}
 
 // PIECES: 16-byte copies per producer thread and slab, at least 180 CK / 8 / 256
 template <int MODE, int PIECES>
@@ -168,37 +160,36 @@ __global__ void __launch_bounds__(kSlabThreads, 1) conv_slab_kernel(const SArgs 
         }
         cp_async_wait<0>();
     } else if (warp == kMmaWarp) {
-        // the whole warp walks the loop, so that descriptors and counters are uniform values;
-        // lane 0 issues
-        const uint32_t idesc = instr_desc(UM, N, 0, 0), leader = lane == 0;
-        const int steps = CK >> 4;
-        // descriptor start addresses count 16-byte units, in the low bits: offsets just add
-        const uint64_t wdesc = smem_desc(wbase, (uint32_t)N * 16u, 128, 0);
-        const uint32_t bstep = (uint32_t)N * 2u, astep = 2u * (kPlane >> 4);
-        int local = 0;
-        for (int tile = blockIdx.x; tile < a.num_tiles; tile += gridDim.x, ++local) {
-            const int buf = local % kSlabAcc;
-            const uint32_t ph = ((uint32_t)local / kSlabAcc) & 1u;
-            const bool ok = wait_or_abort_spin(&tempty_bar[buf], ph ^ 1u, abort_flag) &&
-                            wait_or_abort_spin(&full_bar[buf], ph, abort_flag);
-            if (!__all_sync(0xffffffffu, ok)) break;
-            fence_proxy_async_smem();  // cp.async wrote through the generic proxy
-            tc_fence_after();
-            const uint32_t acc = tmem + (uint32_t)(buf * N);
-            const uint64_t adesc = smem_desc(sbase + (uint32_t)buf * a.stage_bytes, kPlane, kSlabW * 16u, 0);
-            uint64_t bd = wdesc;
+        if (elect_one()) {
+            const uint32_t idesc = instr_desc(UM, N, 0, 0);
+            const int steps = CK >> 4;
+            // descriptor start addresses count 16-byte units, in the low bits: offsets just add
+            const uint64_t wdesc = smem_desc(wbase, (uint32_t)N * 16u, 128, 0);
+            const uint32_t bstep = (uint32_t)N * 2u, astep = 2u * (kPlane >> 4);
+            int local = 0;
+            for (int tile = blockIdx.x; tile < a.num_tiles; tile += gridDim.x, ++local) {
+                const int buf = local % kSlabAcc;
+                const uint32_t ph = ((uint32_t)local / kSlabAcc) & 1u;
+                if (!wait_or_abort_spin(&tempty_bar[buf], ph ^ 1u, abort_flag) ||
+                    !wait_or_abort_spin(&full_bar[buf], ph, abort_flag))
+                    break;
+                fence_proxy_async_smem();  // cp.async wrote through the generic proxy
+                tc_fence_after();
+                const uint32_t acc = tmem + (uint32_t)(buf * N);
+                const uint64_t adesc = smem_desc(sbase + (uint32_t)buf * a.stage_bytes, kPlane, kSlabW * 16u, 0);
+                uint64_t bd = wdesc;
 #pragma unroll
-            for (int t = 0; t < 9; ++t) {
-                const int ty = MODE == U_FWD ? t / 3 : 2 - t / 3, tx = MODE == U_FWD ? t % 3 : 2 - t % 3;
-                uint64_t ad = adesc + (uint32_t)(ty * kSlabW + tx);
-                for (int k = 0; k < steps; ++k) {
-                    umma_bf16_if(leader, acc, ad, bd, idesc, (t > 0 || k > 0) ? 1u : 0u);
-                    ad += astep;
-                    bd += bstep;
+                for (int t = 0; t < 9; ++t) {
+                    const int ty = MODE == U_FWD ? t / 3 : 2 - t / 3, tx = MODE == U_FWD ? t % 3 : 2 - t % 3;
+                    uint64_t ad = adesc + (uint32_t)(ty * kSlabW + tx);
+                    for (int k = 0; k < steps; ++k) {
+                        umma_bf16(acc, ad, bd, idesc, (t > 0 || k > 0) ? 1u : 0u);
+                        ad += astep;
+                        bd += bstep;
+                    }
                 }
+                umma_commit(&tfull_bar[buf]);
             }
-            if (leader) umma_commit(&tfull_bar[buf]);
-            __syncwarp();
         }
     } else {
         const int q = warp & 3;                   // TMEM lane quarter

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) conv_tma_kernel(const __grid_c
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = instr_desc(UM, bn, 0, 0);
             uint32_t s = 0, ph = 0;
             int local = 0;

