@@ -687,11 +687,12 @@ rbgs_status umma_conv_backward_weight(const uint16_t *X, const uint16_t *G, floa
     }
     // 3x3 layers: the ring kernel (conv_wgrad_ring.cuh) or the tap-row kernel (conv_wgrad.cuh),
     // whose epilogue adds 16-byte vectors, else the gather kernel below.  The automatic choice
-    // follows the per-layer measurements on GB300 (U-Net layers at 16 x 256^2, TFLOP/s, ring /
-    // tap row / gather): Cin <= 32, 256^2 and 128^2 rows: 88-166 / 45-144 / 75-157; the other
-    // layers with >= 40 tap-row stages per SM and rows >= 64 pixels: 326-514 (tap row) vs
-    // 163-273 (gather); the rest (stages per SM ~20, or 32-pixel rows): 234-317 (gather) vs
-    // 163-275 (tap row).
+    // follows the per-layer measurements on GB300 (U-Net layers at 16 x 264^2, us, ring / tap row /
+    // gather): Cin <= 32: 16->32 70 / 136 / 134, 32->32 72 / 141 / 267, at 132^2 32->64
+    // 42 / 52 / 66; the other layers with >= 40 tap-row stages per SM and rows >= 64 pixels:
+    // 132^2 64->64 72 / 70 / 114, 192->64 537 / 166 / 362, 264^2 96->32 262 / 210 / 637, 66^2
+    // 384->128 - / 112 / 245; the rest (stages per SM ~20, or 33-pixel rows): 33^2 128->256
+    // 256 / 56 / 37, 256->256 553 / 65 / 62.
     if (ks == 3 && kind != RBGS_WGRAD_GATHER && (reinterpret_cast<uintptr_t>(dW) & 15u) == 0) {
         bool launched = false;
         rbgs_status st = RBGS_OK;

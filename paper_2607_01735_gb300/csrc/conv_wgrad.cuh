@@ -45,13 +45,21 @@ constexpr int kWgEpiWarp0 = 9;     // warps 9-12
 constexpr int kWgThreads = 416;
 constexpr int kWgMaxStages = 16;
 constexpr int kWgMinStages = 4;
-constexpr int kWgGoodStages = 6;
 constexpr uint32_t kWgBudget = 210 * 1024;
 constexpr int kWgMaxN = 160;
-// Pixel rows per channel group in a slot: seg, and seg + 2 halo pixels for activations
-// (rounded up to 8).  (Rows padded to 1 mod 8, against bank conflicts between channel
-// groups, measured the same.)
-constexpr int kWgPadG = 0, kWgPadX = 8;
+// Segment: of the lengths up to 160 pixels that leave a ring of kWgMinStages, the one with the
+// least sum over a row's segments of (pixels + 32 for the hand-overs of a stage).  Rows of 264 and
+// 132 pixels so take 144, not 128, of which the padding was 45%; rings deeper than four stages
+// (6 and 8 were tried) gained nothing over it.
+constexpr int kWgMaxSeg = 160;
+constexpr int kWgStageCost = 32;
+// Pixel rows per channel group in a slot: seg + 1 for gradients, seg + 3 for activations with
+// their two halo pixels.  Odd, so that the groups of one pixel, which neighbouring threads write,
+// lie in eight different bank groups.  With lengths of 0 mod 8 all of them fell in one, and the
+// writes of the copies bounded the kernel (us at 16 images, before, and with the segments above:
+// 264^2 96->32 332, now 212; 132^2 64->64 129, now 70; 192->64 270, now 167; 66^2 384->128 187,
+// now 112).
+constexpr int kWgPadG = 1, kWgPadX = 3;
 
 struct WgArgs {
     const uint16_t *X, *G;  // NHWC bf16 activations and output gradient
@@ -112,10 +120,12 @@ __device__ __forceinline__ void wg_combo(const WgArgs &a, int combo, int &ty, in
 // once per kernel, so a stage costs each copy an add, a bounds check and its address.
 constexpr int kWgMaxUnits = 8;
 
+template <int NU>
 struct WgUnits {
-    uint32_t dst[kWgMaxUnits];  // byte offset in the slot
-    int pc[kWgMaxUnits];        // pixel offset from the segment's first pixel (high 16 bits,
+    uint32_t dst[NU];  // byte offset in the slot
+    int pc[NU];        // pixel offset from the segment's first pixel (high 16 bits,
                                 // signed) and channel offset from the tile's first channel
+    int off[NU];       // the same as an element offset: pixel C + channel
     int n;
 };
 
@@ -123,15 +133,17 @@ __device__ __forceinline__ int wg_pack_pc(int pix, int ch) { return (int)((uint3
 
 // Plain layout: unit (pixel p, group g) of ng groups x npix pixels at (g len + p) 16 bytes,
 // image pixel x0 + p + pix0.
-__device__ __forceinline__ WgUnits wg_units_plain(int ng, int npix, int len, int pix0, int ptid) {
-    WgUnits t;
+template <int NU>
+__device__ __forceinline__ WgUnits<NU> wg_units_plain(int ng, int npix, int len, int pix0, int C, int ptid) {
+    WgUnits<NU> t;
     t.n = 0;
 #pragma unroll
-    for (int k = 0; k < kWgMaxUnits; ++k) {
+    for (int k = 0; k < NU; ++k) {
         const int u = ptid + k * kWgProducers;
         const int p = u / ng, g = u - p * ng;
         t.dst[k] = (uint32_t)(g * len + p) * 16u;
         t.pc[k] = wg_pack_pc(p + pix0, g * 8);
+        t.off[k] = (p + pix0) * C + g * 8;
         if (u < ng * npix) t.n = k + 1;
     }
     return t;
@@ -140,14 +152,17 @@ __device__ __forceinline__ WgUnits wg_units_plain(int ng, int npix, int len, int
 // Issues a thread's copies of one staged row: image pixels x0 + pix, channels c0 + ch;
 // pixels outside the image row, channels beyond C and rows outside the image (row_ok
 // false) are zero-filled.
-__device__ __forceinline__ void wg_stage_units(const WgUnits &t, const uint16_t *row, bool row_ok, int C, int c0,
+template <int NU>
+__device__ __forceinline__ void wg_stage_units(const WgUnits<NU> &t, const uint16_t *row, bool row_ok, int C, int c0,
                                                int x0, int W, uint32_t slot) {
+    const uint16_t *first = row + (long)x0 * C + c0;
+    const unsigned w = row_ok ? (unsigned)W : 0u;
+    const int cn = C - c0;
 #pragma unroll
-    for (int k = 0; k < kWgMaxUnits; ++k) {
+    for (int k = 0; k < NU; ++k) {
         if (k < t.n) {
-            const int x = x0 + (t.pc[k] >> 16), c = c0 + (t.pc[k] & 0xFFFF);
-            const bool ok = row_ok && (unsigned)x < (unsigned)W && c < C;
-            cp_async16(slot + t.dst[k], ok ? row + (long)x * C + c : row, ok);
+            const bool ok = (unsigned)(x0 + (t.pc[k] >> 16)) < w && (t.pc[k] & 0xFFFF) < cn;
+            cp_async16(slot + t.dst[k], ok ? first + t.off[k] : row, ok);
         }
     }
 }
@@ -158,8 +173,8 @@ __device__ void wg_produce(const WgArgs &a, uint32_t sbase, uint64_t *full_bar, 
     const int S = a.stages;
     const int ngx = a.xa ? a.ngA : a.ngB, ngg = a.xa ? a.ngB : a.ngA;
     const int lenx = a.xa ? a.lenA : a.lenB, leng = a.xa ? a.lenB : a.lenA;
-    const WgUnits ux = wg_units_plain(ngx, a.seg + 2, lenx, -1, ptid);
-    const WgUnits ug = wg_units_plain(ngg, a.seg, leng, 0, ptid);
+    const WgUnits<kWgMaxUnits> ux = wg_units_plain<kWgMaxUnits>(ngx, a.seg + 2, lenx, -1, a.Cin, ptid);
+    const WgUnits<kWgMaxUnits> ug = wg_units_plain<kWgMaxUnits>(ngg, a.seg, leng, 0, a.Cout, ptid);
     uint32_t s = 0, ph = 0;
     bool live = true;
     WgItem it;
@@ -357,6 +372,9 @@ void wg_tiles(int ndim, int &n_tiles, int &N) {
     N = ((ndim + n_tiles - 1) / n_tiles + 15) / 16 * 16;
 }
 
+// Longest segment considered for rows of W pixels.
+int wg_max_segment(int W) { return W < kWgMaxSeg ? (W + 15) / 16 * 16 : kWgMaxSeg; }
+
 // Plans the launch; false if no layout fits (the caller then uses the gather kernel).
 // Checks, for every slot, that the addresses the descriptors can form stay inside the
 // allocation: B reads stay inside their slot; A reads (128 rows, possibly beyond the
@@ -377,13 +395,10 @@ bool wg_plan(int B, int H, int W, int Cin, int Cout, int sms, WgPlan &pl) {
     a.ngA = (mdim + 7) / 8 < 16 ? (mdim + 7) / 8 : 16;
     a.ngB = a.N / 8;
     a.ncombo = 3 * a.m_tiles * a.n_tiles;
-    // the longest segment that leaves a ring of kWgGoodStages stages, else kWgMinStages
-    const int seg0 = W < 128 ? (W + 15) / 16 * 16 : 128;
-    const int cands[4] = {seg0, 64, 32, 16};
-    for (int ci = 0; ci < 8 && !a.seg; ++ci) {
-        const int seg = cands[ci & 3];
-        const int min_stages = ci < 4 ? kWgGoodStages : kWgMinStages;
-        if ((ci & 3) > 0 && seg >= seg0) continue;
+    long best = 0;
+    for (int seg = wg_max_segment(W); seg >= 16; seg -= 16) {
+        const long cost = (long)((W + seg - 1) / seg) * (seg + kWgStageCost);
+        if (best && cost >= best) continue;
         const int xp = seg + kWgPadX, gp = seg + kWgPadG, nk = seg / 16;
         const int lenA = a.xa ? xp : gp, lenB = a.xa ? gp : xp;
         const uint32_t as = (uint32_t)(a.ngA * lenA * 16), bs = (uint32_t)(a.ngB * lenB * 16);
@@ -392,7 +407,7 @@ bool wg_plan(int B, int H, int W, int Cin, int Cout, int sms, WgPlan &pl) {
         // every staged row fits the producers' unit tables
         const int ngx = a.xa ? a.ngA : a.ngB, ngg = a.xa ? a.ngB : a.ngA;
         if (ngx * (seg + 2) > kWgMaxUnits * kWgProducers || ngg * seg > kWgMaxUnits * kWgProducers) continue;
-        for (int S = kWgMaxStages; S >= min_stages; --S) {
+        for (int S = kWgMaxStages; S >= kWgMinStages; --S) {
             const uint32_t rings = (uint32_t)S * (as + bs);
             const uint32_t a_reach =
                 (uint32_t)(S - 1) * as + (uint32_t)((16 * (nk - 1) + (a.xa ? 2 : 0)) * 16 + 15 * lenA * 16 + 256);
@@ -402,6 +417,7 @@ bool wg_plan(int B, int H, int W, int Cin, int Cout, int sms, WgPlan &pl) {
                 a.b_ring = (uint32_t)S * as;
                 a.stages = S;
                 pl.smem = total + 1024;
+                best = cost;
                 break;
             }
         }

@@ -11,7 +11,7 @@
 // (1024 bytes, the 16-byte chunk ch of pixel row r at position ch ^ r), the MN atoms of a
 // pixel group 1024 bytes apart (LBO) and pixel groups n_atoms 1024 bytes apart (SBO); the
 // pre-shifted copies keep every descriptor start on an atom.  B is the gradient row y,
-// MN-major without swizzle (channel group i, pixel p at (i seg + p) 16 bytes).  (The
+// MN-major without swizzle (channel group i, pixel p at (i (seg + 1) + p) 16 bytes).  (The
 // layouts without swizzle fed the tensor cores at about 45 bytes per clock and SM in this
 // kernel's first form, a third of what the swizzled forward operands reach.)
 //
@@ -34,6 +34,8 @@
 // address a descriptor can form lies inside the allocation.
 
 constexpr int kWrMaxXr = kWgMaxStages + 2;
+constexpr int kWrMinStages = 3;     // longer segments gained more than a fourth stage (32->32: 74 us, not 87)
+constexpr int kWrMaxGUnits = 4;     // copies of a gradient row per producer thread (8 spilled registers)
 
 struct WrArgs {
     const uint16_t *X, *G;  // NHWC bf16 activations and output gradient
@@ -89,19 +91,22 @@ __device__ __forceinline__ bool wr_next(const WrArgs &a, long long &f, long long
 // (tx, pixel p, group g), groups fastest, holds channels 8g.. of image pixel x0 - 1 + p + tx
 // at M row group mg = tx ncc + g: atom (p / 8, mg / 8), pixel row r = p mod 8, chunk
 // (mg mod 8) ^ r.
-__device__ __forceinline__ WgUnits wr_units_x(int ncc, int n_atoms, int seg, int ptid) {
-    WgUnits t;
+__device__ __forceinline__ WgUnits<kWgMaxUnits> wr_units_x(int ncc, int n_atoms, int seg, int C, int ptid) {
+    WgUnits<kWgMaxUnits> t;
     t.n = 0;
 #pragma unroll
     for (int k = 0; k < kWgMaxUnits; ++k) {
         const int u = ptid + k * kWgProducers;
         const int q = u / ncc, g = u - q * ncc;  // q = tx seg + p
         const int tx = q >= 2 * seg ? 2 : (q >= seg ? 1 : 0);
-        const int p = q - tx * seg;
+        // pixels of a group of eight in bit-reversed order: the eight threads that write at a time
+        // then hit eight different chunks (with 2 or 4 chunks per pixel; in order 2 to 4 of them collide)
+        const int pl = q - tx * seg, p = (pl & ~5) | (pl & 1) << 2 | (pl >> 2 & 1);
         const int mg = tx * ncc + g, r8 = p & 7;
         t.dst[k] = ((uint32_t)((p >> 3) * n_atoms + (mg >> 3)) << 10) + ((uint32_t)r8 << 7) +
                    ((uint32_t)((mg & 7) ^ r8) << 4);
         t.pc[k] = wg_pack_pc(p + tx - 1, g * 8);
+        t.off[k] = (p + tx - 1) * C + g * 8;
         if (u < 3 * ncc * seg) t.n = k + 1;
     }
     return t;
@@ -111,8 +116,8 @@ __device__ void wr_produce(const WrArgs &a, uint32_t sbase, uint64_t *full_bar, 
                            uint64_t *xempty_bar, volatile int *abort_flag, long long f, long long f_end) {
     const int ptid = threadIdx.x;  // 0..255
     const int S = a.stages;
-    const WgUnits ux = wr_units_x(a.ncc, a.n_atoms, a.seg, ptid);
-    const WgUnits ug = wg_units_plain(a.N / 8, a.seg, a.seg, 0, ptid);
+    const WgUnits<kWgMaxUnits> ux = wr_units_x(a.ncc, a.n_atoms, a.seg, a.Cin, ptid);
+    const WgUnits<kWrMaxGUnits> ug = wg_units_plain<kWrMaxGUnits>(a.N / 8, a.seg, a.seg + kWgPadG, 0, a.Cout, ptid);
     uint32_t s = 0, ph = 0;
     int xs = 0;         // slot of the next activation row
     uint32_t xph = 0;   // parity of that slot's uses so far
@@ -155,7 +160,7 @@ __device__ void wr_issue(const WrArgs &a, uint32_t sbase, uint32_t tmem, uint64_
                          uint64_t *xempty_bar, uint64_t *tfull_bar, uint64_t *tempty_bar, volatile int *abort_flag,
                          long long f, long long f_end) {
     const uint32_t idesc = instr_desc(UM, a.N, 1, 1);
-    const uint32_t sbo = (uint32_t)a.seg * 16u;                 // B: channel-group stride
+    const uint32_t sbo = (uint32_t)(a.seg + kWgPadG) * 16u;                 // B: channel-group stride
     const uint32_t a_sbo = (uint32_t)a.n_atoms << 10;           // A: pixel-group stride
     const uint64_t a_kstep = (uint64_t)(2u * a_sbo) >> 4;       // 16 pixels, in 16-byte units
     const int S = a.stages;
@@ -326,16 +331,14 @@ bool wr_plan(int B, int H, int W, int Cin, int Cout, int sms, WrPlan &pl) {
     uint32_t tc = 32;
     while ((int)tc < a.nbuf * a.acc_cols) tc <<= 1;
     a.tmem_cols = tc;
-    const int seg0 = W < 128 ? (W + 15) / 16 * 16 : 128;
-    const int cands[4] = {seg0, 64, 32, 16};
-    for (int ci = 0; ci < 8 && !a.seg; ++ci) {
-        const int seg = cands[ci & 3];
-        const int min_stages = ci < 4 ? kWgGoodStages : kWgMinStages;
-        if ((ci & 3) > 0 && seg >= seg0) continue;
+    long best = 0;
+    for (int seg = wg_max_segment(W); seg >= 16; seg -= 16) {
+        const long cost = (long)((W + seg - 1) / seg) * (seg + kWgStageCost);
+        if (best && cost >= best) continue;
         const int nk = seg / 16;
-        if (3 * a.ncc * seg > kWgMaxUnits * kWgProducers || a.N / 8 * seg > kWgMaxUnits * kWgProducers) continue;
-        const uint32_t xs = (uint32_t)(seg / 8 * a.n_atoms) << 10, gs = (uint32_t)(a.N / 8 * seg * 16);
-        for (int S = kWgMaxStages; S >= min_stages; --S) {
+        if (3 * a.ncc * seg > kWgMaxUnits * kWgProducers || a.N / 8 * seg > kWrMaxGUnits * kWgProducers) continue;
+        const uint32_t xs = (uint32_t)(seg / 8 * a.n_atoms) << 10, gs = (uint32_t)(a.N / 8 * (seg + kWgPadG) * 16);
+        for (int S = kWgMaxStages; S >= kWrMinStages; --S) {
             const int xr = S + 2;
             const uint32_t rings = (uint32_t)xr * xs + (uint32_t)S * gs;
             // A reads: MN atoms up to 2 m_tiles - 1 of the last pixel group of the last slot
@@ -348,6 +351,7 @@ bool wr_plan(int B, int H, int W, int Cin, int Cout, int sms, WrPlan &pl) {
                 a.g_ring = (uint32_t)xr * xs;
                 a.stages = S, a.xr = xr;
                 pl.smem = total + 1024;
+                best = cost;
                 break;
             }
         }
