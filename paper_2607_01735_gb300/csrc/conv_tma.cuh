@@ -1,10 +1,11 @@
 // TMA-fed tcgen05 convolution for the data-gradient product (written for the forward
-// product too, which measured faster with the cp.async gathers).  Included by conv_umma.cu
+// product too, where the cp.async gathers are as fast: 16 images, 132^2 192->64 207 us against
+// 191, 66^2 384->128 124 against 120, 33^2 256->256 41 against 33; both read L2 at 7.7 TB/s).  Included by conv_umma.cu
 // inside its anonymous namespace: it shares that file's PTX helpers, bounded waits and
 // wait-failure flag.
 //
-// M tile = a tw x th rectangle of 128 pixels of one image (tw = 128 when W >= 128, else
-// the power of two >= W); N tile = bn output channels.  The K loop runs over (tap t,
+// M tile = a tw x th rectangle of 128 pixels of one image (the shape that covers the image
+// with the fewest tiles); N tile = bn output channels.  The K loop runs over (tap t,
 // channel chunk) pairs; a chunk is 64, 32 or 16 channels, loaded with the 128-, 64- or
 // 32-byte swizzle whose K-major UMMA layout has rows of exactly that width (SBO = 8 rows).
 // When the channels are a single chunk of 16 or 32, a stage carries 4 or 2 taps (each in
@@ -15,7 +16,7 @@
 //      outside the image read zeros, which is the convolution's zero padding;
 //   B: the 3D box of the weights for that tap and chunk, [Cout][taps][Cin] (forward) or
 //      the transposed [taps][Cin][Cout] (data gradient).
-// Roles: warp 0 lane 0 issues the TMA loads, warp 1 lane 0 the MMAs (w/16 per stage) and
+// Roles: one thread of warp 0 issues the TMA loads, one of warp 1 the MMAs (w/16 per stage) and
 // the commits, warps 2-9 drain the double-buffered TMEM accumulators: warp w reads lanes
 // 32 (w mod 4) .. of every other 16-column slice (two warps per lane quarter, since with
 // few output channels the drain, not the MMAs, sets the pace).  Waits are bounded exactly
@@ -121,7 +122,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) conv_tma_kernel(const __grid_c
     const uint32_t tmem = tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             for (int q = 0; q < 3; ++q) {
                 prefetch_tensormap(&maps.a[q]);
                 prefetch_tensormap(&maps.b[q]);
@@ -333,10 +334,13 @@ bool tma_conv_launch(const uint16_t *src, const uint16_t *wts, const float *bias
     a.relu = relu, a.y_fp32 = y_fp32, a.accumulate = accumulate;
     a.M = B * H * W, a.N = N;
     a.bn = pick_bn(N);
-    a.tw = 128;
-    if (W < 128) {
-        a.tw = 1;
-        while (a.tw < W) a.tw <<= 1;
+    // the patch of 128 pixels that covers the image with the fewest tiles, the widest of several
+    // (16 images, data gradient, us, 128 x 1 patches or the one of the next power of two above W,
+    // and this: 132^2 192->64 209, now 121; 66^2 384->128 133, now 103; 128->128 70, now 55)
+    long fewest = 0;
+    for (int tw = 128; tw >= 1; tw >>= 1) {
+        const long t = (long)((W + tw - 1) / tw) * ((H + UM / tw - 1) / (UM / tw));
+        if (!fewest || t < fewest) fewest = t, a.tw = tw;
     }
     a.th = UM / a.tw;
     a.tiles_x = (W + a.tw - 1) / a.tw;
