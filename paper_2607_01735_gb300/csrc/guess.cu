@@ -2,7 +2,7 @@
 // transfinite interpolation of the Dirichlet ring that the network's correction is added
 // to, the network's four input channels, the training target, the guess itself, and the
 // transfer between a fine grid and the training grid (block averages of f down, bilinear
-// interpolation up).  One thread per output point; everything stays on the device.
+// interpolation up).  Everything stays on the device.
 //
 // Transfinite (Coons) interpolation of the ring of an (n+2)^2 grid, g = n+2, at point
 // (i, j) with x = i/(g-1), y = j/(g-1): the blended sum of the four edge interpolants minus
@@ -21,61 +21,92 @@ namespace {
 
 constexpr int kT = 256;
 
-__device__ __forceinline__ double coons(const double *__restrict__ u, int g, int i, int j) {
-    const double x = (double)i / (double)(g - 1), y = (double)j / (double)(g - 1);
-    const double c00 = u[0], c01 = u[g - 1], c10 = u[(size_t)(g - 1) * g], c11 = u[(size_t)(g - 1) * g + g - 1];
-    const double edges = (1.0 - x) * u[j] + x * u[(size_t)(g - 1) * g + j] + (1.0 - y) * u[(size_t)i * g] +
-                         y * u[(size_t)i * g + g - 1];
-    const double corners = (1.0 - x) * (1.0 - y) * c00 + (1.0 - x) * y * c01 + x * (1.0 - y) * c10 + x * y * c11;
-    return edges - corners;
+// The kernels that interpolate walk kRows rows of one column per thread, on blocks of kCols
+// columns.  One thread per point computed x and y by two FP64 divisions, 17 further FP64
+// operations and two 64-bit integer divisions, and the FP64 pipe bounded it (1023^2: input 76 us,
+// assemble 70).  The interpolant is (1-x) n_j + x s_j + (1-y) W_i + y E_i with, per column,
+//   n_j = N_j - ((1-y) c00 + y c01),  s_j = S_j - ((1-y) c10 + y c11):
+// four operations per point, the column's terms once per thread and the row's once per block
+// (input 25 us, assemble 22).
+constexpr int kCols = 128, kRows = 16;
+
+// body(i, j, in, c) for every point of a rows x cols output: c is the interpolant of the g^2
+// grid's ring there, `in` whether the point lies on the grid (c is 0 off it).
+template <class Body>
+__device__ __forceinline__ void walk_coons(const double *__restrict__ u, int g, int rows, int cols, Body body) {
+    __shared__ double row_x[kRows], row_w[kRows], row_e[kRows];
+    const int j = blockIdx.x * kCols + threadIdx.x;
+    const double *south = u + (size_t)(g - 1) * g;
+    double y = 0.0, nj = 0.0, sj = 0.0;
+    if (j < g) {
+        y = (double)j / (double)(g - 1);
+        nj = u[j] - ((1.0 - y) * u[0] + y * u[g - 1]);
+        sj = south[j] - ((1.0 - y) * south[0] + y * south[g - 1]);
+    }
+    for (int i0 = blockIdx.y * kRows; i0 < rows; i0 += gridDim.y * kRows) {
+        __syncthreads();
+        if (threadIdx.x < kRows) {
+            const int i = i0 + threadIdx.x;
+            row_x[threadIdx.x] = (double)i / (double)(g - 1);
+            row_w[threadIdx.x] = i < g ? u[(size_t)i * g] : 0.0;
+            row_e[threadIdx.x] = i < g ? u[(size_t)i * g + g - 1] : 0.0;
+        }
+        __syncthreads();
+        if (j >= cols) continue;
+#pragma unroll 4
+        for (int r = 0; r < kRows; ++r) {
+            const int i = i0 + r;
+            if (i >= rows) break;
+            const bool in = i < g && j < g;
+            const double x = row_x[r];
+            // fused explicitly, so that every kernel rounds alike
+            const double we = __fma_rn(y, row_e[r], __dmul_rn(1.0 - y, row_w[r]));
+            const double c = __fma_rn(1.0 - x, nj, __fma_rn(x, sj, we));
+            body(i, j, in, in ? c : 0.0);
+        }
+    }
 }
 
-__global__ void blend_kernel(const double *__restrict__ u, int g, double *__restrict__ out) {
-    const long total = (long)g * g;
-    for (long q = (long)blockIdx.x * kT + threadIdx.x; q < total; q += (long)gridDim.x * kT)
-        out[q] = coons(u, g, (int)(q / g), (int)(q % g));
+dim3 walk_grid(int rows, int cols) {
+    const int y = (rows + kRows - 1) / kRows;
+    return dim3((unsigned)((cols + kCols - 1) / kCols), (unsigned)(y < 65535 ? y : 65535));
+}
+
+__global__ void __launch_bounds__(kCols) blend_kernel(const double *__restrict__ u, int g, double *__restrict__ out) {
+    walk_coons(u, g, g, g, [=](int i, int j, bool, double c) { out[(size_t)i * g + j] = c; });
 }
 
 // x[(i*size + j)*4 + c]: f (interior), ring mask, ring values, the blend; zero off the grid
-__global__ void input_kernel(const double *__restrict__ f, const double *__restrict__ u, int n, int size,
-                             float *__restrict__ x) {
+__global__ void __launch_bounds__(kCols) input_kernel(const double *__restrict__ f, const double *__restrict__ u, int n,
+                                                      int size, float *__restrict__ x) {
     const int g = n + 2;
-    const long total = (long)size * size;
-    for (long q = (long)blockIdx.x * kT + threadIdx.x; q < total; q += (long)gridDim.x * kT) {
-        const int i = (int)(q / size), j = (int)(q % size);
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i < g && j < g) {
-            const bool ring = i == 0 || j == 0 || i == g - 1 || j == g - 1;
-            v.x = ring ? 0.f : (float)f[(size_t)(i - 1) * n + (j - 1)];
-            v.y = ring ? 1.f : 0.f;
-            v.z = ring ? (float)u[(size_t)i * g + j] : 0.f;
-            v.w = (float)coons(u, g, i, j);
-        }
-        reinterpret_cast<float4 *>(x)[q] = v;
-    }
+    walk_coons(u, g, size, size, [=](int i, int j, bool in, double c) {
+        const bool ring = i == 0 || j == 0 || i == g - 1 || j == g - 1;
+        float4 v = make_float4(0.f, 0.f, 0.f, (float)c);
+        if (in && !ring) v.x = (float)f[(size_t)(i - 1) * n + (j - 1)];
+        if (in && ring) v.y = 1.f, v.z = (float)u[(size_t)i * g + j];
+        reinterpret_cast<float4 *>(x)[(size_t)i * size + j] = v;
+    });
 }
 
 // t = sol - blend on the (n+2)^2 grid, 0 elsewhere on the size^2 grid
-__global__ void target_kernel(const double *__restrict__ sol, const double *__restrict__ u, int n, int size,
-                              float *__restrict__ t) {
+__global__ void __launch_bounds__(kCols) target_kernel(const double *__restrict__ sol, const double *__restrict__ u,
+                                                       int n, int size, float *__restrict__ t) {
     const int g = n + 2;
-    const long total = (long)size * size;
-    for (long q = (long)blockIdx.x * kT + threadIdx.x; q < total; q += (long)gridDim.x * kT) {
-        const int i = (int)(q / size), j = (int)(q % size);
-        t[q] = (i < g && j < g) ? (float)(sol[(size_t)i * g + j] - coons(u, g, i, j)) : 0.f;
-    }
+    walk_coons(u, g, size, size, [=](int i, int j, bool in, double c) {
+        t[(size_t)i * size + j] = in ? (float)(sol[(size_t)i * g + j] - c) : 0.f;
+    });
 }
 
 // u0: the ring of u; interior = blend + pred (pred on the size^2 grid)
-__global__ void assemble_kernel(const double *__restrict__ u, const float *__restrict__ pred, int n, int size,
-                                double *__restrict__ u0) {
+__global__ void __launch_bounds__(kCols) assemble_kernel(const double *__restrict__ u, const float *__restrict__ pred,
+                                                         int n, int size, double *__restrict__ u0) {
     const int g = n + 2;
-    const long total = (long)g * g;
-    for (long q = (long)blockIdx.x * kT + threadIdx.x; q < total; q += (long)gridDim.x * kT) {
-        const int i = (int)(q / g), j = (int)(q % g);
+    walk_coons(u, g, g, g, [=](int i, int j, bool, double c) {
         const bool ring = i == 0 || j == 0 || i == g - 1 || j == g - 1;
-        u0[q] = ring ? u[q] : coons(u, g, i, j) + (double)pred[(size_t)i * size + j];
-    }
+        const size_t q = (size_t)i * g + j;
+        u0[q] = ring ? u[q] : c + (double)pred[(size_t)i * size + j];
+    });
 }
 
 // coarse node c = (ci, cj), 1 <= ci, cj <= nc, sits on fine node (ci r, cj r): fc = the mean
@@ -147,7 +178,7 @@ rbgs_status rbgs_guess_blend(const double *u_ring, int n, double *out, void *cud
         return RBGS_EINVAL;
     }
     const int g = n + 2;
-    blend_kernel<<<blocks_for((long)g * g), kT, 0, (cudaStream_t)cuda_stream>>>(u_ring, g, out);
+    blend_kernel<<<walk_grid(g, g), kCols, 0, (cudaStream_t)cuda_stream>>>(u_ring, g, out);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
@@ -158,7 +189,7 @@ rbgs_status rbgs_guess_input(const double *f, const double *u_ring, int n, int s
         set_error("rbgs_guess_input: n >= 1, size >= n + 2 and a multiple of 8, device buffers required");
         return RBGS_EINVAL;
     }
-    input_kernel<<<blocks_for((long)size * size), kT, 0, (cudaStream_t)cuda_stream>>>(f, u_ring, n, size, x);
+    input_kernel<<<walk_grid(size, size), kCols, 0, (cudaStream_t)cuda_stream>>>(f, u_ring, n, size, x);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
@@ -170,7 +201,7 @@ rbgs_status rbgs_guess_target(const double *sol, const double *u_ring, int n, in
         set_error("rbgs_guess_target: n >= 1, size >= n + 2, device buffers required");
         return RBGS_EINVAL;
     }
-    target_kernel<<<blocks_for((long)size * size), kT, 0, (cudaStream_t)cuda_stream>>>(sol, u_ring, n, size, t);
+    target_kernel<<<walk_grid(size, size), kCols, 0, (cudaStream_t)cuda_stream>>>(sol, u_ring, n, size, t);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
@@ -183,7 +214,7 @@ rbgs_status rbgs_guess_assemble(const double *u_ring, const float *pred, int n, 
         return RBGS_EINVAL;
     }
     const int g = n + 2;
-    assemble_kernel<<<blocks_for((long)g * g), kT, 0, (cudaStream_t)cuda_stream>>>(u_ring, pred, n, size, u0);
+    assemble_kernel<<<walk_grid(g, g), kCols, 0, (cudaStream_t)cuda_stream>>>(u_ring, pred, n, size, u0);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
