@@ -344,13 +344,15 @@ rbgs_status sweeps_f64(rbgs_ctx *c, long nsweeps) {
     return enqueue_sweeps(c, nsweeps, c->stream);
 }
 
-// rho and max |rt| of the current FP64 iterate (synchronises the stream).
-rbgs_status defect_stats(rbgs_ctx *c, double *rho, double *mx) {
+// rho and max |rt| of the current FP64 iterate (synchronises the stream); exact: (float)rt of every
+// point, now in f32.hf, is zero or at least 2^-102.
+rbgs_status defect_stats(rbgs_ctx *c, double *rho, double *mx, bool *exact) {
     rbgs_status st = launch_defect(c, false, 1.0, c->stream);
     if (st != RBGS_OK) return st;
     if ((st = finish_residual(c)) != RBGS_OK) return st;
     const double r2 = c->hsum[0];
-    *mx = c->hsum[2];
+    *mx = std::fabs(c->hsum[2]);
+    *exact = !std::signbit(c->hsum[2]);
     *rho = c->den2 > 0.0 ? std::sqrt(r2) / std::sqrt(c->den2) : std::sqrt(r2);
     if (!std::isfinite(*rho)) {
         set_error("residual is not finite");
@@ -414,12 +416,16 @@ rbgs_status refine_solve(rbgs_ctx *c, double tol, long *done_out, double *rho_ou
     rbgs_status st = ensure_f32(c);
     long done = 0;
     double rho = 0.0, mx = 0.0;
-    if (st == RBGS_OK) st = defect_stats(c, &rho, &mx);
+    bool exact = false;
+    if (st == RBGS_OK) st = defect_stats(c, &rho, &mx, &exact);
     while (st == RBGS_OK && !(rho <= tol) && done < c->opts.max_sweeps) {
         int e = 0;
         std::frexp(mx, &e);  // mx = m 2^e, m in [0.5, 1)
         const double down = std::ldexp(1.0, -e), up = std::ldexp(1.0, e);
-        if ((st = launch_defect(c, true, down, c->stream)) != RBGS_OK) break;
+        // every nonzero |rt| is at least 2^-102, so (float)rt 2^-e is normal: the bits of (float)(rt 2^-e)
+        if (!exact || e > 24) st = launch_defect(c, true, down, c->stream);
+        else if (e != 0) st = launch_scale_defect(c, (float)down, c->stream);
+        if (st != RBGS_OK) break;
         const size_t bytes = (size_t)c->g.rows * c->f32.W * sizeof(float);
         for (int q = 0; q < 2; ++q) {
             if (cudaMemsetAsync(c->f32.u[q], 0, bytes, c->stream) != cudaSuccess) {
@@ -434,7 +440,7 @@ rbgs_status refine_solve(rbgs_ctx *c, double tol, long *done_out, double *rho_ou
         if ((st = inner_sweeps_f32(c, m)) != RBGS_OK) break;
         if ((st = launch_correct(c, up, c->stream)) != RBGS_OK) break;
         done += m;
-        st = defect_stats(c, &rho, &mx);
+        st = defect_stats(c, &rho, &mx, &exact);
     }
     if (done_out) *done_out = done;
     if (rho_out) *rho_out = rho;

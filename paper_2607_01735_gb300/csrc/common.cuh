@@ -177,6 +177,7 @@ bool cluster_sweeps_f32_fit(int n, int W);
 rbgs_status launch_cluster_sweeps_f32(ColourField<float> &fld, long nsweeps, cudaStream_t s);
 // mixed-precision refinement kernels (mixed.cu)
 rbgs_status launch_defect(const rbgs_ctx *c, bool write_r32, double scale, cudaStream_t s);  // -> dsum[0] sum, dsum[2] max
+rbgs_status launch_scale_defect(const rbgs_ctx *c, float scale, cudaStream_t s);
 rbgs_status launch_correct(const rbgs_ctx *c, double scale, cudaStream_t s);
 // fused FP64 update (fused.cu): max |h2 f| of a loaded problem; the scale of a block of
 // nsweeps sweeps with h2 f on its grid; one half-sweep at that scale

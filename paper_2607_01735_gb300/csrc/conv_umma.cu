@@ -645,8 +645,7 @@ rbgs_status umma_conv_forward(const uint16_t *X, const uint16_t *Wt, const float
     rbgs_status st = RBGS_OK;
     if (slab && slab_conv_launch<U_FWD>(X, Wt, bias, Y, nullptr, nullptr, B, H, W, Cin, Cout, ks, relu, y_fp32, 0, s, &st))
         return st;
-    // (the TMA-fed kernel also takes the forward product, but measured slower there than
-    // the cp.async gathers: its weight box reads bn rows 9 Cin apart per tap)
+    // (the TMA-fed kernel also takes the forward product; see conv_tma.cuh)
     UArgs a{};
     a.X = X, a.Wt = Wt, a.bias = bias, a.out = Y;
     a.H = H, a.W = W, a.Cin = Cin, a.Cout = Cout, a.ks = ks, a.relu = relu, a.y_fp32 = y_fp32;

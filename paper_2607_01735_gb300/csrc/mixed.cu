@@ -1,13 +1,14 @@
 // Mixed-precision defect correction: the FP64 update of the refinement loop.
 //
 // One outer step of the refinement (the loop lives in api.cu):
-//   1. rt = h^2 (b - A u) in FP64 and max |rt| (residual.cu, exact max);
+//   1. rt = h^2 (b - A u) in FP64, max |rt| and (float)rt (residual.cu, exact max);
 //   2. e = the binary exponent of max |rt|; r32 = (float)(rt * 2^-e)   (exact scaling,
-//      one rounding to binary32);
+//      one rounding to binary32): (float)rt * 2^-e, the same bits, where e <= 24 and no nonzero
+//      |rt| is below 2^-102, else a second walk;
 //   3. d = m FP32 red-black sweeps of (4 I - Adj) d = r32 from d = 0 with a zero ring
 //      (the update of Eq. (1) with h^2 f replaced by r32);
 //   4. u = u + (double)d * 2^e at interior points   (this file).
-// Steps 1-2 and 4 touch the FP64 iterate; only step 3 runs in FP32.
+// Steps 1 and 4 touch the FP64 iterate; only step 3 runs in FP32.
 #include "common.cuh"
 
 namespace rbgs {
@@ -45,7 +46,28 @@ correct_kernel(double *__restrict__ red, double *__restrict__ black, const float
     }
 }
 
+__global__ void __launch_bounds__(kThreads) scale_kernel(float4 *__restrict__ red, float4 *__restrict__ black, long count,
+                                                         float scale) {
+    float4 *__restrict__ r = blockIdx.y ? black : red;
+    for (long q = (long)blockIdx.x * kThreads + threadIdx.x; q < count; q += (long)gridDim.x * kThreads) {
+        float4 v = r[q];
+        v.x *= scale, v.y *= scale, v.z *= scale, v.w *= scale;
+        r[q] = v;
+    }
+}
+
 }  // namespace
+
+// Rows 1..n of the defect arrays times a power of two (their ring places and padding hold zeros).
+rbgs_status launch_scale_defect(const rbgs_ctx *c, float scale, cudaStream_t s) {
+    const long count = (long)c->g.n * c->f32.W / 4;  // W: a multiple of 64
+    const long blocks = (count + kThreads - 1) / kThreads;
+    scale_kernel<<<dim3((unsigned)(blocks < 8 * 152 ? blocks : 8 * 152), 2), kThreads, 0, s>>>(
+        reinterpret_cast<float4 *>(c->f32.hf[0] + c->f32.W), reinterpret_cast<float4 *>(c->f32.hf[1] + c->f32.W), count,
+        scale);
+    RBGS_LAUNCH_CHECK();
+    return RBGS_OK;
+}
 
 rbgs_status launch_correct(const rbgs_ctx *c, double scale, cudaStream_t s) {
     const int n = c->g.n;

@@ -27,8 +27,11 @@
 // side (Section 2, Eq. (1)).  So after a sweep only the red points are walked: half the
 // work, and the same sum bit for bit (the black partials were exact zeros).
 //
-// The same walk also serves the mixed-precision refinement: max |rt| (exact, order-
-// independent) and the FP32 scaled defect (float)(rt * 2^-e) for the inner solver.
+// The same walk also serves the mixed-precision refinement: with the sum it forms max |rt| (exact,
+// order-independent) and stores (float)rt, from which the scaled defect (float)(rt * 2^-e) follows
+// by an exact multiplication (mixed.cu) unless some rt is far below 1.  (A second walk that formed
+// rt again with the scale known took 0.97 ms an outer step at 8192^2; the multiplication takes 0.08:
+// 200 sweeps in two outer steps 13.8 ms, now 12.1.)
 #include "common.cuh"
 #include "fp64.cuh"
 #include "sweep_impl.cuh"
@@ -70,12 +73,13 @@ __device__ __forceinline__ double sum_partials(const double *partials, int count
     return block_sum<THREADS>(v, smem);
 }
 
-template <int THREADS>
-__device__ __forceinline__ double max_partials(const double *partials, int count, double *smem) {
-    double v = 0.0;
-    for (int q = threadIdx.x; q < count; q += THREADS) v = fmax(v, __ldcg(partials + q));
-    __syncthreads();
-    return block_max<THREADS>(v, smem);
+// (float)r for 2^-126 <= |r| < 2^127 or r = 0 (m: the bits of |r|), rounded to nearest even on the
+// integer pipe: the walk's FP64 pipe is full, and the conversion would be a seventh instruction on
+// it (the walk with it 1.09 ms at 8192^2, with this 0.97).
+__device__ __forceinline__ float narrow(double r, long long m) {
+    const unsigned long long t = (unsigned long long)m + 0x0FFFFFFFull + ((m >> 29) & 1);
+    const unsigned f = m ? (unsigned)(t >> 29) - (896u << 23) : 0u;  // exponent bias 1023 to 127
+    return __uint_as_float(f | ((unsigned)__double2hiint(r) & 0x80000000u));
 }
 
 struct ResidualArgs {
@@ -85,16 +89,19 @@ struct ResidualArgs {
     int lanes;                     // blocks that share a colour's strips
     double *partials;       // sums, then (from kMaxPartials) maxima
     double *out;            // [0] sum rt^2, [2] max |rt|
-    double *host;           // the same in page-locked host memory, and [3] the device status
+    double *host;           // the same in page-locked host memory ([2] negative: see MAX), and [3] the device status
     const int *status;
     unsigned *ticket;
-    float *r32[2];          // WRITE: FP32 colour arrays of pitch W32
+    float *r32[2];          // WRITE, MAX: FP32 colour arrays of pitch W32
     int W32;
     double scale, one;
 };
 
-// MAX: also reduce max |rt|.  WRITE: only store (float)(rt * scale) into the FP32 colour arrays at
-// interior points: the scaled defect that the refinement hands to its FP32 inner solver.
+// MAX: also reduce max |rt| and store (float)rt into the FP32 colour arrays at interior points;
+// host[2] is -max where some 0 < |rt| < 2^-102, whose binary32 form, scaled down by up to 2^24, may
+// have lost bits.  WRITE: only
+// store (float)(rt * scale) there: the scaled defect that the refinement hands to its FP32 inner
+// solver.
 // Values per thread: PTS neighbouring ones of a colour row.  The grid is one wave of resident
 // blocks, each walking every gridDim.x-th strip of the red and then of the black points (a grid
 // of strips ran 1.4 waves at 16384^2).  Small grids give the black points blocks of their own.
@@ -107,6 +114,7 @@ __global__ void __launch_bounds__(kSweepThreads) residual_kernel(const ResidualA
     const double one = a.one;
     const int lane = threadIdx.x & 31;
     double acc = 0.0, mx = 0.0;
+    bool tiny = false;
     const int own = (int)blockIdx.x >= a.lanes ? 1 : 0;  // blocks past `lanes`: the black points alone
     const int last_colour = (int)gridDim.x > a.lanes ? own : a.colours - 1;
     for (int colour = own; colour <= last_colour; ++colour) {
@@ -141,6 +149,7 @@ __global__ void __launch_bounds__(kSweepThreads) residual_kernel(const ResidualA
                     for (int q = 0; q < PTS; ++q) w[q] = mid[q], e[q] = q + 1 < PTS ? mid[q + 1 < PTS ? q + 1 : 0] : x;
                 }
                 const int j0 = 2 * k0 + p;
+                float keep[PTS];
 #pragma unroll
                 for (int q = 0; q < PTS; ++q) {
                     if (!(act && j0 + 2 * q >= 1 && j0 + 2 * q <= n)) continue;
@@ -153,9 +162,21 @@ __global__ void __launch_bounds__(kSweepThreads) residual_kernel(const ResidualA
                         acc = __fma_rn(r, r, acc);
                         // |r| compares as its bits do; a NaN sorts above everything and the sum shows it
                         if (MAX) {
-                            const double m = __longlong_as_double(__double_as_longlong(r) & 0x7FFFFFFFFFFFFFFFll);
-                            mx = __double_as_longlong(m) > __double_as_longlong(mx) ? m : mx;
+                            const long long m = __double_as_longlong(r) & 0x7FFFFFFFFFFFFFFFll;
+                            tiny |= (unsigned long long)(m - 1) < 0x398FFFFFFFFFFFFFull;  // 2^-102: 0x399 << 52
+                            keep[q] = narrow(r, m);
+                            mx = m > __double_as_longlong(mx) ? __longlong_as_double(m) : mx;
                         }
+                    }
+                }
+                if (MAX) {
+                    float *to = r32 + (size_t)i * a.W32 + k0;
+                    if (PTS == 2 && act && j0 >= 1 && j0 + 2 <= n) {
+                        *reinterpret_cast<float2 *>(to) = make_float2(keep[0], keep[PTS - 1]);
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < PTS; ++q)
+                            if (act && j0 + 2 * q >= 1 && j0 + 2 * q <= n) to[q] = keep[q];
                     }
                 }
 #pragma unroll
@@ -168,17 +189,24 @@ __global__ void __launch_bounds__(kSweepThreads) residual_kernel(const ResidualA
     const double t = block_sum<kSweepThreads>(acc, smem);
     if (threadIdx.x == 0) a.partials[slot] = t;
     if (MAX) {
-        __syncthreads();
+        const bool any = __syncthreads_or(tiny);
         const double m = block_max<kSweepThreads>(mx, smem);
-        if (threadIdx.x == 0) a.partials[kMaxPartials + slot] = m;
+        if (threadIdx.x == 0) a.partials[kMaxPartials + slot] = any ? -m : m;
     }
     if (!last_block<kSweepThreads>(a.ticket, blocks)) return;
     const double sum = sum_partials<kSweepThreads>(a.partials, blocks, smem);
     if (threadIdx.x == 0) a.out[0] = a.host[0] = sum, a.host[3] = (double)*a.status;
     if (MAX) {
-        __syncthreads();
-        const double m = max_partials<kSweepThreads>(a.partials + kMaxPartials, blocks, smem);
-        if (threadIdx.x == 0) a.out[2] = a.host[2] = m;
+        bool any = false;
+        double v = 0.0;
+        for (int q = threadIdx.x; q < blocks; q += kSweepThreads) {
+            const double m = __ldcg(a.partials + kMaxPartials + q);
+            any |= m < 0.0;
+            v = fmax(v, fabs(m));
+        }
+        any = __syncthreads_or(any);
+        const double m = block_max<kSweepThreads>(v, smem);
+        if (threadIdx.x == 0) a.out[2] = m, a.host[2] = any ? -m : m;
     }
 }
 
@@ -276,7 +304,7 @@ rbgs_status residual_pass(const rbgs_ctx *c, double scale, cudaStream_t s, bool 
     ResidualArgs a;
     for (int q = 0; q < 2; ++q) {
         a.u[q] = c->f64.u[q], a.hf[q] = c->f64.hf[q];
-        a.r32[q] = WRITE ? c->f32.hf[q] : nullptr;
+        a.r32[q] = WRITE || MAX ? c->f32.hf[q] : nullptr;
     }
     a.n = g.n, a.W = g.W, a.kact = active_width(g.n), a.W32 = c->f32.W;
     a.colours = red_only ? 1 : 2;
@@ -315,7 +343,7 @@ rbgs_status launch_residual_sum(const rbgs_ctx *c, cudaStream_t s) {
     return residual_pass<false, false>(c, 1.0, s, c->black_fresh);
 }
 
-// write_r32 = false: sum rt^2 -> dsum[0], max |rt| -> dsum[2].
+// write_r32 = false: sum rt^2 -> dsum[0], max |rt| -> dsum[2], r32 = (float)rt at interior points.
 // write_r32 = true:  r32 = (float)(rt * scale) at interior points.
 rbgs_status launch_defect(const rbgs_ctx *c, bool write_r32, double scale, cudaStream_t s) {
     return write_r32 ? residual_pass<false, true>(c, scale, s, false) : residual_pass<true, false>(c, scale, s, false);

@@ -104,6 +104,27 @@ def test_refinement_small_grids_bit_exact(n):
     assert abs(rho - rho_ref) <= 1e-12 * max(rho_ref, 1e-300) or rho == rho_ref
 
 
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 20, 2.0 ** 60, 2.0 ** -20, 2.0 ** -90, 2.0 ** -110, 2.0 ** -125, 2.0 ** -140, 2.0 ** -300])
+@pytest.mark.parametrize("n", [3, 130, 1100])
+def test_refinement_defect_at_any_scale(n, scale):
+    """The scaled defect comes from (float)rt where that loses nothing, else from a second walk:
+    residuals above 1 (scaled down), below it (scaled up), around the smallest normal binary32
+    number, and wholly below the binary32 range.  Bit-exact in each."""
+    f, u0 = _problem(n, 900 + n, interior=False)
+    f, u0 = f * scale, u0 * scale
+    h2 = synth.h_squared(n)
+    ref = u0.copy()
+    done_ref, rho_ref, _ = oracle.refine_solve(ref, f, h2, 1e-30, 9, 22)
+    fd, ud = torch.from_numpy(f).cuda(), torch.from_numpy(u0).cuda()
+    out = torch.empty_like(ud)
+    with rb.Solver(n, h2, fd, ud, precision=rb.RBGS_FP32_REFINE, inner_sweeps=9, max_sweeps=22) as s:
+        done, rho, st = s.solve(1e-30, allow_not_converged=True)
+        s.get_solution(out)
+    assert done == done_ref
+    _assert_bits(out.cpu().numpy(), ref)
+    assert abs(rho - rho_ref) <= 1e-12 * max(rho_ref, 1e-300) or rho == rho_ref
+
+
 @pytest.mark.parametrize("kernel,k", [(rb.RBGS_KERNEL_COLOUR, 0), (rb.RBGS_KERNEL_TEMPORAL, 2),
                                       (rb.RBGS_KERNEL_TEMPORAL, 4), (rb.RBGS_KERNEL_TEMPORAL, 8)])
 @pytest.mark.parametrize("n", [33, 150, 520])
