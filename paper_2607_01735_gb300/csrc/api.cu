@@ -32,14 +32,15 @@ namespace {
 constexpr int kMaxN = 1 << 18;
 constexpr long kGraphSweeps = 32;    // sweeps per cached graph
 constexpr int kGraphMaxN = 2048;     // graphs pay off where launches dominate
-// FP64 sweeps in one cooperative launch (persistent.cu) for kPersistMinN <= n <= kPersistMaxN.
+// FP64 sweeps in one cooperative launch (persistent.cu) for kPersistMinN <= n <= kPersistMaxN,
+// where the resident kernel below does not run.
 // Measured on GB300 against one launch per colour (graphs up to 2048): 0.94x at 383^2,
 // 1.15x at 511^2, 1.29x at 1023^2, 1.32x at 4095^2, 1.10x at 16383^2; below ~400 the grid
 // barrier costs more than a graph's launches.  Above 32768 its flattened item index would
 // leave 32 bits.
 constexpr int kPersistMinN = 416;
 // FP32 inner sweeps in one launch of one 16-block cluster (cluster_sweeps.cu) up to this
-// size.  Measured on GB300 against cached graphs of one launch per colour: 1.42x at 63^2,
+// size, where the resident kernel's buffers cannot be allocated.  Measured on GB300 against cached graphs of one launch per colour: 1.42x at 63^2,
 // 1.46x at 127^2, 0.93x at 255^2, 0.49x at 511^2 (16 SMs do not match the whole GPU there).
 constexpr int kClusterMaxN = 160;
 constexpr int kPersistMaxN = 1 << 15;
@@ -53,7 +54,7 @@ constexpr long kFusedChunk = 1024;
 // 16384^2.
 constexpr int kFusedWaveMinN = 512;
 // The resident kernel (resident.cu): FP64 and fused sweeps wherever its tiles fit (up to about
-// 1200^2, resident_plan decides), FP32 inner sweeps up to 1000^2, above which the wavefront is
+// 1376^2, resident_plan decides), FP32 inner sweeps up to 1000^2, above which the wavefront is
 // as fast and needs no cooperative launch.
 constexpr int kResidentMaxN = 2048, kResident32MaxN = 1000;
 constexpr int kWave32MinN = 1001;    // FP32 inner sweeps as wavefront passes from this size on
@@ -593,7 +594,7 @@ rbgs_status rbgs_create(int n, double h2, const double *f, const double *u_init,
     // graphs (the register wavefront reaches the same FP64-pipe limit, with overlap work on
     // top); the FP32 inner sweeps of the refinement run the register wavefront above 1000^2
     // (a sweep at depth 4 against one launch per colour: 4.1 / 3.5 us at 700^2, 4.2 / 5.0 at
-    // 1023^2, 6.2 / 10 at 2047^2) and one launch per colour (with graphs) on smaller grids
+    // 1023^2, 6.2 / 10 at 2047^2) and the resident kernel on smaller grids
     const bool auto_k = o.kernel == RBGS_KERNEL_AUTO && o.tblock_k == 0;
     const bool default_shape = o.fp64_emulate == -1 && o.int_rows <= 0 && (o.sweep_values == 0 || o.sweep_values == 2) &&
                                (o.sweep_rows == 0 || o.sweep_rows == 1) && o.tile_rows == 0;

@@ -291,7 +291,7 @@ bool slab_conv_launch(const uint16_t *src, const uint16_t *wts, const float *bia
     a.relu = relu, a.y_fp32 = y_fp32, a.accumulate = accumulate;
     a.tiles_x = (W + 7) / 8, a.tiles_y = (H + 15) / 16;
     const long tiles = (long)B * a.tiles_x * a.tiles_y;
-    if (tiles > 0x7fffffffL) return false;
+    if (tiles > 0x7fffffffL - 4096) return false;  // a tile index plus a step of the grid stays in range
     a.num_tiles = (int)tiles;
     uint32_t cols = 32;
     while ((int)cols < kSlabAcc * N) cols <<= 1;

@@ -104,12 +104,13 @@ def test_refinement_small_grids_bit_exact(n):
     assert abs(rho - rho_ref) <= 1e-12 * max(rho_ref, 1e-300) or rho == rho_ref
 
 
-@pytest.mark.parametrize("scale", [1.0, 2.0 ** 20, 2.0 ** 60, 2.0 ** -20, 2.0 ** -90, 2.0 ** -110, 2.0 ** -125, 2.0 ** -140, 2.0 ** -300])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 20, 2.0 ** 60, 2.0 ** -20, 2.0 ** -90, 2.0 ** -110, 2.0 ** -125, 2.0 ** -140, 2.0 ** -300, 2.0 ** -500, 2.0 ** 500])
 @pytest.mark.parametrize("n", [3, 130, 1100])
 def test_refinement_defect_at_any_scale(n, scale):
     """The scaled defect comes from (float)rt where that loses nothing, else from a second walk:
     residuals above 1 (scaled down), below it (scaled up), around the smallest normal binary32
-    number, and wholly below the binary32 range.  Bit-exact in each."""
+    number, and wholly below the binary32 range; corrections at
+    the same scales.  Bit-exact in each."""
     f, u0 = _problem(n, 900 + n, interior=False)
     f, u0 = f * scale, u0 * scale
     h2 = synth.h_squared(n)
