@@ -1,6 +1,6 @@
 // TMA-fed tcgen05 convolution for the data-gradient product (written for the forward
-// product too, where the cp.async gathers are as fast: 16 images, 132^2 192->64 207 us against
-// 191, 66^2 384->128 124 against 120, 33^2 256->256 41 against 33; both read L2 at 7.7 TB/s).  Included by conv_umma.cu
+// product too, where the cp.async gathers are faster: 16 images, 132^2 192->64 207 us against
+// 171, 66^2 384->128 124 against 107, 33^2 256->256 41 against 29).  Included by conv_umma.cu
 // inside its anonymous namespace: it shares that file's PTX helpers, bounded waits and
 // wait-failure flag.
 //

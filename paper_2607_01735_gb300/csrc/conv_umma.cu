@@ -257,62 +257,70 @@ __device__ void produce(const UArgs &a, uint32_t sbase, uint32_t stage_bytes, ui
     bool live = true;
 
     if (MODE != U_BWD_WEIGHT) {
-        // K-major A and B: this thread fills rows 8 (rh0 + 4 it) + row_lo, chunk kc.
-        const int row_lo = ptid & 7, kc = (ptid >> 3) & 7, rh0 = ptid >> 6;
-        const uint32_t sw = (uint32_t)(row_lo * 128 + ((kc ^ row_lo) << 4));
+        // K-major A and B: this thread fills rows 8 (rh0 + 4 it) + row_lo, chunk kc.  Eight
+        // neighbouring threads copy the 128 bytes of one row: one line to read, eight banks to write.
+        // The copies bound this kernel, and their instructions with them (a switch added to each
+        // stage cost 8%), so what a copy needs is kept per tile: the taps that lie inside the image
+        // as bits, and pointers that a stage advances by one offset.  Forward, 16 images, us, before
+        // with bounds checks and products per copy, and now: 132^2 192->64 191, 171; 66^2 384->128
+        // 120, 107, 128->128 49, 43; 33^2 256->256 33, 29.
+        const int kc = ptid & 7, row_lo = (ptid >> 3) & 7, rh0 = ptid >> 6;
+        const uint32_t sw = (uint32_t)(row_lo * 128 + ((kc ^ row_lo) << 4)) + (uint32_t)rh0 * 1024u;
         const int CK = MODE == U_FWD ? a.Cin : a.Cout;
         const uint16_t *src = MODE == U_FWD ? a.X : a.G;
+        const int taps = a.ks * a.ks, flip = MODE == U_BWD_DATA ? -1 : 1;
         const int t_init = (kc * 8) / CK, ch_init = kc * 8 - t_init * CK;
-        const int tx_init = t_init % a.ks, ty_init = t_init / a.ks;
+        const int b_copies = (b_vecs - ptid + kProducers - 1) / kProducers;  // of this thread, per stage
+        const long b_row = MODE == U_FWD ? a.K : a.Cout;                    // elements between B's rows
+        const long b_tap = MODE == U_FWD ? a.Cin : (long)a.Cin * a.Cout;    // and between its taps
         for (int tile = blockIdx.x; tile < a.num_tiles && live; tile += gridDim.x) {
             const Tile T = decode_tile<MODE>(a, tile);
-            int pyx[4];
-            long mbase[4];
+            uint32_t inside[4], cols = 0;  // bit t: tap t of the row's pixel; bit it: row it of B
+            const uint16_t *pa[4];
 #pragma unroll
             for (int it = 0; it < 4; ++it) {
                 const int m = T.m0 + (rh0 + 4 * it) * 8 + row_lo;
+                inside[it] = 0;
+                pa[it] = src;
                 if (m < a.M) {
                     const uint32_t r = (uint32_t)m - fdiv((uint32_t)m, a.div_hw) * HW;
-                    const uint32_t y = fdiv(r, a.div_w);
-                    pyx[it] = (int)((y << 16) | (r - y * (uint32_t)a.W));
-                    mbase[it] = (long)m * CK;
-                } else {
-                    pyx[it] = -1;
-                    mbase[it] = 0;
+                    const int y = (int)fdiv(r, a.div_w), x = (int)r - y * a.W;
+                    // tap offsets -1, 0, 1 inside: bits 0..2; the data gradient's taps run backwards
+                    auto near = [&](int v, int n) { return (uint32_t)(v > 0) | 2u | (uint32_t)(v + 1 < n) << 2; };
+                    uint32_t in_x = near(x, a.W), in_y = near(y, a.H);
+                    if (MODE == U_BWD_DATA) in_x = __brev(in_x) >> 29, in_y = __brev(in_y) >> 29;
+                    inside[it] = a.ks == 1 ? 1u
+                                           : ((in_y & 1u) ? in_x : 0u) | ((in_y & 2u) ? in_x << 3 : 0u) |
+                                                 ((in_y & 4u) ? in_x << 6 : 0u);
+                    pa[it] = src + (long)m * CK;
                 }
             }
-            int ch = ch_init, tx = tx_init, ty = ty_init;
+#pragma unroll
+            for (int it = 0; it < kMaxBn * 8 / kProducers; ++it)
+                cols |= (uint32_t)(T.n0 + (rh0 + 4 * it) * 8 + row_lo < a.N) << it;
+            const uint16_t *pb = a.Wt + (long)(T.n0 + rh0 * 8 + row_lo) * b_row;
+            int ch = ch_init, t = t_init;
             for (int kt = 0; kt < T.KT; ++kt) {
                 if (!wait_or_abort(&empty_bar[s], ph ^ 1u, abort_flag)) {
                     live = false;
                     break;
                 }
-                const uint32_t sa = sbase + s * stage_bytes, sb = sa + a_bytes;
-                const bool kval = ty < a.ks;  // tap index < taps
-                int dy = ty - pad, dx = tx - pad;
-                if (MODE == U_BWD_DATA) dy = -dy, dx = -dx;
-                const long delta = ((long)dy * a.W + dx) * CK + ch;
+                const uint32_t sa = sbase + s * stage_bytes + sw, sb = sa + a_bytes;
+                const int ty = t >= 2 * a.ks ? 2 : (t >= a.ks ? 1 : 0), tx = t - ty * a.ks;
+                const int delta = flip * ((ty - pad) * a.W + tx - pad) * CK + ch;
 #pragma unroll
                 for (int it = 0; it < 4; ++it) {
-                    const int yx = pyx[it];
-                    const int y = (yx >> 16) + dy, x = (yx & 0xFFFF) + dx;
-                    const bool ok = kval && yx >= 0 && y >= 0 && y < a.H && x >= 0 && x < a.W;
-                    cp_async16(sa + (uint32_t)(rh0 + 4 * it) * 1024u + sw, ok ? src + mbase[it] + delta : src, ok);
+                    const bool ok = inside[it] >> t & 1u;  // no bit past the last tap
+                    cp_async16(sa + (uint32_t)it * 4096u, ok ? pa[it] + delta : src, ok);
                 }
+                const uint16_t *p = pb + t * b_tap + ch;
+                const uint32_t valid = t < taps ? cols : 0u;
 #pragma unroll
                 for (int it = 0; it < kMaxBn * 8 / kProducers; ++it) {
-                    const int v = ptid + kProducers * it;
-                    if (v >= b_vecs) break;
-                    const int n = T.n0 + (rh0 + 4 * it) * 8 + row_lo;
-                    const bool ok = kval && n < a.N;
-                    const uint16_t *p = a.Wt;
-                    if (ok) {
-                        if (MODE == U_FWD)
-                            p = a.Wt + (long)n * a.K + kt * UK + kc * 8;  // Wt[o][t][c], k = t Cin + c
-                        else
-                            p = a.Wt + ((long)(ty * a.ks + tx) * a.Cin + n) * a.Cout + ch;  // Wt_t[t][c][o]
-                    }
-                    cp_async16(sb + (uint32_t)(rh0 + 4 * it) * 1024u + sw, p, ok);
+                    if (it >= b_copies) break;
+                    const bool ok = valid >> it & 1u;
+                    cp_async16(sb + (uint32_t)it * 4096u, ok ? p : a.Wt, ok);
+                    p += 32 * b_row;
                 }
                 cp_async_commit();
                 ++issued;
@@ -324,10 +332,7 @@ __device__ void produce(const UArgs &a, uint32_t sbase, uint32_t stage_bytes, ui
                     if (++s_arr == (uint32_t)S) s_arr = 0;
                 }
                 ch += UK;
-                while (ch >= CK) {
-                    ch -= CK;
-                    if (++tx == a.ks) tx = 0, ++ty;
-                }
+                while (ch >= CK) ch -= CK, ++t;
                 if (++s == (uint32_t)S) s = 0, ph ^= 1u;
             }
         }
