@@ -45,6 +45,7 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "conv_index.cuh"
 #include "conv_wait.cuh"
 #include "tma.cuh"
 #include "../../include/rbgs_unet.h"
@@ -243,7 +244,8 @@ __device__ __forceinline__ Tile decode_tile(const UArgs &a, int tile) {
 }
 
 // ------------------------------------------------------------------ producers
-template <int MODE>
+// Offset: the type that holds an element offset between neighbouring rows (conv_index.cuh).
+template <int MODE, typename Offset>
 __device__ void produce(const UArgs &a, uint32_t sbase, uint32_t stage_bytes, uint64_t *full_bar,
                         uint64_t *empty_bar, volatile int *abort_flag) {
     const int ptid = threadIdx.x;  // 0..255
@@ -307,7 +309,7 @@ __device__ void produce(const UArgs &a, uint32_t sbase, uint32_t stage_bytes, ui
                 }
                 const uint32_t sa = sbase + s * stage_bytes + sw, sb = sa + a_bytes;
                 const int ty = t >= 2 * a.ks ? 2 : (t >= a.ks ? 1 : 0), tx = t - ty * a.ks;
-                const int delta = flip * ((ty - pad) * a.W + tx - pad) * CK + ch;
+                const Offset delta = tap_offset<Offset>(flip * (ty - pad), flip * (tx - pad), a.W, CK, ch);
 #pragma unroll
                 for (int it = 0; it < 4; ++it) {
                     const bool ok = inside[it] >> t & 1u;  // no bit past the last tap
@@ -527,7 +529,7 @@ __device__ void drain(const UArgs &a, uint32_t tmem, uint64_t *tfull_bar, uint64
 }
 
 // ------------------------------------------------------------------ kernel
-template <int MODE>
+template <int MODE, typename Offset>
 __global__ void __launch_bounds__(kThreads, 1) conv_umma_kernel(const UArgs a) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], tfull_bar[2], tempty_bar[2];
@@ -563,7 +565,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_umma_kernel(const UArgs a) {
     const uint32_t tmem = tmem_slot;
 
     if (warp < kMmaWarp) {
-        produce<MODE>(a, sbase, stage_bytes, full_bar, empty_bar, abort_flag);
+        produce<MODE, Offset>(a, sbase, stage_bytes, full_bar, empty_bar, abort_flag);
     } else if (warp == kMmaWarp) {
         if (elect_one())
             issue_mmas<MODE>(a, sbase, stage_bytes, tmem, full_bar, empty_bar, tfull_bar, tempty_bar, abort_flag);
@@ -619,15 +621,15 @@ void finish_args(UArgs &a, int B) {
     (void)B;
 }
 
-template <int MODE>
+template <int MODE, typename Offset = int>
 rbgs_status launch(const UArgs &a, cudaStream_t s) {
     // set once per kernel instance, thread-safely; a failure is reported on every call
-    static const cudaError_t attr = cudaFuncSetAttribute(conv_umma_kernel<MODE>,
+    static const cudaError_t attr = cudaFuncSetAttribute(conv_umma_kernel<MODE, Offset>,
                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
     RBGS_CUDA(attr);
     const size_t smem = (size_t)a.stages * (UM + a.bn) * UK * 2 + 1024;
     const int grid = a.num_tiles < sm_count() ? a.num_tiles : sm_count();
-    conv_umma_kernel<MODE><<<grid, kThreads, smem, s>>>(a);
+    conv_umma_kernel<MODE, Offset><<<grid, kThreads, smem, s>>>(a);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
@@ -658,7 +660,7 @@ rbgs_status umma_conv_forward(const uint16_t *X, const uint16_t *Wt, const float
     a.bn = pick_bn(a.N);
     finish_args(a, B);
     a.num_tiles = a.m_tiles * a.n_tiles;
-    return launch<U_FWD>(a, s);
+    return offsets_fit_int(W, Cin) ? launch<U_FWD>(a, s) : launch<U_FWD, long>(a, s);
 }
 
 rbgs_status umma_conv_backward_data(const uint16_t *Wtt, const uint16_t *G, float *dX, const uint16_t *Y,
