@@ -108,6 +108,14 @@ int rbgs_conv_get_wgrad_kernel(void);
 
 /*
  * Not in the paper (learned initial guess): library mechanics.
+ * The weight-gradient kernel (RBGS_WGRAD_RING, _TAPROW or _GATHER) that the tcgen05 engines take
+ * for a layer under the current choice, with a 16-byte aligned dW.  -1 for sizes that
+ * rbgs_conv_backward refuses.
+ */
+int rbgs_conv_wgrad_kernel_for(int B, int H, int W, int Cin, int Cout, int ksize);
+
+/*
+ * Not in the paper (learned initial guess): library mechanics.
  * Synchronises `cuda_stream` and reports whether a tcgen05 convolution launched since
  * the last check gave up one of its bounded waits on the tensor cores (RBGS_ETIMEOUT; its
  * output is then incomplete).  Clears the condition.  RBGS_OK otherwise.

@@ -276,6 +276,7 @@ rbgs_status umma_conv_backward_data(const uint16_t *Wtt, const uint16_t *G, floa
                                     bool tma, cudaStream_t s);
 rbgs_status umma_conv_backward_weight(const uint16_t *X, const uint16_t *G, float *dW, int B, int H, int W,
                                       int Cin, int Cout, int ks, int kind, cudaStream_t s);
+int umma_wgrad_kernel_for(int B, int H, int W, int Cin, int Cout, int ks, int kind);
 rbgs_status umma_conv_check(cudaStream_t s);
 
 rbgs_status conv_forward(const uint16_t *X, const uint16_t *Wt, const float *bias, void *Y, int B, int H,
@@ -424,6 +425,11 @@ extern "C" rbgs_status rbgs_conv_set_wgrad_kernel(int kind) {
 }
 
 extern "C" int rbgs_conv_get_wgrad_kernel(void) { return g_wgrad_kind; }
+
+extern "C" int rbgs_conv_wgrad_kernel_for(int B, int H, int W, int Cin, int Cout, int ksize) {
+    if (!conv_shapes_ok(B, H, W, Cin, Cout, ksize)) return -1;
+    return umma_wgrad_kernel_for(B, H, W, Cin, Cout, ksize, g_wgrad_kind);
+}
 
 extern "C" rbgs_status rbgs_conv_check(void *cuda_stream) {
     clear_error();

@@ -16,6 +16,7 @@ __host__ __device__ __forceinline__ Offset tap_offset(int dy, int dx, int W, int
     return (Offset)(dy * W + dx) * C + ch;
 }
 
+// Offsets within W + 2 neighbouring pixels of C channels fit an int.
 inline bool offsets_fit_int(int W, int C) { return ((long)W + 2) * C <= 0x7fffffffL; }
 
 }  // namespace rbgs

@@ -641,6 +641,26 @@ bool sizes_fit(int B, int H, int W) { return (long)B * H * W < (1L << 31) - UK; 
 #include "conv_wgrad.cuh"
 #include "conv_wgrad_ring.cuh"
 
+// 3x3 layers: the ring kernel (conv_wgrad_ring.cuh) or the tap-row kernel (conv_wgrad.cuh),
+// whose epilogue adds 16-byte vectors, else the gather kernel below.  The automatic choice
+// follows the per-layer measurements on GB300 (U-Net layers at 16 x 264^2, us, ring / tap row /
+// gather): Cin <= 32: 16->32 70 / 136 / 134, 32->32 72 / 141 / 267, at 132^2 32->64
+// 42 / 52 / 66; the other layers with >= 40 tap-row stages per SM and rows >= 64 pixels:
+// 132^2 64->64 72 / 70 / 114, 192->64 537 / 166 / 362, 264^2 96->32 262 / 210 / 637, 66^2
+// 384->128 - / 112 / 245; the rest (stages per SM ~20, or 33-pixel rows): 33^2 128->256
+// 256 / 56 / 37, 256->256 553 / 65 / 62.
+// Returns the kernel and, for the first two, fills in its plan.
+int pick_wgrad(int B, int H, int W, int Cin, int Cout, int ks, int kind, bool aligned, WrPlan &ring, WgPlan &taprow) {
+    if (ks != 3 || kind == RBGS_WGRAD_GATHER || !aligned) return RBGS_WGRAD_GATHER;
+    if ((kind == RBGS_WGRAD_RING || (kind == RBGS_WGRAD_AUTO && Cin <= 32)) &&
+        wr_plan(B, H, W, Cin, Cout, sm_count(), ring))
+        return RBGS_WGRAD_RING;
+    if (wg_plan(B, H, W, Cin, Cout, sm_count(), taprow) &&
+        (kind != RBGS_WGRAD_AUTO || (W >= 64 && taprow.a.f_per_cta >= 40)))
+        return RBGS_WGRAD_TAPROW;
+    return RBGS_WGRAD_GATHER;
+}
+
 }  // namespace
 
 rbgs_status umma_conv_forward(const uint16_t *X, const uint16_t *Wt, const float *bias, void *Y, int B, int H,
@@ -691,28 +711,12 @@ rbgs_status umma_conv_backward_weight(const uint16_t *X, const uint16_t *G, floa
         set_error("tcgen05 convolution: at most 2^31 - 64 pixels");
         return RBGS_EINVAL;
     }
-    // 3x3 layers: the ring kernel (conv_wgrad_ring.cuh) or the tap-row kernel (conv_wgrad.cuh),
-    // whose epilogue adds 16-byte vectors, else the gather kernel below.  The automatic choice
-    // follows the per-layer measurements on GB300 (U-Net layers at 16 x 264^2, us, ring / tap row /
-    // gather): Cin <= 32: 16->32 70 / 136 / 134, 32->32 72 / 141 / 267, at 132^2 32->64
-    // 42 / 52 / 66; the other layers with >= 40 tap-row stages per SM and rows >= 64 pixels:
-    // 132^2 64->64 72 / 70 / 114, 192->64 537 / 166 / 362, 264^2 96->32 262 / 210 / 637, 66^2
-    // 384->128 - / 112 / 245; the rest (stages per SM ~20, or 33-pixel rows): 33^2 128->256
-    // 256 / 56 / 37, 256->256 553 / 65 / 62.
-    if (ks == 3 && kind != RBGS_WGRAD_GATHER && (reinterpret_cast<uintptr_t>(dW) & 15u) == 0) {
-        bool launched = false;
-        rbgs_status st = RBGS_OK;
-        if (kind == RBGS_WGRAD_RING || (kind == RBGS_WGRAD_AUTO && Cin <= 32)) {
-            st = wr_launch(X, G, dW, B, H, W, Cin, Cout, s, &launched);
-            if (st != RBGS_OK || launched) return st;
-        }
-        WgPlan pl;
-        const bool fits = wg_plan(B, H, W, Cin, Cout, sm_count(), pl);
-        if (fits && (kind != RBGS_WGRAD_AUTO || (W >= 64 && pl.a.f_per_cta >= 40))) {
-            st = wg_launch(pl, X, G, dW, s);
-            if (st != RBGS_OK) return st;
-            return RBGS_OK;
-        }
+    WrPlan ring;
+    WgPlan taprow;
+    switch (pick_wgrad(B, H, W, Cin, Cout, ks, kind, (reinterpret_cast<uintptr_t>(dW) & 15u) == 0, ring, taprow)) {
+    case RBGS_WGRAD_RING: return wr_launch(ring, X, G, dW, s);
+    case RBGS_WGRAD_TAPROW: return wg_launch(taprow, X, G, dW, s);
+    default: break;
     }
     UArgs a{};
     a.X = X, a.G = G, a.out = dW;
@@ -735,6 +739,12 @@ rbgs_status umma_conv_backward_weight(const uint16_t *X, const uint16_t *G, floa
     chunks = (a.K + chunk - 1) / chunk;  // every chunk non-empty
     a.num_tiles = mn_tiles * chunks;
     return launch<U_BWD_WEIGHT>(a, s);
+}
+
+int umma_wgrad_kernel_for(int B, int H, int W, int Cin, int Cout, int ks, int kind) {
+    WrPlan ring;
+    WgPlan taprow;
+    return pick_wgrad(B, H, W, Cin, Cout, ks, kind, true, ring, taprow);
 }
 
 rbgs_status umma_conv_check(cudaStream_t s) {

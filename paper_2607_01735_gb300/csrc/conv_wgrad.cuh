@@ -404,6 +404,8 @@ bool wg_plan(int B, int H, int W, int Cin, int Cout, int sms, WgPlan &pl) {
         const uint32_t as = (uint32_t)(a.ngA * lenA * 16), bs = (uint32_t)(a.ngB * lenB * 16);
         const uint32_t b_reach = (uint32_t)((16 * (nk - 1) + (a.xa ? 0 : 2)) * 16 + (a.ngB - 1) * lenB * 16 + 256);
         if (b_reach > bs) continue;
+        // a staged row's element offsets (WgUnits::off) fit an int
+        if (!offsets_fit_int(seg, Cin > Cout ? Cin : Cout)) continue;
         // every staged row fits the producers' unit tables
         const int ngx = a.xa ? a.ngA : a.ngB, ngg = a.xa ? a.ngB : a.ngA;
         if (ngx * (seg + 2) > kWgMaxUnits * kWgProducers || ngg * seg > kWgMaxUnits * kWgProducers) continue;
@@ -447,7 +449,7 @@ bool wg_plan(int B, int H, int W, int Cin, int Cout, int sms, WgPlan &pl) {
 }
 
 // Launches the tap-row weight gradient for a plan of wg_plan.
-rbgs_status wg_launch(WgPlan pl, const uint16_t *X, const uint16_t *G, float *dW, cudaStream_t s) {
+rbgs_status wg_launch(WgPlan &pl, const uint16_t *X, const uint16_t *G, float *dW, cudaStream_t s) {
     static const cudaError_t attr = cudaFuncSetAttribute(wgrad_shift_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                          (int)(kWgBudget + 1024));
     RBGS_CUDA(attr);

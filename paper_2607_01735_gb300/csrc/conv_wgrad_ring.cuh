@@ -373,17 +373,13 @@ bool wr_plan(int B, int H, int W, int Cin, int Cout, int sms, WrPlan &pl) {
     return true;
 }
 
-rbgs_status wr_launch(const uint16_t *X, const uint16_t *G, float *dW, int B, int H, int W, int Cin, int Cout,
-                      cudaStream_t s, bool *launched) {
-    *launched = false;
-    WrPlan pl;
-    if (!wr_plan(B, H, W, Cin, Cout, sm_count(), pl)) return RBGS_OK;
+// Launches the ring weight gradient for a plan of wr_plan.
+rbgs_status wr_launch(WrPlan &pl, const uint16_t *X, const uint16_t *G, float *dW, cudaStream_t s) {
     static const cudaError_t attr = cudaFuncSetAttribute(wgrad_ring_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                          (int)(kWgBudget + 1024));
     RBGS_CUDA(attr);
     pl.a.X = X, pl.a.G = G, pl.a.dW = dW;
     wgrad_ring_kernel<<<pl.grid, kWgThreads, pl.smem, s>>>(pl.a);
     RBGS_LAUNCH_CHECK();
-    *launched = true;
     return RBGS_OK;
 }

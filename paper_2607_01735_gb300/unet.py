@@ -49,6 +49,8 @@ def _lib():
         lib.rbgs_conv_set_wgrad_kernel.restype = ci
         lib.rbgs_conv_get_wgrad_kernel.argtypes = []
         lib.rbgs_conv_get_wgrad_kernel.restype = ci
+        lib.rbgs_conv_wgrad_kernel_for.argtypes = [ci] * 6
+        lib.rbgs_conv_wgrad_kernel_for.restype = ci
         lib.rbgs_conv_check.argtypes = [vp]
         lib.rbgs_conv_check.restype = ci
         lib.rbgs_guess_blend.argtypes = [vp, ci, vp, vp]
@@ -108,6 +110,11 @@ def rbgs_conv_set_wgrad_kernel(kind: int) -> None:
 
 def rbgs_conv_get_wgrad_kernel() -> int:
     return int(_lib().rbgs_conv_get_wgrad_kernel())
+
+
+def rbgs_conv_wgrad_kernel_for(B: int, H: int, W: int, Cin: int, Cout: int, ksize: int = 3) -> int:
+    """The weight-gradient kernel taken for a layer: RBGS_WGRAD_RING, _TAPROW or _GATHER."""
+    return int(_lib().rbgs_conv_wgrad_kernel_for(int(B), int(H), int(W), int(Cin), int(Cout), int(ksize)))
 
 
 def rbgs_conv_check(device=None) -> None:

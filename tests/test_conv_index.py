@@ -30,6 +30,7 @@ def lib():
     l = ctypes.CDLL(OUT)
     l.check_tap_offset.argtypes = [ctypes.c_int] * 5
     l.check_tap_offset.restype = ctypes.c_long
+    l.check_offsets_fit_int.argtypes = [ctypes.c_int] * 2
     return l
 
 
@@ -42,3 +43,24 @@ def test_tap_offsets_of_rows_beyond_32_bits(lib, W, C):
         for dx in (-1, 0, 1):
             for ch in (0, 8, C - 8):
                 assert lib.check_tap_offset(dy, dx, W, C, ch) == (dy * W + dx) * C + ch
+
+
+@pytest.mark.parametrize("seg", [16, 144, 160])
+def test_offsets_of_a_staged_row_fit_an_int(lib, seg):
+    """seg + 2 pixels of C channels, at the largest C that fits and the next one accepted."""
+    most = (2 ** 31 - 1) // (seg + 2) // 8 * 8
+    assert lib.check_offsets_fit_int(seg, most) and not lib.check_offsets_fit_int(seg, most + 8)
+
+
+def test_tap_row_weight_gradient_leaves_rows_that_its_offsets_do_not_hold():
+    """The tap-row kernel keeps its copies' offsets within a segment of a row in 32 bits: from
+    2^31 / 18 channels no segment fits, and the gather kernel, whose offsets are 64-bit, runs."""
+    from paper_2607_01735_gb300 import build, unet as un
+    build.build_library()
+    un.rbgs_conv_set_wgrad_kernel(un.RBGS_WGRAD_TAPROW)
+    try:
+        assert un.rbgs_conv_wgrad_kernel_for(1, 1, 161, 1 << 23, 8) == un.RBGS_WGRAD_TAPROW
+        assert un.rbgs_conv_wgrad_kernel_for(1, 1, 161, 1 << 27, 8) == un.RBGS_WGRAD_GATHER
+        assert un.rbgs_conv_wgrad_kernel_for(1, 1, 161, 8, 12) == -1
+    finally:
+        un.rbgs_conv_set_wgrad_kernel(un.RBGS_WGRAD_AUTO)
