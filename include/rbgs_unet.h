@@ -86,7 +86,7 @@ int rbgs_conv_get_engine(void);
  *   RBGS_WGRAD_AUTO   (default) per layer shape, the kernel that measured fastest on GB300
  *                     over the network's layers: RBGS_WGRAD_RING for Cin <= 32;
  *                     RBGS_WGRAD_TAPROW for image rows of at least 64 pixels when its work
- *                     split gives every SM at least 40 stages; RBGS_WGRAD_GATHER otherwise;
+ *                     split gives every SM at least 1200 pixel steps; RBGS_WGRAD_GATHER otherwise;
  *   RBGS_WGRAD_RING   all nine taps per stage: each activation row is staged once as three
  *                     copies shifted by one pixel and kept in a ring while the output rows
  *                     walk down the image (M = 3 Cin rows of (tap column, channel));

@@ -643,12 +643,21 @@ bool sizes_fit(int B, int H, int W) { return (long)B * H * W < (1L << 31) - UK; 
 
 // 3x3 layers: the ring kernel (conv_wgrad_ring.cuh) or the tap-row kernel (conv_wgrad.cuh),
 // whose epilogue adds 16-byte vectors, else the gather kernel below.  The automatic choice
-// follows the per-layer measurements on GB300 (U-Net layers at 16 x 264^2, us, ring / tap row /
-// gather): Cin <= 32: 16->32 70 / 136 / 134, 32->32 72 / 141 / 267, at 132^2 32->64
-// 42 / 52 / 66; the other layers with >= 40 tap-row stages per SM and rows >= 64 pixels:
-// 132^2 64->64 72 / 70 / 114, 192->64 537 / 166 / 362, 264^2 96->32 262 / 210 / 637, 66^2
-// 384->128 - / 112 / 245; the rest (stages per SM ~20, or 33-pixel rows): 33^2 128->256
-// 256 / 56 / 37, 256->256 553 / 65 / 62.
+// follows the per-layer measurements on GB300 (U-Net layers, us):
+//   Cin <= 32: the ring.  16 images, ring / tap row / gather: 264^2 16->32 72 / 137 / 136, 32->32
+//     74 / 143 / 269, 132^2 32->64 44 / 54 / 68;
+//   rows of 64 pixels and more, and kTapRowPixels pixel steps for each CTA (stages times the
+//     segment's pixels, so a longer segment with fewer stages is the same work): the tap row, whose
+//     fixed costs (filling the ring, one drain of three accumulators per item) are paid by then.
+//     Pixel steps, gather / tap row: 66^2 128->128 880 41.0 / 46.7, 1120 49.5 / 48.7, 1280 56.9 /
+//     48.1, 1680 72.1 / 69.3; 66^2 64->128 880 29.6 / 29.7, 1280 35.4 / 32.0, 1520 39.1 / 40.2,
+//     1680 47.2 / 43.7; 66^2 384->128 720 36.5 / 36.9, 1280 69.7 / 44.6, 5120 248 / 112; 132^2
+//     64->64 864 22.2 / 19.7, 1584 35.6 / 26.9, 6048 115 / 73.7; 264^2 96->32 75.8 / 42.5 and
+//     132^2 192->64 92 / 53 at batches 2 and 4;
+//   the rest: the gather kernel (33-pixel rows, 16 images, gather / tap row: 128->256 39 / 57,
+//     256->256 63 / 67).
+constexpr int kTapRowPixels = 1200;
+
 // Returns the kernel and, for the first two, fills in its plan.
 int pick_wgrad(int B, int H, int W, int Cin, int Cout, int ks, int kind, bool aligned, WrPlan &ring, WgPlan &taprow) {
     if (ks != 3 || kind == RBGS_WGRAD_GATHER || !aligned) return RBGS_WGRAD_GATHER;
@@ -656,7 +665,7 @@ int pick_wgrad(int B, int H, int W, int Cin, int Cout, int ks, int kind, bool al
         wr_plan(B, H, W, Cin, Cout, sm_count(), ring))
         return RBGS_WGRAD_RING;
     if (wg_plan(B, H, W, Cin, Cout, sm_count(), taprow) &&
-        (kind != RBGS_WGRAD_AUTO || (W >= 64 && taprow.a.f_per_cta >= 40)))
+        (kind != RBGS_WGRAD_AUTO || (W >= 64 && taprow.a.f_per_cta * taprow.a.seg >= kTapRowPixels)))
         return RBGS_WGRAD_TAPROW;
     return RBGS_WGRAD_GATHER;
 }
