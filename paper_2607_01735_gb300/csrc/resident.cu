@@ -9,15 +9,14 @@
 // a block needs its halo's black values again (the red ones are recomputed), 2K rows and K values
 // of a colour row deep, from its eight neighbours: no wait on any other block.
 //
-// Exchange: a slot of global memory per black point and parity of the period.  A value travels
-// with the period's number in the same 64-bit word (a binary64 or int64 value as two words, a
-// binary32 value as one), so a reader that finds the number has the value: no fences, no flags,
-// one trip through L2.  Two parities suffice: a block writes the slots of period q + 2 only after
-// it has read its neighbours' period q + 1 values, which they wrote after reading its period q
-// ones.  The numbers continue from launch to launch (the last block to finish advances them in
-// device memory), so nothing is cleared, and a captured launch can be replayed.  Every wait is
-// bounded: after kPolls polls, or when another block has given up, the block records a status
-// and leaves; the host reports it as RBGS_ETIMEOUT at its next synchronising call.
+// Exchange: a slot of global memory per black point and parity of the period, which holds the
+// value with the period's number (tile_exchange.cuh).  Two parities suffice: a block writes the
+// slots of period q + 2 only after it has read its neighbours' period q + 1 values, which they
+// wrote after reading its period q ones.  The numbers continue from launch to launch (the last
+// block to finish advances them in device memory), so nothing is cleared, and a captured launch
+// can be replayed.  Every wait is bounded: after kRPolls polls, or when another block has given
+// up, the block records a status and leaves; the host reports it as RBGS_ETIMEOUT at its next
+// synchronising call.
 //
 // Tile and period: chosen per grid size from a model of the three costs (plan below): the
 // updates of the shrinking regions, a fixed cost per half-sweep (the chain of dependent
@@ -40,6 +39,7 @@
 #include "fixed64.cuh"
 #include "fp64.cuh"
 #include "sweep_impl.cuh"
+#include "tile_exchange.cuh"
 
 namespace rbgs {
 namespace {
@@ -92,36 +92,12 @@ __device__ __forceinline__ double r_update(double hf, double vn, double vs, doub
     return update_f64<false>(0, hf, vn, vs, vw, ve, one);
 }
 
-__device__ __forceinline__ void put(unsigned long long *slot, uint64_t bits, unsigned seq) {
-    const unsigned long long s = (unsigned long long)seq << 32;
-    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(slot), "l"(s | (uint32_t)bits),
-                 "l"(s | (uint32_t)(bits >> 32))
-                 : "memory");
-}
-__device__ __forceinline__ void put(unsigned long long *slot, uint32_t bits, unsigned seq) {
-    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(slot), "l"(((unsigned long long)seq << 32) | bits)
-                 : "memory");
-}
-// true when the slot holds period seq's value, then in `bits`
-__device__ __forceinline__ bool get(const unsigned long long *slot, uint64_t &bits, unsigned seq) {
-    unsigned long long a, b;
-    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(slot) : "memory");
-    bits = (uint64_t)(uint32_t)a | ((uint64_t)(uint32_t)b << 32);
-    return (unsigned)(a >> 32) == seq && (unsigned)(b >> 32) == seq;
-}
-__device__ __forceinline__ bool get(const unsigned long long *slot, uint32_t &bits, unsigned seq) {
-    unsigned long long a;
-    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(a) : "l"(slot) : "memory");
-    bits = (uint32_t)a;
-    return (unsigned)(a >> 32) == seq;
-}
-
 template <typename T>
 __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const RArgs<T> a) {
     using S = typename ResTypes<T>::S;
     using Bits = typename std::conditional<sizeof(T) == 8, uint64_t, uint32_t>::type;
     constexpr bool FUSED = std::is_same<T, int64_t>::value;
-    constexpr int kWords = sizeof(T) / 4;  // 64-bit words per slot
+    constexpr int kWords = kSlotWords<Bits>;
     extern __shared__ __align__(16) unsigned char r_shared[];
     __shared__ Region regions[2 * kMaxPeriod];
     __shared__ int s_nrcv, s_abort;
@@ -138,7 +114,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const RArgs<T> a
     T *sf = su + 2 * plane;
     int2 *rcv = reinterpret_cast<int2 *>(sf + 2 * plane);  // halo points: {shared element, grid element}
 
-    if (*reinterpret_cast<volatile int *>(a.status) != 0) return;  // a wait of an earlier launch gave up
+    if (block_given_up(a.status)) return;  // a wait of an earlier launch gave up
     unsigned long long ew = 0;
     if (FUSED) ew = a.words[2];
     const bool ok_scale = ew != kNoScale;
@@ -213,7 +189,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const RArgs<T> a
                 if (publish && (i < ra + 2 * K || i >= rb - 2 * K || k < ka + K || k >= kb - K)) {
                     Bits b;
                     __builtin_memcpy(&b, &v, sizeof(T));
-                    put(slots + ((size_t)i * W + k) * kWords, b, seq);
+                    slot_put(slots + ((size_t)i * W + k) * kWords, b, seq);
                 }
             }
         }
@@ -236,37 +212,9 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const RArgs<T> a
         if (left == 0) break;
         kk = (int)(left < K ? left : K);
         // the halo's black values of this period
-        const unsigned long long *slots = a.slots + (seq & 1u) * parity_words;
-        for (int base = 0; base < nrcv; base += 4 * kRThreads) {
-            unsigned pend = 0;
-            int2 ent[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int at = base + tid + q * kRThreads;
-                if (at < nrcv) ent[q] = rcv[at], pend |= 1u << q;
-            }
-            uint32_t polls = 0;
-            while (pend) {
-                Bits b[4];
-                bool hit[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) hit[q] = ((pend >> q) & 1u) && get(slots + (size_t)ent[q].y * kWords, b[q], seq);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (hit[q]) {
-                        __builtin_memcpy(&su[ent[q].x], &b[q], sizeof(T));
-                        pend &= ~(1u << q);
-                    }
-                }
-                if (pend && (++polls >= kRPolls || ((polls & 1023u) == 0 && *reinterpret_cast<volatile int *>(a.status) != 0))) {
-                    atomicOr(a.status, 2);
-                    s_abort = 1;
-                    break;
-                }
-            }
-        }
-        __syncthreads();
-        if (s_abort) return;
+        if (!receive_slots<T, Bits, kRThreads>(su, rcv, nrcv, a.slots + (seq & 1u) * parity_words, seq, a.status,
+                                               &s_abort, kRPolls))
+            return;
     }
     if constexpr (!FUSED) {
         for (int q = tid; q < plane; q += kRThreads) {
