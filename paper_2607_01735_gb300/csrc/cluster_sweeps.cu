@@ -17,8 +17,10 @@
 // blocks of the cluster run the same number of barriers (the sweep count is a kernel
 // argument); nothing waits on anything outside the cluster.
 #include <atomic>
+#include <memory>
 
 #include "common.cuh"
+#include "per_device.cuh"
 
 namespace rbgs {
 namespace {
@@ -121,9 +123,11 @@ size_t cluster_smem(int n, int W) {
 
 template <int CS>
 bool cluster_fits(int n, int W) {
-    // largest shared memory per block known to fit, per CS (the occupancy query runs once
-    // per new maximum)
-    static std::atomic<int> checked_bytes{-1};
+    // largest shared memory per block known to fit, per CS and device (the occupancy query runs
+    // once per new maximum)
+    static PerDevice<std::shared_ptr<std::atomic<int>>> known_fit;
+    const std::shared_ptr<std::atomic<int>> held = known_fit.get([] { return std::make_shared<std::atomic<int>>(-1); });
+    std::atomic<int> &checked_bytes = *held;
     const size_t smem = cluster_smem<CS>(n, W);
     if (smem > 200 * 1024) return false;
     const int known = checked_bytes.load();

@@ -263,9 +263,8 @@ __global__ void __launch_bounds__(kSlabThreads, 1) conv_slab_kernel(const SArgs 
 
 template <int MODE, int PIECES>
 bool slab_run(const SArgs &a, cudaStream_t s) {
-    static const cudaError_t attr = cudaFuncSetAttribute(conv_slab_kernel<MODE, PIECES>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSlabSmem);
-    if (attr != cudaSuccess) return false;
+    static PerDevice<cudaError_t> limit;
+    if (raise_smem(limit, conv_slab_kernel<MODE, PIECES>, kSlabSmem) != cudaSuccess) return false;
     const int grid = a.num_tiles < sm_count() ? a.num_tiles : sm_count();
     conv_slab_kernel<MODE, PIECES><<<grid, kSlabThreads, kSlabSmem, s>>>(a);
     return true;

@@ -383,13 +383,8 @@ bool tma_conv_launch(const uint16_t *src, const uint16_t *wts, const float *bias
             return true;
         }
     }
-    static const cudaError_t attr = [] {  // set once per instance, thread-safely
-        const cudaError_t e = cudaFuncSetAttribute(conv_tma_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)(kTmaRing + 1024));
-        if (e != cudaSuccess) cudaGetLastError();
-        return e;
-    }();
-    if (attr != cudaSuccess) {
+    static PerDevice<cudaError_t> limit;
+    if (raise_smem(limit, conv_tma_kernel<MODE>, kTmaRing + 1024) != cudaSuccess) {
         set_error("cudaFuncSetAttribute failed for the TMA convolution");
         *st = RBGS_ECUDA;
         return true;

@@ -47,6 +47,7 @@
 #include "common.cuh"
 #include "conv_index.cuh"
 #include "conv_wait.cuh"
+#include "per_device.cuh"
 #include "tma.cuh"
 #include "../../include/rbgs_unet.h"
 
@@ -582,7 +583,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_umma_kernel(const UArgs a) {
 
 // ------------------------------------------------------------------ host side
 int sm_count() {
-    static const int sms = [] {  // initialised once, thread-safely
+    static PerDevice<int> sms;
+    return sms.get([] {
         int dev = 0, v = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -590,8 +592,7 @@ int sm_count() {
             v = 1;
         }
         return v > 0 ? v : 1;
-    }();
-    return sms;
+    });
 }
 
 // N tile for K-major B: the fewest tiles of at most 256 columns, each a multiple of 16.
@@ -623,10 +624,8 @@ void finish_args(UArgs &a, int B) {
 
 template <int MODE, typename Offset = int>
 rbgs_status launch(const UArgs &a, cudaStream_t s) {
-    // set once per kernel instance, thread-safely; a failure is reported on every call
-    static const cudaError_t attr = cudaFuncSetAttribute(conv_umma_kernel<MODE, Offset>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-    RBGS_CUDA(attr);
+    static PerDevice<cudaError_t> limit;
+    RBGS_CUDA(raise_smem(limit, conv_umma_kernel<MODE, Offset>, kMaxSmem));
     const size_t smem = (size_t)a.stages * (UM + a.bn) * UK * 2 + 1024;
     const int grid = a.num_tiles < sm_count() ? a.num_tiles : sm_count();
     conv_umma_kernel<MODE, Offset><<<grid, kThreads, smem, s>>>(a);

@@ -450,9 +450,8 @@ bool wg_plan(int B, int H, int W, int Cin, int Cout, int sms, WgPlan &pl) {
 
 // Launches the tap-row weight gradient for a plan of wg_plan.
 rbgs_status wg_launch(WgPlan &pl, const uint16_t *X, const uint16_t *G, float *dW, cudaStream_t s) {
-    static const cudaError_t attr = cudaFuncSetAttribute(wgrad_shift_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         (int)(kWgBudget + 1024));
-    RBGS_CUDA(attr);
+    static PerDevice<cudaError_t> limit;
+    RBGS_CUDA(raise_smem(limit, wgrad_shift_kernel, kWgBudget + 1024));
     pl.a.X = X, pl.a.G = G, pl.a.dW = dW;
     wgrad_shift_kernel<<<pl.grid, kWgThreads, pl.smem, s>>>(pl.a);
     RBGS_LAUNCH_CHECK();

@@ -375,9 +375,8 @@ bool wr_plan(int B, int H, int W, int Cin, int Cout, int sms, WrPlan &pl) {
 
 // Launches the ring weight gradient for a plan of wr_plan.
 rbgs_status wr_launch(WrPlan &pl, const uint16_t *X, const uint16_t *G, float *dW, cudaStream_t s) {
-    static const cudaError_t attr = cudaFuncSetAttribute(wgrad_ring_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         (int)(kWgBudget + 1024));
-    RBGS_CUDA(attr);
+    static PerDevice<cudaError_t> limit;
+    RBGS_CUDA(raise_smem(limit, wgrad_ring_kernel, kWgBudget + 1024));
     pl.a.X = X, pl.a.G = G, pl.a.dW = dW;
     wgrad_ring_kernel<<<pl.grid, kWgThreads, pl.smem, s>>>(pl.a);
     RBGS_LAUNCH_CHECK();

@@ -24,6 +24,7 @@
 #include "common.cuh"
 #include "fp64.cuh"
 #include "grid_barrier.cuh"
+#include "per_device.cuh"
 #include "sweep_impl.cuh"
 
 namespace rbgs {
@@ -137,9 +138,9 @@ __global__ void __launch_bounds__(kPThreads) persistent_sweeps(const PArgs<T> a)
 // Blocks the grid needs (at most what can be resident at once).
 template <typename T, int NP>
 int persistent_grid(int n) {
-    // resident blocks of the whole GPU, per template instance (initialised once, thread-safely;
-    // 0 when the query fails)
-    static const long cap = [] {
+    // resident blocks of the whole GPU, per template instance and device (0 when the query fails)
+    static PerDevice<long> resident;
+    const long cap = resident.get([] {
         int dev = 0, sms = 0, per_sm = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -149,7 +150,7 @@ int persistent_grid(int n) {
             return 0L;
         }
         return (long)per_sm * sms;
-    }();
+    });
     const long items = (long)n * ((active_width(n) + 2 * NP - 1) / (2 * NP));
     const long want = (items + kPThreads - 1) / kPThreads;
     return (int)(want < cap ? want : cap);

@@ -38,6 +38,7 @@
 #include "common.cuh"
 #include "fixed64.cuh"
 #include "fp64.cuh"
+#include "per_device.cuh"
 #include "sweep_impl.cuh"
 #include "tile_exchange.cuh"
 
@@ -235,7 +236,8 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const RArgs<T> a
 }
 
 int device_sms() {
-    static const int sms = [] {
+    static PerDevice<int> sms;
+    return sms.get([] {
         int dev = 0, v = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -243,8 +245,7 @@ int device_sms() {
             v = 0;
         }
         return v;
-    }();
-    return sms;
+    });
 }
 
 template <typename T>
@@ -306,9 +307,8 @@ ResidentPlan plan_for(int n) {
 template <typename T>
 rbgs_status run_resident(RArgs<T> &a, const ResidentPlan &pl, long nsweeps, cudaStream_t s) {
     const size_t smem = resident_smem<T>(pl.rows, pl.vals, pl.period);
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(resident_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-    RBGS_CUDA(attr);
+    static PerDevice<cudaError_t> limit;
+    RBGS_CUDA(raise_smem(limit, resident_kernel<T>, kSmemMax));
     a.gx = pl.gx, a.gy = pl.gy, a.period = pl.period;
     a.pitch = pl.vals + 2 * pl.period + 2, a.erows = pl.rows + 4 * pl.period;
     a.sweeps = nsweeps;

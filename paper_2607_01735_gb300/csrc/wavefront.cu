@@ -48,6 +48,7 @@
 #include "common.cuh"
 #include "fixed64.cuh"
 #include "fp64.cuh"
+#include "per_device.cuh"
 #include "sweep_impl.cuh"
 
 namespace rbgs {
@@ -88,14 +89,7 @@ __device__ __forceinline__ double wf_update(double hf, double vn, double vs, dou
     return update_f64<false>(0, hf, vn, vs, vw, ve, one);
 }
 
-// P values at a 16-byte aligned address
-template <typename T, int P>
-__device__ __forceinline__ void wf_read(T *v, const T *p) {
-    constexpr int V = 16 / (int)sizeof(T);
-#pragma unroll
-    for (int q = 0; q < P; q += V) *reinterpret_cast<int4 *>(v + q) = *reinterpret_cast<const int4 *>(p + q);
-}
-
+// P values at a 16-byte aligned address: from global memory, from shared memory, to global
 template <typename T, int P>
 __device__ __forceinline__ void wf_ldg(T (&v)[P], const T *p) {
     constexpr int V = 16 / (int)sizeof(T);
@@ -350,7 +344,8 @@ __global__ void __launch_bounds__(kWfThreads, wf_blocks<T, K>()) wavefront_kerne
 }
 
 int sm_count_wf() {
-    static const int sms = [] {  // initialised once, thread-safely
+    static PerDevice<int> sms;
+    return sms.get([] {
         int dev = 0, v = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) {
@@ -358,8 +353,7 @@ int sm_count_wf() {
             v = 152;
         }
         return v;
-    }();
-    return sms;
+    });
 }
 
 template <typename T, int K, int P, int MODE>
@@ -368,7 +362,8 @@ rbgs_status run_pass(WfArgs<T> &a, cudaStream_t s) {
     a.halo = (K + P - 1) / P * P;
     a.ow = 32 * P - 2 * a.halo;
     a.strips = (a.kmax + a.ow - 1) / a.ow;
-    static const int per_sm = [] {  // resident blocks per SM, per template instance; 0: set-up failed
+    static PerDevice<int> resident;  // blocks per SM, per template instance; 0: set-up failed
+    const int per_sm = resident.get([] {
         int v = 0;
         if (cudaFuncSetAttribute(wavefront_kernel<T, K, P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem) != cudaSuccess ||
@@ -378,7 +373,7 @@ rbgs_status run_pass(WfArgs<T> &a, cudaStream_t s) {
             v = 0;
         }
         return v;
-    }();
+    });
     if (per_sm < 1) {
         set_error("wavefront pass: no resident block fits");
         return RBGS_ECUDA;

@@ -1,0 +1,81 @@
+"""Which kernels the library's host code launches, and where: run over a stand-in CUDA runtime
+(fake_runtime.py) that enforces the launch rules of each device.  CPU only."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import fake_runtime
+import paper_2607_01735_gb300 as rb
+from fake_runtime import Context
+
+
+@pytest.fixture(scope="module")
+def loaded():
+    return fake_runtime.load()
+
+
+@pytest.fixture
+def lib(loaded):
+    loaded.fake_reset()
+    yield loaded
+    loaded.fake_reset()
+
+
+# ------------------------------------------------------------------ a second device
+@pytest.mark.parametrize("n,opts", [(1023, {}), (1368, {}), (1023, {"fma": 1}), (1500, {"fma": 1}), (4095, {}),
+                                    (900, {"kernel": rb.RBGS_KERNEL_WAVEFRONT})])
+def test_sweeps_run_on_a_second_device(lib, n, opts):
+    """A kernel's raised shared-memory limit belongs to the device it was raised on."""
+    for device in (0, 1):
+        lib.fake_set_device(device)
+        c = Context(lib, n, **opts)
+        st, calls = c.sweep(40)
+        assert st == 0, lib.rbgs_last_error()
+        assert calls and all(d == device for kind, _, _, d in calls if kind != "graph")
+        c.close()
+
+
+def test_refined_solve_runs_on_a_second_device(lib):
+    for device in (0, 1):
+        lib.fake_set_device(device)
+        c = Context(lib, 900, precision=rb.RBGS_FP32_REFINE, max_sweeps=200, inner_sweeps=100)
+        assert lib.rbgs_solve(c.ctx, 0.0, None, None) in (rb.RBGS_OK, rb.RBGS_ENOTCONV), lib.rbgs_last_error()
+        c.close()
+
+
+def test_cooperative_launches_fit_a_smaller_second_device(lib):
+    lib.fake_set_sms(2, 60)  # a device that no other test uses: its SM count is asked for once
+    for n, opts in ((511, {}), (511, {"fma": 1}), (4095, {})):
+        for device, sms in ((0, 152), (2, 60)):
+            lib.fake_set_device(device)
+            c = Context(lib, n, **opts)
+            st, calls = c.sweep(40)
+            assert st == 0, lib.rbgs_last_error()
+            blocks = [b for kind, name, b, _ in calls if kind == "cooperative"]
+            assert blocks and (n > 2048 or max(blocks) <= sms)
+            c.close()
+
+
+@pytest.mark.parametrize("Cin,Cout", [(32, 32), (128, 128), (192, 64)])
+def test_convolutions_run_on_a_second_device(lib, Cin, Cout):
+    B, H, W = 2, 66, 66
+    aligned = lambda n: (lambda a: a[(-a.ctypes.data % 16) // a.itemsize:])(np.zeros(n + 64, np.uint16))
+    x, w, g, t = (aligned(k) for k in (B * H * W * Cin, 9 * Cin * Cout, B * H * W * Cout, 9 * Cin * Cout))
+    y, dx, dw = (np.zeros(k, np.float32) for k in (B * H * W * Cout, B * H * W * Cin, 9 * Cin * Cout))
+    p = lambda a: ctypes.c_void_p(a.ctypes.data)
+    lib.rbgs_conv_set_engine(2)  # gathers: tensor maps need a driver
+    try:
+        for device in (0, 1):
+            lib.fake_set_device(device)
+            for engine in (2, 0):
+                lib.rbgs_conv_set_engine(engine)
+                assert lib.rbgs_conv_forward(p(x), p(w), None, p(y), B, H, W, Cin, Cout, 3, 0, 1, None) == 0
+            lib.rbgs_conv_set_engine(2)
+            for kind in (1, 2, 3):
+                lib.rbgs_conv_set_wgrad_kernel(kind)
+                assert lib.rbgs_conv_backward(p(x), p(w), p(g), p(dx), p(dw), None, p(t), B, H, W, Cin, Cout, 3, 0,
+                                              None) == 0, lib.rbgs_last_error()
+    finally:
+        lib.rbgs_conv_set_wgrad_kernel(0)
+        lib.rbgs_conv_set_engine(0)
