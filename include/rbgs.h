@@ -71,11 +71,12 @@ typedef enum {
     RBGS_KERNEL_AUTO = 0,     /* FP64 sweeps, bit-exact or fused, with the default launch-shape
                                  options: all sweeps of a call in one cooperative launch with
                                  tiles of the grid held in shared memory, where they fit (n up
-                                 to about 1370); above that PERSISTENT for 416 <= n <= 32768
-                                 (fused: see fma), else COLOUR.  FP32 inner sweeps of
-                                 RBGS_FP32_REFINE with tblock_k = 0: tiles in shared memory for
-                                 n <= 1000, WAVEFRONT (depth 4) above, else COLOUR.  Sweeps of
-                                 the tiled form wait within the launch (RBGS_ETIMEOUT)         */
+                                 to 1368 on 152 SMs) and the launch is not refused; else
+                                 PERSISTENT for 416 <= n <= 32768 (fused: see fma), else
+                                 COLOUR.  FP32 inner sweeps of RBGS_FP32_REFINE with
+                                 tblock_k = 0: tiles in shared memory for n <= 1000,
+                                 WAVEFRONT (depth 4) above, else COLOUR.  Sweeps of the tiled
+                                 form wait within the launch (RBGS_ETIMEOUT)                  */
     RBGS_KERNEL_COLOUR = 1,   /* one launch per colour (half-sweep kernels)               */
     RBGS_KERNEL_TEMPORAL = 2, /* several sweeps per shared-memory tile, halo recompute      */
     RBGS_KERNEL_WAVEFRONT = 3,/* several sweeps per pass, a register wavefront per strip   */

@@ -197,11 +197,12 @@ rbgs_status ensure_f64_alt(rbgs_ctx *c) {
     return RBGS_OK;
 }
 
-// The resident kernel's plan and exchange slots for this context's grid; without room for the
-// slots the kernel is not used (r.slots stays NULL).
+// The resident kernel's plan and exchange slots for this context's grid; where it cannot run, or
+// without room for the slots, it is not used (r.use stays false).
 void prepare_resident(rbgs_ctx *c, ResidentState &r, int W, int kind) {
     r.plan = resident_plan(c->g.n, kind);
     if (r.plan.rows == 0) return;
+    r.use = true;
     const size_t bytes = resident_slot_bytes(c->g.n, W, kind);
     if (cudaMalloc(&r.slots, bytes) != cudaSuccess || cudaMalloc(&r.epoch, 2 * sizeof(unsigned)) != cudaSuccess ||
         cudaMemsetAsync(r.slots, 0, bytes, c->stream) != cudaSuccess ||
@@ -211,7 +212,13 @@ void prepare_resident(rbgs_ctx *c, ResidentState &r, int W, int kind) {
         cudaFree(r.epoch);
         r.slots = nullptr;
         r.epoch = nullptr;
+        r.use = false;
     }
+}
+
+// The FP64 sweeps of a context whose grid the resident kernel does not take.
+int kernel_without_resident(int n) {
+    return n >= kPersistMinN && n <= kPersistMaxN ? RBGS_KERNEL_PERSISTENT : RBGS_KERNEL_COLOUR;
 }
 
 // FP32 correction, scaled defect and (for the temporal inner kernel) the partner buffers.
@@ -313,9 +320,11 @@ rbgs_status sweeps_f64(rbgs_ctx *c, long nsweeps) {
             nsweeps -= m;
             rbgs_status st = launch_fused_prepare(c, m, c->stream);
             if (st != RBGS_OK) return st;
-            if (c->res64.slots && m >= 2) {
-                if ((st = launch_resident_sweeps_fused(c, m, c->stream)) != RBGS_OK) return st;
-                continue;
+            if (c->res64.use && m >= 2) {
+                st = launch_resident_sweeps_fused(c, m, c->stream);
+                if (st == RBGS_OK) continue;
+                if (st != kLaunchRefused) return st;
+                c->res64.use = false;
             }
             if (c->tq[0] && m >= kFusedWaveMin) {
                 if ((st = launch_fused_wave_sweeps(c, m, c->stream)) != RBGS_OK) return st;
@@ -332,7 +341,11 @@ rbgs_status sweeps_f64(rbgs_ctx *c, long nsweeps) {
         }
         return RBGS_OK;
     }
-    if (c->kernel == kKernelResident && nsweeps >= 2) return launch_resident_sweeps_f64(c, nsweeps, c->stream);
+    if (c->kernel == kKernelResident && nsweeps >= 2) {
+        const rbgs_status st = launch_resident_sweeps_f64(c, nsweeps, c->stream);
+        if (st != kLaunchRefused) return st;
+        c->kernel = kernel_without_resident(c->g.n);
+    }
     if (use_persistent(c)) return launch_persistent_sweeps<double>(c->f64, nsweeps, c->pcounter, c->dstatus, c->stream);
     if (c->kernel == RBGS_KERNEL_COLOUR && c->g.n <= kGraphMaxN && nsweeps >= kGraphSweeps) {
         rbgs_status st = ensure_graph(c);
@@ -363,7 +376,11 @@ rbgs_status defect_stats(rbgs_ctx *c, double *rho, double *mx, bool *exact) {
 }
 
 rbgs_status inner_sweeps_f32(rbgs_ctx *c, long m) {
-    if (c->res32.slots && m >= 2) return launch_resident_sweeps_f32(c, m, c->stream);
+    if (c->res32.use && m >= 2) {
+        const rbgs_status st = launch_resident_sweeps_f32(c, m, c->stream);
+        if (st != kLaunchRefused) return st;
+        c->res32.use = false;
+    }
     // small grids: all m sweeps in one launch of one thread-block cluster
     if (c->kernel32 == RBGS_KERNEL_COLOUR && c->opts.tile_rows == 0 && c->g.n <= kClusterMaxN &&
         cluster_sweeps_f32_fit(c->g.n, c->f32.W))
@@ -657,15 +674,14 @@ rbgs_status rbgs_create(int n, double h2, const double *f, const double *u_init,
     ok = ok && (!c->fused || cudaMalloc(&c->fwords, 3 * sizeof(unsigned long long)) == cudaSuccess);
     if (ok && c->kernel == kKernelResident) {
         prepare_resident(c, c->res64, c->g.W, 0);
-        if (!c->res64.slots)
-            c->kernel = n >= kPersistMinN && n <= kPersistMaxN ? RBGS_KERNEL_PERSISTENT : RBGS_KERNEL_COLOUR;
+        if (!c->res64.use) c->kernel = kernel_without_resident(n);
     } else if (ok && c->fused && o.kernel == RBGS_KERNEL_AUTO && o.tile_rows == 0 && o.sweep_values == 0 &&
                n <= kResidentMaxN) {
         prepare_resident(c, c->res64, c->g.W, 2);
     }
     // the wavefront's buffers; without room for them the half-sweeps run one launch per colour
     if (ok && c->fused && o.kernel == RBGS_KERNEL_AUTO && o.tile_rows == 0 && o.sweep_values == 0 &&
-        n >= kFusedWaveMinN && !c->res64.slots) {
+        n >= kFusedWaveMinN && !c->res64.use) {
         const size_t qbytes = c->g.colour_elems() * sizeof(int64_t);
         if (cudaMalloc(&c->tq[0], qbytes) != cudaSuccess || cudaMalloc(&c->tq[1], qbytes) != cudaSuccess) {
             cudaGetLastError();

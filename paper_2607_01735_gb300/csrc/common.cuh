@@ -73,9 +73,14 @@ struct ResidentPlan {
 
 struct ResidentState {
     ResidentPlan plan;
-    unsigned long long *slots;  // exchange slots (NULL: the kernel is not used)
+    unsigned long long *slots;  // exchange slots
     unsigned *epoch;            // [0] number of the last period, [1] scratch
+    bool use;                   // false: no plan, no room for the slots, or its launch was refused
 };
+
+// Internal status: a cooperative launch was refused (it does not fit the SMs that this process may
+// use); nothing has run, and the caller takes another path.
+constexpr rbgs_status kLaunchRefused = (rbgs_status)-1;
 
 }  // namespace rbgs
 
@@ -166,6 +171,8 @@ rbgs_status launch_persistent_sweeps(ColourField<T> &fld, long nsweeps, unsigned
                                      cudaStream_t s);
 // all sweeps of a small grid in one cooperative launch, tiles in shared memory (resident.cu).
 // kind 0: FP64, 1: FP32 inner sweeps, 2: fused.  nsweeps >= 2
+// (the plan has no rows where the kernel does not fit the grid or cannot run on this device);
+// kLaunchRefused: nothing was launched
 ResidentPlan resident_plan(int n, int kind);
 size_t resident_slot_bytes(int n, int W, int kind);
 rbgs_status launch_resident_sweeps_f64(const rbgs_ctx *c, long nsweeps, cudaStream_t s);

@@ -272,9 +272,29 @@ struct Costs<int64_t> {
     static constexpr double warp = 117, chain = 590, exchange = 1550;
 };
 
+// The current device takes a cooperative launch of this kernel with one block on every SM.
+template <typename T>
+bool can_run() {
+    static PerDevice<cudaError_t> limit;
+    static PerDevice<bool> fits;
+    if (raise_smem(limit, resident_kernel<T>, kSmemMax) != cudaSuccess) return false;
+    return fits.get([] {
+        int dev = 0, coop = 0, per_sm = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, resident_kernel<T>, kRThreads, kSmemMax) !=
+                cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        return coop != 0 && per_sm >= 1;
+    });
+}
+
 template <typename T>
 ResidentPlan plan_for(int n) {
     ResidentPlan best{};
+    if (!can_run<T>()) return best;
     double best_cost = 0.0;
     const int kint = n / 2 + 1, sms = device_sms();
     for (int K = 1; K <= kMaxPeriod; ++K) {
@@ -307,15 +327,18 @@ ResidentPlan plan_for(int n) {
 template <typename T>
 rbgs_status run_resident(RArgs<T> &a, const ResidentPlan &pl, long nsweeps, cudaStream_t s) {
     const size_t smem = resident_smem<T>(pl.rows, pl.vals, pl.period);
-    static PerDevice<cudaError_t> limit;
-    RBGS_CUDA(raise_smem(limit, resident_kernel<T>, kSmemMax));
     a.gx = pl.gx, a.gy = pl.gy, a.period = pl.period;
     a.pitch = pl.vals + 2 * pl.period + 2, a.erows = pl.rows + 4 * pl.period;
     a.sweeps = nsweeps;
     a.one = 1.0;
     void *args[] = {&a};
-    RBGS_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(resident_kernel<T>), dim3(pl.gx * pl.gy),
-                                          dim3(kRThreads), args, smem, s));
+    const cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(resident_kernel<T>),
+                                                      dim3(pl.gx * pl.gy), dim3(kRThreads), args, smem, s);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        return kLaunchRefused;
+    }
+    RBGS_CUDA(e);
     return RBGS_OK;
 }
 

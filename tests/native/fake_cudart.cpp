@@ -30,6 +30,7 @@ int g_coop = 1;              // the device attribute
 int g_refuse = 0;            // cooperative launches fail as too large
 size_t g_in_use = 0, g_limit = (size_t)-1;
 float g_elapsed = 1.0f;
+double g_host[4];            // first values of page-locked memory, where residuals are read
 struct Config {
     dim3 g, b;
     size_t smem;
@@ -75,6 +76,7 @@ void fake_reset() {
     g_log.clear();
     for (int &s : g_sms) s = 152;
     g_coop = 1, g_refuse = 0, g_limit = (size_t)-1, g_elapsed = 1.0f;
+    g_host[0] = g_host[1] = 1.0, g_host[2] = 0.5, g_host[3] = 0.0;  // rho = 1, max |rt| = 0.5, no status
     t_device = 0, t_last = cudaSuccess;
 }
 void fake_clear_log() { std::lock_guard<std::mutex> lock(g_m); g_log.clear(); }
@@ -158,7 +160,11 @@ cudaError_t cudaFree(void *p) {
     if (it != g_alloc.end()) g_in_use -= it->second, g_alloc.erase(it), std::free(p);
     return cudaSuccess;
 }
-cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { *p = std::calloc(n ? n : 1, 1); return cudaSuccess; }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) {
+    *p = std::calloc(n ? n : 1, 1);
+    if (n == sizeof g_host) std::memcpy(*p, g_host, n);
+    return cudaSuccess;
+}
 cudaError_t cudaMallocHost(void **p, size_t n) { return cudaHostAlloc(p, n, 0); }
 cudaError_t cudaFreeHost(void *p) { std::free(p); return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t) { std::memset(p, v, n); return cudaSuccess; }

@@ -7,7 +7,7 @@ import pytest
 
 import fake_runtime
 import paper_2607_01735_gb300 as rb
-from fake_runtime import Context
+from fake_runtime import Context, launches
 
 
 @pytest.fixture(scope="module")
@@ -40,7 +40,10 @@ def test_refined_solve_runs_on_a_second_device(lib):
     for device in (0, 1):
         lib.fake_set_device(device)
         c = Context(lib, 900, precision=rb.RBGS_FP32_REFINE, max_sweeps=200, inner_sweeps=100)
-        assert lib.rbgs_solve(c.ctx, 0.0, None, None) in (rb.RBGS_OK, rb.RBGS_ENOTCONV), lib.rbgs_last_error()
+        lib.fake_clear_log()
+        assert lib.rbgs_solve(c.ctx, 0.0, None, None) == rb.RBGS_ENOTCONV, lib.rbgs_last_error()
+        inner = [kind for kind, name, _, _ in launches(lib) if "resident" in name]
+        assert inner == ["cooperative"] * 2
         c.close()
 
 
@@ -79,3 +82,47 @@ def test_convolutions_run_on_a_second_device(lib, Cin, Cout):
     finally:
         lib.rbgs_conv_set_wgrad_kernel(0)
         lib.rbgs_conv_set_engine(0)
+
+
+# ------------------------------------------------------------------ refused cooperative launches
+def _kinds(calls):
+    return {kind for kind, *_ in calls}
+
+
+@pytest.mark.parametrize("n,opts", [(31, {}), (255, {}), (255, {"fma": 1}), (900, {"fma": 1})])
+def test_sweeps_go_on_when_the_cooperative_launch_is_refused(lib, n, opts):
+    """A process that may use only part of the SMs has cooperative launches refused: the sweeps
+    then run one launch per colour, and later calls do not try again."""
+    c = Context(lib, n, **opts)
+    lib.fake_cooperative(1, 1)
+    for k in (40, 2, 40):
+        st, calls = c.sweep(k)
+        assert st == 0, lib.rbgs_last_error()
+        assert calls and _kinds(calls) <= {"plain", "graph"}
+        assert not any("resident" in name for _, name, _, _ in calls)
+    lib.fake_cooperative(1, 0)
+    st, calls = c.sweep(40)
+    assert st == 0 and _kinds(calls) <= {"plain", "graph"}
+    c.close()
+
+
+def test_refinement_goes_on_when_the_cooperative_launch_is_refused(lib):
+    for n in (127, 511):
+        c = Context(lib, n, precision=rb.RBGS_FP32_REFINE, max_sweeps=200, inner_sweeps=100)
+        lib.fake_cooperative(1, 1)
+        lib.fake_clear_log()
+        assert lib.rbgs_solve(c.ctx, 0.0, None, None) == rb.RBGS_ENOTCONV, lib.rbgs_last_error()
+        assert "cooperative" not in _kinds(launches(lib))
+        lib.fake_cooperative(1, 0)
+        c.close()
+
+
+def test_device_without_cooperative_launches(lib):
+    """The attribute is asked for once per device: this one is used by no other test."""
+    lib.fake_set_device(3)
+    lib.fake_cooperative(0, 0)
+    for opts in ({}, {"fma": 1}):
+        c = Context(lib, 255, **opts)
+        st, calls = c.sweep(40)
+        assert st == 0 and calls and _kinds(calls) <= {"plain", "graph"}
+        c.close()
