@@ -34,7 +34,8 @@
  * Devices and threads: a context lives on the device that is current when rbgs_create
  * runs; call it with that device current (the library does not switch devices).  Calls
  * on one context must not overlap in time; separate contexts may be used from separate
- * threads at once.
+ * threads at once.  Contexts at work on several streams share the device: the kernels that
+ * would fill it (n <= 2048) then take a part each, with the same results.
  */
 #ifndef RBGS_H
 #define RBGS_H

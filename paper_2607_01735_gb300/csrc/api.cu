@@ -58,6 +58,13 @@ constexpr int kFusedWaveMinN = 512;
 // as fast and needs no cooperative launch.
 constexpr int kResidentMaxN = 2048, kResident32MaxN = 1000;
 constexpr int kWave32MinN = 1001;    // FP32 inner sweeps as wavefront passes from this size on
+// Sharing the device among solvers at work on several streams (wave_parts, inner_sweeps_f32).
+constexpr int kShareMaxN = 2048, kShareMostParts = 8;
+// Tiled FP32 grids above kShareWave32MinN run wavefront passes of a part of the device when
+// streams n exceeds kShareWave32: tiles of a part hold few of their rows to themselves.  500
+// sweeps by threads, tiles / passes: 8 x 800^2 6.7 / 5.3 ms, 8 x 1000^2 10.5 / 6.3; on 4 streams
+// 4 x 800^2 3.9 and 4 x 1000^2 5.5 by tiles, 4 x 1100^2 4.6 by passes.
+constexpr int kShareWave32MinN = 700, kShareWave32 = 3500;
 // Residual checks without a new minimum of rho after which a solve stops (opts.stall_checks 0).
 constexpr int kDefaultStallChecks = 64;
 
@@ -125,6 +132,7 @@ rbgs_status load_problem(rbgs_ctx *c, const double *f, const double *u_init) {
     if ((st = stage_in(c, u_init, (size_t)g.rows * g.rows, &uview)) != RBGS_OK) return st;
     if ((st = enqueue_pack(c, fview, uview)) != RBGS_OK) return st;
     RBGS_CUDA(cudaStreamSynchronize(c->stream));  // the reduction wrote hsum[1]
+    stream_idle(c->device, c->stream);
     c->den2 = c->hsum[1];
     return RBGS_OK;
 }
@@ -200,9 +208,9 @@ rbgs_status ensure_f64_alt(rbgs_ctx *c) {
 // The resident kernel's plan and exchange slots for this context's grid; where it cannot run, or
 // without room for the slots, it is not used (r.use stays false).
 void prepare_resident(rbgs_ctx *c, ResidentState &r, int W, int kind) {
-    r.plan = resident_plan(c->g.n, kind);
-    if (r.plan.rows == 0) return;
-    r.use = true;
+    r.plan[0] = resident_plan(c->g.n, kind);
+    if (r.plan[0].rows == 0) return;
+    r.use = r.planned[0] = true;
     const size_t bytes = resident_slot_bytes(c->g.n, W, kind);
     if (cudaMalloc(&r.slots, bytes) != cudaSuccess || cudaMalloc(&r.epoch, 2 * sizeof(unsigned)) != cudaSuccess ||
         cudaMemsetAsync(r.slots, 0, bytes, c->stream) != cudaSuccess ||
@@ -239,6 +247,18 @@ rbgs_status ensure_f32(rbgs_ctx *c) {
     if (c->kernel32 == RBGS_KERNEL_COLOUR && c->opts.kernel == RBGS_KERNEL_AUTO && c->opts.tblock_k == 0 &&
         c->opts.tile_rows == 0 && c->g.n <= kResident32MaxN)
         prepare_resident(c, c->res32, c->f32.W, 1);
+    // partner buffers for inner_sweeps_f32's passes; without room for them it does without
+    if (c->res32.use && c->g.n > kShareWave32MinN) {
+        for (int q = 0; q < 2; ++q) {
+            if (cudaMalloc(&c->f32.alt[q], bytes) != cudaSuccess ||
+                cudaMemsetAsync(c->f32.alt[q], 0, bytes, c->stream) != cudaSuccess) {
+                cudaGetLastError();
+                cudaFree(c->f32.alt[q]);
+                c->f32.alt[q] = nullptr;
+                break;
+            }
+        }
+    }
     return RBGS_OK;
 }
 
@@ -254,6 +274,7 @@ rbgs_status status_error(int status) {
 rbgs_status check_device_status(rbgs_ctx *c) {
     RBGS_CUDA(cudaMemcpyAsync(c->hstatus, c->dstatus, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     RBGS_CUDA(cudaStreamSynchronize(c->stream));
+    stream_idle(c->device, c->stream);
     return status_error(*c->hstatus);
 }
 
@@ -261,6 +282,7 @@ rbgs_status check_device_status(rbgs_ctx *c) {
 // into hsum (page-locked: no copies).
 rbgs_status finish_residual(rbgs_ctx *c) {
     RBGS_CUDA(cudaStreamSynchronize(c->stream));
+    stream_idle(c->device, c->stream);
     return status_error((int)c->hsum[3]);
 }
 
@@ -276,7 +298,7 @@ rbgs_status enqueue_sweeps(rbgs_ctx *c, long nsweeps, cudaStream_t s) {
     if (c->kernel == RBGS_KERNEL_TEMPORAL) return launch_temporal_sweeps(c, nsweeps, s);
     if (c->kernel == RBGS_KERNEL_WAVEFRONT) {
         const long passes = nsweeps / c->tblock_k;
-        const rbgs_status st = launch_wavefront_passes<double>(c->f64, c->tblock_k, passes, s);
+        const rbgs_status st = launch_wavefront_passes<double>(c->f64, c->tblock_k, passes, 1, s);
         if (st != RBGS_OK) return st;
         nsweeps -= passes * c->tblock_k;
     }
@@ -308,6 +330,19 @@ rbgs_status ensure_graph(rbgs_ctx *c) {
     return RBGS_OK;
 }
 
+// Parts of the device that a wavefront pass fills one of, as many as there are streams at work:
+// its segments are then longer and recompute fewer rows of their neighbours (1100^2 FP32: 6 rows
+// with 16 more on the whole device, 38 with 16 on an eighth).  On grids of more than kShareMaxN the
+// overlap is small and a pass always takes the device.  us: about what the passes take alone.
+int wave_parts(const rbgs_ctx *c, int streams, double us) {
+    if (c->g.n > kShareMaxN) return 1;
+    stream_busy(c->device, c->stream, us);
+    return streams < kShareMostParts ? streams : kShareMostParts;
+}
+
+// Streams that share the device with this context's next sweeps (counted up to kShareMaxN).
+int sharing(const rbgs_ctx *c) { return c->g.n > kShareMaxN ? 1 : streams_sharing(c->device, c->stream); }
+
 // nsweeps FP64 sweeps: one cooperative launch, cached graphs of kGraphSweeps sweeps on small
 // grids, or direct / temporally blocked launches.
 rbgs_status sweeps_f64(rbgs_ctx *c, long nsweeps) {
@@ -320,14 +355,16 @@ rbgs_status sweeps_f64(rbgs_ctx *c, long nsweeps) {
             nsweeps -= m;
             rbgs_status st = launch_fused_prepare(c, m, c->stream);
             if (st != RBGS_OK) return st;
+            const int streams = sharing(c);
             if (c->res64.use && m >= 2) {
-                st = launch_resident_sweeps_fused(c, m, c->stream);
+                st = launch_resident_sweeps_fused(c, m, streams, c->stream);
                 if (st == RBGS_OK) continue;
                 if (st != kLaunchRefused) return st;
                 c->res64.use = false;
             }
             if (c->tq[0] && m >= kFusedWaveMin) {
-                if ((st = launch_fused_wave_sweeps(c, m, c->stream)) != RBGS_OK) return st;
+                const int parts = wave_parts(c, streams, (double)m * (6.0 + c->g.n * (double)c->g.n / 0.7e6));
+                if ((st = launch_fused_wave_sweeps(c, m, parts, c->stream)) != RBGS_OK) return st;
                 continue;
             }
             if (m >= kGraphSweeps) {
@@ -342,7 +379,7 @@ rbgs_status sweeps_f64(rbgs_ctx *c, long nsweeps) {
         return RBGS_OK;
     }
     if (c->kernel == kKernelResident && nsweeps >= 2) {
-        const rbgs_status st = launch_resident_sweeps_f64(c, nsweeps, c->stream);
+        const rbgs_status st = launch_resident_sweeps_f64(c, nsweeps, sharing(c), c->stream);
         if (st != kLaunchRefused) return st;
         c->kernel = kernel_without_resident(c->g.n);
     }
@@ -376,8 +413,11 @@ rbgs_status defect_stats(rbgs_ctx *c, double *rho, double *mx, bool *exact) {
 }
 
 rbgs_status inner_sweeps_f32(rbgs_ctx *c, long m) {
-    if (c->res32.use && m >= 2) {
-        const rbgs_status st = launch_resident_sweeps_f32(c, m, c->stream);
+    const int streams = sharing(c);
+    // large tiled grids when many streams are at work: wavefront passes of a part of the device
+    const bool wave = c->res32.use && c->g.n > kShareWave32MinN && streams * c->g.n > kShareWave32 && c->f32.alt[1];
+    if (c->res32.use && !wave && m >= 2) {
+        const rbgs_status st = launch_resident_sweeps_f32(c, m, streams, c->stream);
         if (st != kLaunchRefused) return st;
         c->res32.use = false;
     }
@@ -386,7 +426,7 @@ rbgs_status inner_sweeps_f32(rbgs_ctx *c, long m) {
         cluster_sweeps_f32_fit(c->g.n, c->f32.W))
         return launch_cluster_sweeps_f32(c->f32, m, c->stream);
     // full inner blocks of one-launch-per-colour sweeps on small grids: a cached graph
-    if (c->kernel32 == RBGS_KERNEL_COLOUR && m == c->inner_sweeps && c->g.n <= kGraphMaxN) {
+    if (!wave && c->kernel32 == RBGS_KERNEL_COLOUR && m == c->inner_sweeps && c->g.n <= kGraphMaxN) {
         if (!c->graph32) {
             cudaGraph_t graph = nullptr;
             RBGS_CUDA(cudaStreamBeginCapture(c->capture, cudaStreamCaptureModeThreadLocal));
@@ -411,11 +451,12 @@ rbgs_status inner_sweeps_f32(rbgs_ctx *c, long m) {
         RBGS_CUDA(cudaGraphLaunch(c->graph32, c->stream));
         return RBGS_OK;
     }
-    if (c->kernel32 == RBGS_KERNEL_TEMPORAL || c->kernel32 == RBGS_KERNEL_WAVEFRONT) {
+    if (wave || c->kernel32 == RBGS_KERNEL_TEMPORAL || c->kernel32 == RBGS_KERNEL_WAVEFRONT) {
         const int k = c->tblock_k32;
         const long passes = m / k;
-        if (c->kernel32 == RBGS_KERNEL_WAVEFRONT) {
-            const rbgs_status st = launch_wavefront_passes<float>(c->f32, k, passes, c->stream);
+        if (wave || c->kernel32 == RBGS_KERNEL_WAVEFRONT) {
+            const int parts = wave_parts(c, streams, (double)m * (3.0 + c->g.n * (double)c->g.n / 1.9e6));
+            const rbgs_status st = launch_wavefront_passes<float>(c->f32, k, passes, parts, c->stream);
             if (st != RBGS_OK) return st;
         } else {
             for (long q = 0; q < passes; ++q) {
@@ -798,6 +839,7 @@ rbgs_status rbgs_get_solution(rbgs_t c, double *u_out) {
     if (st != RBGS_OK) return st;
     RBGS_CUDA(cudaMemcpyAsync(u_out, c->staging, count * sizeof(double), cudaMemcpyDefault, c->stream));
     RBGS_CUDA(cudaStreamSynchronize(c->stream));
+    stream_idle(c->device, c->stream);
     return RBGS_OK;
 }
 
@@ -917,6 +959,7 @@ rbgs_status rbgs_run_stream(rbgs_t c, int count, const double *const *f, const d
 void rbgs_destroy(rbgs_t c) {
     if (!c) return;
     cudaStreamSynchronize(c->stream);
+    stream_idle(c->device, c->stream);
     free_ctx(c);
 }
 

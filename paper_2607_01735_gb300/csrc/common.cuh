@@ -66,13 +66,18 @@ inline Geometry make_geometry(int n) { return Geometry{n, colour_width(n), n + 2
 constexpr int kMaxPartials = 8192;
 
 // Tiles of the resident kernel (resident.cu): gx x gy of them, each of at most rows rows and
-// vals values of a colour row, `period` sweeps between exchanges.  rows == 0: does not fit.
+// vals values of a colour row, `period` sweeps between exchanges; microseconds a sweep by the
+// model.  rows == 0: does not fit.
 struct ResidentPlan {
     int gx, gy, rows, vals, period;
+    double us;
 };
 
+constexpr int kResidentShares = 8;  // plans for 1 to 16 streams that share the device
+
 struct ResidentState {
-    ResidentPlan plan;
+    ResidentPlan plan[kResidentShares];  // [0]: the whole device
+    bool planned[kResidentShares];
     unsigned long long *slots;  // exchange slots
     unsigned *epoch;            // [0] number of the last period, [1] scratch
     bool use;                   // false: no plan, no room for the slots, or its launch was refused
@@ -161,23 +166,28 @@ template <typename T>
 rbgs_status launch_temporal_pass(ColourField<T> &fld, int k, int *status, cudaStream_t s);
 rbgs_status launch_sweeps_f32(const ColourField<float> &fld, long nsweeps, cudaStream_t s);
 // register-wavefront passes of k sweeps each between fld.u and fld.alt, which are swapped so
-// that the result is in fld.u (wavefront.cu)
+// that the result is in fld.u; each fills one of `parts` equal parts of the device (wavefront.cu)
 template <typename T>
-rbgs_status launch_wavefront_passes(ColourField<T> &fld, int k, long passes, cudaStream_t s);
+rbgs_status launch_wavefront_passes(ColourField<T> &fld, int k, long passes, int parts, cudaStream_t s);
 // nsweeps FP64 sweeps of fld in cooperative launches with a bounded grid barrier between
 // the colours (persistent.cu); a barrier that gives up sets *status
 template <typename T>
 rbgs_status launch_persistent_sweeps(ColourField<T> &fld, long nsweeps, unsigned *counter, int *status,
                                      cudaStream_t s);
+// Streams of the process that share the device with a launch on s about now, s among them (1:
+// alone); a launch on s takes about us microseconds more; s has been waited for (stream_share.cu)
+int streams_sharing(int device, cudaStream_t s);
+void stream_busy(int device, cudaStream_t s, double us);
+void stream_idle(int device, cudaStream_t s);
 // all sweeps of a small grid in one cooperative launch, tiles in shared memory (resident.cu).
 // kind 0: FP64, 1: FP32 inner sweeps, 2: fused.  nsweeps >= 2
 // (the plan has no rows where the kernel does not fit the grid or cannot run on this device);
-// kLaunchRefused: nothing was launched
+// kLaunchRefused: nothing was launched.  streams: how many share the device
 ResidentPlan resident_plan(int n, int kind);
 size_t resident_slot_bytes(int n, int W, int kind);
-rbgs_status launch_resident_sweeps_f64(const rbgs_ctx *c, long nsweeps, cudaStream_t s);
-rbgs_status launch_resident_sweeps_f32(const rbgs_ctx *c, long nsweeps, cudaStream_t s);
-rbgs_status launch_resident_sweeps_fused(const rbgs_ctx *c, long nsweeps, cudaStream_t s);
+rbgs_status launch_resident_sweeps_f64(rbgs_ctx *c, long nsweeps, int streams, cudaStream_t s);
+rbgs_status launch_resident_sweeps_f32(rbgs_ctx *c, long nsweeps, int streams, cudaStream_t s);
+rbgs_status launch_resident_sweeps_fused(rbgs_ctx *c, long nsweeps, int streams, cudaStream_t s);
 // FP32 inner sweeps in one launch of one thread-block cluster, d held in its shared memory
 // (cluster_sweeps.cu); usable when d of an n^2 grid with row pitch W fits the cluster
 bool cluster_sweeps_f32_fit(int n, int W);
@@ -193,6 +203,6 @@ rbgs_status launch_fused_prepare(const rbgs_ctx *c, long long nsweeps, cudaStrea
 rbgs_status launch_fused_half_sweep(const rbgs_ctx *c, int colour, cudaStream_t s);
 // nsweeps (>= kFusedWaveMin) fused sweeps at that scale in register-wavefront passes (wavefront.cu)
 constexpr long kFusedWaveMin = 4;
-rbgs_status launch_fused_wave_sweeps(const rbgs_ctx *c, long nsweeps, cudaStream_t s);
+rbgs_status launch_fused_wave_sweeps(const rbgs_ctx *c, long nsweeps, int parts, cudaStream_t s);
 
 }  // namespace rbgs

@@ -357,7 +357,7 @@ int sm_count_wf() {
 }
 
 template <typename T, int K, int P, int MODE>
-rbgs_status run_pass(WfArgs<T> &a, cudaStream_t s) {
+rbgs_status run_pass(WfArgs<T> &a, int parts, cudaStream_t s) {
     constexpr size_t smem = wf_smem<T, K, P>();
     a.halo = (K + P - 1) / P * P;
     a.ow = 32 * P - 2 * a.halo;
@@ -378,7 +378,7 @@ rbgs_status run_pass(WfArgs<T> &a, cudaStream_t s) {
         set_error("wavefront pass: no resident block fits");
         return RBGS_ECUDA;
     }
-    const long capacity = (long)per_sm * kWfWarps * sm_count_wf();
+    const long capacity = (long)per_sm * kWfWarps * sm_count_wf() / parts;
     const long rows = a.n + 2, sides = a.strips > 1 ? 2 : 1, inner = a.strips - sides;
     // One wave of items, all of about the same length.  A step of an edge strip takes longer (its
     // checks), and a wave is as long as its longest item, so edge strips are cut into shorter
@@ -415,7 +415,7 @@ rbgs_status run_pass(WfArgs<T> &a, cudaStream_t s) {
 // nsweeps = (whole passes) k sweeps of fld through its partner buffer; the buffers are
 // swapped when the result ends up there.
 template <typename T, int K, int P>
-rbgs_status run_field(ColourField<T> &fld, long passes, cudaStream_t s) {
+rbgs_status run_field(ColourField<T> &fld, long passes, int parts, cudaStream_t s) {
     WfArgs<T> a{};
     a.hf0 = fld.hf[0], a.hf1 = fld.hf[1];
     a.n = fld.n, a.W = fld.W, a.kmax = (fld.n + 3) / 2, a.one = 1.0;
@@ -423,7 +423,8 @@ rbgs_status run_field(ColourField<T> &fld, long passes, cudaStream_t s) {
     for (long q = 0; q < passes; ++q) {
         a.in = buf[q & 1][1];
         a.o0 = buf[(q & 1) ^ 1][0], a.o1 = buf[(q & 1) ^ 1][1];
-        const rbgs_status st = q + 1 == passes ? run_pass<T, K, P, kWfLast>(a, s) : run_pass<T, K, P, 0>(a, s);
+        const rbgs_status st = q + 1 == passes ? run_pass<T, K, P, kWfLast>(a, parts, s)
+                                                 : run_pass<T, K, P, 0>(a, parts, s);
         if (st != RBGS_OK) return st;
     }
     if (passes & 1) {
@@ -438,33 +439,35 @@ rbgs_status run_field(ColourField<T> &fld, long passes, cudaStream_t s) {
 }
 
 template <int MODE>
-rbgs_status run_fused(WfArgs<int64_t> &a, int k, cudaStream_t s) {
-    return k == 2 ? run_pass<int64_t, 2, 2, MODE>(a, s) : run_pass<int64_t, 3, 2, MODE>(a, s);
+rbgs_status run_fused(WfArgs<int64_t> &a, int k, int parts, cudaStream_t s) {
+    return k == 2 ? run_pass<int64_t, 2, 2, MODE>(a, parts, s) : run_pass<int64_t, 3, 2, MODE>(a, parts, s);
 }
 
 }  // namespace
 
 template <>
-rbgs_status launch_wavefront_passes<double>(ColourField<double> &fld, int k, long passes, cudaStream_t s) {
+rbgs_status launch_wavefront_passes<double>(ColourField<double> &fld, int k, long passes, int parts,
+                                            cudaStream_t s) {
     switch (k) {
-    case 2: return run_field<double, 2, 2>(fld, passes, s);
-    case 4: return run_field<double, 4, 2>(fld, passes, s);
+    case 2: return run_field<double, 2, 2>(fld, passes, parts, s);
+    case 4: return run_field<double, 4, 2>(fld, passes, parts, s);
     default: set_error("FP64 wavefront depth must be 2 or 4 (got %d)", k); return RBGS_EINVAL;
     }
 }
 
 template <>
-rbgs_status launch_wavefront_passes<float>(ColourField<float> &fld, int k, long passes, cudaStream_t s) {
+rbgs_status launch_wavefront_passes<float>(ColourField<float> &fld, int k, long passes, int parts,
+                                           cudaStream_t s) {
     switch (k) {
-    case 2: return run_field<float, 2, 4>(fld, passes, s);
-    case 4: return run_field<float, 4, 4>(fld, passes, s);
-    case 6: return run_field<float, 6, 4>(fld, passes, s);
+    case 2: return run_field<float, 2, 4>(fld, passes, parts, s);
+    case 4: return run_field<float, 4, 4>(fld, passes, parts, s);
+    case 6: return run_field<float, 6, 4>(fld, passes, parts, s);
     default: set_error("FP32 wavefront depth must be 2, 4 or 6 (got %d)", k); return RBGS_EINVAL;
     }
 }
 
 // nsweeps fused sweeps (>= kFusedWaveMin) at the scale the last launch_fused_prepare chose.
-rbgs_status launch_fused_wave_sweeps(const rbgs_ctx *c, long nsweeps, cudaStream_t s) {
+rbgs_status launch_fused_wave_sweeps(const rbgs_ctx *c, long nsweeps, int parts, cudaStream_t s) {
     WfArgs<int64_t> a{};
     a.hf0 = c->hq[0], a.hf1 = c->hq[1];
     a.d0 = c->f64.u[0], a.d1 = c->f64.u[1];
@@ -481,9 +484,9 @@ rbgs_status launch_fused_wave_sweeps(const rbgs_ctx *c, long nsweeps, cudaStream
         const int k = nsweeps == 4 || nsweeps == 2 ? 2 : depth;
         a.in = first ? reinterpret_cast<const int64_t *>(c->f64.u[1]) : c->tq[at];
         a.o1 = c->tq[at ^ 1];
-        const rbgs_status st = first              ? run_fused<kWfIn>(a, k, s)
-                               : k == nsweeps ? run_fused<kWfLast>(a, k, s)
-                                              : run_fused<0>(a, k, s);
+        const rbgs_status st = first              ? run_fused<kWfIn>(a, k, parts, s)
+                               : k == nsweeps ? run_fused<kWfLast>(a, k, parts, s)
+                                              : run_fused<0>(a, k, parts, s);
         if (st != RBGS_OK) return st;
         first = false;
         at ^= 1;

@@ -126,3 +126,33 @@ def test_device_without_cooperative_launches(lib):
         st, calls = c.sweep(40)
         assert st == 0 and calls and _kinds(calls) <= {"plain", "graph"}
         c.close()
+
+
+# ------------------------------------------------------------------ several solvers at once
+def _tiles(calls):
+    return [blocks for kind, name, blocks, _ in calls if kind == "cooperative" and "resident" in name]
+
+
+@pytest.mark.parametrize("n,opts", [(127, {}), (255, {"fma": 1})])
+def test_solvers_on_several_streams_share_the_device(lib, n, opts):
+    """A launch takes the whole device alone, and a part of it while other streams are busy (here:
+    with a second's worth of sweeps each); contexts of one stream or of another device do not count."""
+    lone = Context(lib, n, stream=101, **opts)
+    whole = _tiles(lone.sweep(20)[1])
+    assert whole and whole[0] > 76
+    lone.close()
+    busy = [Context(lib, n, stream=201 + q, **opts) for q in range(7)]
+    parts = [_tiles(c.sweep(1000000)[1])[0] for c in busy]
+    assert parts[0] == whole[0] and all(p <= 152 // 2 for p in parts[1:]) and parts[-1] <= 152 // 6
+    same = Context(lib, n, stream=201, **opts)
+    assert _tiles(same.sweep(20)[1])[0] <= 152 // 6  # six other streams besides its own
+    lib.fake_set_device(1)
+    other = Context(lib, n, stream=301, **opts)
+    assert _tiles(other.sweep(20)[1]) == whole
+    other.close()
+    lib.fake_set_device(0)
+    for c in busy:
+        c.close()  # waits for its stream
+    got = [_tiles(same.sweep(20)[1]) for _ in range(3)]
+    assert got[-1] == whole  # the third launch in a row with no other stream busy
+    same.close()
