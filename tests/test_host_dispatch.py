@@ -156,3 +156,16 @@ def test_solvers_on_several_streams_share_the_device(lib, n, opts):
     got = [_tiles(same.sweep(20)[1]) for _ in range(3)]
     assert got[-1] == whole  # the third launch in a row with no other stream busy
     same.close()
+
+
+# ------------------------------------------------------------------ single sweeps
+@pytest.mark.parametrize("n,kernels", [(255, ["half_sweep"] * 2), (511, ["persistent_sweeps"]),
+                                       (1023, ["persistent_sweeps"]), (4095, ["persistent_sweeps"])])
+def test_a_single_sweep_takes_the_fewest_launches(lib, n, kernels):
+    """One sweep of a grid that several sweeps would run in tiles: the grid-barrier launch from
+    416^2 on, one launch per colour below."""
+    c = Context(lib, n)
+    st, calls = c.sweep(1)
+    assert st == 0 and len(calls) == len(kernels)
+    assert all(want in name for want, (_, name, _, _) in zip(kernels, calls)), calls
+    c.close()
