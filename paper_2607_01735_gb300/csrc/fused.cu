@@ -85,11 +85,18 @@ __global__ void __launch_bounds__(kMaxThreads)
 prepare_kernel(const double *__restrict__ hf0, const double *__restrict__ hf1, const double *__restrict__ u0,
                const double *__restrict__ u1, int64_t *__restrict__ hq0, int64_t *__restrict__ hq1, int n, int W,
                unsigned long long *__restrict__ words, long long nsweeps) {
-    int e = 0;
-    const bool ok = scale_exponent(bitsd(words[0]), bitsd(words[1]), nsweeps, &e);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
-        words[2] = ok ? (unsigned long long)(long long)e : kNoScale;
-    if (!ok) return;
+    __shared__ int s_e, s_ok;
+    // Once per block: it is FP64 work, which all threads would queue for (a call of one fused sweep,
+    // us, by every thread and so: 1300^2 47.2, 39.0; 2047^2 88.0, 69.8; 4095^2 235.6, 182.6).
+    if (threadIdx.x == 0) {
+        int e = 0;
+        s_ok = scale_exponent(bitsd(words[0]), bitsd(words[1]), nsweeps, &e);
+        s_e = e;
+        if (blockIdx.x == 0 && blockIdx.y == 0) words[2] = s_ok ? (unsigned long long)(long long)e : kNoScale;
+    }
+    __syncthreads();
+    if (!s_ok) return;
+    const int e = s_e;
     const int k = 2 * (blockIdx.x * kMaxThreads + threadIdx.x);
     if (k >= W) return;
     for (int i = blockIdx.y; i < n + 2; i += gridDim.y) {
