@@ -169,3 +169,26 @@ def test_a_single_sweep_takes_the_fewest_launches(lib, n, kernels):
     assert st == 0 and len(calls) == len(kernels)
     assert all(want in name for want, (_, name, _, _) in zip(kernels, calls)), calls
     c.close()
+
+
+# ------------------------------------------------------------------ the automatic choice's limits
+@pytest.mark.parametrize("n,opts,kernel", [
+    (1368, {}, "resident"), (1369, {}, "persistent"), (1368, {"fma": 1}, "resident"), (1369, {"fma": 1}, "wavefront"),
+    (3000, {"fma": 1}, "wavefront"), (63, {"fma": 1}, "resident"),
+    (1400, {"fma": 1, "kernel": rb.RBGS_KERNEL_COLOUR}, "fused_half_sweep"), (415, {}, "resident")])
+def test_automatic_choice_of_the_sweeps(lib, n, opts, kernel):
+    c = Context(lib, n, **opts)
+    st, calls = c.sweep(9)
+    names = [name for _, name, _, _ in calls if not any(w in name for w in ("absmax", "prepare"))]
+    assert st == 0 and names and all(kernel in name for name in names), names
+    c.close()
+
+
+@pytest.mark.parametrize("n,kernel", [(127, "resident"), (1000, "resident"), (1001, "wavefront"), (4095, "wavefront")])
+def test_automatic_choice_of_the_inner_sweeps(lib, n, kernel):
+    c = Context(lib, n, precision=rb.RBGS_FP32_REFINE, max_sweeps=100, inner_sweeps=100)
+    lib.fake_clear_log()
+    assert lib.rbgs_solve(c.ctx, 0.0, None, None) == rb.RBGS_ENOTCONV
+    assert any(kernel in name for _, name, _, _ in launches(lib))
+    assert not any(k in name for _, name, _, _ in launches(lib) for k in {"resident", "wavefront"} - {kernel})
+    c.close()
