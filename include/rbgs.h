@@ -106,7 +106,8 @@ typedef struct {
     int team_size;     /* rbgs_solve_batched: 2 or 4 forces the phased plan, in which the largest
                           problems left over after full waves of one block per problem are each
                           solved by a thread-block cluster of team_size blocks; 1: one block per
-                          problem always; 0: the autotuner decides                              */
+                          problem always; 0: the autotuner decides.  With 2 or 4 and tblock_k = 2,
+                          the full waves before that run one problem per cluster of 2 blocks     */
     int fma;           /* FP64 update of rbgs_sweep / rbgs_solve (RBGS_FP64 only):
                           0 (default): bit-exact, (((h2f + N) + S) + W) + E times 0.25 with every
                             step correctly rounded, the same bits as the plain sequential loop;
@@ -260,6 +261,10 @@ rbgs_status rbgs_solve_batched(int nprob, const rbgs_problem *probs, double tol,
  * per block, or one per cluster of 2) and the number solved by clusters in its second.  Any pointer may be NULL.
  */
 void rbgs_batched_last_shape(int *threads, int *blocks_per_sm, int *team, int *first, int *nteam);
+
+/* Not in the paper: library mechanics.  Blocks per problem in the first phase of that call's phased
+ * plan (1, or 2: clusters), 0 without one. */
+int rbgs_batched_last_first_team(void);
 
 /*
  * Relative residual of a natural-layout iterate without allocating memory.  The paper has

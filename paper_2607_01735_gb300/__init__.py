@@ -30,7 +30,8 @@ RBGS_KERNEL_AUTO, RBGS_KERNEL_COLOUR, RBGS_KERNEL_TEMPORAL, RBGS_KERNEL_WAVEFRON
 # Every symbol include/rbgs.h declares.
 EXPORTED = ("rbgs_default_opts", "rbgs_create", "rbgs_sweep", "rbgs_residual", "rbgs_solve",
             "rbgs_get_solution", "rbgs_set_solution", "rbgs_set_problem", "rbgs_solve_batched", "rbgs_destroy",
-            "rbgs_last_error", "rbgs_residual_static", "rbgs_batched_last_shape", "rbgs_run_stream")
+            "rbgs_last_error", "rbgs_residual_static", "rbgs_batched_last_shape", "rbgs_batched_last_first_team",
+            "rbgs_run_stream")
 
 
 class RbgsError(RuntimeError):
@@ -115,6 +116,8 @@ def load_library(path: str | None = None):
     lib.rbgs3d_destroy.restype = None
     lib.rbgs_batched_last_shape.argtypes = [ctypes.POINTER(c_int)] * 5
     lib.rbgs_batched_last_shape.restype = None
+    lib.rbgs_batched_last_first_team.argtypes = []
+    lib.rbgs_batched_last_first_team.restype = c_int
     _lib = lib
     return lib
 
@@ -247,6 +250,12 @@ def rbgs_batched_last_shape() -> dict:
     v = [ctypes.c_int(0) for _ in range(5)]
     load_library().rbgs_batched_last_shape(*[ctypes.byref(x) for x in v])
     return dict(zip(("threads", "blocks_per_sm", "team", "first", "nteam"), (x.value for x in v)))
+
+
+def rbgs_batched_last_first_team() -> int:
+    """rbgs_batched_last_first_team: blocks per problem in the first phase of this thread's last
+    batched solve (0: no such phase)."""
+    return int(load_library().rbgs_batched_last_first_team())
 
 
 def rbgs_residual_static(n: int, h2: float, f, u, rel_out, stream=None) -> None:

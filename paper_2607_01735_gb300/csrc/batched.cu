@@ -838,7 +838,7 @@ extern "C" rbgs_status rbgs_solve_batched(int nprob, const rbgs_problem *probs, 
     }
     if (st == RBGS_OK && o.team_size > 1) {
         // explicit request: the phased plan with clusters of team_size blocks
-        lc = LaunchConfig{1024, 1, o.team_size};
+        lc = LaunchConfig{1024, 1, o.team_size, o.tblock_k == 2 ? 2 : 1};
         if (max_clusters_of(o.team_size) < 1) {
             set_error("clusters of %d blocks of 1024 threads do not fit on this device", o.team_size);
             st = RBGS_EINVAL;
@@ -980,3 +980,5 @@ extern "C" void rbgs_batched_last_shape(int *threads, int *blocks_per_sm, int *t
     if (first) *first = g_last_shape.first;
     if (nteam) *nteam = g_last_shape.nteam;
 }
+
+extern "C" int rbgs_batched_last_first_team(void) { return g_last_shape.first > 0 ? g_last_shape.team1 : 0; }
