@@ -309,13 +309,13 @@ __global__ void relu_grad_kernel(const float4 *__restrict__ dX, const uint2 *__r
 
 // Backward of one layer with its weights already transposed (Wtt).  Gin != NULL: the data
 // gradient goes through the ReLU of the layer before (whose output is X) into Gin as bf16; dX is
-// then scratch, used by the mma.sync engine only.
+// then scratch of the mma.sync engine, and NULL with the others.
 rbgs_status backward_products(const uint16_t *X, const uint16_t *Wt, const uint16_t *G, float *dX, uint16_t *Gin,
                               float *dW, float *db, const uint16_t *Wtt, int B, int H, int W, int Cin, int Cout, int ks,
                               int accumulate, cudaStream_t s) {
     const long P = (long)B * H * W;
     const int taps = ks * ks;
-    if (dX) {
+    if (dX || Gin) {
         if (g_engine != RBGS_CONV_MMA_SYNC) {
             const rbgs_status st = umma_conv_backward_data(Wtt, G, dX, X, Gin, B, H, W, Cin, Cout, ks, accumulate,
                                                            g_engine == RBGS_CONV_TCGEN05, s);

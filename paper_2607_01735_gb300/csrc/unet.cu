@@ -14,6 +14,7 @@
 // Parameters (FP32, in this order per layer): weights [Cout][k][k][Cin], then bias[Cout].
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -262,12 +263,13 @@ struct rbgs_unet {
     uint16_t *wb;               // bf16 copy used by the forward and backward
     uint16_t *wtt;              // transposed weights of every layer (at the weights' offsets)
     long step;
-    // activation / gradient buffers for one (B, H, W)
+    // activation / gradient buffers for one (B, H, W); the gradients' from the first training step on
     int B, H, W;
     std::vector<void *> bufs;
     uint16_t *act[22];          // bf16 activations (see forward for the order)
-    float *gr[22];              // fp32 gradients of the same tensors
-    uint16_t *gbf[2];           // bf16 pre-activation gradients: a layer's and the next one's
+    float *gr[22];              // FP32 gradients of the concatenations and the pooled tensors
+    uint16_t *gbf[2];           // bf16 pre-activation gradients: a layer's and the next one's (NULL: none yet)
+    float *scratch;             // FP32 data gradient of the mma.sync engine (NULL: none yet)
     float *out8, *dloss, *hloss;
 };
 
@@ -281,39 +283,65 @@ enum {
 const int kActCh[A_COUNT] = {16, 32, 32, 32, 64, 64, 64, 128, 128, 128, 256, 256, 384, 128, 128, 192, 64, 64, 96, 32, 32};
 const int kActLv[A_COUNT] = {0, 0, 0, 1, 1, 1, 2, 2, 2, 3, 3, 3, 2, 2, 2, 1, 1, 1, 0, 0, 0};
 
-rbgs_status ensure_buffers(rbgs_unet *net, int B, int H, int W) {
-    if (net->B == B && net->H == H && net->W == W) return RBGS_OK;
+size_t act_elems(const rbgs_unet *net, int a) {
+    return (size_t)net->B * (net->H >> kActLv[a]) * (net->W >> kActLv[a]) * kActCh[a];
+}
+
+// A buffer for the network's current (B, H, W), freed with the others of that size.
+bool alloc_buffer(rbgs_unet *net, size_t bytes, void **p) {
+    if (cudaMalloc(p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        *p = nullptr;
+        return false;
+    }
+    net->bufs.push_back(*p);
+    return true;
+}
+
+void free_buffers(rbgs_unet *net) {
     for (void *p : net->bufs) cudaFree(p);
     net->bufs.clear();
     net->B = net->H = net->W = 0;
-    auto alloc = [&](size_t bytes, void **p) {
-        if (cudaMalloc(p, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            *p = nullptr;
-            return false;
-        }
-        net->bufs.push_back(*p);
-        return true;
-    };
-    size_t gmax = 0;
-    for (int a = 0; a < A_COUNT; ++a) {
-        const long pix = (long)B * (H >> kActLv[a]) * (W >> kActLv[a]);
-        const size_t n = (size_t)pix * kActCh[a];
-        if (!alloc(n * 2, (void **)&net->act[a]) || !alloc(n * 4, (void **)&net->gr[a])) {
-            set_error("U-Net activation buffers: out of device memory");
-            return RBGS_ENOMEM;
-        }
-        gmax = n > gmax ? n : gmax;
-    }
-    const size_t P = (size_t)B * H * W;
-    if (!alloc(gmax * 2, (void **)&net->gbf[0]) || !alloc(gmax * 2, (void **)&net->gbf[1]) ||
-        !alloc(P * 8 * 4, (void **)&net->out8) || !alloc(8, (void **)&net->dloss)) {
+    net->gbf[0] = net->gbf[1] = nullptr;
+    net->scratch = nullptr;
+}
+
+// What a forward pass needs.
+rbgs_status ensure_buffers(rbgs_unet *net, int B, int H, int W) {
+    if (net->B == B && net->H == H && net->W == W) return RBGS_OK;
+    free_buffers(net);
+    net->B = B, net->H = H, net->W = W;
+    bool ok = alloc_buffer(net, (size_t)B * H * W * 8 * 4, (void **)&net->out8) &&
+              alloc_buffer(net, 8, (void **)&net->dloss);
+    for (int a = 0; a < A_COUNT && ok; ++a) ok = alloc_buffer(net, act_elems(net, a) * 2, (void **)&net->act[a]);
+    if (!ok) {
+        free_buffers(net);
         set_error("U-Net buffers: out of device memory");
         return RBGS_ENOMEM;
     }
-    net->B = B;
-    net->H = H;
-    net->W = W;
+    return RBGS_OK;
+}
+
+// What a backward pass needs besides: FP32 gradients where one kernel forms a sum of several
+// (concatenations and poolings), the bf16 ones that a layer hands to the next, as large as the
+// largest output of a layer, and with the mma.sync engine that layer's FP32 data gradient.
+rbgs_status ensure_gradients(rbgs_unet *net) {
+    size_t most = 0;
+    bool ok = true;
+    const bool first = !net->gbf[1];
+    for (int a = 1; a < A_COUNT; ++a) {
+        const bool summed = a == A_C0 || a == A_C1 || a == A_C2 || a == A_P0 || a == A_P1 || a == A_P2;
+        if (!summed) most = std::max(most, act_elems(net, a));
+        if (summed && first && ok) ok = alloc_buffer(net, act_elems(net, a) * 4, (void **)&net->gr[a]);
+    }
+    for (int q = 0; q < 2 && first && ok; ++q) ok = alloc_buffer(net, most * 2, (void **)&net->gbf[q]);
+    if (ok && !net->scratch && rbgs_conv_get_engine() == RBGS_CONV_MMA_SYNC)
+        ok = alloc_buffer(net, most * 4, (void **)&net->scratch);
+    if (!ok) {
+        free_buffers(net);
+        set_error("U-Net gradient buffers: out of device memory");
+        return RBGS_ENOMEM;
+    }
     return RBGS_OK;
 }
 
@@ -411,7 +439,8 @@ rbgs_status backward(rbgs_unet *net) {
     auto conv_bwd = [&](int li, int in, int to) {
         const Layer &L = net->layers[li];
         const rbgs_status st = conv_backward_layer(
-            net->act[in], net->gbf[g], to == NONE ? nullptr : net->gr[in], to == TO_G ? net->gbf[g ^ 1] : nullptr,
+            net->act[in], net->gbf[g], to == TO_F32 ? net->gr[in] : to == TO_G ? net->scratch : nullptr,
+            to == TO_G ? net->gbf[g ^ 1] : nullptr,
             net->grad + L.w_off, net->grad + L.b_off, net->wtt + L.w_off, B, H >> L.level, W >> L.level, L.cin, L.cout,
             L.ks, s);
         if (to == TO_G) g ^= 1;
@@ -566,6 +595,7 @@ rbgs_status rbgs_unet_train_step(rbgs_unet_t net, const float *x, const float *t
         return RBGS_EINVAL;
     }
     UNET_TRY(ensure_buffers(net, B, H, W));
+    UNET_TRY(ensure_gradients(net));
     UNET_TRY(forward(net, x));
     const long P = (long)B * H * W;
     RBGS_CUDA(cudaMemsetAsync(net->dloss, 0, 8, net->stream));  // [0] loss, [1] sum(mask)

@@ -192,3 +192,47 @@ def test_automatic_choice_of_the_inner_sweeps(lib, n, kernel):
     assert any(kernel in name for _, name, _, _ in launches(lib))
     assert not any(k in name for _, name, _, _ in launches(lib) for k in {"resident", "wavefront"} - {kernel})
     c.close()
+
+
+# ------------------------------------------------------------------ the network's buffers
+def test_network_buffers_are_what_a_pass_needs(lib):
+    """A forward pass holds the activations and its output; a training step adds the FP32 gradients
+    of the concatenations and pooled tensors and two bf16 ones, the mma.sync engine one more FP32."""
+    B, H = 2, 64
+    P = B * H * H
+    x, y, m = np.zeros((P, 4), np.float32), np.zeros(P, np.float32), np.ones(P, np.float32)
+    p = lambda a: ctypes.c_void_p(a.ctypes.data)
+    net = ctypes.c_void_p()
+    lib.rbgs_unet_create.argtypes = [ctypes.c_uint64, ctypes.c_void_p, ctypes.POINTER(ctypes.c_void_p)]
+    lib.rbgs_unet_train_step.argtypes = [ctypes.c_void_p] * 4 + [ctypes.c_int] * 3 + [ctypes.c_float] + [ctypes.c_void_p] * 2
+    lib.rbgs_unet_destroy.restype = None
+    before = lib.fake_memory_in_use()
+    assert lib.rbgs_unet_create(1, None, ctypes.byref(net)) == 0
+    weights = lib.fake_memory_in_use()
+    channels = 16 + 32 + 32 + 96 + 32 + 32 + (32 + 64 + 64 + 192 + 64 + 64) / 4 + (64 + 128 + 128 + 384 + 128 + 128) / 16 \
+        + (128 + 256 + 256) / 64
+    acts = int(P * channels * 2) + P * 8 * 4 + 8
+    lib.rbgs_conv_set_engine(2)  # gathers: tensor maps need a driver
+    try:
+        assert lib.rbgs_unet_forward(net, p(x), p(y), B, H, H) == 0
+        assert lib.fake_memory_in_use() - weights == acts
+        step = lambda: lib.rbgs_unet_train_step(net, p(x), p(y), p(m), B, H, H, 1e-3, None, None)
+        summed = 96 + 192 / 4 + 384 / 16 + 32 / 4 + 64 / 16 + 128 / 64
+        for _ in range(2):
+            assert step() == 0, lib.rbgs_last_error()
+            assert lib.fake_memory_in_use() - weights == acts + int(P * summed * 4) + 2 * P * 32 * 2
+        lib.rbgs_conv_set_engine(1)
+        assert step() == 0, lib.rbgs_last_error()
+        assert lib.fake_memory_in_use() - weights == acts + int(P * summed * 4) + 2 * P * 32 * 2 + P * 32 * 4
+        assert lib.rbgs_unet_forward(net, p(x), p(y), 1, H, H) == 0  # another size frees them
+        assert lib.fake_memory_in_use() - weights <= acts
+        # out of memory part way: nothing is kept, and a smaller size still works
+        lib.fake_memory_limit(lib.fake_memory_in_use() + acts)
+        assert lib.rbgs_unet_train_step(net, p(x), p(y), p(m), B, H, H, 1e-3, None, None) == 2
+        assert lib.fake_memory_in_use() == weights
+        assert lib.rbgs_unet_forward(net, p(x), p(y), 1, H, H) == 0
+    finally:
+        lib.rbgs_conv_set_engine(0)
+        lib.fake_memory_limit(2 ** 63)
+        lib.rbgs_unet_destroy(net)
+    assert lib.fake_memory_in_use() == before
