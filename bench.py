@@ -53,7 +53,7 @@ PROFILES = {
                                    "paper_2607_01735_gb300/csrc/fp64.cuh"]),
 }
 PERSIST_MIN_N, PERSIST_MAX_N = 416, 1 << 15
-RESIDENT_MAX_N = 1376  # tiles in shared memory up to here (GB300: 152 SMs)
+RESIDENT_MAX_N = 1368  # tiles in shared memory up to here (220 KB on each of GB300's 152 SMs)
 # side files of a run (nvidia-smi clock samples, trained U-Net parameters)
 OUT_DIR = os.environ.get("RBGS_BENCH_OUT", os.path.join(ROOT, "bench_out"))
 

@@ -118,8 +118,9 @@ typedef struct {
                             divided by 4 is rounded once to binary64 (nearest, ties to even).
                             Integer arithmetic only, so the update leaves the FP64 pipe.  Agrees
                             with the bit-exact iterate to <= 1e-13 relative max-norm after the same
-                            sweeps (the tolerance set for this mode); a non-finite value in u or h2 f makes
-                            that block of sweeps run the bit-exact update.  With kernel AUTO and
+                            sweeps (the tolerance set for this mode); with a non-finite value in u
+                            or h2 f a block of sweeps writes NaN to every interior point (the next
+                            residual gives RBGS_ENONFINITE).  With kernel AUTO and
                             no launch-shape option, tiles in shared memory where they fit, above
                             that register-wavefront passes (two more FP64 arrays of half the grid
                             each); without room for their buffers, and otherwise, one launch per

@@ -48,13 +48,13 @@ constexpr int kPersistMaxN = 1 << 15;
 // max |u| + (sweeps) max |h2 f| / 2 a priori, so shorter blocks keep it tighter; the
 // rescaling pass (max |u|, h2 f onto the grid: about one sweep's traffic) repeats per block.
 constexpr long kFusedChunk = 1024;
-// Fused sweeps as register-wavefront passes (wavefront.cu) from this size on.  Measured per
-// sweep against cached graphs of one launch per colour: 5.6 against 4.4 us at 255^2, 5.7 / 5.8
-// at 511^2, 7.2 / 13.1 at 1023^2, 9.9 / 16.2 at 1500^2, 31 / 96 at 4095^2, 382 / 1021 at
-// 16384^2.
+// Fused sweeps as register-wavefront passes (wavefront.cu) from this size on, where the resident
+// kernel does not run (so from 1369^2 on 152 SMs).  Measured per sweep against cached graphs of one
+// launch per colour: 5.6 against 4.4 us at 255^2, 5.7 / 5.8 at 511^2, 7.2 / 13.1 at 1023^2, 9.9 /
+// 16.2 at 1500^2, 31 / 96 at 4095^2, 382 / 1021 at 16384^2.
 constexpr int kFusedWaveMinN = 512;
-// The resident kernel (resident.cu): FP64 and fused sweeps wherever its tiles fit (up to about
-// 1376^2, resident_plan decides), FP32 inner sweeps up to 1000^2, above which the wavefront is
+// The resident kernel (resident.cu): FP64 and fused sweeps wherever its tiles fit (up to
+// 1368^2 on 152 SMs, resident_plan decides), FP32 inner sweeps up to 1000^2, above which the wavefront is
 // as fast and needs no cooperative launch.
 constexpr int kResidentMaxN = 2048, kResident32MaxN = 1000;
 constexpr int kWave32MinN = 1001;    // FP32 inner sweeps as wavefront passes from this size on

@@ -22,15 +22,21 @@
 // accumulators, four warps each (on the narrowest layers one tile's drain takes longer than its
 // MMAs).  Every wait is bounded as in the other kernels.
 //
-// What bounds it: the MMAs.  One takes 40 to 60 cycles from these layouts without swizzle
-// (128 x 16 bf16 of A at about 70 bytes per clock) for 16 to 32 cycles of products, and its thread
-// waits about 500 cycles per tile at the hand-over; copies alone would take a third of the time.
+// What bounds it: the thread that issues the MMAs.  Cycles per tile at 16 x 264^2, forward, by
+// clock64 around its steps (the readings add 10 to 20% to the time): 16->32 (9 MMAs) 918 to issue
+// and commit, 480 at its two waits, 1692 in all; 32->32 (18) 1636, 490, 2601; 96->32 (54) 3644, 535,
+// 5023.  So an MMA takes 102, 91 and 67 cycles for 16 of products (its A operand is 4 KB of shared
+// memory without swizzle).  A wait takes about 230 cycles on every layer, so that is a poll with its
+// fences and not a wait for others: the producers need 308, 611 and 2321 cycles for a tile's copies
+// and wait 692, 703 and 1365, and a drain takes 909 to 2083, four tiles at a time.
 // Measured on 16 images of 264 x 264 (us; before: gathers forward, TMA data gradient; in
 // brackets: the issuing thread chosen by lane number, see elect_one):
 //   forward 16->32 123, now 56 [88]; 32->32 168, now 82 [115]; 96->32 393, now 154 [217]
 //   at 132 x 132: 32->64 53, now 31 [41]; 64->64 81, now 39 [54]
 //   data gradient 32->32 254, now 105 [117]; 96->32 270, now 187 [180]; at 132 x 132:
 //   64->64 158, now 51 [58]; 32->64 154, now 45 [54]
+// The TMA kernel with the patches it has now, data gradient: 96->32 287 (1 and 4 images: 29.9 and
+// 62.4, here 28.9 and 60.3), 32->32 151; at 132 x 132 64->64 84, 32->64 82.
 
 constexpr int kSlabW = 10, kSlabH = 18;
 constexpr uint32_t kPlane = (kSlabW * kSlabH + 1) * 16;  // an odd number of 16-byte rows: 8 groups of a pixel hit 8 banks

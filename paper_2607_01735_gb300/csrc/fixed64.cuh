@@ -90,8 +90,8 @@ __host__ __device__ __forceinline__ int64_t fixed_quarter(int64_t s) {
 // than Q/4 beyond the largest neighbour, so after t sweeps every |u| <= B + t Q / 2 and
 // every sum (before the division by 4) is at most S = 4 B + (2 nsweeps + 1) Q.  With
 // S = m 2^k, 0.5 <= m < 1, e = 61 - k gives S 2^e < 2^61; e is capped at kFixedMaxE and
-// is 0 when S = 0.  Returns false when B, Q or S is not finite (the caller then runs the
-// bit-exact update instead).  S is formed as (4 B) + ((2 nsweeps + 1) Q), each operation
+// is 0 when S = 0.  Returns false when B, Q or S is not finite (the caller's sweeps then write
+// NaN to every point they update).  S is formed as (4 B) + ((2 nsweeps + 1) Q), each operation
 // correctly rounded, so that every implementation picks the same e.
 __host__ __device__ __forceinline__ bool scale_exponent(double B, double Q, long long nsweeps, int *e) {
 #if defined(__CUDA_ARCH__)

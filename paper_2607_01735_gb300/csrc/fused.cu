@@ -15,11 +15,11 @@
 //   2. prepare_kernel: e = scale_exponent(B, Q, sweeps of the block) into words[2] (or
 //      kNoScale); h2 f of both colours converted once to the fixed-point grid (hq, int64),
 //      so the sweeps read it as is;
-//   3. the block's sweeps: register-wavefront passes of 2 or 3 sweeps (wavefront.cu) from
-//      512^2 on, else, or with a launch-shape option, one launch of fused_half_sweep per
-//      colour.
+//   3. the block's sweeps: in tiles (resident.cu) where those fit, register-wavefront passes of 2
+//      or 3 sweeps (wavefront.cu) above that; with a launch-shape option, or for fewer sweeps than
+//      these take, one launch of fused_half_sweep per colour.
 // A non-finite B or Q (a NaN or Inf in the iterate or in f) leaves no valid scale: the
-// block's half-sweeps then write NaN to every point they update, so the next residual
+// block's sweeps then write NaN to every point they update, so the next residual
 // reports RBGS_ENONFINITE.
 //
 // Work decomposition of fused_half_sweep: that of the bit-exact strip kernel (sweep.cu).  A

@@ -148,8 +148,9 @@ constexpr size_t wf_smem() {
     return (size_t)kWfWarps * wf_ring_rows<K>() * 2 * 32 * P * sizeof(T);
 }
 
-// Resident blocks per SM that the registers are allotted for: 3 (168 registers a thread, no
-// spills) for every instance but float K = 6.  Measured at 16384^2 (fused, K = 3): 382 us a
+// Resident blocks per SM that the registers are allotted for: 3 (168 registers a thread) for every
+// instance but float K = 6 (2: 255).  Spills: none but in float K = 4 (16 to 24 bytes of stack, 20
+// to 36 bytes moved each way) and K = 6 (48 to 56 bytes).  Measured at 16384^2 (fused, K = 3): 382 us a
 // sweep with 3, 394 with 4, 540 with 5 (spills); at 1500^2, 9.9 and 11.5 us with 3 and 4.
 template <typename T, int K>
 constexpr int wf_blocks() {
