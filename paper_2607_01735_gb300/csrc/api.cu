@@ -247,19 +247,23 @@ rbgs_status ensure_f32(rbgs_ctx *c) {
     if (c->kernel32 == RBGS_KERNEL_COLOUR && c->opts.kernel == RBGS_KERNEL_AUTO && c->opts.tblock_k == 0 &&
         c->opts.tile_rows == 0 && c->g.n <= kResident32MaxN)
         prepare_resident(c, c->res32, c->f32.W, 1);
-    // partner buffers for inner_sweeps_f32's passes; without room for them it does without
-    if (c->res32.use && c->g.n > kShareWave32MinN) {
-        for (int q = 0; q < 2; ++q) {
-            if (cudaMalloc(&c->f32.alt[q], bytes) != cudaSuccess ||
-                cudaMemsetAsync(c->f32.alt[q], 0, bytes, c->stream) != cudaSuccess) {
-                cudaGetLastError();
-                cudaFree(c->f32.alt[q]);
-                c->f32.alt[q] = nullptr;
-                break;
-            }
+    return RBGS_OK;
+}
+
+// Partner buffers for passes of a context whose inner sweeps run in tiles; false without room.
+bool ensure_alt32(rbgs_ctx *c) {
+    if (c->f32.alt[1]) return true;
+    const size_t bytes = (size_t)c->g.rows * c->f32.W * sizeof(float);
+    for (int q = 0; q < 2; ++q) {
+        if (!c->f32.alt[q] && (cudaMalloc(&c->f32.alt[q], bytes) != cudaSuccess ||
+                               cudaMemsetAsync(c->f32.alt[q], 0, bytes, c->stream) != cudaSuccess)) {
+            cudaGetLastError();
+            cudaFree(c->f32.alt[q]);
+            c->f32.alt[q] = nullptr;
+            return false;
         }
     }
-    return RBGS_OK;
+    return true;
 }
 
 rbgs_status status_error(int status) {
@@ -419,7 +423,8 @@ rbgs_status defect_stats(rbgs_ctx *c, double *rho, double *mx, bool *exact) {
 rbgs_status inner_sweeps_f32(rbgs_ctx *c, long m) {
     const int streams = sharing(c);
     // large tiled grids when many streams are at work: wavefront passes of a part of the device
-    const bool wave = c->res32.use && c->g.n > kShareWave32MinN && streams * c->g.n > kShareWave32 && c->f32.alt[1];
+    const bool wave = c->res32.use && c->g.n > kShareWave32MinN && streams * c->g.n > kShareWave32 &&
+                      ensure_alt32(c);
     if (c->res32.use && !wave && m >= 2) {
         const rbgs_status st = launch_resident_sweeps_f32(c, m, streams, c->stream);
         if (st != kLaunchRefused) return st;
