@@ -1096,7 +1096,7 @@ def main():
                         "frac": achieved / peak_hbm, "traffic": profiled_traffic(kname, args.emulate),
                         "kernel": kname, "peak_source": hbm_src, "launch_ms": 1e3 * launch_s,
                         "algorithmic_bytes_per_launch": alg_bytes,
-                        "note": ("per pass of 3 sweeps, bound by the integer ALU pipe (72% busy under ncu), not "
+                        "note": ("per pass of 3 sweeps, bound by the integer ALU pipe (74% busy under ncu), not "
                                  "by HBM" if blocked else "per half-sweep") +
                                 "; the sweeps' device time includes the per-block rescaling passes (max |u|, "
                                 "h2 f onto the fixed-point grid)"}

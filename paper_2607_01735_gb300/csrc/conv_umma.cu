@@ -650,7 +650,7 @@ bool sizes_fit(int B, int H, int W) { return (long)B * H * W < (1L << 31) - UK; 
 //     fixed costs (filling the ring, one drain of three accumulators per item) are paid by then.
 //     Pixel steps, gather / tap row: 66^2 128->128 880 41.0 / 46.7, 1120 49.5 / 48.7, 1280 56.9 /
 //     48.1, 1680 72.1 / 69.3; 66^2 64->128 880 29.6 / 29.7, 1280 35.4 / 32.0, 1520 39.1 / 40.2,
-//     1680 47.2 / 43.7; 66^2 384->128 720 36.5 / 36.9, 1280 69.7 / 44.6, 5120 248 / 112; 132^2
+//     1680 47.2 / 43.7 (64^2 1344 42.7 / 44.9); 66^2 384->128 720 36.5 / 36.9, 1280 69.7 / 44.6, 5120 248 / 112; 132^2
 //     64->64 864 22.2 / 19.7, 1584 35.6 / 26.9, 6048 115 / 73.7; 264^2 96->32 75.8 / 42.5 and
 //     132^2 192->64 92 / 53 at batches 2 and 4;
 //   the rest: the gather kernel (33-pixel rows, 16 images, gather / tap row: 128->256 39 / 57,

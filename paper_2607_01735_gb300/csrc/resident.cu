@@ -28,8 +28,8 @@
 // cooperative launch with a grid barrier per colour): FP64 127^2 1.1 us (3.9), 255^2 1.7 (4.0),
 // 511^2 3.4 (6.4), 1023^2 9.7 (14.1), 1190^2 12.9 (19.4); fused 255^2 1.3 us (4.4), 1023^2 4.3
 // (7.2 as wavefront passes); FP32 255^2 0.8 us (3.1), 511^2 1.2 (3.3), 1000^2 2.8 (3.9).  What
-// bounds it: from about 700^2 the FP64 pipe (74% of its rate at 1023^2, the shrinking margins
-// included), below the chain of a half-sweep and the exchange, about 1 us together.
+// bounds it: from about 700^2 the FP64 pipe (70% of its rate at 1023^2 by ncu, the shrinking
+// margins included), below the chain of a half-sweep and the exchange, about 1 us together.
 //
 // Three kinds of values, as in wavefront.cu: double (bit-exact FP64), float (inner sweeps of the
 // refinement) and int64 (the fused update on its block's fixed-point grid; the iterate is

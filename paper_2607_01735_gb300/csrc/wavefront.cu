@@ -33,8 +33,8 @@
 // multiple of P) and neighbouring strips overlap by 2H.  A segment that outputs rows [a, b)
 // starts 2K rows above a and runs 2K-1 rows past b.
 //
-// What bounds it (ncu, fused, K = 3, 8191^2): the integer ALU pipe, 72% busy, 31 warp
-// instructions per 32 updates (one launch per colour: 107), DRAM at 3.6 TB/s.  Measured, a
+// What bounds it (ncu, fused, K = 3, 8191^2): the integer ALU pipe, 74% busy, 30 warp
+// instructions per 32 updates (one launch per colour: 107), DRAM at 3.7 TB/s.  Measured, a
 // sweep: fused 16384^2 382 us = 702 GLUP/s (one launch per colour 1021 us, at 0.95 of the HBM
 // bandwidth); fused 4095^2 31 us (96), 1500^2 9.9 us (16.2); FP32 K = 4 8192^2 36.8 us = 1825
 // GLUP/s (46.7 with the ring of whole rows in registers that also moved the red values).
