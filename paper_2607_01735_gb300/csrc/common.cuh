@@ -85,7 +85,7 @@ struct ResidentState {
 
 // Internal status: a cooperative launch was refused (it does not fit the SMs that this process may
 // use); nothing has run, and the caller takes another path.
-constexpr rbgs_status kLaunchRefused = (rbgs_status)-1;
+constexpr rbgs_status kLaunchRefused = (rbgs_status)7;
 
 }  // namespace rbgs
 

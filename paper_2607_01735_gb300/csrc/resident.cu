@@ -276,12 +276,17 @@ struct Costs<int64_t> {
     static constexpr double warp = 117, chain = 590, exchange = 1550;
 };
 
-// The current device takes a cooperative launch of this kernel with one block on every SM.
+// The current device takes a cooperative launch of this kernel with one block on every SM.  The
+// shared-memory limit is raised for every context, not once per device: the plain launches that
+// this kernel replaced needed none, and a cudaDeviceReset takes it back.
 template <typename T>
 bool can_run() {
-    static PerDevice<cudaError_t> limit;
     static PerDevice<bool> fits;
-    if (raise_smem(limit, resident_kernel<T>, kSmemMax) != cudaSuccess) return false;
+    if (cudaFuncSetAttribute(resident_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) !=
+        cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
     return fits.get([] {
         int dev = 0, coop = 0, per_sm = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||

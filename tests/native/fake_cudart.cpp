@@ -25,7 +25,7 @@ std::map<void *, size_t> g_alloc;
 std::string g_log;
 thread_local int t_device = 0;
 thread_local cudaError_t t_last = cudaSuccess;
-int g_sms[4] = {152, 152, 152, 152};
+int g_sms[8] = {152, 152, 152, 152, 152, 152, 152, 152};
 int g_coop = 1;              // the device attribute
 int g_refuse = 0;            // cooperative launches fail as too large
 size_t g_in_use = 0, g_limit = (size_t)-1;
@@ -84,6 +84,11 @@ const char *fake_log() { return g_log.c_str(); }  // "kind kernel blocks device"
 void fake_set_device(int d) { t_device = d; }
 void fake_set_sms(int d, int n) { g_sms[d] = n; }
 void fake_cooperative(int attribute, int refuse) { g_coop = attribute, g_refuse = refuse; }
+void fake_device_reset() {  // of the current device: raised limits are gone
+    std::lock_guard<std::mutex> lock(g_m);
+    for (auto &e : g_smem_limit)
+        if (e.first.first == t_device) e.second = 48 * 1024;
+}
 void fake_memory_limit(size_t bytes) { g_limit = bytes; }
 size_t fake_memory_in_use() { return g_in_use; }
 

@@ -40,3 +40,5 @@ def test_forward_of_rows_beyond_32_bits():
                     if 0 <= yy < 2 and 0 <= xx < W:
                         ref += wd[:, ty, tx] @ x[0, yy, xx].double()
             assert float((y[0, r, c].double() - ref).abs().max()) <= 0.018, (r, c)
+    del x
+    torch.cuda.empty_cache()

@@ -36,6 +36,18 @@ def test_sweeps_run_on_a_second_device(lib, n, opts):
         c.close()
 
 
+@pytest.mark.parametrize("n,opts", [(127, {}), (1023, {}), (1023, {"fma": 1}), (1500, {"fma": 1})])
+def test_sweeps_run_after_a_device_reset(lib, n, opts):
+    lib.fake_set_device(4)  # used by no other test, whose kernels keep their raised limits
+    for _ in range(2):
+        c = Context(lib, n, **opts)
+        st, calls = c.sweep(40)
+        assert st == 0 and calls, lib.rbgs_last_error()
+        assert n > 1368 or _kinds(calls) <= {"cooperative", "plain"} and any("resident" in k for _, k, _, _ in calls)
+        c.close()
+        lib.fake_device_reset()
+
+
 def test_refined_solve_runs_on_a_second_device(lib):
     for device in (0, 1):
         lib.fake_set_device(device)
