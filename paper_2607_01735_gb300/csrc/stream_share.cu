@@ -45,12 +45,16 @@ public:
     }
     void add(int device, cudaStream_t s, double us) {
         const Clock::time_point now = Clock::now();
-        const auto time = std::chrono::duration_cast<Clock::duration>(std::chrono::duration<double, std::micro>(0.75 * us));
+        const double part = 0.75 * us;
+        const auto time = std::chrono::duration_cast<Clock::duration>(
+            std::chrono::duration<double, std::micro>(part < kMostUs ? part : kMostUs));
         std::lock_guard<std::mutex> lock(mutex_);
         for (int q = 0; q < used_; ++q) {
             Busy &e = busy_[q];
             if (e.device != device || e.stream != s) continue;
             e.until = (e.until > now ? e.until : now) + time;
+            const Clock::time_point most = now + std::chrono::microseconds((long long)kMostUs);
+            if (e.until > most) e.until = most;
             return;
         }
         if (used_ < kBusy) busy_[used_++] = Busy{device, s, now + time};
@@ -72,6 +76,7 @@ private:
         int device, count;
         Clock::time_point when;
     };
+    static constexpr double kMostUs = 1e11;  // a day: any sweep count stays within the clock's range
     static constexpr int kBusy = 64;  // past these the device is shared as finely as it gets
     static constexpr int kSeen = 32;  // launches, none older than 20 ms: twice 16 streams' bursts
     static constexpr std::chrono::milliseconds kSeenTime{20};
@@ -82,6 +87,16 @@ private:
     cudaStream_t last_stream_ = nullptr;
 };
 
+// A launch that is being captured runs later, if at all: it neither counts nor shares.
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &status) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return status != cudaStreamCaptureStatusNone;
+}
+
 BusyStreams &busy_streams() {
     static BusyStreams b;
     return b;
@@ -89,8 +104,10 @@ BusyStreams &busy_streams() {
 
 }  // namespace
 
-int streams_sharing(int device, cudaStream_t s) { return busy_streams().sharing(device, s); }
-void stream_busy(int device, cudaStream_t s, double us) { busy_streams().add(device, s, us); }
+int streams_sharing(int device, cudaStream_t s) { return capturing(s) ? 1 : busy_streams().sharing(device, s); }
+void stream_busy(int device, cudaStream_t s, double us) {
+    if (!capturing(s)) busy_streams().add(device, s, us);
+}
 void stream_idle(int device, cudaStream_t s) { busy_streams().idle(device, s); }
 
 }  // namespace rbgs

@@ -30,6 +30,7 @@ int g_coop = 1;              // the device attribute
 int g_refuse = 0;            // cooperative launches fail as too large
 size_t g_in_use = 0, g_limit = (size_t)-1;
 float g_elapsed = 1.0f;
+cudaStream_t g_capturing = (cudaStream_t)-1;  // a stream that a test says is being captured
 double g_host[4];            // first values of page-locked memory, where residuals are read
 struct Config {
     dim3 g, b;
@@ -78,10 +79,12 @@ void fake_reset() {
     g_coop = 1, g_refuse = 0, g_limit = (size_t)-1, g_elapsed = 1.0f;
     g_host[0] = g_host[1] = 1.0, g_host[2] = 0.5, g_host[3] = 0.0;  // rho = 1, max |rt| = 0.5, no status
     t_device = 0, t_last = cudaSuccess;
+    g_capturing = (cudaStream_t)-1;
 }
 void fake_clear_log() { std::lock_guard<std::mutex> lock(g_m); g_log.clear(); }
 const char *fake_log() { return g_log.c_str(); }  // "kind kernel blocks device" per line
 void fake_set_device(int d) { t_device = d; }
+void fake_capture(void *stream) { g_capturing = (cudaStream_t)stream; }
 void fake_set_sms(int d, int n) { g_sms[d] = n; }
 void fake_cooperative(int attribute, int refuse) { g_coop = attribute, g_refuse = refuse; }
 void fake_device_reset() {  // of the current device: raised limits are gone
@@ -193,7 +196,10 @@ cudaError_t cudaStreamDestroy(cudaStream_t s) { std::free(s); return cudaSuccess
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, enum cudaStreamCaptureMode) { return cudaSuccess; }
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g) { *g = (cudaGraph_t)std::malloc(1); return cudaSuccess; }
-cudaError_t cudaStreamIsCapturing(cudaStream_t, enum cudaStreamCaptureStatus *s) { *s = cudaStreamCaptureStatusNone; return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t st, enum cudaStreamCaptureStatus *s) {
+    *s = st == g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t *e, cudaGraph_t, unsigned long long) { *e = (cudaGraphExec_t)std::malloc(1); return cudaSuccess; }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) {
     std::lock_guard<std::mutex> lock(g_m);

@@ -170,6 +170,32 @@ def test_solvers_on_several_streams_share_the_device(lib, n, opts):
     same.close()
 
 
+def test_captured_launches_neither_share_nor_count(lib):
+    lib.fake_capture.argtypes = [ctypes.c_void_p]
+    lib.fake_set_device(5)
+    busy, caught, later = (Context(lib, 127, stream=q) for q in (401, 402, 403))
+    lib.fake_capture(402)
+    assert _tiles(caught.sweep(1000000)[1])[0] == 152
+    lib.fake_capture(2 ** 64 - 1)
+    assert _tiles(busy.sweep(1000000)[1])[0] == 152  # the captured launch is not at work
+    lib.fake_capture(402)
+    assert _tiles(caught.sweep(1000000)[1])[0] == 152  # and takes the plan it would take alone
+    lib.fake_capture(2 ** 64 - 1)
+    assert _tiles(later.sweep(20)[1])[0] <= 76
+    for c in (busy, caught, later):
+        c.close()
+
+
+def test_any_sweep_count_leaves_the_clock_in_range(lib):
+    lib.fake_set_device(5)
+    a, b = Context(lib, 127, stream=501), Context(lib, 127, stream=502)
+    for k in (2 ** 62, 2 ** 62, 5):
+        assert a.sweep(k)[0] == 0
+    assert _tiles(b.sweep(20)[1])[0] <= 76  # still counted as busy
+    a.close()
+    b.close()
+
+
 # ------------------------------------------------------------------ single sweeps
 @pytest.mark.parametrize("n,kernels", [(255, ["half_sweep"] * 2), (511, ["persistent_sweeps"]),
                                        (1023, ["persistent_sweeps"]), (4095, ["persistent_sweeps"])])
