@@ -27,13 +27,15 @@ constexpr int kT = 256;
 // assemble 70).  The interpolant is (1-x) n_j + x s_j + (1-y) W_i + y E_i with, per column,
 //   n_j = N_j - ((1-y) c00 + y c01),  s_j = S_j - ((1-y) c10 + y c11):
 // four operations per point, the column's terms once per thread and the row's once per block
-// (input 25 us, assemble 22).
+// (input 25 us, assemble 22).  Small grids take fewer rows per block (walk_rows): with 16 a call at
+// 31^2 or 127^2 took 8.2 (blend) and 10.3 us (the others), now 5.2 to 6.2 (6.2 by one thread per point).
 constexpr int kCols = 128, kRows = 16;
 
 // body(i, j, in, c) for every point of a rows x cols output: c is the interpolant of the g^2
 // grid's ring there, `in` whether the point lies on the grid (c is 0 off it).
 template <class Body>
-__device__ __forceinline__ void walk_coons(const double *__restrict__ u, int g, int rows, int cols, Body body) {
+__device__ __forceinline__ void walk_coons(const double *__restrict__ u, int g, int rows, int cols, int per,
+                                           Body body) {
     __shared__ double row_x[kRows], row_w[kRows], row_e[kRows];
     const int j = blockIdx.x * kCols + threadIdx.x;
     const double *south = u + (size_t)(g - 1) * g;
@@ -43,9 +45,9 @@ __device__ __forceinline__ void walk_coons(const double *__restrict__ u, int g, 
         nj = u[j] - ((1.0 - y) * u[0] + y * u[g - 1]);
         sj = south[j] - ((1.0 - y) * south[0] + y * south[g - 1]);
     }
-    for (int i0 = blockIdx.y * kRows; i0 < rows; i0 += gridDim.y * kRows) {
+    for (int i0 = blockIdx.y * per; i0 < rows; i0 += gridDim.y * per) {
         __syncthreads();
-        if (threadIdx.x < kRows) {
+        if ((int)threadIdx.x < per) {
             const int i = i0 + threadIdx.x;
             row_x[threadIdx.x] = (double)i / (double)(g - 1);
             row_w[threadIdx.x] = i < g ? u[(size_t)i * g] : 0.0;
@@ -56,7 +58,7 @@ __device__ __forceinline__ void walk_coons(const double *__restrict__ u, int g, 
 #pragma unroll 4
         for (int r = 0; r < kRows; ++r) {
             const int i = i0 + r;
-            if (i >= rows) break;
+            if (r >= per || i >= rows) break;
             const bool in = i < g && j < g;
             const double x = row_x[r];
             // fused explicitly, so that every kernel rounds alike
@@ -67,20 +69,28 @@ __device__ __forceinline__ void walk_coons(const double *__restrict__ u, int g, 
     }
 }
 
+// Rows per block: kRows, fewer on grids that would leave the GPU with less than about a block per SM
+// (a thread walks its rows one after another).
+int walk_rows(int rows, int cols) {
+    const long per = (long)rows * ((cols + kCols - 1) / kCols) / 152;
+    return (int)(per < 1 ? 1 : per > kRows ? kRows : per);
+}
+
 dim3 walk_grid(int rows, int cols) {
-    const int y = (rows + kRows - 1) / kRows;
+    const int per = walk_rows(rows, cols), y = (rows + per - 1) / per;
     return dim3((unsigned)((cols + kCols - 1) / kCols), (unsigned)(y < 65535 ? y : 65535));
 }
 
-__global__ void __launch_bounds__(kCols) blend_kernel(const double *__restrict__ u, int g, double *__restrict__ out) {
-    walk_coons(u, g, g, g, [=](int i, int j, bool, double c) { out[(size_t)i * g + j] = c; });
+__global__ void __launch_bounds__(kCols) blend_kernel(const double *__restrict__ u, int g, int per,
+                                                      double *__restrict__ out) {
+    walk_coons(u, g, g, g, per, [=](int i, int j, bool, double c) { out[(size_t)i * g + j] = c; });
 }
 
 // x[(i*size + j)*4 + c]: f (interior), ring mask, ring values, the blend; zero off the grid
 __global__ void __launch_bounds__(kCols) input_kernel(const double *__restrict__ f, const double *__restrict__ u, int n,
-                                                      int size, float *__restrict__ x) {
+                                                      int size, int per, float *__restrict__ x) {
     const int g = n + 2;
-    walk_coons(u, g, size, size, [=](int i, int j, bool in, double c) {
+    walk_coons(u, g, size, size, per, [=](int i, int j, bool in, double c) {
         const bool ring = i == 0 || j == 0 || i == g - 1 || j == g - 1;
         float4 v = make_float4(0.f, 0.f, 0.f, (float)c);
         if (in && !ring) v.x = (float)f[(size_t)(i - 1) * n + (j - 1)];
@@ -91,18 +101,18 @@ __global__ void __launch_bounds__(kCols) input_kernel(const double *__restrict__
 
 // t = sol - blend on the (n+2)^2 grid, 0 elsewhere on the size^2 grid
 __global__ void __launch_bounds__(kCols) target_kernel(const double *__restrict__ sol, const double *__restrict__ u,
-                                                       int n, int size, float *__restrict__ t) {
+                                                       int n, int size, int per, float *__restrict__ t) {
     const int g = n + 2;
-    walk_coons(u, g, size, size, [=](int i, int j, bool in, double c) {
+    walk_coons(u, g, size, size, per, [=](int i, int j, bool in, double c) {
         t[(size_t)i * size + j] = in ? (float)(sol[(size_t)i * g + j] - c) : 0.f;
     });
 }
 
 // u0: the ring of u; interior = blend + pred (pred on the size^2 grid)
 __global__ void __launch_bounds__(kCols) assemble_kernel(const double *__restrict__ u, const float *__restrict__ pred,
-                                                         int n, int size, double *__restrict__ u0) {
+                                                         int n, int size, int per, double *__restrict__ u0) {
     const int g = n + 2;
-    walk_coons(u, g, g, g, [=](int i, int j, bool, double c) {
+    walk_coons(u, g, g, g, per, [=](int i, int j, bool, double c) {
         const bool ring = i == 0 || j == 0 || i == g - 1 || j == g - 1;
         const size_t q = (size_t)i * g + j;
         u0[q] = ring ? u[q] : c + (double)pred[(size_t)i * size + j];
@@ -178,7 +188,7 @@ rbgs_status rbgs_guess_blend(const double *u_ring, int n, double *out, void *cud
         return RBGS_EINVAL;
     }
     const int g = n + 2;
-    blend_kernel<<<walk_grid(g, g), kCols, 0, (cudaStream_t)cuda_stream>>>(u_ring, g, out);
+    blend_kernel<<<walk_grid(g, g), kCols, 0, (cudaStream_t)cuda_stream>>>(u_ring, g, walk_rows(g, g), out);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
@@ -189,7 +199,8 @@ rbgs_status rbgs_guess_input(const double *f, const double *u_ring, int n, int s
         set_error("rbgs_guess_input: n >= 1, size >= n + 2 and a multiple of 8, device buffers required");
         return RBGS_EINVAL;
     }
-    input_kernel<<<walk_grid(size, size), kCols, 0, (cudaStream_t)cuda_stream>>>(f, u_ring, n, size, x);
+    input_kernel<<<walk_grid(size, size), kCols, 0, (cudaStream_t)cuda_stream>>>(f, u_ring, n, size,
+                                                                                 walk_rows(size, size), x);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
@@ -201,7 +212,8 @@ rbgs_status rbgs_guess_target(const double *sol, const double *u_ring, int n, in
         set_error("rbgs_guess_target: n >= 1, size >= n + 2, device buffers required");
         return RBGS_EINVAL;
     }
-    target_kernel<<<walk_grid(size, size), kCols, 0, (cudaStream_t)cuda_stream>>>(sol, u_ring, n, size, t);
+    target_kernel<<<walk_grid(size, size), kCols, 0, (cudaStream_t)cuda_stream>>>(sol, u_ring, n, size,
+                                                                                  walk_rows(size, size), t);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
@@ -214,7 +226,8 @@ rbgs_status rbgs_guess_assemble(const double *u_ring, const float *pred, int n, 
         return RBGS_EINVAL;
     }
     const int g = n + 2;
-    assemble_kernel<<<walk_grid(g, g), kCols, 0, (cudaStream_t)cuda_stream>>>(u_ring, pred, n, size, u0);
+    assemble_kernel<<<walk_grid(g, g), kCols, 0, (cudaStream_t)cuda_stream>>>(u_ring, pred, n, size, walk_rows(g, g),
+                                                                              u0);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
