@@ -386,7 +386,10 @@ rbgs_status run_pass(WfArgs<T> &a, int parts, cudaStream_t s) {
     // segments, by a factor between the two costs: 16384^2 fused, factor 1 / 1.7 / 2.2 / 2.8 /
     // 4: 613 / 424 / 395 / 382 / 412 us a sweep; 8192^2 FP32, 1 / 1.5 / 2.5 / 4: 53.4 / 41.5 /
     // 36.8 / 40.2 us.
-    constexpr double edge_cost = std::is_same<T, float>::value ? 2.5 : 2.75;
+    // In FP64 the adds take most of a step, and the factor is 1.3 (40 sweeps of depth 2 / 4, ms, by 1 /
+    // 1.3 / 1.6 / 2.75: 2047^2 1.98 / 1.98 / 2.12 / 2.27 and 2.35 / 2.43 / 2.43 / 2.57, 3000^2 3.52 / 3.53 /
+    // 3.52 / 3.85 and 4.03 / 3.87 / 3.99 / 4.17, 8191^2 20.4 / 20.2 / 20.2 / 20.8 and 23.7 / 22.2 / 22.4 / 23.1).
+    constexpr double edge_cost = std::is_same<T, float>::value ? 2.5 : std::is_same<T, double>::value ? 1.3 : 2.75;
     auto even = [&](double h) {
         long v = (long)std::ceil(h);
         v = v < kWfMinRows ? kWfMinRows : v > rows ? rows : v;
