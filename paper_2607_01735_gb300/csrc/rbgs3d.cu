@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <cmath>
 #include <new>
+#include <type_traits>
 
 #include "../../include/rbgs3d.h"
 #include "common.cuh"
@@ -160,17 +161,38 @@ half_sweep3_kernel(double *__restrict__ self, const double *__restrict__ other, 
     }
 }
 
-// Per-block sums of rt^2 over the interior points of colour C, the same walk as a half-sweep
+// Both colours' arrays of a reduction.
+struct Fields3 {
+    const double *u[2], *hf[2];
+};
+
+// The colour that a block of a reduction walks, its number among the colour's blocks and how many
+// these are.  C 0, 1: all blocks; kBoth: the first half of the blocks red, the others black.
+constexpr int kBoth = 2;
+struct Share3 {
+    int colour, block, blocks;
+};
+template <int C>
+__device__ __forceinline__ Share3 share3() {
+    if (C != kBoth) return Share3{C, (int)blockIdx.x, (int)gridDim.x};
+    const int half = gridDim.x >> 1, c = (int)blockIdx.x >= half ? 1 : 0;
+    return Share3{c, (int)blockIdx.x - c * half, half};
+}
+
+// Per-block sums of rt^2 over the interior points of a colour, the same walk as a half-sweep
 // (places and chunks of planes as a grid-stride loop over `tasks` = x_blocks * chunks).
 template <int C>
 __global__ void __launch_bounds__(kThreads3)
-residual3_kernel(const double *__restrict__ self, const double *__restrict__ other, const double *__restrict__ hf,
-                 int n, int W, Pairs3 npairs, int chunk, int x_blocks, int tasks, double one,
+residual3_kernel(const Fields3 fld, int n, int W, Pairs3 npairs, int chunk, int x_blocks, int tasks, double one,
                  double *__restrict__ partials) {
     __shared__ double smem[kThreads3 / 32];
+    const Share3 sh = share3<C>();
+    const int colour = sh.colour;
+    const double *__restrict__ self = colour ? fld.u[1] : fld.u[0], *__restrict__ other = colour ? fld.u[0] : fld.u[1];
+    const double *__restrict__ hf = colour ? fld.hf[1] : fld.hf[0];
     const size_t plane = (size_t)(n + 2) * W;
     double acc = 0.0;
-    for (int task = blockIdx.x; task < tasks; task += gridDim.x) {
+    for (int task = sh.block; task < tasks; task += sh.blocks) {
         const Place3 pl = place3(task % x_blocks, n, npairs);
         if (!pl.act) continue;
         const int i0 = 1 + task / x_blocks * chunk, i1 = min(n, i0 + chunk - 1);
@@ -180,7 +202,7 @@ residual3_kernel(const double *__restrict__ self, const double *__restrict__ oth
             const double2 vs = ldg2(other + at + plane);
             const double2 vw = ldg2(other + at - W), ve = ldg2(other + at + W);
             const double2 f2 = ldg2(hf + at), me = ldg2(self + at);
-            const int p = (i + pl.j + C) & 1;
+            const int p = (i + pl.j + colour) & 1;
             const bool in = p ? pl.m0 + 2 < W : pl.m0 > 0;
             const double x = in ? __ldg(other + at + (p ? 2 : -1)) : 0.0;
             double s0 = add_fma(add_fma(add_fma(add_fma(f2.x, vn.x, one), vs.x, one), vw.x, one), ve.x, one);
@@ -199,21 +221,24 @@ residual3_kernel(const double *__restrict__ self, const double *__restrict__ oth
     if (threadIdx.x == 0) partials[blockIdx.x] = t;
 }
 
-// Per-block sums of (h^2 b)^2 over the interior points of colour C: h2 f plus, in N, S, W, E, D,
+// Per-block sums of (h^2 b)^2 over the interior points of a colour: h2 f plus, in N, S, W, E, D,
 // U order, the neighbours on the shell.  The same walk and the same order of additions as
 // residual3_kernel, so rho is exactly 1 for u = 0 inside and on the shell.  Only points next
 // to the shell read u; everywhere else b is h2 f and the walk streams it.
 template <int C>
 __global__ void __launch_bounds__(kThreads3)
-norm3_kernel(const double *__restrict__ other, const double *__restrict__ hf, int n, int W, Pairs3 npairs, int chunk,
-             int x_blocks, int tasks, double *__restrict__ partials) {
+norm3_kernel(const Fields3 fld, int n, int W, Pairs3 npairs, int chunk, int x_blocks, int tasks,
+             double *__restrict__ partials) {
     __shared__ double smem[kThreads3 / 32];
+    const Share3 sh = share3<C>();
+    const int colour = sh.colour;
+    const double *__restrict__ other = colour ? fld.u[0] : fld.u[1], *__restrict__ hf = colour ? fld.hf[1] : fld.hf[0];
     const int L = n + 2;
     const size_t plane = (size_t)L * W;
-    // a shell neighbour of a point of colour C has the other colour
+    // a shell neighbour of a point has the other colour
     auto shell = [&](int i, int j, int k) { return other[((size_t)i * L + j) * W + (k >> 1)]; };
     double acc = 0.0;
-    for (int task = blockIdx.x; task < tasks; task += gridDim.x) {
+    for (int task = sh.block; task < tasks; task += sh.blocks) {
         const Place3 pl = place3(task % x_blocks, n, npairs);
         if (!pl.act) continue;
         const int j = pl.j, i0 = 1 + task / x_blocks * chunk, i1 = min(n, i0 + chunk - 1);
@@ -232,7 +257,7 @@ norm3_kernel(const double *__restrict__ other, const double *__restrict__ hf, in
         }
         for (; i <= i1; ++i, row += plane) {
             const double2 f2 = ldg2(row);
-            const int k0 = 2 * pl.m0 + ((i + j + C) & 1);
+            const int k0 = 2 * pl.m0 + ((i + j + colour) & 1);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const int k = k0 + 2 * q;
@@ -319,34 +344,43 @@ Walk3 walk3(int n) {
     return w;
 }
 
-// sum rt^2 into dsum[0] (stream-ordered)
-rbgs_status enqueue_residual3(rbgs3d_ctx *c) {
+// Runs a reduction over both colours and adds its partials, red ones first: one launch for both
+// where the blocks of both run at once (a residual of 7^3 / 33^3 / 63^3 / 64^3 takes 24.6 / 25.9 /
+// 28.7 / 27.9 us, with a launch per colour 27.9 / 27.6 / 37.9 / 32.0), else one per colour, whose
+// parity is then a constant (95^3 52, 300^3 524 us).
+template <class Launch>
+rbgs_status reduce3(rbgs3d_ctx *c, double *out, Launch launch) {
     const Walk3 w = walk3(c->n);
     const int tasks = w.x_blocks * w.chunks, blocks = std::min(tasks, kBlocks3);
-    residual3_kernel<0><<<blocks, kThreads3, 0, c->stream>>>(c->u[0], c->u[1], c->hf[0], c->n, c->W, w.npairs, w.chunk,
-                                                             w.x_blocks, tasks, 1.0, c->partials);
+    const Fields3 fld{{c->u[0], c->u[1]}, {c->hf[0], c->hf[1]}};
+    if (2 * blocks <= grid_for((size_t)1 << 40)) {
+        launch(std::integral_constant<int, kBoth>(), 2 * blocks, fld, w, tasks, c->partials);
+    } else {
+        launch(std::integral_constant<int, 0>(), blocks, fld, w, tasks, c->partials);
+        RBGS_LAUNCH_CHECK();
+        launch(std::integral_constant<int, 1>(), blocks, fld, w, tasks, c->partials + blocks);
+    }
     RBGS_LAUNCH_CHECK();
-    residual3_kernel<1><<<blocks, kThreads3, 0, c->stream>>>(c->u[1], c->u[0], c->hf[1], c->n, c->W, w.npairs, w.chunk,
-                                                             w.x_blocks, tasks, 1.0, c->partials + blocks);
-    RBGS_LAUNCH_CHECK();
-    final3_kernel<<<1, kThreads3, 0, c->stream>>>(c->partials, 2 * blocks, c->dsum);
+    final3_kernel<<<1, kThreads3, 0, c->stream>>>(c->partials, 2 * blocks, out);
     RBGS_LAUNCH_CHECK();
     return RBGS_OK;
 }
 
+// sum rt^2 into dsum[0] (stream-ordered)
+rbgs_status enqueue_residual3(rbgs3d_ctx *c) {
+    return reduce3(c, c->dsum, [c](auto C, int blocks, const Fields3 &fld, const Walk3 &w, int tasks, double *partials) {
+        residual3_kernel<decltype(C)::value><<<blocks, kThreads3, 0, c->stream>>>(fld, c->n, c->W, w.npairs, w.chunk,
+                                                                                  w.x_blocks, tasks, 1.0, partials);
+    });
+}
+
 // sum (h^2 b)^2 into dsum[1] (stream-ordered)
 rbgs_status enqueue_norm3(rbgs3d_ctx *c) {
-    const Walk3 w = walk3(c->n);
-    const int tasks = w.x_blocks * w.chunks, blocks = std::min(tasks, kBlocks3);
-    norm3_kernel<0><<<blocks, kThreads3, 0, c->stream>>>(c->u[1], c->hf[0], c->n, c->W, w.npairs, w.chunk, w.x_blocks,
-                                                         tasks, c->partials);
-    RBGS_LAUNCH_CHECK();
-    norm3_kernel<1><<<blocks, kThreads3, 0, c->stream>>>(c->u[0], c->hf[1], c->n, c->W, w.npairs, w.chunk, w.x_blocks,
-                                                         tasks, c->partials + blocks);
-    RBGS_LAUNCH_CHECK();
-    final3_kernel<<<1, kThreads3, 0, c->stream>>>(c->partials, 2 * blocks, c->dsum + 1);
-    RBGS_LAUNCH_CHECK();
-    return RBGS_OK;
+    return reduce3(c, c->dsum + 1, [c](auto C, int blocks, const Fields3 &fld, const Walk3 &w, int tasks,
+                                       double *partials) {
+        norm3_kernel<decltype(C)::value><<<blocks, kThreads3, 0, c->stream>>>(fld, c->n, c->W, w.npairs, w.chunk,
+                                                                              w.x_blocks, tasks, partials);
+    });
 }
 
 }  // namespace

@@ -49,6 +49,18 @@ def test_3d_bit_exact_against_oracle(n):
     assert abs(rho - want) <= max(1e-12, n ** 3 * 2.0 ** -53) * want
 
 
+@pytest.mark.parametrize("n", [80, 81, 82, 83, 84, 85])
+def test_3d_reductions_on_either_side_of_the_one_launch_rule(n):
+    """rho's two sums, both colours in one launch up to about 81^3 and one launch each from there:
+    n^3 terms in any order, so n^3 roundings of 2^-53 at most."""
+    f, u0 = _random3(n, 7 * n)
+    h2 = 1.0 / (n + 1) ** 2
+    with rb.Solver3D(n, h2, torch.from_numpy(f).cuda(), torch.from_numpy(u0).cuda()) as s:
+        rho = s.residual()
+    want = oracle.residual3d(u0, f, h2)[0]
+    assert abs(rho - want) <= n ** 3 * 2.0 ** -53 * want
+
+
 def test_3d_host_buffers_and_manufactured_history():
     n = 31
     f, phi, h = _manufactured(n)
